@@ -17,10 +17,10 @@
 //                cache bytes it streams.
 //   attn_encoder one block per (sentence, head, chunk of 4..32 queries): K and V of
 //                the head staged in shared memory, keys masked past the
-//                source length.
-//   attn_encoder_mma  the same on the int8 tensor cores (mma.sync, exact int32)
-//                for d_h = 64 and up to 256 keys: scores as one product, the
-//                weights split into bytes for the context products.
+//                source length (small grids, and d_h = 128).
+//   attn_encoder_tc  the same for d_h = 32 and 64 on the tensor cores (mma.sync
+//                on fp16 integers, exact): one block per (sentence, head,
+//                16..64 queries).
 #include <type_traits>
 
 #include "common.cuh"
@@ -34,6 +34,11 @@ constexpr int DEC_MAX_KEYS = 1024;
 MNMT_DEV uint32_t vec_word(uint32_t v, int) { return v; }
 MNMT_DEV uint32_t vec_word(const uint2 &v, int k) { return k ? v.y : v.x; }
 MNMT_DEV uint32_t vec_word(const uint4 &v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
+
+// the exact form of a context code (q8_context's undecided values)
+__device__ __noinline__ float att_ctx_exact(long long n, long long z, float rho) {
+    return (float)q8(rn32_div(n, z), rho);
+}
 
 // XS = false: one block per row, one warp per head.  XS = true (cross
 // attention with beams): one block per sentence, one warp per (beam, head) --
@@ -264,10 +269,12 @@ __global__ void __launch_bounds__(32 * ENC_WARPS) attn_encoder(AttnEncArgs a, in
             }
         }
         const size_t o = ((size_t)b * S + qi) * a.d + h * DH + lane * EPL;
+        const float iz = __frcp_rn(__ll2float_rn(Z));
 #pragma unroll
         for (int u = 0; u < EPL; u++) {
-            long long N = (long long)hi[u] * 4096 + lo[u];
-            const int8_t v = q8_quotient(N, Z, a.rho, rn32_div);
+            const int8_t v = q8_context_hl(hi[u], lo[u], iz, a.rho, [&]() {
+                return att_ctx_exact((long long)hi[u] * 4096 + lo[u], Z, a.rho);
+            });
             a.ctx[o + u] = v;
             if (a.ctx16) a.ctx16[o + u] = __short2half_rn(v);
         }
@@ -276,124 +283,121 @@ __global__ void __launch_bounds__(32 * ENC_WARPS) attn_encoder(AttnEncArgs a, in
 }
 
 // ---------------------------------------------------------------------------
-// encoder self-attention on the int8 tensor cores (mma.sync m16n8k32, exact
-// int32 accumulation), d_h = 64 and up to 256 keys.  Same arithmetic as
-// attn_encoder: the scores q . k_j are the same exact integers; the weights E_j
-// in [0, 2^24] are split into four bytes E_j = sum_k e_kj 2^(8k), each byte a
-// u8 operand of its own product with V (sum_j e_kj v_j[e] <= 256 * 255 * 128 <
-// 2^31: exact), and N_e = sum_k 2^(8k) (sum_j e_kj v_j[e]) is rebuilt in int64.
+// encoder self-attention on the tensor cores (mma.sync m16n8k16, fp16 operands,
+// fp32 accumulation), d_h = 32 or 64.  Same integers as attn_encoder: codes and
+// weight pieces are fp16 integers, and every sum stays within 2^24, so fp32
+// holds it exactly in any order.
+//   scores   q . k_j: 64 products of at most 2^14.
+//   context  E_j in [0, 2^24] is split into bytes, E_j = e0 + 2^8 e1 + 2^16 e2
+//            with e2 <= 256; each sum_j e_kj v_j[e] is at most
+//            512 * 256 * 128 = 2^24.
+// The fp16 form is used because the int8 one is slow on this part: mma.sync s8
+// measures 542 operations per clock and SM, f16 2048.
 //
-// One block per (sentence, head, 64 queries), four warps of 16 queries each.
-// Shared memory: Q [64][64] and K [Sp][64] in 64-byte rows, V^T [64][Sp], and
-// per warp the weight bytes [4][16][Sp] (Sp = key count padded to a power of
-// two >= 32), 16-byte chunks XOR-swizzled by row so that ldmatrix phases hit
-// distinct bank groups.  Keys past the source length score -inf (weight 0).
+// One block of four warps per (sentence, head, 16 NW queries): all stage, NW
+// compute, 16 queries each.  K and V are staged once per block as fp16 rows of 2 DH bytes, 16-byte chunks
+// XOR-swizzled by row (ldmatrix without bank conflicts; .trans for V).  The
+// scores are computed twice, for the row maximum and for the weights, which
+// keeps them out of registers; the weights' accumulator fragments are the
+// A fragments of the context products, so they never leave the registers.
+// Bound by issue slots (exp and the byte split), then the tensor pipe.
+// 64 x 100 tokens, 8 heads of 64: 101 us as four int8 products with the weight
+// bytes in shared memory, 31 us so (ncu, cold).
 // ---------------------------------------------------------------------------
-constexpr int ENC_MMA_WARPS = 4;
-
 MNMT_DEV uint32_t att_smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 MNMT_DEV void att_ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
 }
-MNMT_DEV void att_mma_s8(int (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+MNMT_DEV void att_ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
 }
-MNMT_DEV void att_mma_u8s8(int (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// byte offset of (row, 16-byte chunk) in 64-byte rows: chunk ^ (row / 2) % 4
-MNMT_DEV int sw64(int row, int chunk) { return row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4); }
-// byte offset of (row, byte col) in rows of `len` bytes (len = 16 * nch, nch a
-// power of two): chunk ^ (row mod min(nch, 8))
-MNMT_DEV int swl(int row, int col, int len, int msk) {
-    return row * len + ((((col >> 4) ^ (row & msk))) << 4) + (col & 15);
+// byte offset of (row, 16-byte chunk) in rows of 2 DH bytes
+template <int DH>
+MNMT_DEV int att_sw(int row, int chunk) {
+    return DH == 64 ? row * 128 + ((chunk ^ (row & 7)) << 4) : row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4);
 }
 
-__global__ void __launch_bounds__(32 * ENC_MMA_WARPS) attn_encoder_mma(AttnEncArgs a, int Sp) {
+constexpr int ENC_TC_THREADS = 128;
+constexpr long ENC_TC_MIN_TILES = 192;
+
+template <int DH, int NW>
+__global__ void __launch_bounds__(ENC_TC_THREADS) attn_encoder_tc(AttnEncArgs a, int Sp) {
     pdl_grid_wait();
     extern __shared__ __align__(128) uint8_t emm[];
-    constexpr int DH = 64;
+    constexpr int CH = DH / 16;        // 16-code chunks of an int8 row
+    constexpr int KS = DH / 16;        // k-steps of the score product
+    constexpr int NT = DH / 8;         // 8-column tiles of the context
+    constexpr int RB = 2 * DH;         // bytes of an fp16 row
     const int bh = blockIdx.x;
     const int b = bh / a.H, h = bh - b * a.H;
     const int S = a.S;
     int len = a.len[b];
-    len = len < 1 ? 1 : (len > S ? S : len);
-    const int q0 = blockIdx.y * 64;
-    const int nch = Sp >> 4, msk = (nch < 8 ? nch : 8) - 1;
-    uint8_t *Qs = emm;                       // [64][64]
-    uint8_t *Ks = Qs + 64 * 64;              // [Sp][64]
-    uint8_t *Vt = Ks + (size_t)Sp * 64;      // [64][Sp]
-    uint8_t *Es = Vt + (size_t)64 * Sp;      // [warps][4][16][Sp]; first V row-major [Sp][64]
+    len = len < 1 ? 1 : (len > S ? S : len);  // validated on the host path; clamp on the device path
+    const int lp = (len + 15) & ~15;          // keys the products run over
+    const int q0 = blockIdx.y * (16 * NW);
+    uint8_t *Qs = emm;                         // [16 NW][DH] fp16, then the output rows
+    uint8_t *Ks = Qs + 16 * NW * RB;           // [Sp][DH] fp16
+    uint8_t *Vs = Ks + (size_t)Sp * RB;        // [Sp][DH] fp16
     const int ld = 3 * a.d;
-    const int8_t *base = a.qkv + (size_t)b * S * ld;
-    // stage Q (64 queries), K and V (valid keys; the rest zero)
-    for (int i = threadIdx.x; i < 64 * 4; i += blockDim.x) {
-        const int r = i >> 2, c = i & 3, q = q0 + r;
-        int4 v = make_int4(0, 0, 0, 0);
-        if (q < S) v = reinterpret_cast<const int4 *>(base + (size_t)q * ld + h * DH)[c];
-        *reinterpret_cast<int4 *>(Qs + sw64(r, c)) = v;
+    const int8_t *base = a.qkv + (size_t)b * S * ld + h * DH;
+    auto put16 = [&](uint8_t *rows, int r, int c, const int4 v) {
+        uint32_t o[8];
+        codes_to_half2(v.x, o[0], o[1]);
+        codes_to_half2(v.y, o[2], o[3]);
+        codes_to_half2(v.z, o[4], o[5]);
+        codes_to_half2(v.w, o[6], o[7]);
+        *reinterpret_cast<uint4 *>(rows + att_sw<DH>(r, 2 * c)) = make_uint4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<uint4 *>(rows + att_sw<DH>(r, 2 * c + 1)) = make_uint4(o[4], o[5], o[6], o[7]);
+    };
+    const int4 zero = make_int4(0, 0, 0, 0);
+    for (int i = threadIdx.x; i < 16 * NW * CH; i += ENC_TC_THREADS) {
+        const int r = i / CH, c = i % CH, q = q0 + r;
+        put16(Qs, r, c, q < S ? reinterpret_cast<const int4 *>(base + (size_t)q * ld)[c] : zero);
     }
-    for (int i = threadIdx.x; i < Sp * 4; i += blockDim.x) {
-        const int j = i >> 2, c = i & 3;
-        int4 kv = make_int4(0, 0, 0, 0), vv = make_int4(0, 0, 0, 0);
+#pragma unroll 2
+    for (int i = threadIdx.x; i < lp * CH; i += ENC_TC_THREADS) {
+        const int j = i / CH, c = i % CH;
+        int4 kv = zero, vv = zero;
         if (j < len) {
-            kv = reinterpret_cast<const int4 *>(base + (size_t)j * ld + a.d + h * DH)[c];
-            vv = reinterpret_cast<const int4 *>(base + (size_t)j * ld + 2 * a.d + h * DH)[c];
+            kv = reinterpret_cast<const int4 *>(base + (size_t)j * ld + a.d)[c];
+            vv = reinterpret_cast<const int4 *>(base + (size_t)j * ld + 2 * a.d)[c];
         }
-        *reinterpret_cast<int4 *>(Ks + sw64(j, c)) = kv;
-        reinterpret_cast<int4 *>(Es + (size_t)j * DH)[c] = vv;
-    }
-    __syncthreads();
-    // V^T: word (e, keys 4w .. 4w + 3) from four rows of V
-    for (int i = threadIdx.x; i < DH * (Sp >> 2); i += blockDim.x) {
-        const int e = i & (DH - 1), j = 4 * (i >> 6);
-        const uint32_t x = (uint32_t)Es[(size_t)j * DH + e] | ((uint32_t)Es[(size_t)(j + 1) * DH + e] << 8) |
-                           ((uint32_t)Es[(size_t)(j + 2) * DH + e] << 16) |
-                           ((uint32_t)Es[(size_t)(j + 3) * DH + e] << 24);
-        *reinterpret_cast<uint32_t *>(Vt + swl(e, j, Sp, msk)) = x;
+        put16(Ks, j, c, kv);
+        put16(Vs, j, c, vv);
     }
     __syncthreads();
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp >= NW || q0 + warp * 16 >= S) return;
     const int jq = lane >> 3, i8 = lane & 7, g = lane >> 2, tq = lane & 3;
-    uint8_t *Ew = Es + (size_t)warp * 4 * 16 * Sp;
-    // Q fragments of this warp's 16 queries (two k-steps of 32)
-    uint32_t af[2][4];
+    uint32_t af[KS][4];
 #pragma unroll
-    for (int kk = 0; kk < 2; kk++)
-        att_ldmatrix_x4(af[kk], att_smem_u32(Qs + sw64(warp * 16 + (jq & 1) * 8 + i8, kk * 2 + (jq >> 1))));
-    // scores of 16 keys (two n-tiles) per call: exact int32, then fl(acc sigma),
-    // -inf past the source length
+    for (int kk = 0; kk < KS; kk++)
+        att_ldmatrix_x4(af[kk], att_smem_u32(Qs + att_sw<DH>(warp * 16 + (jq & 1) * 8 + i8, kk * 2 + (jq >> 1))));
+    // scores of 16 keys: exact integers, then fl(acc sigma), -inf past the source length
     auto scores16 = [&](int k0, float (&sv)[2][4]) {
-        int acc[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
-        for (int kk = 0; kk < 2; kk++) {
+        for (int kk = 0; kk < KS; kk++) {
             uint32_t r[4];
-            att_ldmatrix_x4(r, att_smem_u32(Ks + sw64(k0 + (jq >> 1) * 8 + i8, kk * 2 + (jq & 1))));
-            att_mma_s8(acc[0], af[kk], r[0], r[1]);
-            att_mma_s8(acc[1], af[kk], r[2], r[3]);
+            att_ldmatrix_x4(r, att_smem_u32(Ks + att_sw<DH>(k0 + (jq >> 1) * 8 + i8, kk * 2 + (jq & 1))));
+            mma_f16_16816(acc[0], af[kk], r[0], r[1]);
+            mma_f16_16816(acc[1], af[kk], r[2], r[3]);
         }
 #pragma unroll
         for (int t = 0; t < 2; t++)
 #pragma unroll
             for (int q = 0; q < 4; q++) {
                 const int key = k0 + t * 8 + tq * 2 + (q & 1);
-                sv[t][q] = key < len ? __fmul_rn(__int2float_rn(acc[t][q]), a.sigma) : -INFINITY;
+                sv[t][q] = key < len ? __fmul_rn(acc[t][q], a.sigma) : -INFINITY;
             }
     };
-    // pass 1: each row's maximum score
     float mx0 = -INFINITY, mx1 = -INFINITY;  // rows g and g + 8
-    for (int k0 = 0; k0 < Sp; k0 += 16) {
+    for (int k0 = 0; k0 < lp; k0 += 16) {
         float sv[2][4];
         scores16(k0, sv);
 #pragma unroll
@@ -407,86 +411,100 @@ __global__ void __launch_bounds__(32 * ENC_MMA_WARPS) attn_encoder_mma(AttnEncAr
         mx0 = fmaxf(mx0, __shfl_xor_sync(0xFFFFFFFFu, mx0, o));
         mx1 = fmaxf(mx1, __shfl_xor_sync(0xFFFFFFFFu, mx1, o));
     }
-    // pass 2: weights E (the scores again), their bytes into shared memory, Z
-    long long z0 = 0, z1 = 0;
-    for (int k0 = 0; k0 < Sp; k0 += 16) {
+    // weights (the scores again), their bytes as fp16 A fragments, the context products
+    uint32_t z0 = 0, z1 = 0;  // at most 128 weights of 2^24 per lane
+    float acc[3][NT][4];
+#pragma unroll
+    for (int L = 0; L < 3; L++)
+#pragma unroll
+        for (int nt = 0; nt < NT; nt++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) acc[L][nt][q] = 0.0f;
+#pragma unroll 1
+    for (int k0 = 0; k0 < lp; k0 += 16) {
         float sv[2][4];
         scores16(k0, sv);
+        uint32_t E[2][4];
 #pragma unroll
         for (int t = 0; t < 2; t++) {
-            int E[4];
 #pragma unroll
-            for (int q = 0; q < 4; q++) E[q] = softmax_weight(__fadd_rn(sv[t][q], -(q < 2 ? mx0 : mx1)));
-            z0 += (long long)E[0] + E[1];
-            z1 += (long long)E[2] + E[3];
-            const int key = k0 + t * 8 + tq * 2;
+            for (int q = 0; q < 4; q++)
+                E[t][q] = (uint32_t)softmax_weight(__fsub_rn(sv[t][q], q < 2 ? mx0 : mx1));
+            z0 += E[t][0] + E[t][1];
+            z1 += E[t][2] + E[t][3];
+        }
+        uint32_t vb[NT / 2][4];
 #pragma unroll
-            for (int L = 0; L < 4; L++) {
-                const uint32_t lo2 = ((uint32_t)(E[0] >> (8 * L)) & 255u) | (((uint32_t)(E[1] >> (8 * L)) & 255u) << 8);
-                const uint32_t hi2 = ((uint32_t)(E[2] >> (8 * L)) & 255u) | (((uint32_t)(E[3] >> (8 * L)) & 255u) << 8);
-                *reinterpret_cast<uint16_t *>(Ew + (size_t)L * 16 * Sp + swl(g, key, Sp, msk)) = (uint16_t)lo2;
-                *reinterpret_cast<uint16_t *>(Ew + (size_t)L * 16 * Sp + swl(g + 8, key, Sp, msk)) = (uint16_t)hi2;
+        for (int nj = 0; nj < NT / 2; nj++)
+            att_ldmatrix_x4_trans(vb[nj],
+                                  att_smem_u32(Vs + att_sw<DH>(k0 + (jq & 1) * 8 + i8, 2 * nj + (jq >> 1))));
+#pragma unroll
+        for (int L = 0; L < 3; L++) {
+            // byte L (byte pair of e2, up to 256) of two weights as fp16: 0x6400 | n is 1024 + n
+            uint32_t ea[4];
+#pragma unroll
+            for (int f = 0; f < 4; f++) {
+                const uint32_t lo = E[f >> 1][2 * (f & 1)], hi = E[f >> 1][2 * (f & 1) + 1];
+                const uint32_t w = L == 2 ? __byte_perm(lo, hi, 0x7632) : __byte_perm(lo, hi, L ? 0x6521 : 0x5410);
+                ea[f] = half2_sub_1024((w & (L == 2 ? 0x01FF01FFu : 0x00FF00FFu)) | 0x64006400u);
+            }
+#pragma unroll
+            for (int nj = 0; nj < NT / 2; nj++) {
+                mma_f16_16816(acc[L][2 * nj], ea, vb[nj][0], vb[nj][1]);
+                mma_f16_16816(acc[L][2 * nj + 1], ea, vb[nj][2], vb[nj][3]);
             }
         }
     }
+    long long Z0 = z0, Z1 = z1;
 #pragma unroll
     for (int o = 1; o < 4; o <<= 1) {
-        z0 += __shfl_xor_sync(0xFFFFFFFFu, z0, o);
-        z1 += __shfl_xor_sync(0xFFFFFFFFu, z1, o);
+        Z0 += __shfl_xor_sync(0xFFFFFFFFu, Z0, o);
+        Z1 += __shfl_xor_sync(0xFFFFFFFFu, Z1, o);
     }
+    // N = a0 + 2^8 a1 + 2^16 a2: fl(2^8 a1 + a0) is off by at most 2^8 + 1, which
+    // makes at most rho 2^-15 of t (Z >= 2^24)
+    const float iz0 = __frcp_rn(__ll2float_rn(Z0)), iz1 = __frcp_rn(__ll2float_rn(Z1));
+    const float slack = __fmul_rn(fabsf(a.rho), 0x1p-15f);
+    uint8_t *Os = Qs + warp * 16 * RB;  // this warp's own query rows: the output as fp16
     __syncwarp();
-    // context: per weight byte L, sum_j e_Lj v_j[e] on the tensor cores (u8 x s8)
-    long long N[8][4];
 #pragma unroll
-    for (int nt = 0; nt < 8; nt++)
+    for (int nt = 0; nt < NT; nt++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) N[nt][q] = 0;
-#pragma unroll 1
-    for (int L = 0; L < 4; L++) {
-        int acc[8][4];
+        for (int hr = 0; hr < 2; hr++) {
+            float c[2];
 #pragma unroll
-        for (int nt = 0; nt < 8; nt++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) acc[nt][q] = 0;
-        const uint8_t *EL = Ew + (size_t)L * 16 * Sp;
-        for (int ks = 0; ks < (Sp >> 5); ks++) {
-            uint32_t ea[4];
-            att_ldmatrix_x4(ea, att_smem_u32(EL + swl((jq & 1) * 8 + i8, (ks * 2 + (jq >> 1)) * 16, Sp, msk)));
-#pragma unroll
-            for (int nj = 0; nj < 4; nj++) {
-                uint32_t r[4];
-                att_ldmatrix_x4(r, att_smem_u32(Vt + swl(nj * 16 + (jq >> 1) * 8 + i8, (ks * 2 + (jq & 1)) * 16, Sp, msk)));
-                att_mma_u8s8(acc[2 * nj], ea, r[0], r[1]);
-                att_mma_u8s8(acc[2 * nj + 1], ea, r[2], r[3]);
+            for (int q = 0; q < 2; q++) {
+                const float a0 = acc[0][nt][2 * hr + q], a1 = acc[1][nt][2 * hr + q], a2 = acc[2][nt][2 * hr + q];
+                const float fn = __fmaf_rn(a2, 65536.0f, __fmaf_rn(a1, 256.0f, a0));
+                c[q] = q8_context(fn, hr ? iz1 : iz0, a.rho, slack, [&]() {
+                    return att_ctx_exact((long long)__float2int_rn(a0) + (long long)__float2int_rn(a1) * 256 +
+                                             (long long)__float2int_rn(a2) * 65536,
+                                         hr ? Z1 : Z0, a.rho);
+                });
             }
+            const __half2 hv = __floats2half2_rn(c[0], c[1]);
+            *reinterpret_cast<__half2 *>(Os + att_sw<DH>(g + 8 * hr, nt) + tq * 4) = hv;
         }
-#pragma unroll
-        for (int nt = 0; nt < 8; nt++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) N[nt][q] += (long long)acc[nt][q] << (8 * L);
+    __syncwarp();
+    // rows of 16 codes per lane: fp16 as they are, int8 from the low byte of 1536 + v
+    for (int i = lane; i < 16 * CH; i += 32) {
+        const int r = i / CH, c = i % CH, qrow = q0 + warp * 16 + r;
+        if (qrow >= S) continue;
+        const uint4 lo = *reinterpret_cast<const uint4 *>(Os + att_sw<DH>(r, 2 * c));
+        const uint4 hi = *reinterpret_cast<const uint4 *>(Os + att_sw<DH>(r, 2 * c + 1));
+        const size_t o = ((size_t)b * S + qrow) * a.d + h * DH + 16 * c;
+        *reinterpret_cast<uint4 *>(a.ctx + o) = make_uint4(half2_to_codes(lo.x, lo.y), half2_to_codes(lo.z, lo.w),
+                                                           half2_to_codes(hi.x, hi.y), half2_to_codes(hi.z, hi.w));
+        if (a.ctx16) {
+            reinterpret_cast<uint4 *>(a.ctx16 + o)[0] = lo;
+            reinterpret_cast<uint4 *>(a.ctx16 + o)[1] = hi;
+        }
     }
-    // row g (q < 2) or g + 8 of the warp's queries, element nt * 8 + 2 tq + (q & 1)
-#pragma unroll
-    for (int nt = 0; nt < 8; nt++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int qrow = q0 + warp * 16 + g + (q >> 1) * 8;
-            if (qrow < S) {
-                const int e = nt * 8 + tq * 2 + (q & 1);
-                const int8_t v = q8_quotient(N[nt][q], q < 2 ? z0 : z1, a.rho, rn32_div);
-                const size_t o = ((size_t)b * S + qrow) * a.d + h * DH + e;
-                a.ctx[o] = v;
-                if (a.ctx16) a.ctx16[o] = __short2half_rn(v);
-            }
-        }
 }
 
-static int enc_mma_keys(int S) {
-    int sp = 32;
-    while (sp < S) sp <<= 1;
-    return sp;
-}
-static size_t enc_mma_smem(int Sp) { return 64 * 64 + (size_t)Sp * 64 * 2 + (size_t)ENC_MMA_WARPS * 4 * 16 * Sp; }
+template <int DH>
+static size_t enc_tc_smem(int S, int nw) { return (size_t)(16 * nw + 2 * ((S + 15) & ~15)) * 2 * DH; }
+
 template <int DH>
 static cudaError_t launch_enc(const AttnEncArgs &a, cudaStream_t st) {
     size_t smem = (size_t)a.S * (DH + 16) + (size_t)a.S * DH + (size_t)ENC_WARPS * a.S * sizeof(int);
@@ -500,21 +518,36 @@ static cudaError_t launch_enc(const AttnEncArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <int DH, int NW>
+static cudaError_t launch_enc_tc_nw(const AttnEncArgs &a, cudaStream_t st) {
+    const dim3 grid(a.B * a.H, (a.S + 16 * NW - 1) / (16 * NW));
+    launch_pdl(attn_encoder_tc<DH, NW>, grid, ENC_TC_THREADS, enc_tc_smem<DH>(a.S, NW), st, a, (a.S + 15) & ~15);
+    return cudaGetLastError();
+}
+
+// warps (16 queries each) per block: four share a staging of K and V; fewer
+// when that would leave SMs without a block or hold warps without queries
+template <int DH>
+static cudaError_t launch_enc_tc(const AttnEncArgs &a, cudaStream_t st) {
+    const int tiles = (a.S + 15) / 16;
+    int nw = tiles >= 3 ? 4 : tiles;
+    while (nw > 1 && (long)a.B * a.H * ((tiles + nw - 1) / nw) < device_sm_count()) nw >>= 1;
+    if (nw == 4) return launch_enc_tc_nw<DH, 4>(a, st);
+    if (nw == 2) return launch_enc_tc_nw<DH, 2>(a, st);
+    return launch_enc_tc_nw<DH, 1>(a, st);
+}
+
 cudaError_t launch_attention_encoder(const AttnEncArgs &a, cudaStream_t st) {
     if (a.S < 1 || a.S > ENC_MAX_KEYS) return cudaErrorInvalidValue;
-    // the tensor-core kernel when its grid fills the GPU (a handful of
-    // sentences run faster on the dp4a kernel's finer query chunks)
-    if (a.dh == 64 && a.S <= 256 && (long)a.B * a.H * ((a.S + 63) / 64) >= device_sm_count()) {
-        const int Sp = enc_mma_keys(a.S);
-        dim3 grid(a.B * a.H, (a.S + 63) / 64);
-        launch_pdl(attn_encoder_mma, grid, 32 * ENC_MMA_WARPS, enc_mma_smem(Sp), st, a, Sp);
-        return cudaGetLastError();
-    }
+    // few 16-query tiles: the dp4a kernel, one query per warp, has the shorter
+    // chain (encode of one 46-token sentence, 12 layers: 402 against 440 us;
+    // equal at 192 tiles; 8 x 100 tokens, 224 tiles: 634 against 561 us)
+    const bool tc = (long)a.B * a.H * ((a.S + 15) / 16) > ENC_TC_MIN_TILES;
     switch (a.dh) {
         case 32:
-            return launch_enc<32>(a, st);
+            return tc ? launch_enc_tc<32>(a, st) : launch_enc<32>(a, st);
         case 64:
-            return launch_enc<64>(a, st);
+            return tc ? launch_enc_tc<64>(a, st) : launch_enc<64>(a, st);
         case 128:
             return launch_enc<128>(a, st);
         default:
@@ -541,9 +574,15 @@ cudaError_t attention_init() {
     if (!err) err = cudaFuncSetAttribute(attn_encoder<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc(32));
     if (!err) err = cudaFuncSetAttribute(attn_encoder<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc(64));
     if (!err) err = cudaFuncSetAttribute(attn_encoder<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc(128));
-    if (!err)
-        err = cudaFuncSetAttribute(attn_encoder_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)enc_mma_smem(256));
+    auto enc_tc = [&](auto k, size_t smem) {
+        if (!err) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+    enc_tc(attn_encoder_tc<32, 1>, enc_tc_smem<32>(ENC_MAX_KEYS, 1));
+    enc_tc(attn_encoder_tc<32, 2>, enc_tc_smem<32>(ENC_MAX_KEYS, 2));
+    enc_tc(attn_encoder_tc<32, 4>, enc_tc_smem<32>(ENC_MAX_KEYS, 4));
+    enc_tc(attn_encoder_tc<64, 1>, enc_tc_smem<64>(ENC_MAX_KEYS, 1));
+    enc_tc(attn_encoder_tc<64, 2>, enc_tc_smem<64>(ENC_MAX_KEYS, 2));
+    enc_tc(attn_encoder_tc<64, 4>, enc_tc_smem<64>(ENC_MAX_KEYS, 4));
     return err;
 }
 }  // namespace mnmt

@@ -7,6 +7,7 @@
 // the fixed-point LayerNorm and softmax sums).
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -120,8 +121,13 @@ MNMT_DEV float exp_own(float x) {
 }
 
 // softmax weight on the 2^-24 grid: rne(exp(x) * 2^24), x <= 0
+// (the float-to-integer conversion runs at 17 lanes per clock and SM on this
+// part, an addition at 130: below 2^23 the rounding is an addition of 2^23,
+// whose ulp is 1; from 2^23 on the value is an integer, read off its bits)
 MNMT_DEV int32_t softmax_weight(float x) {
-    return __float2int_rn(__fmul_rn(exp_own(x), 16777216.0f));
+    const float w = __fmul_rn(exp_own(x), 16777216.0f);
+    return w < 0x1p23f ? (int32_t)(__float_as_uint(__fadd_rn(w, 0x1p23f)) - 0x4B000000u)
+                       : (int32_t)(__float_as_uint(w) - 0x4A800000u);
 }
 
 // natural log in double for z >= 1: z = f 2^k, f in [sqrt(1/2), sqrt(2)),
@@ -202,6 +208,36 @@ MNMT_DEV int dot16(int4 a, int4 b, int acc) {
     acc = __dp4a(a.z, b.z, acc);
     acc = __dp4a(a.w, b.w, acc);
     return acc;
+}
+
+// ---------------------------------------------------------------------------
+// int8 codes as fp16 (exact) and back without conversion instructions: for an
+// unsigned byte u, 0x6400 | u is the fp16 1024 + u; the code v = u - 128 has
+// u = v ^ 0x80.  The fp16 1536 + v has v's two's complement as its low byte.
+// ---------------------------------------------------------------------------
+MNMT_DEV uint32_t h2_sub(uint32_t x, uint32_t y) {
+    const __half2 r = __hsub2(*reinterpret_cast<const __half2 *>(&x), *reinterpret_cast<const __half2 *>(&y));
+    return *reinterpret_cast<const uint32_t *>(&r);
+}
+MNMT_DEV uint32_t half2_sub_1024(uint32_t x) { return h2_sub(x, 0x64006400u); }
+// four codes (bytes of w, lowest first) -> (v0, v1), (v2, v3)
+MNMT_DEV void codes_to_half2(int w, uint32_t &lo, uint32_t &hi) {
+    const uint32_t u = (uint32_t)w ^ 0x80808080u;
+    lo = h2_sub(__byte_perm(u, 0x64646464u, 0x4140), 0x64806480u);  // 1152 = 1024 + 128
+    hi = h2_sub(__byte_perm(u, 0x64646464u, 0x4342), 0x64806480u);
+}
+// (v0, v1), (v2, v3) -> four codes
+MNMT_DEV uint32_t half2_to_codes(uint32_t lo, uint32_t hi) {
+    return __byte_perm(h2_sub(lo, 0xE600E600u), h2_sub(hi, 0xE600E600u), 0x6420);  // v + 1536
+}
+
+// d += a b: m16n8k16, fp16 operands, fp32 accumulation
+MNMT_DEV void mma_f16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 // ---------------------------------------------------------------------------
@@ -332,6 +368,30 @@ MNMT_DEV int8_t q8_quotient(long long n, long long z, float rho, ExactDiv exact)
     const int8_t hi = q8(__fmul_rn(sgn, __uint_as_float(qb + 8u)), rho);
     if (lo == hi) return lo;
     return q8(exact(n, z), rho);
+}
+
+// q8(nearest float to N / Z, rho) from an approximation fN of N and invZ =
+// fl(1 / fl(Z)), Z >= 2^24: t = fl(fl(fN invZ) rho) is off the exact chain by
+// at most eight relative roundings of 2^-24 (two in fN, fl(Z), fl(1/Z), two
+// products; the quotient and the product of the exact chain; < 2^-20) plus
+// `slack`, what fN's absolute error makes of t.  Where t lies further from a
+// rounding boundary than that (all but ~1e-4 of the values), rne(t) is the
+// code; else exact() decides.  (A NaN clamps to -127, as in q8.)  Returns the
+// code as an integer-valued float.  (q8_quotient converts two 64-bit integers
+// per value, at 2 lanes per clock and SM on this part.)
+template <typename Exact>
+MNMT_DEV float q8_context(float fN, float invZ, float rho, float slack, Exact exact) {
+    const float t = fminf(fmaxf(__fmul_rn(__fmul_rn(fN, invZ), rho), -127.0f), 127.0f);
+    const float r = __fsub_rn(__fadd_rn(t, 12582912.0f), 12582912.0f);  // rne for |t| < 2^22
+    if (fabsf(__fsub_rn(t, r)) < __fsub_rn(0.5f, __fmaf_rn(fabsf(t), 0x1p-20f, slack))) return r;
+    return exact();
+}
+// the same for N = 4096 hi + lo, |hi|, |lo| < 2^29 (up to 1024 keys): fl(lo) is
+// off by at most 2^5, which makes at most rho 2^-19 of t
+template <typename Exact>
+MNMT_DEV int8_t q8_context_hl(int hi, int lo, float invZ, float rho, Exact exact) {
+    const float fn = __fmaf_rn(__int2float_rn(hi), 4096.0f, __int2float_rn(lo));
+    return (int8_t)__float2int_rn(q8_context(fn, invZ, rho, __fmul_rn(fabsf(rho), 0x1p-18f), exact));
 }
 
 // ---------------------------------------------------------------------------

@@ -296,16 +296,6 @@ MNMT_DEV void topk_insert(unsigned long long (&lst)[KM], int k, unsigned long lo
     }
 }
 
-// rne(exp_own(x) 2^24) for x <= 0, the weight of one softmax term.  Below 2^23
-// the rounding to an integer is done by adding 2^23 (whose ulp is 1) and
-// reading the low bits; the few weights in [2^23, 2^24] (x within ln 2 of
-// the maximum) are integers already.
-MNMT_DEV int32_t softmax_weight_fast(float x) {
-    const float w = __fmul_rn(exp_own(x), 16777216.0f);
-    if (w < 0x1p23f) return (int32_t)(__float_as_uint(__fadd_rn(w, 0x1p23f)) - 0x4B000000u);
-    return __float2int_rn(w);
-}
-
 // Block-wide selection of the n largest keys held in the threads' descending
 // lists lst[0..KL): n rounds of a maximum over the list heads.  The keys land
 // in sel[0..n) (0 where fewer exist); every thread must call it.
@@ -411,8 +401,8 @@ __global__ void __launch_bounds__(NT) beam_rows_kernel(BeamArgs a) {
     // four logits per lane and step: their weights, then one warp vote on
     // whether any of them can enter the warp's list
     auto visit4 = [&](const float4 v, int n0) {
-        const int32_t w4 = softmax_weight_fast(__fsub_rn(v.x, m)) + softmax_weight_fast(__fsub_rn(v.y, m)) +
-                           softmax_weight_fast(__fsub_rn(v.z, m)) + softmax_weight_fast(__fsub_rn(v.w, m));
+        const int32_t w4 = softmax_weight(__fsub_rn(v.x, m)) + softmax_weight(__fsub_rn(v.y, m)) +
+                           softmax_weight(__fsub_rn(v.z, m)) + softmax_weight(__fsub_rn(v.w, m));
         z += w4;  // each weight <= 2^24
         unsigned msk = __ballot_sync(0xFFFFFFFFu, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)) >= thr);
         while (msk) {
@@ -433,11 +423,11 @@ __global__ void __launch_bounds__(NT) beam_rows_kernel(BeamArgs a) {
         if (v4) {
             for (int n = threadIdx.x; n < V / 4; n += NT) {
                 const float4 v = l4[n];
-                z += softmax_weight_fast(__fsub_rn(v.x, m)) + softmax_weight_fast(__fsub_rn(v.y, m)) +
-                     softmax_weight_fast(__fsub_rn(v.z, m)) + softmax_weight_fast(__fsub_rn(v.w, m));
+                z += softmax_weight(__fsub_rn(v.x, m)) + softmax_weight(__fsub_rn(v.y, m)) +
+                     softmax_weight(__fsub_rn(v.z, m)) + softmax_weight(__fsub_rn(v.w, m));
             }
         } else {
-            for (int n = threadIdx.x; n < V; n += NT) z += softmax_weight_fast(__fsub_rn(l[n], m));
+            for (int n = threadIdx.x; n < V; n += NT) z += softmax_weight(__fsub_rn(l[n], m));
         }
     } else if (v4) {
         // four loads in flight per lane before the (branchy) visits

@@ -113,3 +113,17 @@ def test_encoder_attention_tensor_core_long_sources(stream):
     assert ids.shape[1] > 128
     picks = [int(np.argmin(lens)), int(np.argmax(lens))]
     check_taps(blob, cfg, ids, lens, 1, 4, 2, picks, stream)
+
+
+@pytest.mark.parametrize("d,H,B,S", [(128, 4, 52, 1), (128, 4, 50, 16), (192, 3, 40, 17), (192, 3, 22, 48), (128, 4, 13, 65),
+                                     (192, 3, 9, 129), (192, 3, 4, 512), (128, 4, 3, 511)])
+def test_encoder_attention_fp16_tiles(d, H, B, S, stream):
+    """The fp16 tensor-core encoder attention (more than 192 tiles of 16 queries)
+    at one key, whole and ragged 16-key blocks, partly filled query blocks and
+    its largest key count, d_h = 32 and 64."""
+    assert B * H * ((S + 15) // 16) > 192
+    cfg = synth.ModelConfig(1, 1, d, H, 128, 300, d, 1, 1, max_pos=512)
+    blob = synth.build_blob(cfg, 79, gamma_range=(0.5, 1.5))
+    ids, lens = synth.source_batch(cfg.vocab, B, max(1, S // 2), S, 80)
+    ids = np.pad(ids, ((0, 0), (0, S - ids.shape[1])))
+    check_taps(blob, cfg, ids, lens, 1, 4, 1, sorted({int(np.argmin(lens)), int(np.argmax(lens))}), stream)
