@@ -109,7 +109,7 @@ int mnmt_load_weights(const void *blob, size_t bytes, void *cuda_stream, mnmt_mo
 /* Memory-minimal operation (Sec. 4 "Memory Optimization"; the running memory
  * column of Table 2).  MNMT_LOAD_LEAN keeps only the int8 blob and the derived
  * per-column constants on the device (no fp16 copy of the weight codes): every
- * linear of the model's sessions runs on the int8 GEMV / IMMA kernels, with
+ * linear of the model's sessions runs on the kernels that read int8 codes, with
  * results identical to the default load.  flags = 0 is mnmt_load_weights.
  * MNMT_EINVAL for unknown flags. */
 #define MNMT_LOAD_LEAN 1

@@ -275,7 +275,7 @@ struct mnmt_model {
     uint8_t *d_blob;
     __half *d_blob16;  // fp16 copy of every blob byte read as an int8 code (tensor-core operands); null when lean
     int wq;            // weight format of the attention / FFN linears (8, 4, 4 | WQ_MINMAX)
-    int8_t *d_w8;      // symmetric 4-bit linears unpacked to int8 (the IMMA / tensor-core operands); null when lean
+    int8_t *d_w8;      // symmetric 4-bit linears unpacked to int8 (the tiled linears' operands); null when lean
     __half *d_w8_16;   // its fp16 copy
     size_t w8_codes;
     float *d_aux;
@@ -361,7 +361,7 @@ extern "C" int mnmt_load_weights_ex(const void *blob, size_t bytes, void *cuda_s
     };
     // 4-bit linears: rows of at most 16 (and min-max rows always) run on the
     // 4-bit GEMV kernel; for more rows symmetric linears use an int8 copy of
-    // their codes on the IMMA / tensor-core kernels (not kept when lean)
+    // their codes on the tiled kernels (not kept when lean)
     m->wq = L.wq;
     if (L.wq == 4 && !m->lean) {
         size_t codes = 0;
@@ -769,8 +769,8 @@ __half *out16_for(mnmt_session *s, const int8_t *buf, int M) { return tc_rows(s,
 
 // The quantised linear of rows A [M][lda] (Eq. 3 + epilogue e): on the
 // tensor cores when the layer is a dense contraction (M >= TC_MIN_ROWS),
-// reading the fp16 mirror of A that A's producer wrote; else on the IMMA /
-// GEMV kernels.
+// reading the fp16 mirror of A that A's producer wrote; else on the kernels
+// that read the int8 codes (linear.cu).
 cudaError_t run_linear(mnmt_session *s, const int8_t *A, int lda, const Lin &l, int M, const Epi &e,
                        cudaStream_t st) {
     const mnmt_model *m = s->m;

@@ -1,5 +1,5 @@
 // epilogue.cuh -- the fused epilogue of a quantised linear (Sec. 3.3, Fig. 5),
-// shared by the GEMV, IMMA and tcgen05 kernels: dequantise with the
+// shared by the GEMV, tiled mma.sync and tcgen05 kernels: dequantise with the
 // per-channel weight scale, add the full-precision bias, then requantise /
 // ReLU + requantise / gamma-residual / fp32 / K-V cache write.
 #pragma once

@@ -12,11 +12,13 @@
 //                  activation rows sit in shared memory, products use dp4a and
 //                  a lane group's partial sums meet by warp shuffles.  Bound by
 //                  weight bytes (HBM or L2).
-//   linear_mma     other M > 16: CTA tiles of the int8 GEMM on the warp-level s8
-//                  tensor-core instruction (mma.sync m16n8k32, exact int32
-//                  accumulate), cp.async multi-stage pipeline with XOR-swizzled
-//                  shared memory and ldmatrix fragment loads.  sm_103a has no
-//                  int8 form of tcgen05.mma, so this is the exact int8 tensor path.
+//   linear_mma     other M > 16: CTA tiles of the int8 GEMM on the warp-level
+//                  fp16 tensor-core instruction (mma.sync m16n8k16), the codes
+//                  staged as bytes and widened to fp16 in registers; cp.async
+//                  multi-stage pipeline with XOR-swizzled shared memory and
+//                  ldmatrix fragment loads.  sm_103a has no int8 form of
+//                  tcgen05.mma, and its mma.sync s8 runs at a quarter of the f16
+//                  rate (542 against 2048 operations per clock and SM).
 #include "common.cuh"
 #include "epilogue.cuh"
 #include "internal.h"
@@ -137,7 +139,7 @@ __global__ void __launch_bounds__(SM_THREADS) linear_smallm(const int8_t *__rest
 }
 
 // ---------------------------------------------------------------------------
-// tensor-core path (mma.sync s8)
+// tensor-core path (mma.sync f16 on the int8 codes)
 // ---------------------------------------------------------------------------
 MNMT_DEV uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -154,19 +156,21 @@ MNMT_DEV void ldmatrix_x4(uint32_t (&r)[4], uint32_t addr) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
 }
-MNMT_DEV void mma_s8(int (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 // 64-byte shared rows, 16-byte chunks XOR-swizzled by (row / 2) % 4 so that the
 // 8 rows of an ldmatrix phase hit 8 distinct bank groups.
 MNMT_DEV int swz(int row, int chunk) { return row * 64 + ((chunk ^ ((row >> 1) & 3)) << 4); }
 
-template <int BM, int BN, int WARPS_M, int WARPS_N, int STAGES>
+// An ldmatrix of bytes gives a lane four consecutive codes of one row per 16:
+// widened to two fp16 pairs they are the two registers of an m16n8k16 fragment
+// row, for a k order (codes 4 t .. 4 t + 3 of lane t) that A and W share.
+// Products of codes are at most 2^14, so fp32 sums of 1024 of them are exact;
+// BIGK (K > 1024) moves the sums to int32 every 1024.
+// Bound by issue and the tensor pipe together (per warp and k-tile of a
+// 128 x 128 block, 64 products of 8 cycles and ~340 issued instructions, 240 of
+// them the widening).  Against the s8 instruction: 1000 x 1536 x 512 19.1 ->
+// 9.1 us, 512 x 32000 x 512 argmax 158 -> 60 us, 8192 x 2048 x 512 180 -> 59 us.
+template <int BM, int BN, int WARPS_M, int WARPS_N, int STAGES, bool BIGK>
 __global__ void __launch_bounds__(WARPS_M *WARPS_N * 32)
     linear_mma(const int8_t *__restrict__ A, int lda, const int8_t *__restrict__ W, int M, int N, int K,
                Epi e) {
@@ -175,6 +179,7 @@ __global__ void __launch_bounds__(WARPS_M *WARPS_N * 32)
     constexpr int WTM = BM / WARPS_M, WTN = BN / WARPS_N;
     constexpr int MI = WTM / 16, NI = WTN / 8;
     static_assert(NI % 2 == 0, "B fragments are loaded two n8 tiles at a time");
+    static_assert(STAGES * (BM + BN) * BK >= BM * (BN + 16), "the ring holds the int8 output tile");
     pdl_grid_wait();
     if (e.skip && *e.skip) return;
     extern __shared__ __align__(128) uint8_t smem[];
@@ -185,13 +190,17 @@ __global__ void __launch_bounds__(WARPS_M *WARPS_N * 32)
     const int wm = warp / WARPS_N, wn = warp % WARPS_N;
     const int ktiles = K / BK;
 
-    int acc[MI][NI][4];
+    float acc[MI][NI][4];
+    int acci[BIGK ? MI : 1][BIGK ? NI : 1][4];
 #pragma unroll
     for (int i = 0; i < MI; i++)
 #pragma unroll
         for (int j = 0; j < NI; j++)
 #pragma unroll
-            for (int q = 0; q < 4; q++) acc[i][j][q] = 0;
+            for (int q = 0; q < 4; q++) {
+                acc[i][j][q] = 0.0f;
+                if (BIGK) acci[BIGK ? i : 0][BIGK ? j : 0][q] = 0;
+            }
 
     auto load_stage = [&](int stage, int kt) {
         const int k0 = kt * BK;
@@ -230,89 +239,187 @@ __global__ void __launch_bounds__(WARPS_M *WARPS_N * 32)
         const uint8_t *b_s = sB + (kt % STAGES) * BN * BK;
 #pragma unroll
         for (int kk = 0; kk < 2; kk++) {
-            uint32_t af[MI][4];
-            uint32_t bf[NI][2];
+            uint32_t ar[MI][4], br[NI / 2][4];
             const int j = lane >> 3, i8 = lane & 7;
 #pragma unroll
-            for (int mi = 0; mi < MI; mi++) {
-                int row = wm * WTM + mi * 16 + (j & 1) * 8 + i8;
-                ldmatrix_x4(af[mi], smem_u32(a_s + swz(row, kk * 2 + (j >> 1))));
-            }
+            for (int mi = 0; mi < MI; mi++)
+                ldmatrix_x4(ar[mi], smem_u32(a_s + swz(wm * WTM + mi * 16 + (j & 1) * 8 + i8, kk * 2 + (j >> 1))));
 #pragma unroll
-            for (int nj = 0; nj < NI / 2; nj++) {
-                int row = wn * WTN + nj * 16 + (j >> 1) * 8 + i8;
-                uint32_t r[4];
-                ldmatrix_x4(r, smem_u32(b_s + swz(row, kk * 2 + (j & 1))));
-                bf[2 * nj][0] = r[0];
-                bf[2 * nj][1] = r[1];
-                bf[2 * nj + 1][0] = r[2];
-                bf[2 * nj + 1][1] = r[3];
+            for (int nj = 0; nj < NI / 2; nj++)
+                ldmatrix_x4(br[nj], smem_u32(b_s + swz(wn * WTN + nj * 16 + (j >> 1) * 8 + i8, kk * 2 + (j & 1))));
+#pragma unroll
+            for (int h = 0; h < 2; h++) {  // the two k16 steps of these 32 codes
+                uint32_t bf[NI][2];
+#pragma unroll
+                for (int ni = 0; ni < NI; ni++)
+                    codes_to_half2((int)br[ni >> 1][2 * (ni & 1) + h], bf[ni][0], bf[ni][1]);
+#pragma unroll
+                for (int mi = 0; mi < MI; mi++) {
+                    uint32_t af[4];
+                    codes_to_half2((int)ar[mi][2 * h], af[0], af[2]);
+                    codes_to_half2((int)ar[mi][2 * h + 1], af[1], af[3]);
+#pragma unroll
+                    for (int ni = 0; ni < NI; ni++) mma_f16_16816(acc[mi][ni], af, bf[ni][0], bf[ni][1]);
+                }
             }
+        }
+        if (BIGK && ((kt & 15) == 15 || kt == ktiles - 1)) {
 #pragma unroll
             for (int mi = 0; mi < MI; mi++)
 #pragma unroll
-                for (int ni = 0; ni < NI; ni++) mma_s8(acc[mi][ni], af[mi], bf[ni][0], bf[ni][1]);
+                for (int ni = 0; ni < NI; ni++)
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        acci[BIGK ? mi : 0][BIGK ? ni : 0][q] += __float2int_rn(acc[mi][ni][q]);
+                        acc[mi][ni][q] = 0.0f;
+                    }
         }
     }
     cp_async_wait<0>();
+    if (BIGK) {
+#pragma unroll
+        for (int mi = 0; mi < MI; mi++)
+#pragma unroll
+            for (int ni = 0; ni < NI; ni++)
+#pragma unroll
+                for (int q = 0; q < 4; q++) acc[mi][ni][q] = __int2float_rn(acci[BIGK ? mi : 0][BIGK ? ni : 0][q]);
+    }
 
-    const int t = e.t_ptr ? *e.t_ptr : 0;
+    // y in place: lane (g, tq) holds rows g, g + 8 and columns 2 tq, 2 tq + 1 of every 16 x 8 tile
+    const int g = lane >> 2, tq = lane & 3;
+    const int row0 = bm + wm * WTM + g, col0 = bn + wn * WTN + 2 * tq;
+#pragma unroll
+    for (int ni = 0; ni < NI; ni++) {
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const int col = col0 + ni * 8 + c;
+            const float sc = col < N ? __fmul_rn(e.s_x, e.s_w[col]) : 0.0f, bs = col < N ? e.bias[col] : 0.0f;
+#pragma unroll
+            for (int mi = 0; mi < MI; mi++) {
+                acc[mi][ni][c] = __fadd_rn(__fmul_rn(acc[mi][ni][c], sc), bs);
+                acc[mi][ni][2 + c] = __fadd_rn(__fmul_rn(acc[mi][ni][2 + c], sc), bs);
+            }
+        }
+    }
     if (e.mode == EPI_ARGMAX) {
-        // per row: max key over this thread's columns, then over the 4 lanes of a quad
+        // per row: the largest (ordered y, lowest column) of this thread's
+        // columns, the quad's, then the block's (one atomic per row and block)
+        __syncthreads();
+        unsigned long long *best_s = reinterpret_cast<unsigned long long *>(smem);  // [WARPS_N][BM]
 #pragma unroll
         for (int mi = 0; mi < MI; mi++) {
 #pragma unroll
             for (int hr = 0; hr < 2; hr++) {
-                int row = bm + wm * WTM + mi * 16 + (lane >> 2) + hr * 8;
-                unsigned long long best = 0ull;
+                uint32_t bo = 0u, bc = 0u;
 #pragma unroll
                 for (int ni = 0; ni < NI; ni++) {
 #pragma unroll
-                    for (int q = 0; q < 2; q++) {
-                        int col = bn + wn * WTN + ni * 8 + (lane & 3) * 2 + q;
-                        if (row < M && col < N) {
-                            float y = dequant_bias(acc[mi][ni][hr * 2 + q], e.s_x, e.s_w[col], e.bias[col]);
-                            unsigned long long k = pack_key(y, (uint32_t)col);
-                            best = k > best ? k : best;
+                    for (int c = 0; c < 2; c++) {
+                        const uint32_t col = (uint32_t)(col0 + ni * 8 + c);
+                        const uint32_t o = col < (uint32_t)N ? ordered_bits(acc[mi][ni][2 * hr + c]) : 0u;
+                        if (o > bo) {
+                            bo = o;
+                            bc = col;
                         }
                     }
                 }
+                unsigned long long best = bo ? ((unsigned long long)bo << 32) | (0xFFFFFFFFu - bc) : 0ull;
 #pragma unroll
                 for (int o = 1; o < 4; o <<= 1) {
                     unsigned long long w2 = __shfl_xor_sync(0xFFFFFFFFu, best, o);
                     best = w2 > best ? w2 : best;
                 }
-                if ((lane & 3) == 0 && row < M) atomicMax(e.keys + row, best);
+                if (tq == 0) best_s[wn * BM + wm * WTM + mi * 16 + hr * 8 + g] = best;
             }
+        }
+        __syncthreads();
+        for (int r = threadIdx.x; r < BM && bm + r < M; r += NT) {
+            unsigned long long best = best_s[r];
+#pragma unroll
+            for (int w = 1; w < WARPS_N; w++) best = best_s[w * BM + r] > best ? best_s[w * BM + r] : best;
+            atomicMax(e.keys + bm + r, best);
         }
         return;
     }
-    if (e.mode == EPI_RESID) {
-        // every residual load first: the stores may alias them
-        float r[MI][NI][4];
+    if (e.mode == EPI_RESID || e.mode == EPI_F32) {
+        // two adjacent columns per access where they are 8-byte aligned; every
+        // residual load of an m-tile before its stores
+        const bool v2 = e.ldf % 2 == 0 && (reinterpret_cast<uintptr_t>(e.f32) & 7) == 0;
 #pragma unroll
-        for (int mi = 0; mi < MI; mi++)
+        for (int mi = 0; mi < MI; mi++) {
+            if (e.mode == EPI_RESID) {
+                float r[NI][4];
+#pragma unroll
+                for (int ni = 0; ni < NI; ni++)
+#pragma unroll
+                    for (int hr = 0; hr < 2; hr++) {
+                        const int row = row0 + mi * 16 + hr * 8, col = col0 + ni * 8;
+                        const float *p = e.f32 + (size_t)row * e.ldf + col;
+                        float2 v = make_float2(0.0f, 0.0f);
+                        if (row < M && col + 1 < N && v2) v = *reinterpret_cast<const float2 *>(p);
+                        else if (row < M) {
+                            if (col < N) v.x = p[0];
+                            if (col + 1 < N) v.y = p[1];
+                        }
+                        r[ni][2 * hr] = v.x;
+                        r[ni][2 * hr + 1] = v.y;
+                    }
+#pragma unroll
+                for (int ni = 0; ni < NI; ni++)
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        acc[mi][ni][q] = __fadd_rn(__fmul_rn(e.gamma, r[ni][q]), acc[mi][ni][q]);
+            }
 #pragma unroll
             for (int ni = 0; ni < NI; ni++)
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    int row = bm + wm * WTM + mi * 16 + (lane >> 2) + (q >> 1) * 8;
-                    int col = bn + wn * WTN + ni * 8 + (lane & 3) * 2 + (q & 1);
-                    r[mi][ni][q] = (row < M && col < N) ? e.f32[(size_t)row * e.ldf + col] : 0.0f;
+                for (int hr = 0; hr < 2; hr++) {
+                    const int row = row0 + mi * 16 + hr * 8, col = col0 + ni * 8;
+                    float *p = e.f32 + (size_t)row * e.ldf + col;
+                    if (row < M && col + 1 < N && v2) {
+                        *reinterpret_cast<float2 *>(p) = make_float2(acc[mi][ni][2 * hr], acc[mi][ni][2 * hr + 1]);
+                    } else if (row < M) {
+                        if (col < N) p[0] = acc[mi][ni][2 * hr];
+                        if (col + 1 < N) p[1] = acc[mi][ni][2 * hr + 1];
+                    }
                 }
+        }
+        return;
+    }
+    const int t = e.t_ptr ? *e.t_ptr : 0;
+    if ((e.mode == EPI_Q8 || e.mode == EPI_RELU_Q8) && !e.out16 && e.ldo % 16 == 0 &&
+        (reinterpret_cast<uintptr_t>(e.out) & 15) == 0) {
+        // int8 rows through shared memory (rows of BN + 16 bytes), 16 bytes per store
+        constexpr int LDS = BN + 16;
+        __syncthreads();
 #pragma unroll
-        for (int mi = 0; mi < MI; mi++)
+        for (int ni = 0; ni < NI; ni++) {
+            const int col = col0 + ni * 8;
+            const float i0 = col < N ? e.inv_out[col] : 0.0f, i1 = col + 1 < N ? e.inv_out[col + 1] : 0.0f;
 #pragma unroll
-            for (int ni = 0; ni < NI; ni++)
+            for (int mi = 0; mi < MI; mi++)
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    int row = bm + wm * WTM + mi * 16 + (lane >> 2) + (q >> 1) * 8;
-                    int col = bn + wn * WTN + ni * 8 + (lane & 3) * 2 + (q & 1);
-                    if (row < M && col < N)
-                        e.f32[(size_t)row * e.ldf + col] =
-                            __fadd_rn(__fmul_rn(e.gamma, r[mi][ni][q]),
-                                      dequant_bias(acc[mi][ni][q], e.s_x, e.s_w[col], e.bias[col]));
+                for (int hr = 0; hr < 2; hr++) {
+                    float y0 = acc[mi][ni][2 * hr], y1 = acc[mi][ni][2 * hr + 1];
+                    if (e.mode == EPI_RELU_Q8) {
+                        y0 = y0 > 0.0f ? y0 : 0.0f;
+                        y1 = y1 > 0.0f ? y1 : 0.0f;
+                    }
+                    *reinterpret_cast<uint16_t *>(smem + (wm * WTM + mi * 16 + hr * 8 + g) * LDS + wn * WTN + ni * 8 + 2 * tq) =
+                        (uint16_t)__byte_perm(q8_bits(y0, i0), q8_bits(y1, i1), 0x0040);
                 }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < BM * (BN / 16); i += NT) {
+            const int r = i / (BN / 16), c = (i % (BN / 16)) * 16, row = bm + r, col = bn + c;
+            if (row >= M || col >= N) continue;
+            const uint4 v = *reinterpret_cast<const uint4 *>(smem + r * LDS + c);
+            if (col + 16 <= N) {
+                *reinterpret_cast<uint4 *>(e.out + (size_t)row * e.ldo + col) = v;
+            } else {
+                for (int b = 0; col + b < N; b++) e.out[(size_t)row * e.ldo + col + b] = (int8_t)smem[r * LDS + c + b];
+            }
+        }
         return;
     }
 #pragma unroll
@@ -321,9 +428,8 @@ __global__ void __launch_bounds__(WARPS_M *WARPS_N * 32)
         for (int ni = 0; ni < NI; ni++)
 #pragma unroll
             for (int q = 0; q < 4; q++) {
-                int row = bm + wm * WTM + mi * 16 + (lane >> 2) + (q >> 1) * 8;
-                int col = bn + wn * WTN + ni * 8 + (lane & 3) * 2 + (q & 1);
-                if (row < M && col < N) epi_store(e, row, col, acc[mi][ni][q], t);
+                const int row = row0 + mi * 16 + (q >> 1) * 8, col = col0 + ni * 8 + (q & 1);
+                if (row < M && col < N) epi_store_y(e, row, col, acc[mi][ni][q], t);
             }
 }
 
@@ -332,8 +438,12 @@ __global__ void __launch_bounds__(WARPS_M *WARPS_N * 32)
 // ---------------------------------------------------------------------------
 template <int BM, int BN, int WM, int WN, int STAGES>
 static cudaError_t mma_attr() {
-    return cudaFuncSetAttribute(linear_mma<BM, BN, WM, WN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                STAGES * (BM + BN) * 64);
+    cudaError_t err = cudaFuncSetAttribute(linear_mma<BM, BN, WM, WN, STAGES, false>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, STAGES * (BM + BN) * 64);
+    if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(linear_mma<BM, BN, WM, WN, STAGES, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   STAGES * (BM + BN) * 64);
+    return err;
 }
 
 // Opt the tensor-core kernels into their shared memory (once per process,
@@ -370,7 +480,7 @@ static cudaError_t launch_small(const int8_t *A, int lda, const int8_t *W, int M
 template <int BM, int BN, int WM, int WN, int STAGES>
 static cudaError_t launch_mma(const int8_t *A, int lda, const int8_t *W, int M, int N, int K, const Epi &e,
                               cudaStream_t st) {
-    auto k = linear_mma<BM, BN, WM, WN, STAGES>;
+    auto k = K > 1024 ? linear_mma<BM, BN, WM, WN, STAGES, true> : linear_mma<BM, BN, WM, WN, STAGES, false>;
     size_t smem = (size_t)STAGES * (BM + BN) * 64;
     dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
     launch_pdl(k, grid, WM * WN * 32, smem, st, A, lda, W, M, N, K, e);
@@ -388,7 +498,7 @@ cudaError_t launch_linear(const int8_t *A, int lda, const int8_t *W, int M, int 
         return launch_small<16>(A, lda, W, M, N, K, e, st);
     }
     // up to 64 rows over few output tiles (narrow N): chunks of 16 rows over
-    // the grid's y dimension spread the work over more blocks than the IMMA
+    // the grid's y dimension spread the work over more blocks than the 64 x 64
     // tiling would (the weights are re-read per chunk, from L2)
     const long tiles64 = (long)((M + 63) / 64) * ((N + 63) / 64);
     if (M <= SMALL_CHUNKED_MAX_M && K <= 2048 && tiles64 < 8) return launch_small<16>(A, lda, W, M, N, K, e, st);

@@ -219,3 +219,21 @@ def test_attention_context_on_rounding_ties(rho):
     mnmt.mnmt_attention_decode(dev(q), dev(Kc), dev(Vc), dev(n_keys), R, H, dh, T, sigma, np.float32(rho), ctx)
     ref = O.attention_decode(q, Kc, Vc, n_keys, sigma, np.float32(rho))
     assert np.array_equal(host(ctx), ref)
+
+
+@pytest.mark.parametrize("M,N,K,mode", [(17, 33, 1024, mnmt.EPI_F32), (65, 130, 1088, mnmt.EPI_RESID), (130, 64, 3136, mnmt.EPI_F32),
+                                        (128, 129, 64, mnmt.EPI_Q8), (127, 2048, 1024, mnmt.EPI_RELU_Q8),
+                                        (1500, 1700, 2112, mnmt.EPI_Q8), (1500, 1702, 128, mnmt.EPI_RESID)])
+def test_linear_fp16_products_edges(M, N, K, mode):
+    """The tiled int8 linear at its edges: codes of +-127 and -128 in rows that
+    add up to +-2^24 over 1024 products (the largest exact fp32 sum), K past
+    1024 (sums moved to int32), partial tiles of both block sizes, rows whose
+    int8 or fp32 segments are not aligned."""
+    A, W, s_w, b, inv, s_x = _lin_inputs(M + N + K, M, N, K)
+    A[0], W[0] = -128, -128
+    A[1], W[1] = 127, -128
+    resid = synth.uniform_f32(6, "r", (M, N), -3, 3) if mode == mnmt.EPI_RESID else None
+    got = _gpu_linear(A, W, s_w, b, inv, s_x, mode, np.float32(0.875), resid)
+    ref = O.linear(A, W, s_w, b, s_x, mode, inv_out=inv, gamma=np.float32(0.875), resid=resid)
+    v = np.uint8 if got.dtype == np.int8 else np.uint32
+    assert np.array_equal(got.view(v), ref.view(v))
