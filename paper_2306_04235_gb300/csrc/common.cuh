@@ -253,13 +253,25 @@ MNMT_DEV void mma_f16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, 
 // Exact roundings to fp32 with integer operations only (no double precision,
 // which is slow on this part).
 // ---------------------------------------------------------------------------
+// the float nearest S (ties to even), as __ll2float_rn, which runs at 2 lanes
+// per clock and SM on this part: the top 32 significant bits, with the rest
+// folded into the lowest one, round to 24 as the whole would
+MNMT_DEV float ll2float(long long S) {
+    const unsigned long long a = S < 0 ? 0ull - (unsigned long long)S : (unsigned long long)S;
+    const int sh = __clzll((long long)(a | 1ull));
+    const unsigned long long t = a << sh;
+    const float f = __uint2float_rn((uint32_t)(t >> 32) | ((uint32_t)t ? 1u : 0u));
+    const uint32_t b = __float_as_uint(f) + ((uint32_t)(32 - sh) << 23);
+    return a == 0ull ? 0.0f : __uint_as_float(b | (S < 0 ? 0x80000000u : 0u));
+}
+
 // nearest float (ties to even) to S * 2^e, subnormals included
 MNMT_DEV float rn32_pow2(long long S, int e) {
     if (S == 0) return 0.0f;
     {
         // fast path: the integer rounds to float once (half to even); scaling
         // by 2^e is exact while the result stays a normal float
-        const float f = __ll2float_rn(S);
+        const float f = ll2float(S);
         const uint32_t fb = __float_as_uint(f);
         const int fe = (int)((fb >> 23) & 0xFFu) + e;
         if (fe >= 1 && fe <= 254) return __uint_as_float(fb + ((uint32_t)e << 23));
@@ -314,6 +326,26 @@ MNMT_DEV float rn32_scaled_div(long long S, int e, int d) {
     const unsigned long long num = a << t;
     const unsigned long long q = num / z, r = num - q * z;
     const float f = rn32_pow2((long long)(2ull * q + (r != 0ull ? 1ull : 0ull)), e - k - t - 1);
+    return S < 0 ? -f : f;
+}
+
+// rn32_scaled_div for |S| < 2^63 with its 64-bit division replaced by a
+// multiply-high by zm = floor(2^64 / z) (host-computed; d = z 2^kd, z odd): for
+// a numerator below 2^63 the estimate is the quotient or one less, which the
+// remainder corrects
+MNMT_DEV float rn32_scaled_mul(long long S, int e, int kd, unsigned z, unsigned long long zm) {
+    if (z == 1u) return rn32_pow2(S, e - kd);
+    if (S == 0) return 0.0f;
+    const unsigned long long a = S < 0 ? 0ull - (unsigned long long)S : (unsigned long long)S;
+    const int nb = 64 - __clzll(a);
+    const int t = nb < 62 ? 62 - nb : 0;
+    const unsigned long long num = a << t;
+    unsigned long long q = __umul64hi(num, zm), r = num - q * z;
+    if (r >= z) {
+        q++;
+        r -= z;
+    }
+    const float f = rn32_pow2((long long)(2ull * q + (r != 0ull ? 1ull : 0ull)), e - kd - t - 1);
     return S < 0 ? -f : f;
 }
 
@@ -420,6 +452,34 @@ MNMT_DEV long long warp_sum_exact(long long v) {
     p1 = __reduce_add_sync(0xFFFFFFFFu, p1);
     p2 = __reduce_add_sync(0xFFFFFFFFu, p2);
     return (long long)p0 + (long long)p1 * (1LL << 20) + (long long)p2 * (1LL << 40);
+}
+
+// sum over v[0..N) of fx_scale(v[i], 52 - e) for |v[i]| <= 2^e, -70 <= e <= 33,
+// without conversions or 64-bit shifts per term: T = rne(v 2^(52-e)) is taken
+// apart as A 2^30 + B 2^8 + C, A = rne(v 2^(22-e)), B and C the same of the
+// remainder 22 and 8 bits down.  Each rounding is an addition of 1.5 2^23, whose
+// sum's low bits are the integer; each remainder is exact (a multiple of v's
+// ulp, shorter than v); and A 2^30 + B 2^8 is even, so rounding the last
+// remainder rounds T.  |A| <= 2^22, so int32 sums hold 2^9 terms.
+template <int N>
+MNMT_DEV long long fx_sum(const float (&v)[N], int e) {
+    auto p2 = [](int k) { return __uint_as_float((uint32_t)(127 + k) << 23); };
+    const float s22 = p2(22 - e), s44 = p2(44 - e), s52 = p2(52 - e);
+    const float u22 = p2(e - 22), u44 = p2(e - 44);
+    uint32_t sa = 0, sb = 0, sc = 0;
+#pragma unroll
+    for (int i = 0; i < N; i++) {
+        const float ta = __fmaf_rn(v[i], s22, 12582912.0f);
+        const float r1 = __fmaf_rn(-__fsub_rn(ta, 12582912.0f), u22, v[i]);
+        const float tb = __fmaf_rn(r1, s44, 12582912.0f);
+        const float r2 = __fmaf_rn(-__fsub_rn(tb, 12582912.0f), u44, r1);
+        const float tc = __fmaf_rn(r2, s52, 12582912.0f);
+        sa += __float_as_uint(ta);
+        sb += __float_as_uint(tb);
+        sc += __float_as_uint(tc);
+    }
+    const uint32_t off = (uint32_t)N * 0x4B400000u;  // the bits of 1.5 2^23, N times
+    return (long long)(int)(sa - off) * (1LL << 30) + (long long)(int)(sb - off) * 256 + (int)(sc - off);
 }
 
 // LayerNorm of one row held by a warp (x[u] = element u*32 + lane); gv / bv

@@ -237,3 +237,27 @@ def test_linear_fp16_products_edges(M, N, K, mode):
     ref = O.linear(A, W, s_w, b, s_x, mode, inv_out=inv, gamma=np.float32(0.875), resid=resid)
     v = np.uint8 if got.dtype == np.int8 else np.uint32
     assert np.array_equal(got.view(v), ref.view(v))
+
+
+@pytest.mark.parametrize("M,d", [(301, 4), (301, 128), (333, 132), (301, 384), (700, 516), (301, 768), (301, 1020), (302, 1024), (2500, 512)])
+@pytest.mark.parametrize("scale", [1.0, 1e-12, 1e-25, 3e6])
+def test_layernorm_warp_rows(M, d, scale):
+    """The warp-per-row LayerNorm (more than 300 rows): ragged and whole
+    float4 counts per lane, odd factors of d, rows within fx_sum's range and,
+    at the two small scales, the term-by-term forms of the variance and of both
+    sums; rows with values far below the largest (every piece of a term)."""
+    r = (synth.Stream(M + d, "r").normal(M * d).reshape(M, d) * scale + scale * 0.1).astype(np.float32)
+    r[0, : d // 2] = 7.0 * scale
+    r[1] = r[1] * np.exp2(-synth.Stream(9, "e").randint(0, 60, d).astype(np.float64))
+    r[2] = 0.0
+    g = synth.uniform_f32(d, "g", (d,), 0.5, 1.5)
+    b = synth.uniform_f32(d, "b", (d,), -0.2, 0.2)
+    inv = np.float32(127 / 4.0)
+    of = torch.zeros((M, d), dtype=torch.float32, device="cuda")
+    oq = torch.zeros((M, d), dtype=torch.int8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    mnmt.mnmt_layernorm(dev(r), dev(g), dev(b), M, d, inv, of, oq, status)
+    ref_f, ref_q = O.layernorm(r, g, b, inv)
+    assert host(status)[0] == 0
+    assert np.array_equal(host(of).view(np.uint32), ref_f.view(np.uint32))
+    assert np.array_equal(host(oq), ref_q)
