@@ -71,3 +71,43 @@ def test_fake_quant_rejects_bad_scale():
     with pytest.raises(mnmt.MnmtError) as ei:
         mnmt.mnmt_fake_quant(x, 4, 0.0, y=x)
     assert ei.value.code == mnmt.EINVAL
+
+
+@pytest.mark.parametrize("scale_g", [1.0, 1e-30, 1e-42, 1e37])
+@pytest.mark.parametrize("off,n", [(0, 4099), (1, 4099), (0, 7), (0, 1 << 16)])
+def test_fake_quant_backward_pair_sums(scale_g, off, n):
+    """The scale gradient's groups of eight: products inside the range of the
+    exact fp32 pairs, below and above it (summed in fp64), all-zero groups,
+    remainders and unaligned arrays.  Bound: fp64 addition of n terms."""
+    s = np.float32(0.041)
+    x, g = _x(n + off, n + off, 0.6), (_x(n + 5, n + off, 1.0) * np.float32(scale_g)).astype(np.float32)
+    x[off + 3::97] = 0.0
+    x[off + 5::31] = np.float32(9.0)     # clamped
+    g[off: off + 40] = 0.0
+    dx, dg = dev(x)[off:], dev(g)[off:]
+    gx, y = torch.empty(n + off, dtype=torch.float32, device="cuda")[off:], torch.empty(n + off, dtype=torch.float32, device="cuda")[off:]
+    gs = torch.empty(1, dtype=torch.float64, device="cuda")
+    mnmt.mnmt_fake_quant(dx, n, s, 0.0, 8, False, y)
+    mnmt.mnmt_fake_quant_backward(dx, dg, n, s, gx, gs)
+    rgx, rgs, _ = O.fake_quant_backward(x[off:], g[off:], s, 8, 0.0, False)
+    ry, _ = O.fake_quant(x[off:], s, 8, 0.0, False)
+    assert np.array_equal(host(y).view(np.uint32), ry.view(np.uint32))
+    assert np.array_equal(host(gx).view(np.uint32), rgx.view(np.uint32))
+    terms = np.abs(g[off:].astype(np.float64)) * 127
+    assert abs(float(host(gs)[0]) - rgs) <= n * 2.0 ** -53 * float(terms.sum())
+
+
+def test_fake_quant_backward_non_finite():
+    """An infinite or NaN gradient reaches the scale gradient as in fp64."""
+    n = 64
+    x = _x(1, n, 0.6)
+    x[9], x[11] = 0.3, 0.31
+    for bad in (np.inf, np.nan):
+        g = np.ones(n, np.float32)
+        g[9] = bad
+        gx = torch.empty(n, dtype=torch.float32, device="cuda")
+        gs = torch.empty(1, dtype=torch.float64, device="cuda")
+        mnmt.mnmt_fake_quant_backward(dev(x), dev(g), n, 0.041, gx, gs)
+        rgx, rgs, _ = O.fake_quant_backward(x, g, np.float32(0.041), 8, 0.0, False)
+        assert np.array_equal(host(gx).view(np.uint32), rgx.view(np.uint32))
+        assert np.array_equal(np.array([float(host(gs)[0])]), np.array([rgs]), equal_nan=True)
