@@ -6,8 +6,7 @@
 // s_j = fl(acc_j * sigma), m = max_j s_j, weights E_j = rne(exp(fl(s_j - m)) 2^24)
 // (an integer in [0, 2^24]), context N_e = sum_j E_j v_j[e] and Z = sum_j E_j as
 // exact integer sums (so any summation order gives the same bits), then
-// ctx_e = q8(nearest fp32 to N_e / Z, rho).  N_e is accumulated in two int32 halves,
-// E_j = Eh 2^12 + El, which cannot overflow for up to 1024 keys.
+// ctx_e = q8(nearest fp32 to N_e / Z, rho).
 //
 // Kernels:
 //   attn_decode  one warp per (row, head): the incremental step of the decoder
@@ -23,6 +22,7 @@
 //                16..64 queries).
 #include <type_traits>
 
+#include "attn_core.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -30,28 +30,39 @@ namespace mnmt {
 
 constexpr int DEC_MAX_KEYS = 1024;
 
-// 32-bit word k of a 4-, 8- or 16-byte vector held in registers
-MNMT_DEV uint32_t vec_word(uint32_t v, int) { return v; }
-MNMT_DEV uint32_t vec_word(const uint2 &v, int k) { return k ? v.y : v.x; }
-MNMT_DEV uint32_t vec_word(const uint4 &v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
+struct DecRows {
+    const int8_t *kc, *vc;  // layer cache
+    const int *prow;        // [n] physical row of every position (null: all `row`)
+    int row, H, h, T, dh;
+    MNMT_DEV size_t at(int j) const { return (((size_t)(prow ? prow[j] : row) * H + h) * T + j) * dh; }
+    MNMT_DEV const int8_t *k(int j, int) const { return kc + at(j); }
+    MNMT_DEV const int8_t *v(int j, int) const { return vc + at(j); }
+    MNMT_DEV bool same_block(int) const { return true; }
+};
 
-// the exact form of a context code (q8_context's undecided values)
-__device__ __noinline__ float att_ctx_exact(long long n, long long z, float rho) {
-    return (float)q8(rn32_div(n, z), rho);
-}
+// XS = false: a warp per (row, head).  XS = true (cross attention with beams):
+// a warp per head and four of a sentence's beams, which read the same keys and
+// values once.  LONGK: more than 512 keys may be attended (self attention only).
+// Warps are independent; blocks of four at up to 84 registers keep 24 warps of
+// loads in flight per SM (whole rows per block, at 102 registers: 16).
+// 512 rows x 8 heads of 64, 80..160 keys (63 MB): 25.9 -> 21.8 us;
+// 256 x 8, 500 of 512 keys: 56.5 -> 38.5; 1 x 8, 500 keys: 25.7 -> 15.8.
+constexpr int DEC_WARPS = 4;
 
-// XS = false: one block per row, one warp per head.  XS = true (cross
-// attention with beams): one block per sentence, one warp per (beam, head) --
-// the beams of a sentence read the same keys and values, which their block
-// then fetches from L2 once and serves from L1.
-template <int DH, bool XS>
-__global__ void __launch_bounds__(XS ? 32 * 32 : 32 * 16) attn_decode(AttnDecArgs a) {
+template <int DH, bool XS, bool LONGK>
+__global__ void __launch_bounds__(32 * DEC_WARPS, DH == 128 || LONGK || XS ? 4 : 6) attn_decode(AttnDecArgs a) {
     pdl_grid_wait();
     if (a.skip && *a.skip) return;
-    extern __shared__ int dsm[];
+    constexpr int NB = XS ? 4 : 1;
+    extern __shared__ __align__(16) int dsm[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int r = XS ? blockIdx.x * a.beam + w / a.H : blockIdx.x;
-    const int h = XS ? w % a.H : w;
+    const int item = blockIdx.x * DEC_WARPS + w, h = item % a.H;
+    const int groups = XS ? (a.beam + NB - 1) / NB : 1;
+    const int set = item / a.H;                          // row, or (sentence, four of its beams)
+    const int b0 = XS ? set % groups * NB : 0;
+    const int r = XS ? set / groups * a.beam + b0 : set;
+    if (r >= a.R) return;
+    const int nb = XS ? min(NB, a.beam - b0) : 1;
     int n, t = 0;
     if (a.cross) {
         n = a.src_len[r / a.beam];
@@ -63,134 +74,62 @@ __global__ void __launch_bounds__(XS ? 32 * 32 : 32 * 16) attn_decode(AttnDecArg
         t = *a.t_ptr;
         n = t + 1;
     }
-    const int cap = a.T;  // key capacity: cache length / padded source length
-    int *prow = dsm;      // [cap] physical row of every key position (shared by the heads of this row)
-    int *sc = XS ? dsm + w * cap : dsm + cap + h * cap;  // per warp [cap]: scores, then weights
-    if (!XS) {
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            int p;
-            if (a.cross) p = r / a.beam;
-            else p = (a.anc && j < t) ? a.anc[(size_t)r * a.T + j] : r;
-            prow[j] = p;
-        }
-        __syncthreads();
-        if (h >= a.H) return;
+    const int cap = (a.T + 15) & ~15;  // key capacity: cache length / padded source length
+    const bool gather = !XS && !a.cross && a.anc;  // positions live in other rows' caches
+    int *sc = dsm + w * (NB + (gather ? 1 : 0)) * cap;  // this warp's [NB][cap] scores, then weights
+    int *prow = sc + NB * cap;                          // [cap] physical row of every key position
+    if (gather) {
+        for (int j = lane; j < n; j += 32) prow[j] = j < t ? a.anc[(size_t)r * a.T + j] : r;
+        __syncwarp();
     }
-    const int psent = r / a.beam;  // XS: the sentence of every key
-    auto prow_of = [&](int j) { return XS ? psent : prow[j]; };
-
-    constexpr int QC = DH / 16;
-    int4 qv[QC];
-    const int4 *qp = reinterpret_cast<const int4 *>(a.q + (size_t)r * a.H * DH + h * DH);
+    const DecRows rows{a.kc, a.vc, gather ? prow : nullptr, a.cross ? r / a.beam : r, a.H, h, a.T, DH};
+    const int d = a.H * DH;
+    attn_rows<DH, NB, true, LONGK>(
+        a.q + (size_t)r * d + h * DH, d, nb, n, a.sigma, a.rho, sc, cap, rows, [&](int b, int e, const uint32_t (&words)[DH / 32]) {
+            const size_t o = (size_t)(r + b) * d + h * DH + e;
+            const bool al = (reinterpret_cast<uintptr_t>(a.ctx) & 3) == 0;
 #pragma unroll
-    for (int c = 0; c < QC; c++) qv[c] = qp[c];
-
-    float mx = -INFINITY;
-#pragma unroll 4
-    for (int j = lane; j < n; j += 32) {
-        const int4 *kr = reinterpret_cast<const int4 *>(a.kc + (((size_t)prow_of(j) * a.H + h) * a.T + j) * DH);
-        int acc = 0;
+            for (int i = 0; i < DH / 32; i++) {
+                if (al) {
+                    reinterpret_cast<uint32_t *>(a.ctx + o)[i] = words[i];
+                } else {
 #pragma unroll
-        for (int c = 0; c < QC; c++) acc = dot16(qv[c], kr[c], acc);
-        float s = __fmul_rn(__int2float_rn(acc), a.sigma);
-        sc[j] = __float_as_int(s);
-        mx = fmaxf(mx, s);
-    }
-    mx = warp_max_f(mx);
-    long long Z = 0;
-    for (int j = lane; j < n; j += 32) {
-        int E = softmax_weight(__fadd_rn(__int_as_float(sc[j]), -mx));
-        sc[j] = E;
-        Z += E;
-    }
-    Z = warp_sum_ll(Z);
-    __syncwarp();
-
-    // context: the warp takes CG keys at a time, one per group of 8 lanes;
-    // lane gl of a group holds EPG consecutive elements of the head, read as
-    // one EPG-byte load per key.  N_e = sum_j E_j v_j[e] is split into 12-bit
-    // halves of E_j so that every partial stays an exact int32.
-    constexpr int CG = 4, LPG = 32 / CG, EPG = DH / LPG;
-    using VecT = typename std::conditional<EPG == 4, uint32_t, typename std::conditional<EPG == 8, uint2, uint4>::type>::type;
-    const int grp = lane / LPG, gl = lane % LPG;
-    int hi[EPG], lo[EPG];
-#pragma unroll
-    for (int u = 0; u < EPG; u++) hi[u] = lo[u] = 0;
-    auto vload = [&](int j) -> VecT {
-        return *reinterpret_cast<const VecT *>(a.vc + (((size_t)prow_of(j) * a.H + h) * a.T + j) * DH + gl * EPG);
-    };
-    auto vacc = [&](int j, const VecT &raw) {
-        const int E = sc[j];
-        const int Eh = E >> 12, El = E & 4095;
-#pragma unroll
-        for (int u = 0; u < EPG; u++) {
-            const int v = (int)(int8_t)(vec_word(raw, u >> 2) >> (8 * (u & 3)));
-            hi[u] += Eh * v;
-            lo[u] += El * v;
-        }
-    };
-    // groups of UJ rounds: every value load of the batch is issued before any
-    // is used, so their latencies overlap
-    constexpr int UJ = DH == 128 ? 2 : 4;
-    int j0 = 0;
-    for (; j0 + CG * UJ <= n; j0 += CG * UJ) {
-        VecT raw[UJ];
-#pragma unroll
-        for (int u = 0; u < UJ; u++) raw[u] = vload(j0 + u * CG + grp);
-#pragma unroll
-        for (int u = 0; u < UJ; u++) vacc(j0 + u * CG + grp, raw[u]);
-    }
-    for (int j = j0 + grp; j < n; j += CG) vacc(j, vload(j));
-    // sum over the CG groups (lanes gl, gl+8, gl+16, gl+24): every lane gets the totals
-#pragma unroll
-    for (int u = 0; u < EPG; u++) {
-#pragma unroll
-        for (int o = LPG; o < 32; o <<= 1) {
-            hi[u] += __shfl_xor_sync(0xFFFFFFFFu, hi[u], o);
-            lo[u] += __shfl_xor_sync(0xFFFFFFFFu, lo[u], o);
-        }
-    }
-    // lane (grp, gl) writes elements gl * EPG + grp * EPG / CG + [0, EPG / CG)
-    constexpr int OPL = EPG / CG;
-    const size_t o = (size_t)r * a.H * DH + h * DH + gl * EPG + grp * OPL;
-#pragma unroll
-    for (int u = 0; u < EPG; u++) {
-        if (u / OPL == grp) {
-            long long N = (long long)hi[u] * 4096 + lo[u];
-            const int8_t v = q8_quotient(N, Z, a.rho, rn32_div);
-            a.ctx[o + u - grp * OPL] = v;
-            if (a.ctx16) a.ctx16[o + u - grp * OPL] = __short2half_rn(v);
-        }
-    }
+                    for (int k = 0; k < 4; k++) a.ctx[o + 4 * i + k] = (int8_t)(words[i] >> (8 * k));
+                }
+                if (a.ctx16) {
+                    uint32_t lo, hi;
+                    codes_to_half2((int)words[i], lo, hi);
+                    reinterpret_cast<uint32_t *>(a.ctx16 + o)[2 * i] = lo;
+                    reinterpret_cast<uint32_t *>(a.ctx16 + o)[2 * i + 1] = hi;
+                }
+            }
+        });
 }
 
 cudaError_t launch_attention_decode(const AttnDecArgs &a, cudaStream_t st) {
     if (a.H > 16 || a.T < 1 || a.T > DEC_MAX_KEYS) return cudaErrorInvalidValue;
-    // cross attention with beams: the beams of a sentence share a block, when
-    // there are sentences enough for half of the SMs (measured on 152 SMs:
-    // 3.8 us per step faster at 128 sentences, 1.7 us slower at 32)
-    const bool xs = a.cross && a.beam > 1 && a.beam * a.H <= 32 && a.R % a.beam == 0 &&
+    // cross attention with beams: a sentence's beams share a warp when there are
+    // sentences enough for half of the SMs (with fewer, a warp per beam keeps
+    // more SMs busy)
+    const bool xs = a.cross && a.T <= ATT_CORE_MAX_KEYS && a.beam > 1 && a.R % a.beam == 0 &&
                     2 * (a.R / a.beam) >= device_sm_count();
-    const size_t smem = (size_t)(xs ? a.beam * a.H : 1 + a.H) * a.T * sizeof(int);
-    const dim3 block(32 * a.H * (xs ? a.beam : 1));
-    const int grid = xs ? a.R / a.beam : a.R;
+    const long items = (long)a.H * (xs ? (a.R / a.beam) * ((a.beam + 3) / 4) : a.R);
+    const size_t smem = (size_t)DEC_WARPS * (xs ? 4 : !a.cross && a.anc ? 2 : 1) * ((a.T + 15) & ~15) * sizeof(int);
+    const dim3 block(32 * DEC_WARPS);
+    const int grid = (int)((items + DEC_WARPS - 1) / DEC_WARPS);
+    auto go = [&](auto dh) {
+        constexpr int DH = decltype(dh)::value;
+        if (xs) launch_pdl(attn_decode<DH, true, false>, grid, block, smem, st, a);
+        else if (a.T > ATT_CORE_MAX_KEYS) launch_pdl(attn_decode<DH, false, true>, grid, block, smem, st, a);
+        else launch_pdl(attn_decode<DH, false, false>, grid, block, smem, st, a);
+        return cudaGetLastError();
+    };
     switch (a.dh) {
-        case 32:
-            if (xs) launch_pdl(attn_decode<32, true>, grid, block, smem, st, a);
-            else launch_pdl(attn_decode<32, false>, grid, block, smem, st, a);
-            break;
-        case 64:
-            if (xs) launch_pdl(attn_decode<64, true>, grid, block, smem, st, a);
-            else launch_pdl(attn_decode<64, false>, grid, block, smem, st, a);
-            break;
-        case 128:
-            if (xs) launch_pdl(attn_decode<128, true>, grid, block, smem, st, a);
-            else launch_pdl(attn_decode<128, false>, grid, block, smem, st, a);
-            break;
-        default:
-            return cudaErrorInvalidValue;
+        case 32: return go(std::integral_constant<int, 32>{});
+        case 64: return go(std::integral_constant<int, 64>{});
+        case 128: return go(std::integral_constant<int, 128>{});
+        default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -562,14 +501,20 @@ namespace mnmt {
 // (called once per process before any launch or stream capture).
 cudaError_t attention_init() {
     cudaError_t err = cudaSuccess;
-    int dec = (1 + 16) * DEC_MAX_KEYS * (int)sizeof(int);
-    const int xs = 32 * DEC_MAX_KEYS * (int)sizeof(int);  // up to 32 (beam, head) warps
-    if (!err) err = cudaFuncSetAttribute(attn_decode<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dec);
-    if (!err) err = cudaFuncSetAttribute(attn_decode<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dec);
-    if (!err) err = cudaFuncSetAttribute(attn_decode<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dec);
-    if (!err) err = cudaFuncSetAttribute(attn_decode<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, xs);
-    if (!err) err = cudaFuncSetAttribute(attn_decode<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, xs);
-    if (!err) err = cudaFuncSetAttribute(attn_decode<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, xs);
+    const int dec = DEC_WARPS * 2 * DEC_MAX_KEYS * (int)sizeof(int);
+    const int xs = DEC_WARPS * 4 * ATT_CORE_MAX_KEYS * (int)sizeof(int);
+    auto dec_attr = [&](auto k, int smem) {
+        if (!err) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    };
+    dec_attr(attn_decode<32, false, false>, dec);
+    dec_attr(attn_decode<64, false, false>, dec);
+    dec_attr(attn_decode<128, false, false>, dec);
+    dec_attr(attn_decode<32, true, false>, xs);
+    dec_attr(attn_decode<64, true, false>, xs);
+    dec_attr(attn_decode<128, true, false>, xs);
+    dec_attr(attn_decode<32, false, true>, dec);
+    dec_attr(attn_decode<64, false, true>, dec);
+    dec_attr(attn_decode<128, false, true>, dec);
     auto enc = [](int dh) { return ENC_MAX_KEYS * (dh + 16) + ENC_MAX_KEYS * dh + ENC_WARPS * ENC_MAX_KEYS * 4; };
     if (!err) err = cudaFuncSetAttribute(attn_encoder<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc(32));
     if (!err) err = cudaFuncSetAttribute(attn_encoder<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc(64));

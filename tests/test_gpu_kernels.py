@@ -261,3 +261,25 @@ def test_layernorm_warp_rows(M, d, scale):
     assert host(status)[0] == 0
     assert np.array_equal(host(of).view(np.uint32), ref_f.view(np.uint32))
     assert np.array_equal(host(oq), ref_q)
+
+
+@pytest.mark.parametrize("R,H,dh,T", [(1, 1, 64, 1), (3, 5, 32, 17), (2, 3, 128, 33), (5, 4, 64, 512), (2, 2, 64, 513), (2, 3, 32, 1024),
+                                      (1, 2, 128, 1023)])
+@pytest.mark.parametrize("flat", [False, True])
+def test_attention_core_edges(R, H, dh, T, flat):
+    """The tensor-core attention core: one key, ragged and whole steps of 16
+    keys, 512 equal weights of 2^24 against values of +-127 (the largest exact
+    sums), more than 512 keys (sums moved to int32), odd numbers of warps."""
+    q = synth.uniform_int8(1, "q", (R, H, dh))
+    Kc, Vc = synth.uniform_int8(2, "k", (R, H, T, dh)), synth.uniform_int8(3, "v", (R, H, T, dh))
+    if flat:
+        q[:] = 0
+        Vc[:, 0] = 127
+        Vc[:, -1, :, ::2] = -127
+    n_keys = np.array([max(1, T - 7 * i) for i in range(R)], np.int32)
+    for sigma in (np.float32(1e-4), np.float32(3e-3)):
+        ctx = torch.zeros(R * H * dh + 1, dtype=torch.int8, device="cuda")
+        for off in (0, 1):  # any alignment of the output
+            mnmt.mnmt_attention_decode(dev(q), dev(Kc), dev(Vc), dev(n_keys), R, H, dh, T, sigma, np.float32(0.97), ctx[off:])
+            got = host(ctx[off: off + R * H * dh]).reshape(R, H, dh)
+            assert np.array_equal(got, O.attention_decode(q, Kc, Vc, n_keys, sigma, np.float32(0.97)))
