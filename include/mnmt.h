@@ -217,8 +217,9 @@ int64_t mnmt_debug_tap(mnmt_session *s, int32_t tap, int32_t layer, void *host_d
 /* Which decode-step implementation the session uses for the batch encoded
  * last: 1 = the single thread-block-cluster step (greedy batches of at most 4
  * sentences whose shapes fit one cluster's shared memory), 0 = the multi-kernel
- * step; negative on error.  Setting MNMT_DECODE_CLUSTER=0 in the environment
- * before the first decode of a batch forces the multi-kernel step.  Both give
+ * step (whose decoder layers run as one kernel where the model's shape allows
+ * it, else a kernel per operation); negative on error.  Setting MNMT_DECODE_CLUSTER=0 in the environment
+ * before the first decode of a batch forces the kernel-per-operation step.  Both give
  * bit-identical results. */
 int mnmt_session_decode_path(mnmt_session *s);
 

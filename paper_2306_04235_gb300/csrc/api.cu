@@ -70,6 +70,7 @@ static int lib_init() {
     if (e == cudaSuccess) e = attention_init();
     if (e == cudaSuccess) e = rows_init();
     if (e == cudaSuccess) e = decode_cluster_init();
+    if (e == cudaSuccess) e = decode_rows_init();
     if (e == cudaSuccess) e = linear_tc_init();
     if (e != cudaSuccess) return fail(MNMT_ECUDA, "kernel set-up failed: %s", cudaGetErrorString(e));
     g_init_done[dev] = true;
@@ -591,6 +592,14 @@ struct mnmt_session {
     int dc_nc = 0;
     size_t dc_smem = 0;
     int dc_flags = -1;  // the compiled-in model bits of its step kernel (dc_flags)
+    // batched decode step on clusters of 8 dr_nb rows
+    DrParams *d_dr = nullptr;
+    uint8_t *dr_w = nullptr;  // the decoder's weights as it consumes them
+    bool rows_ok = false;   // the model and the session allow it
+    bool use_rows = false;
+    int dr_nb = 0, dr_hpc = 0, dr_nc = 0, dr_clusters = 0;
+    int dr_packed = 0;      // heads per CTA that dr_w is packed for
+    size_t dr_smem = 0;
 };
 
 static int poison(mnmt_session *s, int code) {
@@ -639,6 +648,12 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
         off += (bytes + 255) & ~(size_t)255;
         return at;
     };
+    // the batched decode step (decode_rows.cu), where greedy batches too small
+    // for it have the single-cluster one: its packed weights live in the arena
+    const char *tc_env = std::getenv("MNMT_TC");
+    const bool rows_ok = tc_ok && !(tc_env && tc_env[0] == '0') && c.pre_ln && m->dec_self[0].qkv.w &&
+                         (beam > 1 || max_batch > DC_RMAX) && dr_shape_ok(c.d_model, c.n_heads, c.d_ffn, c.d_embed, c.n_dec);
+    const size_t drw_bytes = rows_ok ? dr_bytes(c.d_model, c.d_ffn, c.n_dec) : 0;
     const size_t qkv_bytes = lean ? std::max(ME * 3 * d, rows * F) : ME * 3 * d;
     size_t o_resid = piece(rows * d * 4), o_act = piece(rows * (d > F ? d : F)), o_qkv = piece(qkv_bytes),
            o_ctx = lean ? o_act : piece(rows * d), o_hid = lean ? o_qkv : piece(rows * F), o_qbuf = piece(R * d),
@@ -650,7 +665,8 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
            o_anc = piece(R * max_len * 4), o_keys = piece(R * 8), o_cand = piece(R * beam * 8),
            o_logits = piece(beam > 1 ? R * V * 4 : 256), o_outids = piece((size_t)max_batch * max_len * 4),
            o_outlens = piece((size_t)max_batch * 4), o_outsc = piece((size_t)max_batch * 4),
-           o_state = piece(ST_N * 4), o_dc = piece(sizeof(DcParams)), o_dcln = piece((6 * L + 2) * d * 4);
+           o_state = piece(ST_N * 4), o_dc = piece(sizeof(DcParams)), o_dcln = piece((6 * L + 2) * d * 4),
+           o_dr = piece(rows_ok ? sizeof(DrParams) : 0), o_drw = piece(drw_bytes);
     const size_t kmax = std::max(d, std::max(F, (size_t)c.d_embed));
     const bool tc_any = tc_ok && rows >= TC_MIN_ROWS;
     size_t o_a16 = piece(tc_any ? rows * kmax * 2 : 256);
@@ -701,17 +717,16 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
     s->state = reinterpret_cast<int *>(a + o_state);
     s->d_dc = reinterpret_cast<DcParams *>(a + o_dc);
     s->dc_ln = reinterpret_cast<float *>(a + o_dcln);
+    s->d_dr = reinterpret_cast<DrParams *>(a + o_dr);
     s->a16 = reinterpret_cast<__half *>(a + o_a16);
     s->act16 = reinterpret_cast<__half *>(a + o_act16);
     s->ctx16 = reinterpret_cast<__half *>(a + o_ctx16);
     s->hid16 = reinterpret_cast<__half *>(a + o_hid16);
     s->encq16 = reinterpret_cast<__half *>(a + o_encq16);
-    {
-        const char *v = std::getenv("MNMT_TC");
-        s->use_tc = tc_ok && !(v && v[0] == '0') && rows >= TC_MIN_ROWS;
-    }
-    if (cudaMemsetAsync(s->arena, 0, off, m->stream) != cudaSuccess ||
-        cudaStreamSynchronize(m->stream) != cudaSuccess) {
+    s->use_tc = tc_ok && !(tc_env && tc_env[0] == '0') && rows >= TC_MIN_ROWS;
+    s->rows_ok = rows_ok;
+    s->dr_w = a + o_drw;
+    if (cudaMemsetAsync(s->arena, 0, off, m->stream) != cudaSuccess || cudaStreamSynchronize(m->stream) != cudaSuccess) {
         mnmt_session_free(s);
         return fail(MNMT_ECUDA, "arena initialisation failed");
     }
@@ -932,8 +947,8 @@ static int dc_flags(const mnmt_config &c, const mnmt_model *m, int R, int att_lw
     return (c.pre_ln ? 1 : 0) | (m->factorised ? 2 : 0) | (R * c.d_model > 256 ? 4 : 0) | (att_lw << 3);
 }
 
-// one decoder step for all B*k hypotheses (captured into a graph)
-int issue_decode_step(mnmt_session *s) {
+// the embedding and every decoder layer of one step, a kernel per operation
+int issue_decoder_layers(mnmt_session *s) {
     mnmt_model *m = s->m;
     const mnmt_config &c = m->c;
     const int d = c.d_model, F = c.d_ffn, H = c.n_heads, dh = d / H;
@@ -942,25 +957,6 @@ int issue_decode_step(mnmt_session *s) {
     const int *done = s->state + ST_DONE;
     int *t_ptr = s->state + ST_T;
     int *status = s->state + ST_STATUS;
-    if (s->use_cluster) {
-        LK(launch_decode_cluster(s->d_dc, dh, s->dc_nc, s->dc_smem, m->wq != 8, R == 1, s->dc_flags, st));
-        GreedyArgs g;
-        g.keys = s->keys;
-        g.tok = s->tok;
-        g.fin = s->fin;
-        g.hist = s->hist;
-        g.t_ptr = t_ptr;
-        g.done = s->state + ST_DONE;
-        g.tmax_ptr = s->state + ST_TMAX;
-        g.R = R;
-        g.T = s->Tcap;
-        g.eos = c.eos_id;
-        g.pad = c.pad_id;
-        g.pending = s->state + ST_PENDING;
-        LK(launch_vocab_greedy(s->act, m->out.w, m->out.s, m->out.b, m->s_dout, R, c.vocab, d, s->keys,
-                               s->state + ST_TICKET, g, s->dc_nc, st));
-        return MNMT_OK;
-    }
     {
         EmbedArgs e;
         std::memset(&e, 0, sizeof(e));
@@ -1078,6 +1074,43 @@ int issue_decode_step(mnmt_session *s) {
             rc = ln_after_residual(s, R, m->dec_final, Fb.ln, m->s_dout, s->act, done);
         }
         if (rc) return rc;
+    }
+    return MNMT_OK;
+}
+
+// one decoder step for all B*k hypotheses (captured into a graph)
+int issue_decode_step(mnmt_session *s) {
+    mnmt_model *m = s->m;
+    const mnmt_config &c = m->c;
+    const int d = c.d_model, H = c.n_heads, dh = d / H;
+    const int R = s->B * s->k;
+    cudaStream_t st = m->stream;
+    const int *done = s->state + ST_DONE;
+    int *t_ptr = s->state + ST_T;
+    int *status = s->state + ST_STATUS;
+    if (s->use_cluster) {
+        LK(launch_decode_cluster(s->d_dc, dh, s->dc_nc, s->dc_smem, m->wq != 8, R == 1, s->dc_flags, st));
+        GreedyArgs g;
+        g.keys = s->keys;
+        g.tok = s->tok;
+        g.fin = s->fin;
+        g.hist = s->hist;
+        g.t_ptr = t_ptr;
+        g.done = s->state + ST_DONE;
+        g.tmax_ptr = s->state + ST_TMAX;
+        g.R = R;
+        g.T = s->Tcap;
+        g.eos = c.eos_id;
+        g.pad = c.pad_id;
+        g.pending = s->state + ST_PENDING;
+        LK(launch_vocab_greedy(s->act, m->out.w, m->out.s, m->out.b, m->s_dout, R, c.vocab, d, s->keys,
+                               s->state + ST_TICKET, g, s->dc_nc, st));
+        return MNMT_OK;
+    }
+    if (s->use_rows) {
+        LK(launch_decode_rows(s->d_dr, s->dr_nb, s->dr_hpc, s->dr_nc, s->dr_clusters, s->dr_smem, st));
+    } else if (int rc = issue_decoder_layers(s)) {
+        return rc;
     }
     if (s->k == 1) {
         Epi e = base_epi(EPI_ARGMAX, m->s_dout, m->out);
@@ -1213,6 +1246,85 @@ int setup_cluster_step(mnmt_session *s) {
     return MNMT_OK;
 }
 
+// The batched step (decode_rows.cu) where the single-cluster step does not
+// apply: as few rows per cluster as still keep every cluster resident at once
+// (a second wave of clusters would double the step), one head per CTA before
+// two: 15 clusters of eight CTAs fit on 152 SMs, 36 of four.  It was faster than
+// the kernel-per-operation step at every batch measured (12+2 layers, d = 256,
+// beam 4, 1 .. 64 sentences: 139 -> 115 .. 216 -> 158 us per step; 6+6 layers,
+// d = 512, 1 .. 128 sentences: 314 -> 292 .. 665 -> 621).
+// MNMT_DECODE_CLUSTER=0 forces the kernel-per-operation step.
+int setup_rows_step(mnmt_session *s) {
+    mnmt_model *m = s->m;
+    const mnmt_config &c = m->c;
+    s->use_rows = false;
+    const char *env = getenv("MNMT_DECODE_CLUSTER");
+    if (!s->rows_ok || s->use_cluster || (env && env[0] == '0')) return MNMT_OK;
+    const int R = s->B * s->k;
+    static_assert(sizeof(DrParams) % 16 == 0, "the parameter block is copied in 16-byte chunks");
+    DrParams P;
+    std::memset(&P, 0, sizeof(P));
+    P.R = R; P.d = c.d_model; P.H = c.n_heads; P.F = c.d_ffn; P.E = c.d_embed; P.V = c.vocab; P.T = s->Tcap;
+    P.n_dec = c.n_dec; P.beam = s->k;
+    P.stream = s->dr_w;
+    P.emb_q = m->emb_q; P.emb_s = m->emb_s; P.pe = m->pe; P.emb_scale = m->emb_scale;
+    if (m->factorised) { P.proj_w = m->proj.w; P.proj_s = m->proj.s; P.proj_b = m->proj.b; }
+    P.fin_g = m->dec_final.g; P.fin_b = m->dec_final.b; P.inv_dout = 1.0f / m->s_dout;
+    P.tok = s->tok; P.src_len = s->src_lens; P.anc = s->anc; P.t_ptr = s->state + ST_T; P.done = s->state + ST_DONE;
+    P.act_out = s->act; P.act16_out = out16_for(s, s->act, R); P.resid_out = s->resid; P.status = s->state + ST_STATUS;
+    for (int l = 0; l < c.n_dec; l++) {
+        const SelfBlk &A = m->dec_self[l];
+        const CrossBlk &X = m->dec_cross[l];
+        const FfnBlk &Fb = m->dec_ffn[l];
+        DrLayer &Y = P.layer[l];
+        Y.ln1_g = A.ln.g; Y.ln1_b = A.ln.b; Y.ln2_g = X.ln.g; Y.ln2_b = X.ln.b; Y.ln3_g = Fb.ln.g; Y.ln3_b = Fb.ln.b;
+        Y.inv_in1 = 1.0f / A.s_in; Y.inv_in2 = 1.0f / X.s_in; Y.inv_in3 = 1.0f / Fb.s_in;
+        Y.sigma1 = A.sigma; Y.rho1 = A.rho; Y.sigma2 = X.sigma; Y.rho2 = X.rho;
+        Y.lin[0] = DrLin{A.qkv.s, A.qkv.b, A.inv_qkv, A.s_in, 0.0f};
+        Y.lin[1] = DrLin{A.o.s, A.o.b, nullptr, A.s_ctx, A.gamma};
+        Y.lin[2] = DrLin{X.q.s, X.q.b, X.inv_q, X.s_in, 0.0f};
+        Y.lin[3] = DrLin{X.o.s, X.o.b, nullptr, X.s_ctx, X.gamma};
+        Y.lin[4] = DrLin{Fb.w1.s, Fb.w1.b, Fb.inv_h, Fb.s_in, 0.0f};
+        Y.lin[5] = DrLin{Fb.w2.s, Fb.w2.b, nullptr, Fb.s_h, Fb.gamma};
+        Y.self_k = s->sk + l * s->sk_layer; Y.self_v = s->sv + l * s->sk_layer;
+        Y.cross_k = s->ck + l * s->ck_layer; Y.cross_v = s->cv + l * s->ck_layer;
+    }
+    // laid out for the session's longest source: only S changes with the batch
+    P.S = s->Smax;
+    for (const auto &v : {std::pair<int, int>{1, 1}, {2, 1}, {4, 1}, {2, 2}, {4, 2}}) {
+        const int nb = v.first, hpc = v.second;
+        const size_t smem = dr_layout(P, nb, hpc, 227 * 1024);
+        if (smem == (size_t)-1) continue;
+        const int clusters = (R + 8 * nb - 1) / (8 * nb), fit = dr_max_clusters(nb, hpc, P.nc, smem);
+        if (fit < 1) continue;
+        s->use_rows = true;
+        s->dr_nb = nb;
+        s->dr_hpc = hpc;
+        s->dr_clusters = clusters;
+        s->dr_smem = smem;
+        if (clusters <= fit) break;
+    }
+    if (!s->use_rows) return MNMT_OK;
+    dr_layout(P, s->dr_nb, s->dr_hpc, 227 * 1024);
+    s->dr_nc = P.nc;
+    if (s->dr_packed != s->dr_hpc) {
+        DrPack pk;
+        std::memset(&pk, 0, sizeof(pk));
+        pk.n_dec = c.n_dec;
+        for (int l = 0; l < c.n_dec; l++) {
+            const int8_t *const w[6] = {m->dec_self[l].qkv.w, m->dec_self[l].o.w,  m->dec_cross[l].q.w,
+                                        m->dec_cross[l].o.w,  m->dec_ffn[l].w1.w, m->dec_ffn[l].w2.w};
+            std::memcpy(pk.w[l], w, sizeof(w));
+        }
+        CK(dr_pack(pk, P.d, P.H, s->dr_hpc, P.F, s->dr_w, m->stream));
+        s->dr_packed = s->dr_hpc;
+    }
+    P.S = s->S;
+    CK(cudaMemcpyAsync(s->d_dr, &P, sizeof(P), cudaMemcpyHostToDevice, m->stream));
+    CK(cudaStreamSynchronize(m->stream));  // P lives on this stack frame
+    return MNMT_OK;
+}
+
 // capture `steps` consecutive decode steps into one executable graph
 int capture_steps(mnmt_session *s, int steps, cudaGraphExec_t *out) {
     cudaStream_t st = s->m->stream;
@@ -1256,12 +1368,13 @@ int capture_steps(mnmt_session *s, int steps, cudaGraphExec_t *out) {
 
 int ensure_graph(mnmt_session *s) {
     if (s->gexec && s->graph_B == s->B && s->graph_S == s->S) return MNMT_OK;
-    if (s->gexec && s->graph_B == s->B && s->use_cluster) {
-        // the cluster step reads the padded source length from its parameter
+    if (s->gexec && s->graph_B == s->B && (s->use_cluster || s->use_rows)) {
+        // the cluster steps read the padded source length from their parameter
         // block: update it in stream order and keep the captured graphs
         s->dc_S = s->S;
-        CK(cudaMemcpyAsync(reinterpret_cast<uint8_t *>(s->d_dc) + offsetof(DcParams, S), &s->dc_S, sizeof(int),
-                           cudaMemcpyHostToDevice, s->m->stream));
+        uint8_t *at = s->use_cluster ? reinterpret_cast<uint8_t *>(s->d_dc) + offsetof(DcParams, S)
+                                     : reinterpret_cast<uint8_t *>(s->d_dr) + offsetof(DrParams, S);
+        CK(cudaMemcpyAsync(at, &s->dc_S, sizeof(int), cudaMemcpyHostToDevice, s->m->stream));
         s->graph_S = s->S;
         return MNMT_OK;
     }
@@ -1271,12 +1384,13 @@ int ensure_graph(mnmt_session *s) {
             *ge = nullptr;
         }
     int rc = setup_cluster_step(s);
+    if (!rc) rc = setup_rows_step(s);
     if (rc) return rc;
     if ((rc = capture_steps(s, 1, &s->gexec))) return rc;
     // the cluster step also gets a graph of GRAPH_STEPS steps, inside which
     // each step's kernel starts while the previous step's vocabulary kernel
     // runs (programmatic dependent launch)
-    if (s->use_cluster && (rc = capture_steps(s, GRAPH_STEPS, &s->gexec_n))) return rc;
+    if ((s->use_cluster || s->use_rows) && (rc = capture_steps(s, GRAPH_STEPS, &s->gexec_n))) return rc;
     s->graph_B = s->B;
     s->graph_S = s->S;
     return MNMT_OK;
