@@ -577,6 +577,7 @@ struct mnmt_session {
     int32_t *src_ids, *src_lens, *tok, *fin, *hist, *parents, *anc, *out_ids, *out_lens;
     float *out_scores;
     unsigned long long *keys, *cand;
+    int *arrive;        // [Bmax] beam rows of a sentence that finished the step
     int *state;
     int *h_state = nullptr;  // pinned mirror of state, then a second slot for the look-ahead copy
     cudaEvent_t ev_look = nullptr;  // marks the look-ahead copy of translate's decode loop
@@ -663,6 +664,7 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
            o_tok = piece(R * 4), o_fin = piece(R * 4), o_cum = piece(R * 4),
            o_hist = piece((size_t)max_len * R * 4), o_par = piece((size_t)max_len * R * 4),
            o_anc = piece(R * max_len * 4), o_keys = piece(R * 8), o_cand = piece(R * beam * 8),
+           o_arrive = piece(beam > 1 ? (size_t)max_batch * 4 : 0),
            o_logits = piece(beam > 1 ? R * V * 4 : 256), o_outids = piece((size_t)max_batch * max_len * 4),
            o_outlens = piece((size_t)max_batch * 4), o_outsc = piece((size_t)max_batch * 4),
            o_state = piece(ST_N * 4), o_dc = piece(sizeof(DcParams)), o_dcln = piece((6 * L + 2) * d * 4),
@@ -710,6 +712,7 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
     s->anc = reinterpret_cast<int32_t *>(a + o_anc);
     s->keys = reinterpret_cast<unsigned long long *>(a + o_keys);
     s->cand = reinterpret_cast<unsigned long long *>(a + o_cand);
+    s->arrive = reinterpret_cast<int *>(a + o_arrive);
     s->logits = reinterpret_cast<float *>(a + o_logits);
     s->out_ids = reinterpret_cast<int32_t *>(a + o_outids);
     s->out_lens = reinterpret_cast<int32_t *>(a + o_outlens);
@@ -1148,6 +1151,7 @@ int issue_decode_step(mnmt_session *s) {
         b.t_ptr = t_ptr;
         b.done = s->state + ST_DONE;
         b.ticket = s->state + ST_TICKET;
+        b.arrive = s->arrive;
         b.tmax_ptr = s->state + ST_TMAX;
         b.B = s->B;
         b.k = s->k;

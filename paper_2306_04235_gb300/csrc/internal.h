@@ -196,6 +196,7 @@ struct BeamArgs {
     int32_t *anc;              // [R][T]
     unsigned long long *cand;  // [R][k] row candidates
     int *t_ptr, *done, *ticket;   // ticket[0..1]: arrival and running counters
+    int *arrive;                  // [B] rows of a sentence done (0 between steps)
     const int *tmax_ptr;          // steps of this translation (device)
     int B, k, V, T, eos, pad;     // T: cache / history capacity
     int *status;

@@ -659,50 +659,48 @@ __global__ void __launch_bounds__(NT) beam_rows_kernel(BeamArgs a) {
     block_select<KM, NT>(top, k, out, s_key);
 }
 
-// per sentence: best k of the k*k row candidates; reorder state
-__global__ void __launch_bounds__(256) beam_select_kernel(BeamArgs a) {
-    pdl_grid_wait();
-    if (*a.done) return;
-    const int b = blockIdx.x;
+// per sentence: best k of the k*k row candidates; reorder state (every thread
+// of the block; anc_old: [k][T] shared)
+MNMT_DEV void beam_select_sentence(const BeamArgs &a, int b, int nt, int nsent, int *anc_old) {
     const int k = a.k, V = a.V, T = a.T;
     const int t = *a.t_ptr;
-    __shared__ unsigned long long cand[BEAM_MAX * BEAM_MAX];
     __shared__ unsigned long long sel[BEAM_MAX];
     __shared__ int pfin[BEAM_MAX];
-    __shared__ int s_all;
-    extern __shared__ int anc_old[];  // [k][T]
+    __shared__ int s_all, s_last;
     const int r0 = b * k;
-    for (int i = threadIdx.x; i < k * k; i += blockDim.x) cand[i] = a.cand[(size_t)r0 * k + i];
-    for (int i = threadIdx.x; i < k; i += blockDim.x) pfin[i] = a.fin[r0 + i];
-    for (int i = threadIdx.x; i < k * t; i += blockDim.x) {
+    if (threadIdx.x < 32) {
+        // k rounds of a maximum over the k*k keys, eight per lane at most (keys
+        // are unique; at k = 4 one per lane).  Read from L2: rows on other SMs
+        // may have written them in this launch.
+        const int lane = threadIdx.x, per = (k * k + 31) >> 5;
+        unsigned long long mine[BEAM_MAX * BEAM_MAX / 32];
+#pragma unroll
+        for (int i = 0; i < BEAM_MAX * BEAM_MAX / 32; i++)
+            mine[i] = i < per && i * 32 + lane < k * k ? __ldcg(a.cand + (size_t)r0 * k + i * 32 + lane) : 0ull;
+        const int f = lane < k ? a.fin[r0 + lane] : 0;
+        if (lane < k) pfin[lane] = f;
+        int all = 1;
+        for (int i = 0; i < k; i++) {
+            unsigned long long m = mine[0];
+#pragma unroll
+            for (int j = 1; j < BEAM_MAX * BEAM_MAX / 32; j++) m = mine[j] > m ? mine[j] : m;
+            const unsigned long long best = warp_max_u64(m);
+#pragma unroll
+            for (int j = 0; j < BEAM_MAX * BEAM_MAX / 32; j++)
+                if (mine[j] == best) mine[j] = 0ull;
+            if (lane == 0) sel[i] = best;
+            const uint32_t idx = key_index(best);
+            const int p = (int)(idx / (uint32_t)V), n = (int)(idx - (uint32_t)p * V);
+            all &= __shfl_sync(0xFFFFFFFFu, f, p) || n == a.eos;
+        }
+        if (lane == 0) s_all = all;
+    }
+    for (int i = threadIdx.x; i < k * t; i += nt) {
         int rr = i / t, j = i - rr * t;
         anc_old[rr * T + j] = a.anc[(size_t)(r0 + rr) * T + j];
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        // k rounds of selection over k*k keys (unique keys, descending)
-        for (int i = 0; i < k; i++) {
-            unsigned long long best = 0ull;
-            int bi = 0;
-            for (int j = 0; j < k * k; j++)
-                if (cand[j] > best) {
-                    best = cand[j];
-                    bi = j;
-                }
-            sel[i] = best;
-            cand[bi] = 0ull;
-        }
-        int all = 1;
-        for (int i = 0; i < k; i++) {
-            uint32_t idx = key_index(sel[i]);
-            int p = (int)(idx / (uint32_t)V), n = (int)(idx - (uint32_t)p * V);
-            int f = pfin[p] || n == a.eos;
-            all &= f;
-        }
-        s_all = all;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
+    for (int i = threadIdx.x; i < k; i += nt) {
         unsigned long long key = sel[i];
         uint32_t idx = key_index(key);
         int p = (int)(idx / (uint32_t)V), n = (int)(idx - (uint32_t)p * V);
@@ -714,20 +712,19 @@ __global__ void __launch_bounds__(256) beam_select_kernel(BeamArgs a) {
         a.parents[(size_t)t * (a.B * k) + r] = p;
     }
     // ancestry: new row i takes parent p's positions 0..t-1 and p's own slot at t
-    for (int x = threadIdx.x; x < k * (t + 1); x += blockDim.x) {
+    for (int x = threadIdx.x; x < k * (t + 1); x += nt) {
         int i = x / (t + 1), j = x - i * (t + 1);
         uint32_t idx = key_index(sel[i]);
         int p = (int)(idx / (uint32_t)V);
         a.anc[(size_t)(r0 + i) * T + j] = (j < t) ? anc_old[p * T + j] : r0 + p;
     }
-    // the last block to finish decides whether every sentence is done
-    __shared__ int s_last;
+    // the last sentence to finish decides whether every sentence is done
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         if (!s_all) atomicAdd(a.ticket + 1, 1);  // sentences still running
         int prev = atomicAdd(a.ticket, 1);
-        s_last = prev == (int)gridDim.x - 1;
+        s_last = prev == nsent - 1;
     }
     __syncthreads();
     if (s_last && threadIdx.x == 0) {
@@ -740,11 +737,188 @@ __global__ void __launch_bounds__(256) beam_select_kernel(BeamArgs a) {
     }
 }
 
+__global__ void __launch_bounds__(256) beam_select_kernel(BeamArgs a) {
+    pdl_grid_wait();
+    if (*a.done) return;
+    extern __shared__ int anc_old[];  // [k][T]
+    beam_select_sentence(a, blockIdx.x, 256, gridDim.x, anc_old);
+}
+
+// ---------------------------------------------------------------------------
+// The same step for vocabularies of 4096 to 4096 NV entries (rows of whole,
+// aligned float4s), one block of 1024 threads per row and the row in registers:
+// the logits are read once, and the block that finishes a sentence's last row
+// selects for the sentence (no second kernel).
+//   threshold  the KC-th largest of the 32 warps' maxima: at least KC logits
+//              reach it and few more (about 9 of them for KC = 8), so listing
+//              those that do is a compare per logit and a handful of insertions;
+//   candidates the row's KC best logits, taken from that list by warp 1 while
+//              warp 0 computes lambda; then as in beam_rows_kernel, with its
+//              full scan where the candidates may not be exact.
+// Bound by issue (exp_own per logit) and the latency of its serial parts.
+// 128 rows of 32000 (32 x beam 4): step 128 -> 113 us with one launch less;
+// 512 rows: 621 -> 607.
+// ---------------------------------------------------------------------------
+constexpr int BRR_THREADS = 1024;
+constexpr int BRR_LIST = 256;
+
+template <int KM, int NV>
+__global__ void __launch_bounds__(BRR_THREADS, 1) beam_rows_reg_kernel(BeamArgs a) {
+    pdl_grid_wait();
+    if (*a.done) return;
+    constexpr int KC = KM + 4, NT = BRR_THREADS;
+    const int r = blockIdx.x, k = a.k, V = a.V;
+    const int lb = r % k;  // beam index within the sentence
+    unsigned long long *out = a.cand + (size_t)r * k;
+    extern __shared__ int anc_old[];  // [k][T]
+    __shared__ float s_mx[32], s_lam;
+    __shared__ long long s_z[32];
+    __shared__ unsigned long long s_list[BRR_LIST], s_cand[KC], s_key[32];
+    __shared__ int s_cnt, s_full, s_mine;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const float NI = -INFINITY;
+    if (a.fin[r]) {
+        // a finished hypothesis offers itself once, unchanged, with token PAD
+        if (threadIdx.x < k) out[threadIdx.x] = threadIdx.x == 0 ? pack_key(a.cum[r], (uint32_t)(lb * V + a.pad)) : 0ull;
+    } else {
+        const float *l = a.logits + (size_t)r * V;
+        const float4 *l4 = reinterpret_cast<const float4 *>(l);
+        const int n4 = V >> 2;
+        float4 v[NV];
+        float mx = NI;
+#pragma unroll
+        for (int i = 0; i < NV; i++) {
+            const int n = i * NT + threadIdx.x;
+            v[i] = n < n4 ? l4[n] : make_float4(NI, NI, NI, NI);
+        }
+#pragma unroll
+        for (int i = 0; i < NV; i++) mx = fmaxf(mx, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
+        mx = warp_max_f(mx);
+        if (lane == 0) s_mx[warp] = mx;
+        if (threadIdx.x == 0) s_cnt = 0;
+        __syncthreads();
+        const float wm = s_mx[lane];
+        const float m = warp_max_f(wm);
+        int rank = 0;  // of this lane's warp maximum (ties by lane)
+#pragma unroll
+        for (int i = 0; i < 32; i++) {
+            const float o = __shfl_sync(0xFFFFFFFFu, wm, i);
+            rank += (o > wm || (o == wm && i < lane)) ? 1 : 0;
+        }
+        const unsigned at = __ballot_sync(0xFFFFFFFFu, rank == KC - 1);
+        const float thr = at ? __shfl_sync(0xFFFFFFFFu, wm, __ffs(at) - 1) : NI;
+        uint32_t z = 0;  // at most 4 NV weights of 2^24
+#pragma unroll
+        for (int i = 0; i < NV; i++) {
+            z += (uint32_t)(softmax_weight(__fsub_rn(v[i].x, m)) + softmax_weight(__fsub_rn(v[i].y, m)) +
+                            softmax_weight(__fsub_rn(v[i].z, m)) + softmax_weight(__fsub_rn(v[i].w, m)));
+            if (fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)) >= thr && i * NT + (int)threadIdx.x < n4) {
+                const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (e[q] >= thr) {
+                        const int p = atomicAdd(&s_cnt, 1);
+                        if (p < BRR_LIST) s_list[p] = pack_key(e[q], (uint32_t)(4 * (i * NT + (int)threadIdx.x) + q));
+                    }
+            }
+        }
+        const long long zw = (long long)__reduce_add_sync(0xFFFFFFFFu, z & 0xFFFFu) +
+                             ((long long)__reduce_add_sync(0xFFFFFFFFu, z >> 16) << 16);
+        if (lane == 0) s_z[warp] = zw;
+        __syncthreads();
+        const int cnt = s_cnt;
+        if (warp == 0) {
+            const long long Z = warp_sum_ll(s_z[lane]);
+            // lambda = ln Z - 24 ln 2 (log of the normaliser of the 2^-24 weights)
+            if (lane == 0) s_lam = __double2float_rn(__dadd_rn(log_own(__ll2double_rn(Z)), -0x1.0a2b23f3bab73p+4));
+        } else if (warp == 1 && cnt <= BRR_LIST) {
+            unsigned long long key[BRR_LIST / 32];
+#pragma unroll
+            for (int i = 0; i < BRR_LIST / 32; i++) key[i] = i * 32 + lane < cnt ? s_list[i * 32 + lane] : 0ull;
+            for (int j = 0; j < KC; j++) {
+                unsigned long long mk = key[0];
+#pragma unroll
+                for (int i = 1; i < BRR_LIST / 32; i++) mk = key[i] > mk ? key[i] : mk;
+                const unsigned long long best = warp_max_u64(mk);
+#pragma unroll
+                for (int i = 0; i < BRR_LIST / 32; i++)
+                    if (key[i] == best) key[i] = 0ull;
+                if (lane == 0) s_cand[j] = best;
+            }
+        }
+        __syncthreads();
+        const float lam = s_lam, cum = a.cum[r];
+        if (warp == 0) {
+            // final keys of the KC best logits; the k best of them, best first
+            const unsigned long long cand = lane < KC && cnt <= BRR_LIST ? s_cand[lane] : 0ull;
+            float sc = 0.0f;
+            unsigned long long fk = 0ull;
+            if (cand) {
+                sc = __fadd_rn(cum, __fsub_rn(__fsub_rn(key_value(cand), m), lam));
+                fk = pack_key(sc, (uint32_t)(lb * V) + key_index(cand));
+            }
+            const float sc_last = __shfl_sync(0xFFFFFFFFu, sc, KC - 1);
+            const bool whole = __shfl_sync(0xFFFFFFFFu, cand, KC - 1) != 0ull;  // KC candidates
+            unsigned long long kth = 0ull;
+            for (int i = 0; i < k; i++) {
+                const unsigned long long best = warp_max_u64(fk);
+                if (fk == best) fk = 0ull;
+                if (lane == i) kth = best;
+            }
+            // every other element scores <= sc_last; it cannot displace the k-th
+            // key unless it can tie its score
+            const unsigned long long kk = __shfl_sync(0xFFFFFFFFu, kth, k - 1);
+            const bool exact = whole && sc_last < key_value(kk);
+            if (exact && lane < k) out[lane] = kth;
+            if (lane == 0) s_full = !exact;
+        }
+        __syncthreads();
+        if (s_full) {
+            // full scan of the scores (a tie at the candidate boundary; always
+            // while dead beams score -inf)
+            unsigned long long top[KM];
+#pragma unroll
+            for (int i = 0; i < KM; i++) top[i] = 0ull;
+            for (int n = threadIdx.x; n < V; n += NT)
+                topk_insert<KM>(top, k, pack_key(__fadd_rn(cum, __fsub_rn(__fsub_rn(l[n], m), lam)), (uint32_t)(lb * V + n)));
+            block_select<KM, NT>(top, k, out, s_key);
+        }
+    }
+    // the row's candidates are out; the last row of the sentence selects
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_mine = atomicAdd(a.arrive + r / k, 1) == k - 1;
+    }
+    __syncthreads();
+    if (!s_mine) return;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        a.arrive[r / k] = 0;
+    }
+    __syncthreads();
+    beam_select_sentence(a, r / k, NT, a.B, anc_old);
+}
+
+template <int KM>
+static cudaError_t launch_beam_rows_reg(const BeamArgs &a, cudaStream_t st) {
+    const size_t smem = (size_t)a.k * a.T * sizeof(int);
+    if (a.V <= 8192) launch_pdl(beam_rows_reg_kernel<KM, 2>, a.B * a.k, BRR_THREADS, smem, st, a);
+    else launch_pdl(beam_rows_reg_kernel<KM, 8>, a.B * a.k, BRR_THREADS, smem, st, a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_beam_step(const BeamArgs &a, cudaStream_t st) {
     if (a.k < 1 || a.k > BEAM_MAX) return cudaErrorInvalidValue;
     int R = a.B * a.k;
-    // up to one row per SM: the plain scan (its simple loops keep more loads
-    // in flight per warp); more rows: the candidate pass
+    if (a.V >= 4096 && a.V <= 32768 && a.V % 4 == 0 && (reinterpret_cast<uintptr_t>(a.logits) & 15) == 0) {
+        if (a.k <= 4) return launch_beam_rows_reg<4>(a, st);
+        if (a.k <= 8) return launch_beam_rows_reg<8>(a, st);
+        return launch_beam_rows_reg<16>(a, st);
+    }
+    // other vocabularies: several passes over the logits.  Up to one row per
+    // SM: the plain scan (its simple loops keep more loads in flight per warp);
+    // more rows: the candidate pass
     if (R <= device_sm_count()) {
         if (a.k <= 4) launch_pdl(beam_rows_kernel<4, BR_THREADS, false>, R, BR_THREADS, 0, st, a);
         else if (a.k <= 8) launch_pdl(beam_rows_kernel<8, BR_THREADS, false>, R, BR_THREADS, 0, st, a);
@@ -788,11 +962,21 @@ __global__ void finalize_kernel(FinalArgs a) {
     a.out_scores[b] = a.k > 1 ? a.cum[b * a.k] : 0.0f;
 }
 
-// Opt the beam reorder kernel into the shared memory of its largest shape
+// Opt the beam reorder kernels into the shared memory of their largest shape
 // (k = 16 hypotheses x 1024 positions); once per process, before any capture.
 cudaError_t rows_init() {
-    return cudaFuncSetAttribute(beam_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                BEAM_MAX * 1024 * (int)sizeof(int));
+    const int anc = BEAM_MAX * 1024 * (int)sizeof(int);
+    cudaError_t err = cudaFuncSetAttribute(beam_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, anc);
+    auto reg = [&](auto k) {
+        if (err == cudaSuccess) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, anc);
+    };
+    reg(beam_rows_reg_kernel<4, 2>);
+    reg(beam_rows_reg_kernel<4, 8>);
+    reg(beam_rows_reg_kernel<8, 2>);
+    reg(beam_rows_reg_kernel<8, 8>);
+    reg(beam_rows_reg_kernel<16, 2>);
+    reg(beam_rows_reg_kernel<16, 8>);
+    return err;
 }
 
 cudaError_t launch_finalize(const FinalArgs &a, cudaStream_t st) {

@@ -466,3 +466,30 @@ def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, 
             tr.close()
     for a, b in zip(out["1"], out["0"]):
         assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
+
+
+@pytest.mark.parametrize("V,beam", [(4096, 4), (8192, 2), (8196, 4), (20000, 3), (32768, 5), (5000, 16), (32764, 8)])
+@pytest.mark.parametrize("flat", [False, True])
+def test_beam_rows_in_registers(V, beam, flat, stream):
+    """The beam step that keeps a row's logits in registers: its vocabulary
+    limits, every list size, beams that share a 32-byte sector of candidates;
+    flat: an output bias that makes hundreds of logits tie (the candidate list
+    overflows and the row is scanned in full), with EOS among the first."""
+    cfg = synth.ModelConfig(1, 1, 64, 1, 64, V, 64, 1, 1, max_pos=32)
+    bias = {i: 40.0 for i in range(0, 900)} if flat else None
+    blob = synth.build_blob(cfg, 17, gamma_range=(0.5, 1.5), out_bias=bias)
+    if flat:  # equal logits: the tied embedding rows of the biased ids zeroed
+        off = 64
+        b = bytearray(blob)
+        b[off: off + 900 * 64] = bytes(900 * 64)
+        blob = bytes(b)
+    ids, lens = synth.source_batch(V, 5, 3, 9, 8)
+    T = 7
+    tr = mnmt.Translator(blob, 5, ids.shape[1], beam, T, stream)
+    try:
+        g_ids, g_len, g_sc = tr.translate(ids, lens, T)
+    finally:
+        tr.close()
+    o_ids, o_len, o_sc = O.translate(blob, ids, lens, beam, T)
+    assert np.array_equal(g_ids, o_ids) and np.array_equal(g_len, o_len)
+    assert np.array_equal(g_sc.view(np.uint32), o_sc.view(np.uint32))
