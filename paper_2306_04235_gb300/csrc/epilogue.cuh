@@ -56,6 +56,48 @@ MNMT_DEV void epi_store_y(const Epi &e, int m, int n, float y, int t) {
     }
 }
 
+// Sums over the LPC lanes of a group (lane sl of it) of V accumulators each,
+// scattered: in every step a lane hands half of its values to its partner and
+// keeps the other half, so a group of 8 lanes with 32 values takes 28 shuffles
+// instead of 96 and each lane ends with V / LPC of them to finish.  Value i of
+// the result is the caller's value gemv_first(sl) + i; when V < LPC, several
+// lanes end with the same value and gemv_owner picks one.
+template <int V, int LPC>
+MNMT_DEV void gemv_reduce(int (&acc)[V], int sl) {
+    int n = V;
+#pragma unroll
+    for (int o = LPC / 2; o > 0; o >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = (sl & o) != 0;
+#pragma unroll
+            for (int i = 0; i < V / 2; i++) {
+                if (i < n) {
+                    const int send = up ? acc[i] : acc[i + n], keep = up ? acc[i + n] : acc[i];
+                    acc[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
+                }
+            }
+        } else {
+            acc[0] += __shfl_xor_sync(0xFFFFFFFFu, acc[0], o);
+        }
+    }
+}
+template <int V, int LPC>
+MNMT_DEV int gemv_first(int sl) {
+    int n = V, at = 0;
+#pragma unroll
+    for (int o = LPC / 2; o > 0; o >>= 1)
+        if (n > 1) {
+            n >>= 1;
+            if (sl & o) at += n;
+        }
+    return at;
+}
+template <int V, int LPC>
+MNMT_DEV bool gemv_owner(int sl) {
+    return V >= LPC || (sl & (LPC / V - 1)) == 0;
+}
+
 // epilogue of one output element; accf = fl(acc), the accumulator rounded to
 // fp32 (exact for |acc| <= 2^24)
 MNMT_DEV void epi_store_f(const Epi &e, int m, int n, float accf, int t) {

@@ -33,6 +33,11 @@ constexpr int SMALL_CHUNKED_MAX_M = 64;
 
 // MT: rows held (>= M); LPC: lanes per weight row (K/16 chunks spread over
 // LPC lanes); U: weight rows in flight per lane group.
+// Bound by latency at these sizes.  The first weights are read before the rows
+// of A are staged, and the lanes of a group share the reduction and the
+// epilogue (gemv_reduce; one lane per group finishing all of a column's rows
+// took as long as the products).  8 x 2048 x 512: 5.3 -> 2.8 us; 16 x 1536 x
+// 512: 8.2 -> 3.6; 1 x 32000 x 256 argmax: 5.2 -> 4.4.
 template <int MT, int LPC, int U>
 __global__ void __launch_bounds__(SM_THREADS) linear_smallm(const int8_t *__restrict__ A, int lda,
                                                            const int8_t *__restrict__ W, int M, int N,
@@ -40,7 +45,24 @@ __global__ void __launch_bounds__(SM_THREADS) linear_smallm(const int8_t *__rest
     pdl_grid_wait();
     if (e.skip && *e.skip) return;
     extern __shared__ int4 smA[];  // [MT][K/16]
+    __shared__ unsigned long long s_best[MT];
+    constexpr int NW = SM_THREADS / 32;
+    constexpr int GPW = 32 / LPC;        // lane groups per warp
+    constexpr int CPB = NW * GPW * U;    // columns per block pass
+    constexpr int V = U * MT;
     const int kc = K >> 4;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int grp = lane / LPC, sl = lane % LPC;
+    // column of (warp, group, u): base + (u * NW + warp) * GPW + grp
+    auto wload = [&](int base, int c, int4 (&w)[U]) {
+#pragma unroll
+        for (int u = 0; u < U; u++) {
+            const int n = base + (u * NW + warp) * GPW + grp;
+            w[u] = (n < N && c < kc) ? __ldg(reinterpret_cast<const int4 *>(W + (size_t)n * K) + c) : make_int4(0, 0, 0, 0);
+        }
+    };
+    int4 w[U];
+    wload(blockIdx.x * CPB, sl, w);  // on its way while the rows of A are staged
     // blockIdx.y selects the chunk of MT rows this block computes
     const int m0 = blockIdx.y * MT;
     A += (size_t)m0 * lda;
@@ -49,92 +71,64 @@ __global__ void __launch_bounds__(SM_THREADS) linear_smallm(const int8_t *__rest
         int m = i / kc, c = i - m * kc;
         smA[i] = (m < M) ? reinterpret_cast<const int4 *>(A + (size_t)m * lda)[c] : make_int4(0, 0, 0, 0);
     }
+    if (threadIdx.x < MT) s_best[threadIdx.x] = 0ull;
     __syncthreads();
     const int t = e.t_ptr ? *e.t_ptr : 0;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int GPW = 32 / LPC;              // lane groups per warp
-    constexpr int CPB = (SM_THREADS / 32) * GPW * U;  // columns per block pass
-    const int grp = lane / LPC, sl = lane % LPC;
     const bool argmax = e.mode == EPI_ARGMAX;
-    unsigned long long best[MT];
+    constexpr int PER = V >= LPC ? V / LPC : 1;  // outputs a lane finishes per pass
+    const int first = gemv_first<V, LPC>(sl);
+    const bool owner = gemv_owner<V, LPC>(sl);
+    unsigned long long best[PER];
 #pragma unroll
-    for (int m = 0; m < MT; m++) best[m] = 0ull;
+    for (int i = 0; i < PER; i++) best[i] = 0ull;
 
     for (int base = blockIdx.x * CPB; base < N; base += gridDim.x * CPB) {
-        int acc[U][MT];
+        int acc[V];
 #pragma unroll
-        for (int u = 0; u < U; u++)
-#pragma unroll
-            for (int m = 0; m < MT; m++) acc[u][m] = 0;
-        // column of (warp, group, u): base + (u * 8 + warp) * GPW + grp
+        for (int i = 0; i < V; i++) acc[i] = 0;
         for (int c0 = 0; c0 < kc; c0 += LPC) {
-            int c = c0 + sl;
-            int4 w[U];
-#pragma unroll
-            for (int u = 0; u < U; u++) {
-                int n = base + (u * (SM_THREADS / 32) + warp) * GPW + grp;
-                w[u] = (n < N && c < kc) ? __ldg(reinterpret_cast<const int4 *>(W + (size_t)n * K) + c)
-                                         : make_int4(0, 0, 0, 0);
-            }
+            const int c = c0 + sl;
+            if (c0 || base != (int)blockIdx.x * CPB) wload(base, c, w);
             if (c < kc) {
 #pragma unroll
                 for (int m = 0; m < MT; m++) {
                     int4 a = smA[m * kc + c];
 #pragma unroll
-                    for (int u = 0; u < U; u++) acc[u][m] = dot16(a, w[u], acc[u][m]);
+                    for (int u = 0; u < U; u++) acc[u * MT + m] = dot16(a, w[u], acc[u * MT + m]);
                 }
             }
         }
+        gemv_reduce<V, LPC>(acc, sl);
+        // every residual load first: the stores may alias them
+        float r[PER];
+        if (e.mode == EPI_RESID) {
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-#pragma unroll
-            for (int m = 0; m < MT; m++) {
-#pragma unroll
-                for (int o = LPC / 2; o > 0; o >>= 1) acc[u][m] += __shfl_xor_sync(0xFFFFFFFFu, acc[u][m], o);
+            for (int i = 0; i < PER; i++) {
+                const int u = (first + i) / MT, m = (first + i) % MT, n = base + (u * NW + warp) * GPW + grp;
+                r[i] = owner && n < N && m < M ? e.f32[(size_t)(m0 + m) * e.ldf + n] : 0.0f;
             }
-            int n = base + (u * (SM_THREADS / 32) + warp) * GPW + grp;
-            if (sl == 0 && n < N) {
-                if (argmax) {
+        }
 #pragma unroll
-                    for (int m = 0; m < MT; m++) {
-                        if (m < M) {
-                            float y = dequant_bias(acc[u][m], e.s_x, e.s_w[n], e.bias[n]);
-                            unsigned long long k = pack_key(y, (uint32_t)n);
-                            best[m] = k > best[m] ? k : best[m];
-                        }
-                    }
-                } else if (e.mode == EPI_RESID) {
-                    // every residual load first: the stores may alias them
-                    float r[MT];
-#pragma unroll
-                    for (int m = 0; m < MT; m++) r[m] = m < M ? e.f32[(size_t)(m0 + m) * e.ldf + n] : 0.0f;
-#pragma unroll
-                    for (int m = 0; m < MT; m++)
-                        if (m < M)
-                            e.f32[(size_t)(m0 + m) * e.ldf + n] =
-                                __fadd_rn(__fmul_rn(e.gamma, r[m]),
-                                          dequant_bias(acc[u][m], e.s_x, e.s_w[n], e.bias[n]));
-                } else {
-#pragma unroll
-                    for (int m = 0; m < MT; m++)
-                        if (m < M) epi_store(e, m0 + m, n, acc[u][m], t);
-                }
+        for (int i = 0; i < PER; i++) {
+            const int u = (first + i) / MT, m = (first + i) % MT, n = base + (u * NW + warp) * GPW + grp;
+            if (!owner || n >= N || m >= M) continue;
+            const float y = dequant_bias(acc[i], e.s_x, e.s_w[n], e.bias[n]);
+            if (argmax) {
+                const unsigned long long k = pack_key(y, (uint32_t)n);
+                best[i] = k > best[i] ? k : best[i];
+            } else if (e.mode == EPI_RESID) {
+                e.f32[(size_t)(m0 + m) * e.ldf + n] = __fadd_rn(__fmul_rn(e.gamma, r[i]), y);
+            } else {
+                epi_store_y(e, m0 + m, n, y, t);
             }
         }
     }
     if (argmax) {
-        __shared__ unsigned long long red[SM_THREADS / 32][MT];
 #pragma unroll
-        for (int m = 0; m < MT; m++) {
-            unsigned long long v = warp_max_u64(best[m]);
-            if (lane == 0) red[warp][m] = v;
-        }
+        for (int i = 0; i < PER; i++)
+            if (best[i]) atomicMax(&s_best[(first + i) % MT], best[i]);
         __syncthreads();
-        if (threadIdx.x < MT && (int)threadIdx.x < M) {
-            unsigned long long v = 0;
-            for (int w = 0; w < SM_THREADS / 32; w++) v = red[w][threadIdx.x] > v ? red[w][threadIdx.x] : v;
-            atomicMax(e.keys + m0 + threadIdx.x, v);
-        }
+        if (threadIdx.x < MT && (int)threadIdx.x < M) atomicMax(e.keys + m0 + threadIdx.x, s_best[threadIdx.x]);
     }
 }
 
@@ -454,27 +448,36 @@ cudaError_t linear_init() {
     return err;
 }
 
+template <int MT, int LPC, int U>
+static cudaError_t launch_small_u(const int8_t *A, int lda, const int8_t *W, int M, int N, int K, const Epi &e,
+                                  cudaStream_t st) {
+    constexpr int CPB = (SM_THREADS / 32) * (32 / LPC) * U;
+    int blocks = (N + CPB - 1) / CPB;
+    if (blocks > 4 * 152) blocks = 4 * 152;
+    const dim3 grid(blocks, (M + MT - 1) / MT);  // row chunks of MT, one per grid row
+    launch_pdl(linear_smallm<MT, LPC, U>, grid, SM_THREADS, (size_t)MT * K, st, A, lda, W, M, N, K, e);
+    return cudaGetLastError();
+}
+
+// two weight rows per lane group and pass, or one where that leaves fewer
+// blocks than SMs
+template <int MT, int LPC>
+static cudaError_t launch_small_t(const int8_t *A, int lda, const int8_t *W, int M, int N, int K, const Epi &e,
+                                  cudaStream_t st) {
+    constexpr int CPB2 = (SM_THREADS / 32) * (32 / LPC) * 2;
+    const long blocks = (long)((N + CPB2 - 1) / CPB2) * ((M + MT - 1) / MT);
+    return blocks >= 152 ? launch_small_u<MT, LPC, 2>(A, lda, W, M, N, K, e, st)
+                         : launch_small_u<MT, LPC, 1>(A, lda, W, M, N, K, e, st);
+}
+
 template <int MT>
 static cudaError_t launch_small(const int8_t *A, int lda, const int8_t *W, int M, int N, int K, const Epi &e,
                                 cudaStream_t st) {
     const int kc = K / 16;
-    const int chunks = (M + MT - 1) / MT;  // row chunks of MT, one per grid row
-    size_t smem = (size_t)MT * kc * 16;
-    int lpc = kc >= 32 ? 32 : (kc >= 16 ? 16 : 8);
-    constexpr int U = 2;
-    int cpb = (SM_THREADS / 32) * (32 / lpc) * U;
-    int blocks = (N + cpb - 1) / cpb;
-    if (blocks > 4 * 152) blocks = 4 * 152;
-    if (smem > 48 * 1024) return cudaErrorInvalidValue;  // K <= 3072 at M <= 16
-    const dim3 grid(blocks, chunks);
-    if (lpc == 32) {
-        launch_pdl(linear_smallm<MT, 32, U>, grid, SM_THREADS, smem, st, A, lda, W, M, N, K, e);
-    } else if (lpc == 16) {
-        launch_pdl(linear_smallm<MT, 16, U>, grid, SM_THREADS, smem, st, A, lda, W, M, N, K, e);
-    } else {
-        launch_pdl(linear_smallm<MT, 8, U>, grid, SM_THREADS, smem, st, A, lda, W, M, N, K, e);
-    }
-    return cudaGetLastError();
+    if ((size_t)MT * K > 48 * 1024) return cudaErrorInvalidValue;  // K <= 3072 at M <= 16
+    if (kc >= 32) return launch_small_t<MT, 32>(A, lda, W, M, N, K, e, st);
+    if (kc >= 16) return launch_small_t<MT, 16>(A, lda, W, M, N, K, e, st);
+    return launch_small_t<MT, 8>(A, lda, W, M, N, K, e, st);
 }
 
 template <int BM, int BN, int WM, int WN, int STAGES>

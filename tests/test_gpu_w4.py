@@ -150,3 +150,33 @@ def test_w4_cluster_step_matches_oracle(wq, B, shape, stream):
         tr.close()
     o_ids, o_len, _ = O.translate(blob, ids, lens, 1, T, n_threads=B)
     assert np.array_equal(g_ids, o_ids) and np.array_equal(g_len, o_len)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1, 32), (2, 3, 64), (3, 70, 128), (7, 65, 288), (16, 131, 544), (33, 500, 1056), (9, 6000, 96)])
+@pytest.mark.parametrize("asym", [False, True])
+def test_gemv_lane_split_edges(M, N, K, asym):
+    """Both GEMV kernels where the outputs are spread over a group's lanes:
+    fewer values than lanes, every group width, ragged columns and rows, one
+    and two weight rows per group; int8 rows in mode F32, 4-bit rows in F32 and
+    argmax."""
+    A = synth.uniform_int8(M, "A", (M, K))
+    s_w, b = synth.uniform_f32(1, "s", (N,), 1e-4, 3e-4), synth.uniform_f32(2, "b", (N,), -0.5, 0.5)
+    dA, ds, db = (torch.from_numpy(x).cuda() for x in (A, s_w, b))
+    f = torch.zeros((M, N), device="cuda")
+    if M <= 16 and not asym:
+        W = synth.uniform_int8(N, "W", (N, K))
+        mnmt.mnmt_linear(dA, torch.from_numpy(W).cuda(), ds, db, 0.02, None, 1.0, M, N, K, mnmt.EPI_F32, None, f)
+        ref = O.linear(A, W, s_w, b, np.float32(0.02), O.MODE_F32)
+        assert np.array_equal(f.cpu().numpy().view(np.uint32), ref.view(np.uint32))
+    u = (synth.uniform_int8(N + 1, "u", (N, K)).view(np.uint8) & 15).astype(np.uint8)
+    u = np.maximum(u, 1) if not asym else u
+    m = synth.uniform_f32(3, "m", (N,), -2e-3, -1e-3) if asym else None
+    Wp = synth.pack4(u)
+    dm = torch.from_numpy(m).cuda() if asym else None
+    dW = torch.from_numpy(Wp).cuda()
+    mnmt.mnmt_linear_w4(dA, dW, ds, dm, db, 0.02, None, 1.0, M, N, K, mnmt.EPI_F32, None, f)
+    ref = O.linear_w4(A, Wp, s_w, m, b, np.float32(0.02), O.MODE_F32, asym)
+    assert np.array_equal(f.cpu().numpy().view(np.uint32), ref.view(np.uint32))
+    keys = torch.zeros(M, dtype=torch.int64, device="cuda")
+    mnmt.mnmt_linear_w4(dA, dW, ds, dm, db, 0.02, None, 1.0, M, N, K, mnmt.EPI_ARGMAX, None, None, keys)
+    assert np.array_equal(mnmt.argmax_from_keys(keys.cpu().numpy()), ref.argmax(1))
