@@ -668,12 +668,14 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
            o_logits = piece(beam > 1 ? R * V * 4 : 256), o_outids = piece((size_t)max_batch * max_len * 4),
            o_outlens = piece((size_t)max_batch * 4), o_outsc = piece((size_t)max_batch * 4),
            o_state = piece(ST_N * 4), o_dc = piece(sizeof(DcParams)), o_dcln = piece((6 * L + 2) * d * 4),
-           o_dr = piece(rows_ok ? sizeof(DrParams) : 0), o_drw = piece(drw_bytes);
+           o_dr = piece(rows_ok ? sizeof(DrParams) : 0);
     const size_t kmax = std::max(d, std::max(F, (size_t)c.d_embed));
     const bool tc_any = tc_ok && rows >= TC_MIN_ROWS;
     size_t o_a16 = piece(tc_any ? rows * kmax * 2 : 256);
     size_t o_act16 = piece(tc_any ? rows * kmax * 2 : 256), o_ctx16 = piece(tc_any ? rows * d * 2 : 256),
            o_hid16 = piece(tc_any ? rows * F * 2 : 256), o_encq16 = piece(tc_any ? ME * d * 2 : 256);
+    const size_t zeroed = off;
+    const size_t o_drw = piece(drw_bytes);  // packed before its first use
     s->arena_bytes = off;
     if (cudaMalloc(&s->arena, off) != cudaSuccess) {
         delete s;
@@ -729,7 +731,7 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
     s->use_tc = tc_ok && !(tc_env && tc_env[0] == '0') && rows >= TC_MIN_ROWS;
     s->rows_ok = rows_ok;
     s->dr_w = a + o_drw;
-    if (cudaMemsetAsync(s->arena, 0, off, m->stream) != cudaSuccess || cudaStreamSynchronize(m->stream) != cudaSuccess) {
+    if (cudaMemsetAsync(s->arena, 0, zeroed, m->stream) != cudaSuccess || cudaStreamSynchronize(m->stream) != cudaSuccess) {
         mnmt_session_free(s);
         return fail(MNMT_ECUDA, "arena initialisation failed");
     }
