@@ -771,9 +771,23 @@ const __half *w16_of(const mnmt_model *m, const int8_t *w) {
     return m->d_blob16 + (w - reinterpret_cast<const int8_t *>(m->d_blob));
 }
 
-// does a linear of M rows run on the tensor cores (then its input comes from
-// the fp16 mirror its producer wrote)
-bool tc_rows(const mnmt_session *s, int M) { return s->use_tc && (size_t)M >= TC_MIN_ROWS; }
+// does the linear l of M rows run on the tcgen05 kernel (then its input comes
+// from the fp16 mirror its producer wrote), or on the kernels that read int8
+// codes?  The latter start faster (no TMEM, no barriers; mma.sync), the former
+// has the throughput and splits a long K.  Both measured in graphs, us:
+//   0.13 GMAC, K = 256 (512 x 1024): 3.7 / 5.3;  0.4 GMAC, K = 512: 6.9 / 6.3;
+//   0.8 GMAC, K = 512 (1024 x 1536): 9.4 / 8.9;  1.6 GMAC: 18.4 / 11.3
+//   K = 768: equal up to 0.15 GMAC; K = 1024 (512 x 256): 8.6 / 7.1, but the
+//   GEMV's 16-row chunks (narrow layers of up to 64 rows): 3.3 / 6.4
+//   fp32 rows of 32000 logits, K = 256: 32 rows 11.7 / 9.8, 128 rows 12.6 / 15.7,
+//   512 rows 34.5 / 42.9; K = 512: 20.3 / 17.8 and 60.9 / 47.1
+bool tc_linear(const mnmt_session *s, int M, const Lin &l, bool f32_out = false) {
+    if (!s->use_tc || (size_t)M < TC_MIN_ROWS) return false;
+    if (f32_out && l.k <= 256 && M >= 128) return false;
+    const long tiles64 = (long)((M + 63) / 64) * ((l.n + 63) / 64);
+    if (M <= 64 && l.k <= 1024 && tiles64 < 8) return false;
+    return l.k > 768 || (double)M * l.n * l.k > 3e8;
+}
 
 // fp16 mirror of one of the session's int8 activation buffers
 __half *mirror16(mnmt_session *s, const int8_t *buf) {
@@ -784,18 +798,20 @@ __half *mirror16(mnmt_session *s, const int8_t *buf) {
     return nullptr;
 }
 
-// the fp16 copy a producer of buf (M rows) must also write, or null
-__half *out16_for(mnmt_session *s, const int8_t *buf, int M) { return tc_rows(s, M) ? mirror16(s, buf) : nullptr; }
+// the fp16 copy that a producer of buf (M rows), read by the linear l, must
+// also write, or null
+__half *out16_for(mnmt_session *s, const int8_t *buf, int M, const Lin &l, bool f32_out = false) {
+    return tc_linear(s, M, l, f32_out) ? mirror16(s, buf) : nullptr;
+}
 
-// The quantised linear of rows A [M][lda] (Eq. 3 + epilogue e): on the
-// tensor cores when the layer is a dense contraction (M >= TC_MIN_ROWS),
-// reading the fp16 mirror of A that A's producer wrote; else on the kernels
-// that read the int8 codes (linear.cu).
+// The quantised linear of rows A [M][lda] (Eq. 3 + epilogue e), by tc_linear on
+// the tcgen05 kernel, reading the fp16 mirror of A that A's producer wrote, or
+// on the kernels that read the int8 codes (linear.cu).
 cudaError_t run_linear(mnmt_session *s, const int8_t *A, int lda, const Lin &l, int M, const Epi &e,
                        cudaStream_t st) {
     const mnmt_model *m = s->m;
     if (l.bits == 4 && ((size_t)M <= 16 || !l.w)) return launch_linear_w4(A, lda, l.wp, l.m, M, l.n, l.k, e, st);
-    if (tc_rows(s, M) && l.k % 16 == 0) {
+    if (tc_linear(s, M, l, e.mode == EPI_F32) && l.k % 16 == 0) {
         const __half *w16 = w16_of(m, l.w);
         const __half *a16 = mirror16(s, A);
         int lda16 = lda;
@@ -822,8 +838,9 @@ cudaError_t run_linear(mnmt_session *s, const int8_t *A, int lda, const Lin &l, 
 
 // LayerNorm after a residual update.  Pre-LN: q8(LN_next(r)) into act (r kept).
 // Post-LN: r = LN_this(r) in place, act = q8(r).
+// next: the linear that reads act_out.
 int ln_after_residual(mnmt_session *s, int M, const LnP &ln_pre_next, const LnP &ln_post_this, float s_next,
-                      int8_t *act_out, const int *skip) {
+                      int8_t *act_out, const int *skip, const Lin &next, bool next_f32 = false) {
     mnmt_model *m = s->m;
     LnArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -832,7 +849,7 @@ int ln_after_residual(mnmt_session *s, int M, const LnP &ln_pre_next, const LnP 
     a.d = m->c.d_model;
     a.inv = 1.0f / s_next;
     a.out_q = act_out;
-    a.out16 = out16_for(s, act_out, M);
+    a.out16 = out16_for(s, act_out, M, next, next_f32);
     a.status = s->state + ST_STATUS;
     a.skip = skip;
     if (m->c.pre_ln) {
@@ -873,7 +890,7 @@ int run_encoder(mnmt_session *s, int B, int S) {
         e.V = c.vocab;
         e.r = s->resid;
         e.out_q = s->act;
-        e.out16 = out16_for(s, s->act, M);
+        e.out16 = out16_for(s, s->act, M, m->enc_self[0].qkv);
         if (c.pre_ln) {
             e.ln_g = m->enc_self[0].ln.g;
             e.ln_b = m->enc_self[0].ln.b;
@@ -894,7 +911,7 @@ int run_encoder(mnmt_session *s, int B, int S) {
         std::memset(&at, 0, sizeof(at));
         at.qkv = s->qkv;
         at.ctx = s->ctx;
-        at.ctx16 = out16_for(s, s->ctx, M);
+        at.ctx16 = out16_for(s, s->ctx, M, A.o);
         at.len = s->src_lens;
         at.B = B;
         at.S = S;
@@ -909,12 +926,12 @@ int run_encoder(mnmt_session *s, int B, int S) {
         e.ldf = d;
         e.gamma = A.gamma;
         LK(run_linear(s, s->ctx, d, A.o, M, e, st));  // N = d, K = d
-        int rc = ln_after_residual(s, M, Fb.ln, A.ln, Fb.s_in, s->act, nullptr);
+        int rc = ln_after_residual(s, M, Fb.ln, A.ln, Fb.s_in, s->act, nullptr, Fb.w1);
         if (rc) return rc;
         e = base_epi(EPI_RELU_Q8, Fb.s_in, Fb.w1);
         e.inv_out = Fb.inv_h;
         e.out = s->hid;
-        e.out16 = out16_for(s, s->hid, M);
+        e.out16 = out16_for(s, s->hid, M, Fb.w2);
         e.ldo = F;
         LK(run_linear(s, s->act, d, Fb.w1, M, e, st));  // N = F, K = d
         e = base_epi(EPI_RESID, Fb.s_h, Fb.w2);
@@ -924,9 +941,9 @@ int run_encoder(mnmt_session *s, int B, int S) {
         LK(run_linear(s, s->hid, F, Fb.w2, M, e, st));  // N = d, K = F
         if (l + 1 < c.n_enc) {
             const SelfBlk &An = m->enc_self[l + 1];
-            rc = ln_after_residual(s, M, An.ln, Fb.ln, An.s_in, s->act, nullptr);
+            rc = ln_after_residual(s, M, An.ln, Fb.ln, An.s_in, s->act, nullptr, An.qkv);
         } else {
-            rc = ln_after_residual(s, M, m->enc_final, Fb.ln, m->s_enc, s->enc_q, nullptr);
+            rc = ln_after_residual(s, M, m->enc_final, Fb.ln, m->s_enc, s->enc_q, nullptr, m->dec_cross[0].kv);
         }
         if (rc) return rc;
     }
@@ -982,7 +999,7 @@ int issue_decoder_layers(mnmt_session *s) {
         e.V = c.vocab;
         e.r = s->resid;
         e.out_q = s->act;
-        e.out16 = out16_for(s, s->act, R);
+        e.out16 = out16_for(s, s->act, R, m->dec_self[0].qkv);
         if (c.pre_ln) {
             e.ln_g = m->dec_self[0].ln.g;
             e.ln_b = m->dec_self[0].ln.b;
@@ -1015,7 +1032,7 @@ int issue_decoder_layers(mnmt_session *s) {
         at.kc = s->sk + l * s->sk_layer;
         at.vc = s->sv + l * s->sk_layer;
         at.ctx = s->ctx;
-        at.ctx16 = out16_for(s, s->ctx, R);
+        at.ctx16 = out16_for(s, s->ctx, R, A.o);
         at.R = R;
         at.H = H;
         at.dh = dh;
@@ -1034,7 +1051,7 @@ int issue_decoder_layers(mnmt_session *s) {
         e.gamma = A.gamma;
         e.skip = done;
         LK(run_linear(s, s->ctx, d, A.o, R, e, st));  // N = d, K = d
-        int rc = ln_after_residual(s, R, X.ln, A.ln, X.s_in, s->act, done);
+        int rc = ln_after_residual(s, R, X.ln, A.ln, X.s_in, s->act, done, X.q);
         if (rc) return rc;
         e = base_epi(EPI_Q8, X.s_in, X.q);
         e.inv_out = X.inv_q;
@@ -1057,12 +1074,12 @@ int issue_decoder_layers(mnmt_session *s) {
         e.gamma = X.gamma;
         e.skip = done;
         LK(run_linear(s, s->ctx, d, X.o, R, e, st));  // N = d, K = d
-        rc = ln_after_residual(s, R, Fb.ln, X.ln, Fb.s_in, s->act, done);
+        rc = ln_after_residual(s, R, Fb.ln, X.ln, Fb.s_in, s->act, done, Fb.w1);
         if (rc) return rc;
         e = base_epi(EPI_RELU_Q8, Fb.s_in, Fb.w1);
         e.inv_out = Fb.inv_h;
         e.out = s->hid;
-        e.out16 = out16_for(s, s->hid, R);
+        e.out16 = out16_for(s, s->hid, R, Fb.w2);
         e.ldo = F;
         e.skip = done;
         LK(run_linear(s, s->act, d, Fb.w1, R, e, st));  // N = F, K = d
@@ -1074,9 +1091,9 @@ int issue_decoder_layers(mnmt_session *s) {
         LK(run_linear(s, s->hid, F, Fb.w2, R, e, st));  // N = d, K = F
         if (l + 1 < c.n_dec) {
             const SelfBlk &An = m->dec_self[l + 1];
-            rc = ln_after_residual(s, R, An.ln, Fb.ln, An.s_in, s->act, done);
+            rc = ln_after_residual(s, R, An.ln, Fb.ln, An.s_in, s->act, done, An.qkv);
         } else {
-            rc = ln_after_residual(s, R, m->dec_final, Fb.ln, m->s_dout, s->act, done);
+            rc = ln_after_residual(s, R, m->dec_final, Fb.ln, m->s_dout, s->act, done, m->out, s->k > 1);
         }
         if (rc) return rc;
     }
@@ -1277,7 +1294,7 @@ int setup_rows_step(mnmt_session *s) {
     if (m->factorised) { P.proj_w = m->proj.w; P.proj_s = m->proj.s; P.proj_b = m->proj.b; }
     P.fin_g = m->dec_final.g; P.fin_b = m->dec_final.b; P.inv_dout = 1.0f / m->s_dout;
     P.tok = s->tok; P.src_len = s->src_lens; P.anc = s->anc; P.t_ptr = s->state + ST_T; P.done = s->state + ST_DONE;
-    P.act_out = s->act; P.act16_out = out16_for(s, s->act, R); P.resid_out = s->resid; P.status = s->state + ST_STATUS;
+    P.act_out = s->act; P.act16_out = out16_for(s, s->act, R, m->out, s->k > 1); P.resid_out = s->resid; P.status = s->state + ST_STATUS;
     for (int l = 0; l < c.n_dec; l++) {
         const SelfBlk &A = m->dec_self[l];
         const CrossBlk &X = m->dec_cross[l];
