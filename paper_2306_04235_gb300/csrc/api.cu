@@ -25,6 +25,7 @@
 #include <string>
 #include <vector>
 
+#include "decode_rows.h"
 #include "internal.h"
 
 using namespace mnmt;

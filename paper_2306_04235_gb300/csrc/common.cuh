@@ -392,34 +392,14 @@ MNMT_DEV float rn32_div(long long n, long long z) {
     return n < 0 ? -q : q;
 }
 
-// q8(nearest float to n / z, rho): the quantised attention context of Eq. 2.
-// The approximate quotient fl(fl(n) / fl(z)) is within 2^-22 (relative) of
-// the exact rounded one -- three roundings of 2^-24 each, plus the exact
-// quotient's own -- which is at most 4 ulp, 8 across a binade boundary;
-// fl(x * rho), the rounding and the clamp are monotone in x, so when both ends
-// of the +-8-ulp bracket give the same code, so does the exact quotient.  Only
-// a bracket that straddles a rounding boundary needs the exact quotient.
-template <typename ExactDiv>
-MNMT_DEV int8_t q8_quotient(long long n, long long z, float rho, ExactDiv exact) {
-    if (n == 0) return q8(0.0f, rho);
-    const unsigned long long a = n < 0 ? 0ull - (unsigned long long)n : (unsigned long long)n;
-    const uint32_t qb = __float_as_uint(__fdiv_rn(__ull2float_rn(a), __ll2float_rn(z)));
-    const float sgn = n < 0 ? -1.0f : 1.0f;
-    const int8_t lo = q8(__fmul_rn(sgn, __uint_as_float(qb - 8u)), rho);
-    const int8_t hi = q8(__fmul_rn(sgn, __uint_as_float(qb + 8u)), rho);
-    if (lo == hi) return lo;
-    return q8(exact(n, z), rho);
-}
-
-// q8(nearest float to N / Z, rho) from an approximation fN of N and invZ =
-// fl(1 / fl(Z)), Z >= 2^24: t = fl(fl(fN invZ) rho) is off the exact chain by
+// q8(nearest float to N / Z, rho), the quantised attention context of Eq. 2,
+// from an approximation fN of N and invZ = fl(1 / fl(Z)), Z >= 2^24: t = fl(fl(fN invZ) rho) is off the exact chain by
 // at most eight relative roundings of 2^-24 (two in fN, fl(Z), fl(1/Z), two
 // products; the quotient and the product of the exact chain; < 2^-20) plus
 // `slack`, what fN's absolute error makes of t.  Where t lies further from a
 // rounding boundary than that (all but ~1e-4 of the values), rne(t) is the
 // code; else exact() decides.  (A NaN clamps to -127, as in q8.)  Returns the
-// code as an integer-valued float.  (q8_quotient converts two 64-bit integers
-// per value, at 2 lanes per clock and SM on this part.)
+// code as an integer-valued float.
 template <typename Exact>
 MNMT_DEV float q8_context(float fN, float invZ, float rho, float slack, Exact exact) {
     const float t = fminf(fmaxf(__fmul_rn(__fmul_rn(fN, invZ), rho), -127.0f), 127.0f);
@@ -432,7 +412,7 @@ MNMT_DEV float q8_context(float fN, float invZ, float rho, float slack, Exact ex
 template <typename Exact>
 MNMT_DEV int8_t q8_context_hl(int hi, int lo, float invZ, float rho, Exact exact) {
     const float fn = __fmaf_rn(__int2float_rn(hi), 4096.0f, __int2float_rn(lo));
-    return (int8_t)__float2int_rn(q8_context(fn, invZ, rho, __fmul_rn(fabsf(rho), 0x1p-18f), exact));
+    return (int8_t)(__float_as_uint(__fadd_rn(q8_context(fn, invZ, rho, __fmul_rn(fabsf(rho), 0x1p-18f), exact), 12582912.0f)) & 0xFFu);
 }
 
 // ---------------------------------------------------------------------------
@@ -442,7 +422,8 @@ MNMT_DEV int8_t q8_context_hl(int hi, int lo, float invZ, float rho, Exact exact
 // integer below 2^52, summed in int64, so any reduction order gives the same
 // bits; each sum / d is rounded once to fp32 (rn32_scaled_div); rstd =
 // 1 / sqrt(var + 1e-5) in IEEE fp32; returns false if |x| >= 2^32.
-// warp LayerNorm over a row held as VPL values per lane (element u*32 + lane)
+// warp LayerNorm over a row held as VPL values per lane (element u*32 + lane, 0
+// past d)
 // ---------------------------------------------------------------------------
 // exact warp sum of int64 values with |v| < 2^58 per lane: three 20-bit
 // pieces summed by single-instruction warp reductions
@@ -482,44 +463,6 @@ MNMT_DEV long long fx_sum(const float (&v)[N], int e) {
     return (long long)(int)(sa - off) * (1LL << 30) + (long long)(int)(sb - off) * 256 + (int)(sc - off);
 }
 
-// LayerNorm of one row held by a warp (x[u] = element u*32 + lane); gv / bv
-// are the matching gamma / beta values, loaded by the caller
-template <int VPL>
-MNMT_DEV bool warp_layernorm_v(const float (&x)[VPL], int d, const float (&gv)[VPL], const float (&bv)[VPL],
-                               float (&out)[VPL], int lane) {
-    unsigned amax_bits = 0;
-#pragma unroll
-    for (int u = 0; u < VPL; u++)
-        if (u * 32 + lane < d) amax_bits = max(amax_bits, __float_as_uint(x[u]) & 0x7FFFFFFFu);
-    const float amax = __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, amax_bits));
-    if (!(amax < 0x1p32f)) return false;
-    const int ea = exp_bound(amax);
-    long long s1 = 0;
-#pragma unroll
-    for (int u = 0; u < VPL; u++)
-        if (u * 32 + lane < d) s1 += fx_scale(x[u], 52 - ea);
-    s1 = warp_sum_exact(s1);
-    const float mu = rn32_scaled_div(s1, ea - 52, d);
-    float c[VPL];
-    unsigned bmax_bits = 0;
-#pragma unroll
-    for (int u = 0; u < VPL; u++) {
-        c[u] = __fsub_rn(x[u], mu);
-        if (u * 32 + lane < d) bmax_bits = max(bmax_bits, __float_as_uint(c[u]) & 0x7FFFFFFFu);
-    }
-    const int eb = exp_bound(__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, bmax_bits)));
-    long long s2 = 0;
-#pragma unroll
-    for (int u = 0; u < VPL; u++)
-        if (u * 32 + lane < d) s2 += fx_scale(__fmul_rn(c[u], c[u]), 52 - 2 * eb);
-    s2 = warp_sum_exact(s2);
-    const float var = rn32_scaled_div(s2, 2 * eb - 52, d);
-    const float rstd = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(var, 1e-5f)));
-#pragma unroll
-    for (int u = 0; u < VPL; u++) out[u] = __fadd_rn(__fmul_rn(__fmul_rn(c[u], rstd), gv[u]), bv[u]);
-    return true;
-}
-
 template <int VPL>
 MNMT_DEV bool warp_layernorm(const float (&x)[VPL], int d, const float *__restrict__ g,
                              const float *__restrict__ b, float (&out)[VPL], int lane) {
@@ -531,23 +474,35 @@ MNMT_DEV bool warp_layernorm(const float (&x)[VPL], int d, const float *__restri
     if (!(amax < 0x1p32f)) return false;
     const int ea = exp_bound(amax);
     long long s1 = 0;
+    if (ea >= -70) {
+        s1 = fx_sum<VPL>(x, ea);
+    } else {
 #pragma unroll
-    for (int u = 0; u < VPL; u++)
-        if (u * 32 + lane < d) s1 += fx_scale(x[u], 52 - ea);
-    s1 = warp_sum_exact(s1);
-    const float mu = rn32_scaled_div(s1, ea - 52, d);
+        for (int u = 0; u < VPL; u++) s1 += fx_scale(x[u], 52 - ea);
+    }
+    const float mu = rn32_scaled_div(warp_sum_exact(s1), ea - 52, d);
     float c[VPL];
     unsigned bmax_bits = 0;
 #pragma unroll
     for (int u = 0; u < VPL; u++) {
-        c[u] = __fsub_rn(x[u], mu);
-        if (u * 32 + lane < d) bmax_bits = max(bmax_bits, __float_as_uint(c[u]) & 0x7FFFFFFFu);
+        c[u] = u * 32 + lane < d ? __fsub_rn(x[u], mu) : 0.0f;
+        bmax_bits = max(bmax_bits, __float_as_uint(c[u]) & 0x7FFFFFFFu);
     }
     const int eb = exp_bound(__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, bmax_bits)));
     long long s2 = 0;
+    if (eb >= -36) {
+        float c2[VPL];
+        const float su = __uint_as_float((uint32_t)(127 - eb) << 23);
 #pragma unroll
-    for (int u = 0; u < VPL; u++)
-        if (u * 32 + lane < d) s2 += fx_scale(__fmul_rn(c[u], c[u]), 52 - 2 * eb);
+        for (int u = 0; u < VPL; u++) {
+            const float cs = __fmul_rn(c[u], su);
+            c2[u] = __fmul_rn(cs, cs);
+        }
+        s2 = fx_sum<VPL>(c2, 0);
+    } else {
+#pragma unroll
+        for (int u = 0; u < VPL; u++) s2 += fx_scale(__fmul_rn(c[u], c[u]), 52 - 2 * eb);
+    }
     s2 = warp_sum_exact(s2);
     const float var = rn32_scaled_div(s2, 2 * eb - 52, d);
     const float rstd = __fdiv_rn(1.0f, __fsqrt_rn(__fadd_rn(var, 1e-5f)));
@@ -557,11 +512,6 @@ MNMT_DEV bool warp_layernorm(const float (&x)[VPL], int d, const float *__restri
         if (i < d) out[u] = __fadd_rn(__fmul_rn(__fmul_rn(c[u], rstd), g[i]), b[i]);
     }
     return true;
-}
-
-MNMT_DEV bool warp_layernorm16(const float (&x)[16], int d, const float *g, const float *b, float (&out)[16],
-                               int lane) {
-    return warp_layernorm<16>(x, d, g, b, out, lane);
 }
 
 // device-side status word: first error wins

@@ -79,13 +79,14 @@ MNMT_DEV void dc_grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory
 MNMT_DEV void dc_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 // out-of-line copies of the exact roundings (one copy of the code each)
-__device__ __noinline__ float dc_rn32_div(long long n, long long z) { return rn32_div(n, z); }
+__device__ __noinline__ float dc_q8_exact(long long n, long long z, float rho) { return (float)q8(rn32_div(n, z), rho); }
+__device__ __noinline__ long long dc_fx_scale(float v, int shift) { return fx_scale(v, shift); }
 __device__ __noinline__ float dc_rn32_pow2_full(long long s, int e) { return rn32_pow2(s, e); }
 // the common case inline (one conversion, exact while the result is a normal
 // float), the rest out of line
 MNMT_DEV float dc_rn32_pow2(long long s, int e) {
     if (s != 0) {
-        const uint32_t fb = __float_as_uint(__ll2float_rn(s));
+        const uint32_t fb = __float_as_uint(ll2float(s));
         const int fe = (int)((fb >> 23) & 0xFFu) + e;
         if (fe >= 1 && fe <= 254) return __uint_as_float(fb + ((uint32_t)e << 23));
     }
@@ -265,9 +266,11 @@ __device__ __noinline__ void dc_layernorm(float *r, int R, int d, const float *g
         dc_row_extremes(mm, dc_row_of<RM>(e0, d, R), nc, hi, lo);
         const float am = fmaxf(fabsf(hi), fabsf(lo));
         if (!(am < 0x1p32f) && lane == 0) set_status(status, MNMT_EOVERFLOW);
-        const int sh = 52 - exp_bound(am);
-        long long v = fx_scale(r[e0 + lane], sh);
-        if (two) v += fx_scale(r[e0 + 32 + lane], sh);
+        const int ea = exp_bound(am);
+        const float x2[2] = {r[e0 + lane], two ? r[e0 + 32 + lane] : 0.0f};
+        long long v;
+        if (ea >= -70 && ea <= 33) v = two ? fx_sum<2>(x2, ea) : fx_sum<1>(reinterpret_cast<const float(&)[1]>(x2), ea);
+        else v = dc_fx_scale(x2[0], 52 - ea) + dc_fx_scale(x2[1], 52 - ea);
         const long long s = warp_sum_exact(v);
         if (lane == 0) part_l[e0 >> cs] = s;
     }
@@ -281,12 +284,14 @@ __device__ __noinline__ void dc_layernorm(float *r, int R, int d, const float *g
         const int ea = exp_bound(fmaxf(fabsf(hi), fabsf(lo)));
         const float mu = dc_rn32_scaled(dc_row_sum(part_l, row, spr), ea - 52, kd, dodd, zm);
         const int eb = exp_bound(fmaxf(fabsf(__fsub_rn(hi, mu)), fabsf(__fsub_rn(lo, mu))));
-        const int sh = 52 - 2 * eb;
-        const float cv = __fsub_rn(r[e0 + lane], mu);
-        long long v = fx_scale(__fmul_rn(cv, cv), sh);
-        if (two) {
-            const float cw2 = __fsub_rn(r[e0 + 32 + lane], mu);
-            v += fx_scale(__fmul_rn(cw2, cw2), sh);
+        const float cv = __fsub_rn(r[e0 + lane], mu), cv2 = two ? __fsub_rn(r[e0 + 32 + lane], mu) : 0.0f;
+        long long v;
+        if (eb >= -36 && eb <= 34) {
+            const float su = __uint_as_float((uint32_t)(127 - eb) << 23), c1 = __fmul_rn(cv, su), c2 = __fmul_rn(cv2, su);
+            const float q2[2] = {__fmul_rn(c1, c1), __fmul_rn(c2, c2)};
+            v = two ? fx_sum<2>(q2, 0) : fx_sum<1>(reinterpret_cast<const float(&)[1]>(q2), 0);
+        } else {
+            v = dc_fx_scale(__fmul_rn(cv, cv), 52 - 2 * eb) + dc_fx_scale(__fmul_rn(cv2, cv2), 52 - 2 * eb);
         }
         const long long s = warp_sum_exact(v);
         if (lane == 0) part_l[64 + (e0 >> cs)] = s;
@@ -436,11 +441,12 @@ __device__ __forceinline__ void dc_attention(const DcParams &P, int l, int cross
             // context, the KPI lanes of a group sharing its 4 elements
             if (live) {
                 constexpr int UPL = 4 / KPI;
+                const float iz = __frcp_rn(ll2float(z));
 #pragma unroll
                 for (int u = 0; u < 4; u++)
                     if (u / UPL == kg)
-                        ctx[(size_t)m * P.d + h * DH + el + u] =
-                            q8_quotient((long long)hi[u] * 4096 + lo[u], z, rho, dc_rn32_div);
+                        ctx[(size_t)m * P.d + h * DH + el + u] = q8_context_hl(
+                            hi[u], lo[u], iz, rho, [&]() { return dc_q8_exact((long long)hi[u] * 4096 + lo[u], z, rho); });
             }
             __syncthreads();
             continue;
@@ -460,7 +466,8 @@ __device__ __forceinline__ void dc_attention(const DcParams &P, int l, int cross
                     Z += pz[ii * wpi + w];
                 }
                 const int m2 = dc_row_of<RM>(it2, H, R), h2 = it2 - m2 * H;
-                ctx[(size_t)m2 * P.d + h2 * DH + e] = q8_quotient(N, Z, rho, dc_rn32_div);
+                const float c = q8_context(ll2float(N), __frcp_rn(ll2float(Z)), rho, 0.0f, [&]() { return dc_q8_exact(N, Z, rho); });
+                ctx[(size_t)m2 * P.d + h2 * DH + e] = (int8_t)(__float_as_uint(__fadd_rn(c, 12582912.0f)) & 0xFFu);
             }
         }
         __syncthreads();

@@ -33,6 +33,7 @@
 
 #include "attn_core.cuh"
 #include "common.cuh"
+#include "decode_rows.h"
 #include "internal.h"
 #include "mbarrier.cuh"
 
