@@ -780,11 +780,12 @@ const __half *w16_of(const mnmt_model *m, const int8_t *w) {
 //   0.8 GMAC, K = 512 (1024 x 1536): 9.4 / 8.9;  1.6 GMAC: 18.4 / 11.3
 //   K = 768: equal up to 0.15 GMAC; K = 1024 (512 x 256): 8.6 / 7.1, but the
 //   GEMV's 16-row chunks (narrow layers of up to 64 rows): 3.3 / 6.4
-//   fp32 rows of 32000 logits, K = 256: 32 rows 11.7 / 9.8, 128 rows 12.6 / 15.7,
-//   512 rows 34.5 / 42.9; K = 512: 20.3 / 17.8 and 60.9 / 47.1
+//   fp32 rows of 32000 logits, K = 256: 32 rows 11.4 / 9.4, 128 rows 12.8 / 15.6,
+//   192 rows 20.6 / 16.1, 512 rows 34.4 / 25.9; K = 512: 128 rows 20.1 / 17.6, 512
+//   rows 60.3 / 30.8; of 8000, K = 256: 256 rows 7.5 / 9.3, 640 rows 15.7 / 14.8
 bool tc_linear(const mnmt_session *s, int M, const Lin &l, bool f32_out = false) {
     if (!s->use_tc || (size_t)M < TC_MIN_ROWS) return false;
-    if (f32_out && l.k <= 256 && M >= 128) return false;
+    if (f32_out && l.k <= 256 && M >= 128) return (double)M * l.n * l.k > 1.2e9;
     const long tiles64 = (long)((M + 63) / 64) * ((l.n + 63) / 64);
     if (M <= 64 && l.k <= 1024 && tiles64 < 8) return false;
     return l.k > 768 || (double)M * l.n * l.k > 3e8;

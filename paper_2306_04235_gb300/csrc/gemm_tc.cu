@@ -12,7 +12,7 @@
 // them with one fp32 addition, which returns fl(acc) -- the correctly rounded
 // exact sum, the same value as (float)acc of the int32 accumulator.
 //
-// Pipeline (persistent CTAs, 128 x BN output tiles, 320 threads):
+// Pipeline (linear_tc: persistent CTAs, 128 x BN output tiles, 320 threads):
 //   warp 0 lane 0   TMA producer: 128-byte-swizzled 128x64 (A) and BNx64 (W)
 //                   fp16 tiles into a STAGES-deep shared-memory ring;
 //   warp 1          allocates two TMEM accumulator buffers; lane 0 issues
@@ -23,6 +23,8 @@
 //                   32*(w%4)..+31 = tile rows, half of the columns) and apply
 //                   the fused epilogue of the linear while the MMAs of the
 //                   next tile fill the other buffer.
+// Large grids run linear_tc2 on CTA pairs, with tiles of 256 rows and an
+// epilogue that moves outputs and residuals by TMA (see its header).
 // Grids of few 128 x 64 tiles run linear_tc_sk instead: the same pipeline for
 // one tile per CTA, K split over a 2- or 4-CTA cluster, the partials reduced
 // exactly in int32 through distributed shared memory (see its header).
@@ -469,6 +471,551 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc(const __grid_constant
 }
 
 // ---------------------------------------------------------------------------
+// 256 x BN tiles on CTA pairs (tcgen05 cta_group::2).  Each CTA of a pair stages
+// its 128 rows of A and BN / 2 of the rows of W and holds its 128 rows of the
+// accumulator:
+//   warp 0    TMA producer in both CTAs; all copies complete on the leader's
+//             (rank 0) full barrier;
+//   warp 1    in the leader, one thread issues the pair's tcgen05.mma; commits
+//             are multicast, so both CTAs' slots and accumulators follow;
+//   warps 2-9 epilogue of the CTA's own rows: 32 rows x BN / 2 columns per warp.
+// TMEM holds two accumulator buffers, or one of two chunks of 256 columns, which
+// is then read into registers and released at once.
+//
+// What bounded the 128 x 256 tiles of one CTA that this replaces was their
+// epilogue, 12 (codes) to 40 (residual) thousand cycles a tile against 4 to 8
+// thousand of products: loads and stores of one row per lane pass a first-level
+// cache that the ring leaves a few KB of, and the release of the accumulator
+// waited for them.  Here outputs and residuals move by TMA through two 4 KB
+// blocks per warp (32 rows x 128 bytes, swizzled: a lane's 16-byte accesses meet
+// no bank conflict); the first residuals of a tile are under way before its
+// accumulator is ready, the accumulator is released once it is in registers, and
+// a tile's column constants are read while the previous tile is finished.  What
+// is left of the epilogue (5 thousand cycles a 256-wide tile, codes) runs under
+// the next tile's products.
+// 256 columns: 64 KB of operands feed 128 x 256 x 64 products per SM, as much as
+// shared memory moves (128 bytes a cycle, written once and read once) in the 512
+// cycles that the tensor core takes; 128 columns: 620 cycles a k-block for half
+// of the products.  Four stages, 128 KB in flight, are what two staging blocks a
+// warp leave room for.
+// Tried and not better: k-blocks brought to L2 ahead of the ring, pairs starting
+// at different k-blocks, residuals of the second two blocks brought to L2 early.
+// us, 128 x 256 tiles of one CTA -> here (before and after, inputs larger than L2):
+//   16384 x 512 x 2048 residual    57.6 -> 43.0;  K = 512     35.6 -> 24.5
+//   16384 x 2048 x 512 codes       46.5 -> 40.2;  N = 1536    38.5 -> 33.6
+//   6400 x 512 x 2048 residual     29.1 -> 24.3;  K = 512     20.9 -> 15.7
+//   512 x 32000 x 512 fp32         45.8 -> 30.0;  256 rows    27.2 -> 19.6
+//   8192 x 8192 x 1024 codes       96.8 -> 90.2;  2048, fp32 281.3 -> 196 (1400 TFLOP/s)
+// ---------------------------------------------------------------------------
+constexpr int T2_BLK = 4096;  // one staging block: 32 rows x 128 bytes
+
+template <int BN>
+struct T2Layout {
+    static constexpr int STAGES = BN == 256 ? 4 : 6;
+    static constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2;
+    static constexpr uint32_t STAGE = A_BYTES + (BN / 2) * TC_BK * 2;     // A rows, then W rows
+    static constexpr uint32_t OFF_STG = STAGES * STAGE;                   // [8 warps][2] blocks
+    static constexpr uint32_t OFF_COLS = OFF_STG + TC_EPI_WARPS * 2 * T2_BLK;  // [2][3][BN] fp32
+    static constexpr uint32_t OFF_BARS = OFF_COLS + 2 * 3 * BN * 4;
+    // full, empty, acc_full[2], acc_empty[2], done, residual[8 warps][2]
+    static constexpr int NBARS = 2 * STAGES + 5 + 2 * TC_EPI_WARPS;
+    static constexpr uint32_t OFF_MISC = OFF_BARS + NBARS * 8;
+    static constexpr uint32_t BYTES = OFF_MISC + 16;
+    static constexpr size_t SMEM = 1024 + BYTES;
+};
+
+__device__ __forceinline__ uint32_t t2_mapa(uint32_t local, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    return r;
+}
+// tile load into this CTA's shared memory, completing on a barrier of either CTA of the pair
+__device__ __forceinline__ void t2_load(uint32_t dst, const CUtensorMap *tm, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+        "%3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+// tile store from this CTA's shared memory; outside the matrix nothing is written
+__device__ __forceinline__ void t2_store(const CUtensorMap *tm, int x, int y, uint32_t src) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     reinterpret_cast<uint64_t>(tm)),
+                 "r"(x), "r"(y), "r"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void t2_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// at most N groups of stores still read their blocks
+template <int N>
+__device__ __forceinline__ void t2_store_wait_read() {
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void t2_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+__device__ __forceinline__ void t2_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// arrives on the barrier at this offset in both CTAs once the MMAs issued so far are complete
+__device__ __forceinline__ void t2_commit(uint32_t bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+        "h"((uint16_t)3)
+        : "memory");
+}
+__device__ __forceinline__ void t2_arrive_remote(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+}
+
+// byte of 16-byte chunk c of row r in a block of rows of RB bytes, RB-byte swizzle
+template <int RB>
+__device__ __forceinline__ int t2_chunk(int r, int c) {
+    return 16 * (c ^ (RB == 64 ? (r >> 1) & 3 : r & 7));
+}
+
+// One warp's 32 rows x 32 columns, a row per lane, through a 128-byte-swizzled
+// block: y = fl(fl(a * sc) + b), with RESID fl(fl(gamma * r) + y) of the
+// residuals that the block holds.
+template <bool RESID>
+__device__ __forceinline__ void t2_block_f32(const float (&a)[32], const float *sc, const float *bs, float gamma, uint8_t *blk) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int g = 0; g < 8; g++) {
+        const float4 s4 = *reinterpret_cast<const float4 *>(sc + 4 * g), b4 = *reinterpret_cast<const float4 *>(bs + 4 * g);
+        float4 y = make_float4(__fadd_rn(__fmul_rn(a[4 * g], s4.x), b4.x), __fadd_rn(__fmul_rn(a[4 * g + 1], s4.y), b4.y),
+                               __fadd_rn(__fmul_rn(a[4 * g + 2], s4.z), b4.z), __fadd_rn(__fmul_rn(a[4 * g + 3], s4.w), b4.w));
+        float4 *p = reinterpret_cast<float4 *>(blk + lane * 128 + t2_chunk<128>(lane, g));
+        if (RESID) {
+            const float4 r = *p;
+            y = make_float4(__fadd_rn(__fmul_rn(gamma, r.x), y.x), __fadd_rn(__fmul_rn(gamma, r.y), y.y),
+                            __fadd_rn(__fmul_rn(gamma, r.z), y.z), __fadd_rn(__fmul_rn(gamma, r.w), y.w));
+        }
+        *p = y;
+    }
+}
+
+// One warp's 32 rows x 32 columns (block b of its RB) as codes, a row per lane:
+// [32][RB] codes, RB-byte swizzle; with fp16 copies, [32][64] halves of blocks
+// 2 i and 2 i + 1, 128-byte swizzle.
+template <bool RELU, int RB>
+__device__ __forceinline__ void t2_block_q8(const float (&a)[32], const float *sc, const float *bs, const float *inv, int b,
+                                            uint8_t *codes, uint8_t *halves) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int c = 16 * g + 4 * k;
+            const float4 s4 = *reinterpret_cast<const float4 *>(sc + c), b4 = *reinterpret_cast<const float4 *>(bs + c),
+                         i4 = *reinterpret_cast<const float4 *>(inv + c);
+            auto code = [](float v, float s, float bb, float in) {
+                const float y = __fadd_rn(__fmul_rn(v, s), bb);
+                return q8_bits(RELU && !(y > 0.0f) ? 0.0f : y, in);
+            };
+            w[k] = __byte_perm(__byte_perm(code(a[c], s4.x, b4.x, i4.x), code(a[c + 1], s4.y, b4.y, i4.y), 0x0040),
+                               __byte_perm(code(a[c + 2], s4.z, b4.z, i4.z), code(a[c + 3], s4.w, b4.w, i4.w), 0x0040), 0x5410);
+        }
+        *reinterpret_cast<uint4 *>(codes + lane * RB + t2_chunk<RB>(lane, 2 * b + g)) = make_uint4(w[0], w[1], w[2], w[3]);
+        if (halves) {
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                uint4 h;
+                codes_to_half2((int)w[2 * k], h.x, h.y);
+                codes_to_half2((int)w[2 * k + 1], h.z, h.w);
+                *reinterpret_cast<uint4 *>(halves + lane * 128 + t2_chunk<128>(lane, 4 * (b & 1) + 2 * g + k)) = h;
+            }
+        }
+    }
+}
+
+// destination of 16 codes at (row, col), col a multiple of 16, of the cache-writing modes
+__device__ __forceinline__ int8_t *epi_dst16(const Epi &e, int row, int col, int t) {
+    if (e.mode == EPI_QKV_DEC && col >= e.d) {
+        const int seg = col >= 2 * e.d, c = col - (seg ? 2 * e.d : e.d), h = c / e.dh;
+        return (seg ? e.vc : e.kc) + (((size_t)row * e.H + h) * e.T + t) * e.dh + (c - h * e.dh);
+    }
+    if (e.mode == EPI_KV_CROSS) {
+        const int b = row / e.S, sp = row - b * e.S, seg = col >= e.d, c = col - (seg ? e.d : 0), h = c / e.dh;
+        return (seg ? e.vc : e.kc) + (((size_t)b * e.H + h) * e.S + sp) * e.dh + (c - h * e.dh);
+    }
+    return e.out + (size_t)row * e.ldo + col;
+}
+
+// outs: 1 = tmO describes the output matrix (fp32, or codes), 2 = tmH its fp16 copy
+template <int BN, int NCH>
+__global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constant__ CUtensorMap tmA,
+                                                            const __grid_constant__ CUtensorMap tmB,
+                                                            const __grid_constant__ CUtensorMap tmO,
+                                                            const __grid_constant__ CUtensorMap tmH, int outs, int M, int N,
+                                                            int K, Epi e, int *status) {
+    pdl_grid_wait();
+    using L = T2Layout<BN>;
+    constexpr uint32_t IDESC = idesc_f16(2 * TC_BM, BN);
+    constexpr int STAGES = L::STAGES, ACC_COLS = NCH * BN;
+    constexpr int NBUF = 2 * ACC_COLS <= 512 ? 2 : 1;  // accumulator buffers
+    if (e.skip && *e.skip) return;  // one flag for every CTA of the grid
+
+    extern __shared__ uint8_t tc_raw[];
+    uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(tc_raw) + 1023) & ~(uintptr_t)1023);
+    float *cols = reinterpret_cast<float *>(sm + L::OFF_COLS);
+    const uint32_t bars = s_addr(sm + L::OFF_BARS);
+    auto full_bar = [&](int s) { return bars + 8u * s; };
+    auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
+    auto accf_bar = [&](int b) { return bars + 8u * (2 * STAGES + b); };
+    auto acce_bar = [&](int b) { return bars + 8u * (2 * STAGES + 2 + b); };
+    const uint32_t done_bar = bars + 8u * (2 * STAGES + 4);
+    auto resid_bar = [&](int w) { return bars + 8u * (2 * STAGES + 5 + w); };
+    uint32_t *misc = reinterpret_cast<uint32_t *>(sm + L::OFF_MISC);  // [0] tmem base, [1] abort, [2] consumed
+    volatile uint32_t *abort_flag = misc + 1;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t rank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
+    const int mt = (M + 2 * TC_BM - 1) / (2 * TC_BM);
+    const int nt = (N + BN - 1) / BN, tiles = mt * nt;
+    // the dimension of fewer tiles runs fastest: the larger operand is then read
+    // by pairs that run at the same time
+    auto tile_m = [&](int tile) { return (mt <= nt ? tile % mt : tile / nt) * 2 * TC_BM; };
+    auto tile_n = [&](int tile) { return (mt <= nt ? tile / mt : tile % nt) * BN; };
+    const int nkb = (K + TC_BK - 1) / TC_BK;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; s++) {
+            mbar_init(full_bar(s), 1);
+            mbar_init(empty_bar(s), 1);
+        }
+        for (int b = 0; b < 2; b++) {
+            mbar_init(accf_bar(b), 1);
+            mbar_init(acce_bar(b), 2 * TC_EPI_WARPS);
+        }
+        mbar_init(done_bar, 1);
+        for (int w = 0; w < 2 * TC_EPI_WARPS; w++) mbar_init(resid_bar(w), 1);
+        misc[1] = 0;
+        misc[2] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_addr(misc)), "r"(NBUF * ACC_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        tc_fence_before();
+    }
+    // both CTAs' barriers and accumulators are set up
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = misc[0];
+
+    uint32_t issued = 0;
+    if (warp == 0 && lane == 0) {
+        // ---- TMA producer: this CTA's rows of A and W of all the pair's tiles ----
+        uint32_t it = 0;
+        const uint32_t ring = s_addr(sm);
+        for (int tile = pair; tile < tiles && !*abort_flag; tile += pairs) {
+            const int m0 = tile_m(tile) + (int)rank * TC_BM, n0 = tile_n(tile) + (int)rank * (BN / 2);
+            for (int kb = 0; kb < nkb; kb++, it++) {
+                const int s = (int)(it % STAGES);
+                if (it >= STAGES && !mbar_wait(empty_bar(s), (it / STAGES - 1) & 1)) {
+                    *abort_flag = 1;
+                    set_status(status, MNMT_ETIMEOUT);
+                    break;
+                }
+                // the leader's barrier takes the bytes of both CTAs
+                if (rank == 0) mbar_expect_tx(full_bar(s), 2 * L::STAGE);
+                const uint32_t bar = t2_mapa(full_bar(s), 0);
+                t2_load(ring + s * L::STAGE, &tmA, kb * TC_BK, m0, bar);
+                t2_load(ring + s * L::STAGE + L::A_BYTES, &tmB, kb * TC_BK, n0, bar);
+                issued = it + 1;
+            }
+        }
+    } else if (warp == 1 && lane == 0 && rank == 0) {
+        // ---- MMA issuer of the pair ----
+        uint32_t it = 0, lt = 0;
+        bool failed = false;
+        const uint64_t a_desc = sw128_desc(s_addr(sm)), b_desc = sw128_desc(s_addr(sm) + L::A_BYTES);
+        for (int tile = pair; tile < tiles && !failed; tile += pairs, lt++) {
+            const int buf = (int)(lt % NBUF);
+            if (lt >= NBUF && !mbar_wait(acce_bar(buf), (lt / NBUF - 1) & 1)) {
+                failed = true;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t dbase = tbase + (uint32_t)(buf * ACC_COLS);
+            for (int kb = 0; kb < nkb; kb++, it++) {
+                const int s = (int)(it % STAGES);
+                if (!mbar_wait(full_bar(s), (it / STAGES) & 1)) {
+                    failed = true;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = dbase + (uint32_t)((kb / TC_KB_PER_CHUNK) * BN);
+                const uint64_t ad = a_desc + (uint64_t)((s * L::STAGE) >> 4), bd = b_desc + (uint64_t)((s * L::STAGE) >> 4);
+#pragma unroll
+                for (int k = 0; k < TC_BK / 16; k++)
+                    t2_mma(d, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), IDESC, (uint32_t)((kb % TC_KB_PER_CHUNK) | k));
+                t2_commit(empty_bar(s));
+            }
+            if (!failed) t2_commit(accf_bar(buf));
+        }
+        if (failed) {
+            *abort_flag = 1;
+            set_status(status, MNMT_ETIMEOUT);
+        }
+        pdl_allow_next();     // every MMA of this pair is issued
+        misc[2] = it;         // k-blocks whose copies this thread saw land
+        t2_commit(done_bar);  // arrives in both CTAs once the MMAs have completed
+    } else if (warp == 1 && lane == 0) {
+        pdl_allow_next();  // the leader's trigger decides
+    } else if (warp >= 2) {
+        // ---- epilogue of this CTA's 128 rows ----
+        constexpr int NB = BN / 64, RB = 32 * NB;  // blocks of 32 columns per warp; its columns
+        constexpr int PL = NBUF == 2 ? 1 : NB;     // blocks read at a time: a single buffer is released at once
+        const int ew = warp - 2, q = warp & 3, cw = RB * (ew >> 2);  // rows 32 q .., columns cw ..
+        const int t = e.t_ptr ? *e.t_ptr : 0;
+        const bool f32m = e.mode == EPI_RESID || e.mode == EPI_F32, plain = e.mode == EPI_Q8 || e.mode == EPI_RELU_Q8;
+        const bool tma = outs & 1, h16 = outs & 2, cache = !f32m && !plain && e.mode != EPI_ARGMAX && epi_vec_ok(e) && N % 16 == 0;
+        uint8_t *blk = sm + L::OFF_STG + ew * 2 * T2_BLK;
+        const uint32_t blk_s = s_addr(blk);
+        uint32_t rphase = 0;  // of the two residual barriers, a bit each
+        // thread i carries the constants of a tile's column i
+        const int ti = ew * 32 + lane;
+        float k_sw = 0.0f, k_b = 0.0f, k_inv = 0.0f;
+        auto fetch = [&](int tile) {
+            const int n = tile_n(tile) + ti;
+            if (ti < BN && tile < tiles && n < N) {
+                k_sw = e.s_w[n];
+                k_b = e.bias[n];
+                k_inv = e.inv_out ? e.inv_out[n] : 0.0f;
+            }
+        };
+        fetch(pair);
+        uint32_t lt = 0;
+        for (int tile = pair; tile < tiles; tile += pairs, lt++) {
+            const int n0 = tile_n(tile), row0 = tile_m(tile) + (int)rank * TC_BM + 32 * q, col0 = n0 + cw;
+            const bool mine = row0 < M && col0 < N;
+            float *c_sc = cols + (lt & 1) * 3 * BN, *c_b = c_sc + BN, *c_inv = c_b + BN;
+            if (ti < BN) {
+                c_sc[ti] = __fmul_rn(e.s_x, k_sw);
+                c_b[ti] = k_b;
+                c_inv[ti] = k_inv;
+            }
+            fetch(tile + pairs);
+            const bool resid = tma && e.mode == EPI_RESID && mine;
+            // one thread: the residuals of block b into their staging block, which is free
+            auto load_resid = [&](int b) {
+                const uint32_t rb = resid_bar(2 * ew + (b & 1));
+                mbar_expect_tx(rb, T2_BLK);
+                tma_load_2d(blk_s + (b & 1) * T2_BLK, &tmO, col0 + 32 * b, row0, rb);
+            };
+            if (lane == 0) {
+                t2_store_wait_read<0>();  // both blocks are free again
+                if (resid) {
+                    load_resid(0);
+                    if (col0 + 32 < N) load_resid(1);
+                }
+            }
+            epi_bar_sync();
+            const int buf = (int)(lt % NBUF);
+            bool ok = *abort_flag == 0 && mbar_wait(accf_bar(buf), (lt / NBUF) & 1);
+            if (!ok && *abort_flag == 0) {
+                *abort_flag = 1;
+                set_status(status, MNMT_ETIMEOUT);
+            }
+            tc_fence_after();
+            ok = __all_sync(0xFFFFFFFFu, ok && *abort_flag == 0);
+            if (!ok || !mine) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) t2_arrive_remote(t2_mapa(acce_bar(buf), 0));
+                if (resid) {  // aborted: no residual may be in flight when the CTA ends
+                    if (lane == 0) {
+                        mbar_wait(resid_bar(2 * ew), rphase & 1);
+                        if (col0 + 32 < N) mbar_wait(resid_bar(2 * ew + 1), (rphase >> 1) & 1);
+                    }
+                    rphase ^= col0 + 32 < N ? 3 : 1;
+                }
+                continue;
+            }
+            const uint32_t taddr = tbase + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * ACC_COLS + cw);
+            const float *sc = c_sc + cw, *bs = c_b + cw, *inv = c_inv + cw;
+            uint32_t bk = 0, bi = (uint32_t)col0;  // ARGMAX: the lane's largest ordered value, its lowest column
+            float a[PL][32];
+            auto read = [&](int b, float (&v)[32]) {
+                if constexpr (NCH == 1) {
+                    uint32_t r[32];
+                    tmem_ld32(taddr + 32 * b, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int k = 0; k < 32; k++) v[k] = __uint_as_float(r[k]);
+                } else {
+#pragma unroll
+                    for (int g = 0; g < 2; g++) {
+                        uint32_t r[16], r1[16];
+                        tmem_ld16(taddr + 32 * b + 16 * g, r);
+                        tmem_ld16(taddr + BN + 32 * b + 16 * g, r1);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int k = 0; k < 16; k++) v[16 * g + k] = __fadd_rn(__uint_as_float(r[k]), __uint_as_float(r1[k]));
+                    }
+                }
+            };
+            auto release = [&]() {  // this warp is done with the accumulator buffer
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) t2_arrive_remote(t2_mapa(acce_bar(buf), 0));
+            };
+            if constexpr (PL > 1) {
+#pragma unroll
+                for (int b = 0; b < PL; b++) read(b, a[b]);
+                release();
+            }
+            // one block's code, not NB copies, unless the blocks are in registers: grids
+            // of a few tiles per pair spend their time on instruction fetches
+#pragma unroll(PL > 1 ? NB : 1)
+            for (int b = 0; b < NB; b++) {
+                if constexpr (PL == 1) {
+                    read(b, a[0]);
+                    if (b == NB - 1) release();
+                }
+                if (col0 + 32 * b < N) {
+                    const float(&acc)[32] = a[PL > 1 ? b : 0];
+                    const float *scb = sc + 32 * b, *bsb = bs + 32 * b, *invb = inv + 32 * b;
+                    uint8_t *p = blk + (b & 1) * T2_BLK;
+                    if (e.mode == EPI_ARGMAX) {
+#pragma unroll
+                        for (int g = 0; g < 8; g++) {
+                            const float4 s4 = *reinterpret_cast<const float4 *>(scb + 4 * g), b4 = *reinterpret_cast<const float4 *>(bsb + 4 * g);
+                            const float ss[4] = {s4.x, s4.y, s4.z, s4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                            for (int k = 0; k < 4; k++) {
+                                const int col = col0 + 32 * b + 4 * g + k;
+                                const uint32_t key = ordered_bits(__fadd_rn(__fmul_rn(acc[4 * g + k], ss[k]), bb[k]));
+                                if (key > bk && col < N) {
+                                    bk = key;
+                                    bi = (uint32_t)col;
+                                }
+                            }
+                        }
+                    } else if (f32m && tma) {
+                        if (e.mode == EPI_RESID) {
+                            if (!mbar_wait(resid_bar(2 * ew + (b & 1)), (rphase >> (b & 1)) & 1)) {
+                                *abort_flag = 1;
+                                set_status(status, MNMT_ETIMEOUT);
+                            }
+                            rphase ^= 1u << (b & 1);
+                            t2_block_f32<true>(acc, scb, bsb, e.gamma, p);
+                        } else {
+                            if (b >= 2) {  // the block's earlier store has read it
+                                if (lane == 0) t2_store_wait_read<1>();
+                                __syncwarp();
+                            }
+                            t2_block_f32<false>(acc, scb, bsb, 0.0f, p);
+                        }
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) {
+                            t2_store(&tmO, col0 + 32 * b, row0, blk_s + (b & 1) * T2_BLK);
+                            t2_store_commit();
+                            if (NB == 4 && b == 1 && e.mode == EPI_RESID) {  // the second pair of blocks
+                                t2_store_wait_read<1>();
+                                if (col0 + 64 < N) load_resid(2);
+                                t2_store_wait_read<0>();
+                                if (col0 + 96 < N) load_resid(3);
+                            }
+                        }
+                    } else if ((plain && tma) || cache) {
+                        if (b == 2 && h16) {  // the halves of blocks 0 and 1 have been read
+                            if (lane == 0) t2_store_wait_read<0>();
+                            __syncwarp();
+                        }
+                        if (e.mode == EPI_RELU_Q8)
+                            t2_block_q8<true, RB>(acc, scb, bsb, invb, b, blk, h16 ? blk + T2_BLK : nullptr);
+                        else
+                            t2_block_q8<false, RB>(acc, scb, bsb, invb, b, blk, h16 ? blk + T2_BLK : nullptr);
+                        if (h16 && ((b & 1) || col0 + 32 * (b + 1) >= N)) {
+                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                            __syncwarp();
+                            if (lane == 0) {
+                                t2_store(&tmH, col0 + 64 * (b >> 1), row0, blk_s + T2_BLK);
+                                t2_store_commit();
+                            }
+                        }
+                    } else {
+                        // destinations without 16-byte alignment: one element at a time, a column per lane
+                        __syncwarp();
+#pragma unroll
+                        for (int g = 0; g < 8; g++)
+                            *reinterpret_cast<float4 *>(blk + lane * 128 + t2_chunk<128>(lane, g)) =
+                                make_float4(acc[4 * g], acc[4 * g + 1], acc[4 * g + 2], acc[4 * g + 3]);
+                        __syncwarp();
+                        const int col = col0 + 32 * b + lane;
+                        for (int rl = 0; rl < 32; rl++) {
+                            const float v = *reinterpret_cast<const float *>(blk + rl * 128 + t2_chunk<128>(rl, lane >> 2) + 4 * (lane & 3));
+                            if (row0 + rl < M && col < N) epi_store_f(e, row0 + rl, col, v, t);
+                        }
+                    }
+                }
+            }
+            if (e.mode == EPI_ARGMAX) {  // pack_key(value, column)
+                if (row0 + lane < M) atomicMax(e.keys + row0 + lane, ((unsigned long long)bk << 32) | (0xFFFFFFFFu - bi));
+            } else if (plain && tma) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    t2_store(&tmO, col0, row0, blk_s);
+                    t2_store_commit();
+                }
+            } else if (cache) {
+                __syncwarp();
+                constexpr int LR = RB / 16;  // lanes per row
+                const int c = lane % LR;
+#pragma unroll
+                for (int i = 0; i < LR; i++) {
+                    const int rl = (32 / LR) * i + lane / LR;
+                    if (row0 + rl < M && col0 + 16 * c < N)
+                        *reinterpret_cast<uint4 *>(epi_dst16(e, row0 + rl, col0 + 16 * c, t)) =
+                            *reinterpret_cast<const uint4 *>(blk + rl * RB + t2_chunk<RB>(rl, c));
+                }
+            }
+        }
+        if (lane == 0) t2_store_wait();
+    }
+
+    // ---- teardown: every MMA and copy has completed before either CTA ends ----
+    __syncthreads();
+    if (warp == 0 && lane == 0 && rank == 0 && *abort_flag) {
+        // copies of the pair that the MMA issuer never consumed (bounded waits)
+        for (uint32_t it = misc[2]; it < issued; it++) mbar_wait(full_bar((int)(it % STAGES)), (it / STAGES) & 1);
+    }
+    if (warp == 1) {
+        if (lane == 0) mbar_wait(done_bar, 0);
+        __syncwarp();
+        tc_fence_after();
+    }
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(NBUF * ACC_COLS) : "memory");
+}
+
+// ---------------------------------------------------------------------------
 // int8 codes -> fp16 (exact); 16 codes per thread and step
 // ---------------------------------------------------------------------------
 __global__ void codes_to_f16_kernel(const int8_t *__restrict__ src, int ld_src, __half *__restrict__ dst, int ld_dst,
@@ -780,6 +1327,7 @@ __global__ void wait_timeout_selftest_kernel(int *status) {
 // ---------------------------------------------------------------------------
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 int g_num_sms = 148;
+int g_pairs = 0;  // CTA pairs of linear_tc2 that fit at once
 int g_sk_clusters[5] = {0, 0, 0, 0, 0};  // clusters of S split-K CTAs that fit at once (S = 2, 4)
 
 bool make_map(CUtensorMap *tm, const __half *p, int cols, int rows, int ld, int box_rows) {
@@ -852,10 +1400,68 @@ cudaError_t tc_launch_sk(const CUtensorMap &ta, const CUtensorMap &tb, int M, in
     return cudaLaunchKernelEx(&cfg, linear_tc_sk<S>, ta, tb, M, N, K, e, status);
 }
 
+template <int BN, int NCH>
+cudaLaunchConfig_t tc2_config(int pairs, cudaStream_t st, cudaLaunchAttribute (&attr)[2], bool pdl) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * pairs));
+    cfg.blockDim = dim3(TC_THREADS);
+    cfg.dynamicSmemBytes = T2Layout<BN>::SMEM;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 2 : 1;
+    return cfg;
+}
+
+template <int BN, int NCH>
+cudaError_t tc2_init() {
+    cudaError_t err = cudaFuncSetAttribute(linear_tc2<BN, NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T2Layout<BN>::SMEM);
+    if (err != cudaSuccess) return err;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = tc2_config<BN, NCH>(64, nullptr, attr, false);
+    int n = 0;
+    err = cudaOccupancyMaxActiveClusters(&n, linear_tc2<BN, NCH>, &cfg);
+    if (err == cudaSuccess && (g_pairs == 0 || n < g_pairs)) g_pairs = n;
+    return err;
+}
+
+// map of an output matrix for 32-row boxes of 128 bytes (64 for codes), or
+// false if its alignment does not allow one
+bool make_out_map(CUtensorMap *tm, CUtensorMapDataType type, int esize, void *p, int cols, int rows, int ld, int box_cols) {
+    if (!p || (reinterpret_cast<uintptr_t>(p) & 15) || (size_t)ld * esize % 16) return false;
+    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    cuuint64_t strides[1] = {(cuuint64_t)ld * esize};
+    cuuint32_t box[2] = {(cuuint32_t)box_cols, 32};
+    cuuint32_t estr[2] = {1, 1};
+    return g_encode(tm, type, 2, p, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                    box_cols * esize == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                    CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int BN, int NCH>
+cudaError_t tc2_launch(const CUtensorMap &ta, const CUtensorMap &tb, int M, int N, int K, const Epi &e, int *status, long tiles,
+                       cudaStream_t st) {
+    CUtensorMap to = ta, th = ta;
+    int outs = 0;
+    if (e.mode == EPI_RESID || e.mode == EPI_F32) {
+        outs = make_out_map(&to, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, e.f32, N, M, e.ldf, 32);
+    } else if ((e.mode == EPI_Q8 || e.mode == EPI_RELU_Q8) && make_out_map(&to, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, e.out, N, M, e.ldo, BN / 2)) {
+        outs = !e.out16 ? 1 : make_out_map(&th, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, e.out16, N, M, e.ldo, 64) ? 3 : 0;
+    }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cs = cudaStreamCaptureStatusNone;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg =
+        tc2_config<BN, NCH>((int)(tiles < g_pairs ? tiles : g_pairs), st, attr, cs != cudaStreamCaptureStatusActive);
+    return cudaLaunchKernelEx(&cfg, linear_tc2<BN, NCH>, ta, tb, to, th, outs, M, N, K, e, status);
+}
+
 constexpr int TC_STAGES = 6;
-// 128 x 256 tiles: half the A-tile bytes per FLOP, for grids with enough
-// tiles; with two K chunks the 512-column accumulator fills TMEM, so that
-// variant keeps one accumulator buffer (its epilogue does not overlap)
 constexpr int TC_STAGES_WIDE = 4;
 // 128 x 64 tiles for grids that would leave SMs idle (a few hundred rows):
 // twice the CTAs, and each streams a third fewer bytes per k-block
@@ -877,6 +1483,10 @@ cudaError_t linear_tc_init() {
     if (err == cudaSuccess) err = tc_attr<128, 2, TC_STAGES, 2>();
     if (err == cudaSuccess) err = tc_attr<256, 1, TC_STAGES_WIDE, 2>();
     if (err == cudaSuccess) err = tc_attr<256, 2, TC_STAGES_WIDE, 1>();
+    if (err == cudaSuccess) err = tc2_init<128, 1>();
+    if (err == cudaSuccess) err = tc2_init<128, 2>();
+    if (err == cudaSuccess) err = tc2_init<256, 1>();
+    if (err == cudaSuccess) err = tc2_init<256, 2>();
     if (err == cudaSuccess) err = tc_attr<64, 1, TC_STAGES_NARROW, 2>();
     if (err == cudaSuccess) err = tc_attr<64, 2, TC_STAGES_NARROW, 2>();
     if (err == cudaSuccess) err = tc_sk_init<2>();
@@ -901,19 +1511,43 @@ cudaError_t launch_linear_tc(const __half *A16, int lda, const __half *W16, int 
     if (M <= 0 || N <= 0) return cudaSuccess;
     if (!linear_tc_shape_ok(M, N, K, lda, ldw, A16, W16)) return cudaErrorInvalidValue;
     const bool two_chunks = K > TC_KB_PER_CHUNK * TC_BK;
-    const long tiles_wide = (long)((M + TC_BM - 1) / TC_BM) * ((N + 255) / 256);
-    const bool wide = N >= 256 && tiles_wide >= g_num_sms;
-    const long tiles_128 = (long)((M + TC_BM - 1) / TC_BM) * ((N + 127) / 128);
-    const bool narrow = !wide && tiles_128 < g_num_sms;
+    const int nkb = (K + TC_BK - 1) / TC_BK;
+    const long mt = (M + TC_BM - 1) / TC_BM, mt2 = (M + 2 * TC_BM - 1) / (2 * TC_BM);
+    const long tiles_128 = mt * ((N + 127) / 128), tiles64 = mt * ((N + SK_BN - 1) / SK_BN);
+    const bool f32m = e.mode == EPI_RESID || e.mode == EPI_F32;
+    // CTA pairs, by the waves of 256 x 256 tiles on the pairs and of 128 x 128
+    // tiles on the SMs.  A pair starts later (cluster, 512 TMEM columns) and its
+    // tile takes longer; with K = 512 and codes out 7.2 + 4.4 us a wave against
+    // 4.4 + 3.5, so it wins where 5 w256 + 3 < 4 w128 (M 4000, N 2048: 15.9 us
+    // against 18.0; M 4400, N 1536, where it does not: 15.8 against 15.0).  The fp32 outputs of
+    // 128 x 128 tiles are slower, two waves (M 5000, N 512, residual 20.2; M 300,
+    // N 8192 14.6) than one of pairs (14.7; 12.8); with equal waves they are not.
+    const long p256 = mt2 * ((N + 255) / 256), p128 = mt2 * ((N + 127) / 128);
+    const long w256 = g_pairs > 0 ? (p256 + g_pairs - 1) / g_pairs : 0, w128 = (tiles_128 + g_num_sms - 1) / g_num_sms;
+    const bool pair256 = g_pairs > 0 && N >= 256 && tiles_128 >= g_num_sms && (f32m ? w256 < w128 : 5 * w256 + 3 < 4 * w128);
+    // 256 x 128 tiles: one wave of pairs where 128 x 64 tiles need two and K is
+    // long (M 4000, N 512, K 2048, residual: 18.1 us against 23.1; K 1024: 13.9
+    // against 15.1; K 512: equal; M 2300, N 1024, K 1024, codes: 11.9 against 13.8)
+    const bool pair128 = !pair256 && nkb >= TC_KB_PER_CHUNK && p128 <= g_pairs && tiles64 > g_num_sms;
+    // 128 x 256 tiles of one CTA: one wave that would be two of 128 x 128 (M 1500,
+    // N 2048, codes: K 512 9.5 us against 10.6, K 1024 13.3 against 15.4, K 2048
+    // 19.1 against 23.9; M 2400, N 2048, K 512, residual: 20.1 against 21.1)
+    const long tiles_wide = mt * ((N + 255) / 256);
+    const bool wide = !pair256 && !pair128 && N >= 256 && w128 == 2 && tiles_wide <= g_num_sms;
+    const bool pair = pair256 || pair128, narrow = !pair && tiles_128 < g_num_sms;
     CUtensorMap ta, tb;
-    if (!make_map(&ta, A16, K, M, lda, TC_BM) || !make_map(&tb, W16, K, N, ldw, wide ? 256 : (narrow ? 64 : 128)))
+    if (!make_map(&ta, A16, K, M, lda, TC_BM) || !make_map(&tb, W16, K, N, ldw, wide ? 256 : pair256 ? 128 : pair || narrow ? 64 : 128))
         return cudaErrorInvalidValue;
+    if (pair256)
+        return two_chunks ? tc2_launch<256, 2>(ta, tb, M, N, K, e, status, p256, st)
+                          : tc2_launch<256, 1>(ta, tb, M, N, K, e, status, p256, st);
+    if (pair)
+        return two_chunks ? tc2_launch<128, 2>(ta, tb, M, N, K, e, status, p128, st)
+                          : tc2_launch<128, 1>(ta, tb, M, N, K, e, status, p128, st);
     if (narrow) {
         // split K over a cluster when the 128 x 64 tiles leave SMs idle: S CTAs
         // per tile, each with at most 16 k-blocks (one exact chunk); K of at
         // least 8 k-blocks (measured: splitting 4 k-blocks in two was slower)
-        const long tiles64 = (long)((M + TC_BM - 1) / TC_BM) * ((N + SK_BN - 1) / SK_BN);
-        const int nkb = (K + TC_BK - 1) / TC_BK;
         if (nkb >= 8 && tiles64 * 4 <= g_num_sms && tiles64 <= g_sk_clusters[4])
             return tc_launch_sk<4>(ta, tb, M, N, K, e, status, st);
         if (nkb >= 8 && nkb <= 32 && tiles64 * 2 <= g_num_sms && tiles64 <= g_sk_clusters[2])

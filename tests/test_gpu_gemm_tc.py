@@ -132,6 +132,41 @@ def test_linear_tc_equals_imma_path():
     assert np.array_equal(got, host(out))
 
 
+@pytest.mark.parametrize("M,N,K", [(19300, 528, 64), (9700, 1008, 1032), (4801, 2001, 512), (9600, 1024, 2048),
+                                   (2500, 512, 2048), (1301, 1000, 1032), (1501, 2000, 1032), (3100, 1008, 512)])
+@pytest.mark.parametrize("mode", [mnmt.EPI_Q8, mnmt.EPI_RELU_Q8, mnmt.EPI_RESID, mnmt.EPI_F32, mnmt.EPI_ARGMAX])
+def test_linear_tc_large_grids(M, N, K, mode):
+    """Grids of several 256x256 tiles per CTA pair, of one wave of 256x128 or 128x256 tiles,
+    ragged in M and N, with and without 16-byte rows, one and two accumulator
+    chunks: the first, last and tile-edge rows against the oracle, all rows
+    against the int8 kernel."""
+    A, W, s_w, b, inv, s_x = _inputs(M + 3 * N + K, M, N, K)
+    gamma = np.float32(0.875)
+    Kp = (K + 63) // 64 * 64  # the int8 kernel's reductions, padded with zeros
+    A8, W8 = (dev(np.pad(x, ((0, 0), (0, Kp - K)))) for x in (A, W))
+    resid = synth.uniform_f32(8, "r", (M, N), -3, 3) if mode == mnmt.EPI_RESID else None
+    rows = np.unique(np.concatenate([np.arange(0, 4), np.arange(126, 130), np.arange(254, 258), np.arange(M - 3, M)]))
+    omode = O.MODE_F32 if mode == mnmt.EPI_ARGMAX else mode
+    ref = O.linear(A[rows], W, s_w, b, s_x, omode, inv_out=inv, gamma=gamma,
+                   resid=None if resid is None else resid[rows])
+    if mode == mnmt.EPI_ARGMAX:
+        keys = torch.zeros(M, dtype=torch.int64, device="cuda")
+        _tc(A, W, s_w, b, inv, s_x, mode, keys=keys)
+        logits = torch.empty((M, N), device="cuda")
+        mnmt.mnmt_linear(A8, W8, dev(s_w), dev(b), s_x, None, 1.0, M, N, Kp, mnmt.EPI_F32, None, logits)
+        got = mnmt.argmax_from_keys(host(keys))
+        assert np.array_equal(got, np.argmax(host(logits), axis=1))
+        assert np.array_equal(got[rows], np.argmax(ref, axis=1))
+        return
+    got = _tc(A, W, s_w, b, inv, s_x, mode, gamma, resid)
+    assert _same(got[rows], ref)
+    codes = mode in (mnmt.EPI_Q8, mnmt.EPI_RELU_Q8)
+    q = torch.zeros((M, N), dtype=torch.int8, device="cuda") if codes else None
+    f = None if codes else (dev(resid).clone() if resid is not None else torch.zeros((M, N), device="cuda"))
+    mnmt.mnmt_linear(A8, W8, dev(s_w), dev(b), s_x, dev(inv), float(gamma), M, N, Kp, mode, q, f)
+    assert _same(got, host(q if codes else f))
+
+
 SWEEP_M = [256, 1024, 4096]
 SWEEP_KN = [(256, 1024), (1024, 256), (512, 2048), (2048, 512), (256, 32000)]
 
