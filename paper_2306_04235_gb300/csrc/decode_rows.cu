@@ -34,6 +34,7 @@
 #include "attn_core.cuh"
 #include "common.cuh"
 #include "decode_rows.h"
+#include "epilogue.cuh"
 #include "internal.h"
 #include "mbarrier.cuh"
 
@@ -309,11 +310,16 @@ MNMT_DEV float dr_rn32(long long S, int e, const DrParams &P) {
 }
 __device__ __noinline__ long long dr_fx_scale(float v, int shift) { return fx_scale(v, shift); }
 
-// Attention of AR rows of one head by a warp: attn_core's arithmetic in one
-// compact loop over (16 keys, set of values).  A row's position j lives at
+// Attention of AR rows of one head by a warp: attn_core's arithmetic in compact
+// loops over (32 keys, set of rows that reads them).  A row's position j lives at
 // kc / vc + (base[b] + prow[b][j]) rs + 64 j; `same` has a bit per 16 keys at
-// which the rows read the same values.  Z comes out of the products too, as
-// one more column tile of ones.  The codes go to every CTA (send).
+// which the rows read the same keys and values.  Z comes out of the products
+// too, as one more column tile of ones.  The codes go to every CTA (send).
+// Bound by the latency of each step's loads and chains (two warps a scheduler):
+// with a lane per key and a row after the other, 102 to 124 keys of 4 rows took
+// 8.5 thousand cycles of scores, 4 to 6.5 of softmax and 11 to 14 of values, in
+// steps of 32 keys and all rows 6.2, 2.1 and 8.2 (512 rows, d = 512: 601 us a
+// step -> 569; 256 rows 542 -> 509; greedy, 128 rows, 495 -> 445).
 template <int AR>
 __device__ __noinline__ void dr_attention(const DrParams &P, const int8_t *q, int q_ld, int nb, int n, float sigma, float rho,
                                           int *sc, const int8_t *kc, const int8_t *vc, size_t rs, const int *base,
@@ -324,42 +330,69 @@ __device__ __noinline__ void dr_attention(const DrParams &P, const int8_t *q, in
     };
     float mine = -INFINITY;  // lane b: row b's maximum
     {
+        // Four lanes read a key (whole lines per load), 8 keys a load; the sum
+        // scattered over the four leaves lane (g, t) with key 8 t + g of 32.
+        // Every step scores the keys against all rows, in one straight run of
+        // independent sums, and keeps those of the rows that read these keys.
         float mx[AR];
-#pragma unroll
-        for (int b = 0; b < AR; b++) mx[b] = -INFINITY;
-#pragma unroll 1
-        for (int j = lane; j < n; j += 32) {
-            int4 kr[4];
-            const int4 *last = nullptr;
-#pragma unroll
-            for (int b = 0; b < AR; b++) {
-                if (b >= nb) break;
-                const int4 *kp = reinterpret_cast<const int4 *>(kc + at(j, b));
-                if (kp != last) {
-#pragma unroll
-                    for (int c = 0; c < 4; c++) kr[c] = kp[c];
-                    last = kp;
-                }
-                int acc = 0;
-#pragma unroll
-                for (int c = 0; c < 4; c++) acc = dot16(reinterpret_cast<const int4 *>(q + b * q_ld)[c], kr[c], acc);
-                const float s = __fmul_rn(__int2float_rn(acc), sigma);
-                sc[b * cap + j] = __float_as_int(s);
-                mx[b] = fmaxf(mx[b], s);
-            }
-        }
+        int4 qr[AR], nx[4];
 #pragma unroll
         for (int b = 0; b < AR; b++) {
-            const float m = warp_max_f(mx[b]);
-            if (lane == b) mine = m;
+            mx[b] = -INFINITY;
+            qr[b] = *reinterpret_cast<const int4 *>(q + (b < nb ? b : 0) * q_ld + 16 * t);
+        }
+        auto kload = [&](int j0, int b) {
+#pragma unroll
+            for (int i = 0; i < 4; i++) nx[i] = *reinterpret_cast<const int4 *>(kc + at(min(j0 + 8 * i + g, n - 1), b) + 16 * t);
+        };
+        kload(0, 0);
+        int j0 = 0, b = 0;
+#pragma unroll 1
+        while (j0 < n) {
+            int4 kr[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) kr[i] = nx[i];
+            const bool one = AR == 1 || ((same >> (j0 >> 4)) & 3u) == 3u, next = one || b + 1 == nb;
+            const int j1 = next ? j0 + 32 : j0, b1 = next ? 0 : b + 1, j = j0 + 8 * t + g;
+            if (j1 < n) kload(j1, b1);  // the next keys are on their way during this step
+#pragma unroll
+            for (int r = 0; r < AR; r++) {
+                int acc[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) acc[i] = dot16(qr[r], kr[i], 0);
+                gemv_reduce<4, 4>(acc, t);
+                const float s = __fmul_rn(__int2float_rn(acc[0]), sigma);
+                if (j < n && (one || r == b)) {
+                    sc[r * cap + j] = __float_as_int(s);
+                    mx[r] = fmaxf(mx[r], s);
+                }
+            }
+            j0 = j1;
+            b = b1;
+        }
+#pragma unroll
+        for (int r = 0; r < AR; r++) {
+            const float m = warp_max_f(mx[r]);
+            if (lane == r) mine = m;
         }
     }
+    __syncwarp();
     const int n16 = (n + 15) & ~15;
+    {
+        float m[AR];
+#pragma unroll
+        for (int r = 0; r < AR; r++) m[r] = __shfl_sync(0xFFFFFFFFu, mine, r);
 #pragma unroll 1
-    for (int b = 0; b < nb; b++) {
-        const float m = __shfl_sync(0xFFFFFFFFu, mine, b);
-        for (int j = lane; j < n16; j += 32)
-            sc[b * cap + j] = j < n ? softmax_weight(__fsub_rn(__int_as_float(sc[b * cap + j]), m)) : 0;
+        for (int j = lane; j < n16; j += 32) {  // the rows' chains of one key run side by side
+            float v[AR];
+#pragma unroll
+            for (int r = 0; r < AR; r++) v[r] = __int_as_float(sc[r * cap + j]);
+#pragma unroll
+            for (int r = 0; r < AR; r++) {
+                const int w = softmax_weight(__fsub_rn(v[r], m[r]));
+                sc[r * cap + j] = j < n ? w : 0;
+            }
+        }
     }
     __syncwarp();
     float acc[9][4];
@@ -369,49 +402,52 @@ __device__ __noinline__ void dr_attention(const DrParams &P, const int8_t *q, in
         for (int i = 0; i < 4; i++) acc[j][i] = 0.0f;
     const int qb = g & 3, sh = g >= 4 ? 8 : 0;
     const int *er = sc + (qb < nb ? qb : 0) * cap + 4 * t;
-    auto vload = [&](int kb, int b, uint2 (&raw)[4]) {
+    uint2 nx[8];
+    auto vload = [&](int j0, int b) {
 #pragma unroll
-        for (int i = 0; i < 4; i++)
-            raw[i] = *reinterpret_cast<const uint2 *>(vc + at(min(kb * 16 + 4 * t + i, n - 1), b) + 8 * g);  // past the end: weight 0
+        for (int i = 0; i < 8; i++)  // past the end: weight 0
+            nx[i] = *reinterpret_cast<const uint2 *>(vc + at(min(j0 + 16 * (i >> 2) + 4 * t + (i & 3), n - 1), b) + 8 * g);
     };
-    const int nkb = n16 >> 4;
-    uint2 nx[4];
-    vload(0, 0, nx);
-    int kb = 0, b = 0;
+    vload(0, 0);
+    int j0 = 0, b = 0;
 #pragma unroll 1
-    while (kb < nkb) {
-        uint2 raw[4];
+    while (j0 < n) {
+        uint2 raw[8];
 #pragma unroll
-        for (int i = 0; i < 4; i++) raw[i] = nx[i];
-        const bool one = (same >> kb) & 1u, next = one || b + 1 == nb;
-        const int kb1 = next ? kb + 1 : kb, b1 = next ? 0 : b + 1;
-        if (kb1 < nkb) vload(kb1, b1, nx);  // the next values are on their way during this step
+        for (int i = 0; i < 8; i++) raw[i] = nx[i];
+        const bool one = AR == 1 || ((same >> (j0 >> 4)) & 3u) == 3u, next = one || b + 1 == nb;
+        const int j1 = next ? j0 + 32 : j0, b1 = next ? 0 : b + 1;
+        if (j1 < n) vload(j1, b1);  // the next values are on their way during this step
         const bool in = qb < nb && (one || qb == b);
-        const uint32_t k01 = in ? 0x00FF00FFu : 0u, k2 = in && g < 4 ? 0x01FF01FFu : 0u;
-        const int4 e = *reinterpret_cast<const int4 *>(er + kb * 16);
-        uint32_t a[4];
-        a[0] = half2_sub_1024((__byte_perm((uint32_t)e.x >> sh, (uint32_t)e.y >> sh, 0x5410) & k01) | 0x64006400u);
-        a[2] = half2_sub_1024((__byte_perm((uint32_t)e.z >> sh, (uint32_t)e.w >> sh, 0x5410) & k01) | 0x64006400u);
-        a[1] = half2_sub_1024((__byte_perm((uint32_t)e.x, (uint32_t)e.y, 0x7632) & k2) | 0x64006400u);
-        a[3] = half2_sub_1024((__byte_perm((uint32_t)e.z, (uint32_t)e.w, 0x7632) & k2) | 0x64006400u);
-        mma_f16_16816(acc[8], a, 0x3C003C00u, 0x3C003C00u);
 #pragma unroll
-        for (int w = 0; w < 2; w++) {
-            uint32_t u[4], bq[4][2];
+        for (int h = 0; h < 2; h++) {
+            const bool inh = in && j0 + 16 * h < n16;
+            const uint32_t k01 = inh ? 0x00FF00FFu : 0u, k2 = inh && g < 4 ? 0x01FF01FFu : 0u;
+            const int4 e = *reinterpret_cast<const int4 *>(er + min(j0 + 16 * h, n16 - 16));
+            uint32_t a[4];
+            a[0] = half2_sub_1024((__byte_perm((uint32_t)e.x >> sh, (uint32_t)e.y >> sh, 0x5410) & k01) | 0x64006400u);
+            a[2] = half2_sub_1024((__byte_perm((uint32_t)e.z >> sh, (uint32_t)e.w >> sh, 0x5410) & k01) | 0x64006400u);
+            a[1] = half2_sub_1024((__byte_perm((uint32_t)e.x, (uint32_t)e.y, 0x7632) & k2) | 0x64006400u);
+            a[3] = half2_sub_1024((__byte_perm((uint32_t)e.z, (uint32_t)e.w, 0x7632) & k2) | 0x64006400u);
+            mma_f16_16816(acc[8], a, 0x3C003C00u, 0x3C003C00u);
 #pragma unroll
-            for (int i = 0; i < 4; i++) u[i] = (w ? raw[i].y : raw[i].x) ^ 0x80808080u;
+            for (int w = 0; w < 2; w++) {
+                uint32_t u[4], bq[4][2];
 #pragma unroll
-            for (int p = 0; p < 2; p++) {
-                const uint32_t lo = __byte_perm(u[2 * p], u[2 * p + 1], 0x5140), hi = __byte_perm(u[2 * p], u[2 * p + 1], 0x7362);
-                bq[0][p] = h2_sub(__byte_perm(lo, 0x64646464u, 0x4140), 0x64806480u);
-                bq[1][p] = h2_sub(__byte_perm(lo, 0x64646464u, 0x4342), 0x64806480u);
-                bq[2][p] = h2_sub(__byte_perm(hi, 0x64646464u, 0x4140), 0x64806480u);
-                bq[3][p] = h2_sub(__byte_perm(hi, 0x64646464u, 0x4342), 0x64806480u);
+                for (int i = 0; i < 4; i++) u[i] = (w ? raw[4 * h + i].y : raw[4 * h + i].x) ^ 0x80808080u;
+#pragma unroll
+                for (int p = 0; p < 2; p++) {
+                    const uint32_t lo = __byte_perm(u[2 * p], u[2 * p + 1], 0x5140), hi = __byte_perm(u[2 * p], u[2 * p + 1], 0x7362);
+                    bq[0][p] = h2_sub(__byte_perm(lo, 0x64646464u, 0x4140), 0x64806480u);
+                    bq[1][p] = h2_sub(__byte_perm(lo, 0x64646464u, 0x4342), 0x64806480u);
+                    bq[2][p] = h2_sub(__byte_perm(hi, 0x64646464u, 0x4140), 0x64806480u);
+                    bq[3][p] = h2_sub(__byte_perm(hi, 0x64646464u, 0x4342), 0x64806480u);
+                }
+#pragma unroll
+                for (int x = 0; x < 4; x++) mma_f16_16816(acc[4 * w + x], a, bq[x][0], bq[x][1]);
             }
-#pragma unroll
-            for (int x = 0; x < 4; x++) mma_f16_16816(acc[4 * w + x], a, bq[x][0], bq[x][1]);
         }
-        kb = kb1;
+        j0 = j1;
         b = b1;
     }
     // as in attn_rows: lanes g < 4 finish the elements 16 t + j of row g, lanes
@@ -681,6 +717,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                     eq = eq && meta[RB + c0] + prow[c0 * cap + j] == meta[RB + c0 + b] + prow[(c0 + b) * cap + j];
                 if (__all_sync(0xFFFFFFFFu, eq)) same |= 1u << kb;
             }
+        if (nb > 1 && nk <= 16 * 31) same |= 0xFFFFFFFFu << ((nk + 15) >> 4);  // no keys there
         if (lane == 0) meta[3 * RB + warp] = (int)same;
     }
 
@@ -834,8 +871,13 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                     pr = nullptr;
                     same = 0xFFFFFFFFu;
                 }
-                dr_attention<AR>(P, qbuf + (c0 + b0) * HC + hl * 64, HC, b1 - b0, n, cross ? Y.sigma2 : Y.sigma1,
-                                 cross ? Y.rho2 : Y.rho1, scw, kc, vc, rs, base, pr, same, out + (uint32_t)(b0 * sa), sa, xbar, nc);
+                auto run = [&](auto rows_c) {
+                    dr_attention<decltype(rows_c)::value>(P, qbuf + (c0 + b0) * HC + hl * 64, HC, b1 - b0, n,
+                                                          cross ? Y.sigma2 : Y.sigma1, cross ? Y.rho2 : Y.rho1, scw, kc, vc, rs,
+                                                          base, pr, same, out + (uint32_t)(b0 * sa), sa, xbar, nc);
+                };
+                if (AR > 1 && b1 - b0 == 1) run(std::integral_constant<int, 1>{});
+                else run(std::integral_constant<int, AR>{});
                 b0 = b1;
             }
             // rows past the batch send zeros: every exchange has its full size
