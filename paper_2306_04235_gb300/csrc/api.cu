@@ -1291,6 +1291,7 @@ int setup_rows_step(mnmt_session *s) {
     std::memset(&P, 0, sizeof(P));
     P.R = R; P.d = c.d_model; P.H = c.n_heads; P.F = c.d_ffn; P.E = c.d_embed; P.V = c.vocab; P.T = s->Tcap;
     P.n_dec = c.n_dec; P.beam = s->k;
+    P.far_caches = ((double)R * s->Tcap + (double)s->B * s->Smax) * 2.0 * c.d_model * c.n_dec > 128e6;  // 129 MB of L2
     P.stream = s->dr_w;
     P.emb_q = m->emb_q; P.emb_s = m->emb_s; P.pe = m->pe; P.emb_scale = m->emb_scale;
     if (m->factorised) { P.proj_w = m->proj.w; P.proj_s = m->proj.s; P.proj_b = m->proj.b; }

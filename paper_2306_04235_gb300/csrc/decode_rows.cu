@@ -119,6 +119,10 @@ MNMT_DEV void dr_send2(uint32_t remote, uint32_t x, uint32_t y, uint32_t bar) {
                  "r"(x), "r"(y), "r"(bar)
                  : "memory");
 }
+// [p, p + bytes) to L2 (16-byte aligned)
+MNMT_DEV void dr_prefetch(const void *p, int bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(p), "r"(bytes) : "memory");
+}
 // barrier over the compute warps
 MNMT_DEV void dr_sync() { asm volatile("bar.sync 1, %0;" ::"n"(DR_WARPS * 32) : "memory"); }
 
@@ -595,6 +599,25 @@ __device__ __noinline__ void dr_layernorm(const DrParams &P, const DrLnRow w, co
     sync();
 }
 
+// One warp: the caches that layer l's attention of these rows and heads reads,
+// to L2.  Caches larger than L2 do not stay there from step to step, and the
+// attention waits for every step of its loads (512 rows 568 -> 555 us a step, 256
+// rows 509 -> 495, greedy 128 rows 444 -> 411; where they stay, 1 % slower).  Not
+// a beam's own keys and values: their rows scatter (559).
+__device__ __noinline__ void dr_prefetch_layer(const DrParams &P, int l, int r0, int rows, int head0, int heads) {
+    const DrLayer &Y = P.layer[l];
+    const int lane = threadIdx.x & 31, s0 = r0 / P.beam, ns = (r0 + rows - 1) / P.beam - s0 + 1, t = *P.t_ptr, per = 2 * heads;
+    for (int k = lane; k < ns * per; k += 32) {
+        const int sent = s0 + k / per, head = head0 + (k % per >> 1), len = P.src_len[sent];
+        dr_prefetch((k & 1 ? Y.cross_v : Y.cross_k) + ((size_t)sent * P.H + head) * P.S * 64,
+                    64 * (len < 1 ? 1 : (len > P.S ? P.S : len)));
+    }
+    for (int k = lane; P.beam == 1 && t > 0 && k < rows * per; k += 32) {
+        const int row = r0 + k / per, head = head0 + (k % per >> 1);
+        dr_prefetch((k & 1 ? Y.self_v : Y.self_k) + ((size_t)row * P.H + head) * P.T * 64, t * 64);
+    }
+}
+
 // NB: the cluster takes 8 NB rows; HPC: heads per CTA (the cluster has H / HPC)
 template <int NB, int HPC>
 __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrParams *__restrict__ Pp) {
@@ -644,12 +667,12 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
 
     if (warp == DR_WARPS) {
         // ---- producer: the CTA's weight stream through the ring ----
-        if (lane == 0) {
-            const uint8_t *src = P.stream + (size_t)c * P.stream_cta;
-            const uint32_t n = (uint32_t)(P.stream_cta / DR_SLOT);
-            uint32_t s = 0, par = 1, i = 0;
-            for (; i < n; i++) {
-                if (i >= (uint32_t)slots && !wait(empty + 8u * s, par)) break;
+        const uint8_t *src = P.stream + (size_t)c * P.stream_cta;
+        const uint32_t n = (uint32_t)(P.stream_cta / DR_SLOT);
+        uint32_t s = 0, par = 1, i = 0;
+        auto feed = [&](uint32_t end) {  // one thread: slots up to `end`; false after a timed-out wait
+            for (; i < end; i++) {
+                if (i >= (uint32_t)slots && !wait(empty + 8u * s, par)) return false;
                 mbar_expect_tx(full + 8u * s, DR_SLOT);
                 bulk_load(dr_smem(ring + s * DR_SLOT), src + (size_t)i * DR_SLOT, DR_SLOT, full + 8u * s);
                 if (++s == (uint32_t)slots) {
@@ -657,11 +680,21 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                     par ^= 1;
                 }
             }
-            // after a timed-out wait: the copies in flight land (bounded) before the CTA ends
-            if (*abort_flag)
-                for (uint32_t k = i > (uint32_t)slots ? i - slots : 0; k < i; k++)
-                    mbar_wait(full + 8u * (k % slots), (k / slots) & 1);
+            return true;
+        };
+        if (!P.far_caches) {
+            if (lane == 0) feed(n);
+        } else {
+            bool ok = true;
+            for (int l = 0; l < P.n_dec && ok; l++) {
+                dr_prefetch_layer(P, l, r0, rows, c * HPC, HPC);
+                if (lane == 0) ok = feed(n / (uint32_t)P.n_dec * (uint32_t)(l + 1));
+                ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+            }
         }
+        // after a timed-out wait: the copies in flight land (bounded) before the CTA ends
+        if (lane == 0 && *abort_flag)
+            for (uint32_t k = i > (uint32_t)slots ? i - slots : 0; k < i; k++) mbar_wait(full + 8u * (k % slots), (k / slots) & 1);
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
         return;

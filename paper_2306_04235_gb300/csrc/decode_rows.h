@@ -36,6 +36,7 @@ struct alignas(16) DrParams {
     float *resid_out;
     int *status;
     // shared-memory carve-up and constants filled by dr_layout
+    int far_caches;  // the decoder's caches exceed L2
     int nc, param_bytes, cap, stride_a, stride_h, slots;
     int off_bar, off_a, off_h, off_y, off_r, off_q, off_red, off_stage, off_prow, off_meta, off_ln, off_ring;
     int ln_w, ln_epl, ln_kd, ln_dodd;  // log2 warps per row, elements per lane; d = ln_dodd 2^ln_kd

@@ -468,6 +468,29 @@ def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, 
         assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
 
 
+@pytest.mark.parametrize("beam,B,n_dec", [(1, 260, 1), (4, 65, 1), (3, 23, 4)])
+def test_batched_cluster_step_with_caches_beyond_l2(beam, B, n_dec, stream, monkeypatch):
+    """Sessions whose caches exceed L2 bring a layer's to it ahead of its
+    attention: the first step (no own keys yet), sentences of one token, beams
+    that straddle clusters, against the kernel-per-operation step."""
+    T = 500
+    cfg = synth.ModelConfig(1, n_dec, 512, 8, 512, 300, 512, 1, 1, max_pos=512)
+    assert (B * beam * T + B * 33) * 2 * 512 * n_dec > 128e6
+    blob = synth.build_blob(cfg, 93, gamma_range=(0.5, 1.5))
+    ids, lens = synth.source_batch(cfg.vocab, B, 1, 33, 7)
+    ids = np.pad(ids, ((0, 0), (0, 33 - ids.shape[1])))
+    out = {}
+    for env in ("1", "0"):
+        monkeypatch.setenv("MNMT_DECODE_CLUSTER", env)
+        tr = mnmt.Translator(blob, B, 33, beam, T, stream)
+        try:
+            out[env] = list(tr.translate(ids, lens, 20)) + [mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_DEC_OUT)]
+        finally:
+            tr.close()
+    for a, b in zip(out["1"], out["0"]):
+        assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
+
+
 @pytest.mark.parametrize("V,beam", [(4096, 4), (8192, 2), (8196, 4), (20000, 3), (32768, 5), (5000, 16), (32764, 8)])
 @pytest.mark.parametrize("flat", [False, True])
 def test_beam_rows_in_registers(V, beam, flat, stream):
