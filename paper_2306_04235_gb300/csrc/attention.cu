@@ -35,22 +35,25 @@ struct DecRows {
     const int *prow;        // [n] physical row of every position (null: all `row`)
     int row, H, h, T, dh;
     MNMT_DEV size_t at(int j) const { return (((size_t)(prow ? prow[j] : row) * H + h) * T + j) * dh; }
-    MNMT_DEV const int8_t *k(int j, int) const { return kc + at(j); }
-    MNMT_DEV const int8_t *v(int j, int) const { return vc + at(j); }
-    MNMT_DEV bool same_block(int) const { return true; }
+    MNMT_DEV const int8_t *k(int j) const { return kc + at(j); }
+    MNMT_DEV const int8_t *v(int j) const { return vc + at(j); }
 };
 
 // XS = false: a warp per (row, head).  XS = true (cross attention with beams):
 // a warp per head and four of a sentence's beams, which read the same keys and
 // values once.  LONGK: more than 512 keys may be attended (self attention only).
-// Warps are independent; blocks of four at up to 84 registers keep 24 warps of
-// loads in flight per SM (whole rows per block, at 102 registers: 16).
-// 512 rows x 8 heads of 64, 80..160 keys (63 MB): 25.9 -> 21.8 us;
-// 256 x 8, 500 of 512 keys: 56.5 -> 38.5; 1 x 8, 500 keys: 25.7 -> 15.8.
+// Warps are independent, in blocks of four, MB of them to an SM: what bounds it
+// is the loads in flight, and whether the grid fits at once.
+// 512 rows x 8 heads of 64, 160 keys (84 MB): 28.0 us with whole rows per block,
+// 26.2 in two waves of 24 warps per SM (6 blocks of 80 registers), 21.3 in one of
+// 28 (7 of 72); 8 of 64 spill, 22.0.  80 keys: 17.8, 17.3, 13.8.  Grids that 24
+// warps per SM hold prefer the registers (256 x 8, 500 of 512 keys: 56.4, 38.2,
+// 39.1).  A key read by DH / 16 lanes instead of one: 512 x 4 heads of 128, 120
+// keys 21.2 -> 17.4; of 64, 1 to 6 %.
 constexpr int DEC_WARPS = 4;
 
-template <int DH, bool XS, bool LONGK>
-__global__ void __launch_bounds__(32 * DEC_WARPS, DH == 128 || LONGK || XS ? 4 : 6) attn_decode(AttnDecArgs a) {
+template <int DH, bool XS, bool LONGK, int MB>
+__global__ void __launch_bounds__(32 * DEC_WARPS, MB) attn_decode(AttnDecArgs a) {
     pdl_grid_wait();
     if (a.skip && *a.skip) return;
     constexpr int NB = XS ? 4 : 1;
@@ -84,7 +87,7 @@ __global__ void __launch_bounds__(32 * DEC_WARPS, DH == 128 || LONGK || XS ? 4 :
     }
     const DecRows rows{a.kc, a.vc, gather ? prow : nullptr, a.cross ? r / a.beam : r, a.H, h, a.T, DH};
     const int d = a.H * DH;
-    attn_rows<DH, NB, true, LONGK>(
+    attn_rows<DH, NB, LONGK>(
         a.q + (size_t)r * d + h * DH, d, nb, n, a.sigma, a.rho, sc, cap, rows, [&](int b, int e, const uint32_t (&words)[DH / 32]) {
             const size_t o = (size_t)(r + b) * d + h * DH + e;
             const bool al = (reinterpret_cast<uintptr_t>(a.ctx) & 3) == 0;
@@ -119,9 +122,11 @@ cudaError_t launch_attention_decode(const AttnDecArgs &a, cudaStream_t st) {
     const int grid = (int)((items + DEC_WARPS - 1) / DEC_WARPS);
     auto go = [&](auto dh) {
         constexpr int DH = decltype(dh)::value;
-        if (xs) launch_pdl(attn_decode<DH, true, false>, grid, block, smem, st, a);
-        else if (a.T > ATT_CORE_MAX_KEYS) launch_pdl(attn_decode<DH, false, true>, grid, block, smem, st, a);
-        else launch_pdl(attn_decode<DH, false, false>, grid, block, smem, st, a);
+        constexpr int MB = DH == 128 ? 4 : 6, MANY = DH == 128 ? 4 : 7;
+        if (xs) launch_pdl(attn_decode<DH, true, false, 4>, grid, block, smem, st, a);
+        else if (a.T > ATT_CORE_MAX_KEYS) launch_pdl(attn_decode<DH, false, true, 4>, grid, block, smem, st, a);
+        else if (grid > MB * device_sm_count()) launch_pdl(attn_decode<DH, false, false, MANY>, grid, block, smem, st, a);
+        else launch_pdl(attn_decode<DH, false, false, MB>, grid, block, smem, st, a);
         return cudaGetLastError();
     };
     switch (a.dh) {
@@ -506,15 +511,17 @@ cudaError_t attention_init() {
     auto dec_attr = [&](auto k, int smem) {
         if (!err) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     };
-    dec_attr(attn_decode<32, false, false>, dec);
-    dec_attr(attn_decode<64, false, false>, dec);
-    dec_attr(attn_decode<128, false, false>, dec);
-    dec_attr(attn_decode<32, true, false>, xs);
-    dec_attr(attn_decode<64, true, false>, xs);
-    dec_attr(attn_decode<128, true, false>, xs);
-    dec_attr(attn_decode<32, false, true>, dec);
-    dec_attr(attn_decode<64, false, true>, dec);
-    dec_attr(attn_decode<128, false, true>, dec);
+    dec_attr(attn_decode<32, false, false, 6>, dec);
+    dec_attr(attn_decode<64, false, false, 6>, dec);
+    dec_attr(attn_decode<32, false, false, 7>, dec);
+    dec_attr(attn_decode<64, false, false, 7>, dec);
+    dec_attr(attn_decode<128, false, false, 4>, dec);
+    dec_attr(attn_decode<32, true, false, 4>, xs);
+    dec_attr(attn_decode<64, true, false, 4>, xs);
+    dec_attr(attn_decode<128, true, false, 4>, xs);
+    dec_attr(attn_decode<32, false, true, 4>, dec);
+    dec_attr(attn_decode<64, false, true, 4>, dec);
+    dec_attr(attn_decode<128, false, true, 4>, dec);
     auto enc = [](int dh) { return ENC_MAX_KEYS * (dh + 16) + ENC_MAX_KEYS * dh + ENC_WARPS * ENC_MAX_KEYS * 4; };
     if (!err) err = cudaFuncSetAttribute(attn_encoder<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc(32));
     if (!err) err = cudaFuncSetAttribute(attn_encoder<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, enc(64));

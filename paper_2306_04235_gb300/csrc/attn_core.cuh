@@ -1,8 +1,9 @@
 // attn_core.cuh -- incremental attention (Eq. 1/2, Fig. 5b) of up to four query
 // rows of one head by one warp, keys and values read from int8 caches.
 //
-//   scores   lane j takes the keys j, j + 32, ...: acc = q . k by dp4a (exact
-//            int32), s = fl(acc sigma); a key row that the rows share is read once.
+//   scores   acc = q . k by dp4a (exact int32), s = fl(acc sigma); a key is read
+//            by DH / 16 lanes, 16 bytes each (a lane per key touched a line for
+//            every 16 bytes), whose sums are scattered over them.
 //   weights  E = rne(exp(s - max) 2^24) in [0, 2^24], kept in shared memory.
 //   context  sum_j E_j v_j on the fp16 tensor cores (mma.sync m16n8k16, 16 keys
 //            per step): E = e0 + 2^8 e1 + 2^16 e2 (e2 <= 256), the operand rows
@@ -20,6 +21,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "epilogue.cuh"
 
 namespace mnmt {
 
@@ -39,42 +41,45 @@ MNMT_DEV uint32_t att_word(uint32_t v, int) { return v; }
 MNMT_DEV uint32_t att_word(const uint2 &v, int k) { return k ? v.y : v.x; }
 MNMT_DEV uint32_t att_word(const uint4 &v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
 
-// Rows: int k(j, b), v(j, b) give the key / value row of position j for query
-// row b; SHARED: the same for every b; same_block(kb): for the 16 keys of step kb.
+// rows.k(j), rows.v(j): the key / value row of position j, for every query row.
 // q: [NB][q_ld] codes of the head (16-byte aligned rows), sc: this warp's
 // [NB][cap] weights, cap a multiple of 16, at least n; n <= ATT_CORE_MAX_KEYS
 // unless LONGK.
 // store(b, e, words): EPG codes from element e of row b.
-template <int DH, int NB, bool SHARED, bool LONGK, typename Rows, typename Store>
+template <int DH, int NB, bool LONGK, typename Rows, typename Store>
 __device__ __forceinline__ void attn_rows(const int8_t *q, int q_ld, int nb, int n, float sigma, float rho, int *sc, int cap,
                         const Rows &rows, const Store &store) {
-    constexpr int QC = DH / 16, EPG = DH / 8, NT = DH / 8;
+    constexpr int LPK = DH / 16, KPL = 32 / LPK, EPG = DH / 8, NT = DH / 8;  // lanes per key, keys per load
     using Vec = typename AttVec<EPG>::T;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int kc = lane % LPK, kg = lane / LPK;
     float mx[NB];
+    int4 qr[NB];
 #pragma unroll
-    for (int b = 0; b < NB; b++) mx[b] = -INFINITY;
+    for (int b = 0; b < NB; b++) {
+        mx[b] = -INFINITY;
+        qr[b] = *reinterpret_cast<const int4 *>(q + (size_t)(b < nb ? b : 0) * q_ld + 16 * kc);
+    }
 #pragma unroll 2
-    for (int j = lane; j < n; j += 32) {
-        int4 kr[QC];
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        int4 kr[LPK];
+#pragma unroll
+        for (int i = 0; i < LPK; i++) kr[i] = *reinterpret_cast<const int4 *>(rows.k(min(j0 + KPL * i + kg, n - 1)) + 16 * kc);
+        const int j = j0 + KPL * kc + kg;  // the key whose sum this lane ends with
 #pragma unroll
         for (int b = 0; b < NB; b++) {
-            if (b > 0 && b >= nb) break;
-            if (b == 0 || !SHARED) {
-                const int4 *kp = reinterpret_cast<const int4 *>(rows.k(j, b));
-                if (b == 0 || kp != reinterpret_cast<const int4 *>(rows.k(j, b - 1))) {
+            int acc[LPK];
 #pragma unroll
-                    for (int c = 0; c < QC; c++) kr[c] = kp[c];
-                }
+            for (int i = 0; i < LPK; i++) acc[i] = dot16(qr[b], kr[i], 0);
+            gemv_reduce<LPK, LPK>(acc, kc);
+            if (j < n && b < nb) {
+                const float s = __fmul_rn(__int2float_rn(acc[0]), sigma);
+                sc[b * cap + j] = __float_as_int(s);
+                mx[b] = fmaxf(mx[b], s);
             }
-            int acc = 0;
-#pragma unroll
-            for (int c = 0; c < QC; c++) acc = dot16(reinterpret_cast<const int4 *>(q + (size_t)b * q_ld)[c], kr[c], acc);
-            const float s = __fmul_rn(__int2float_rn(acc), sigma);
-            sc[b * cap + j] = __float_as_int(s);
-            mx[b] = fmaxf(mx[b], s);
         }
     }
+    __syncwarp();
     const int n16 = (n + 15) & ~15;
     long long Z[NB];
     float iz[NB];
@@ -104,20 +109,20 @@ __device__ __forceinline__ void attn_rows(const int8_t *q, int q_ld, int nb, int
     const int sh = g >= 4 ? 8 : 0;
     const uint32_t m01 = qb < nb ? 0x00FF00FFu : 0u, m2 = qb < nb && g < 4 ? 0x01FF01FFu : 0u;
     const int *er = sc + (qb < nb ? qb : 0) * cap + 4 * t;
-    auto vload = [&](int kb, int b, Vec (&raw)[4]) {
+    auto vload = [&](int kb, Vec (&raw)[4]) {
 #pragma unroll
         for (int i = 0; i < 4; i++) {
             const int key = min(kb * 16 + 4 * t + i, n - 1);  // past the end: weight 0
-            raw[i] = *reinterpret_cast<const Vec *>(rows.v(key, b) + EPG * g);
+            raw[i] = *reinterpret_cast<const Vec *>(rows.v(key) + EPG * g);
         }
     };
-    auto step = [&](int kb, const Vec (&raw)[4], uint32_t k01, uint32_t k2) {
+    auto step = [&](int kb, const Vec (&raw)[4]) {
         const int4 e = *reinterpret_cast<const int4 *>(er + kb * 16);
         uint32_t a[4];
-        a[0] = half2_sub_1024((__byte_perm((uint32_t)e.x >> sh, (uint32_t)e.y >> sh, 0x5410) & k01) | 0x64006400u);
-        a[2] = half2_sub_1024((__byte_perm((uint32_t)e.z >> sh, (uint32_t)e.w >> sh, 0x5410) & k01) | 0x64006400u);
-        a[1] = half2_sub_1024((__byte_perm((uint32_t)e.x, (uint32_t)e.y, 0x7632) & k2) | 0x64006400u);
-        a[3] = half2_sub_1024((__byte_perm((uint32_t)e.z, (uint32_t)e.w, 0x7632) & k2) | 0x64006400u);
+        a[0] = half2_sub_1024((__byte_perm((uint32_t)e.x >> sh, (uint32_t)e.y >> sh, 0x5410) & m01) | 0x64006400u);
+        a[2] = half2_sub_1024((__byte_perm((uint32_t)e.z >> sh, (uint32_t)e.w >> sh, 0x5410) & m01) | 0x64006400u);
+        a[1] = half2_sub_1024((__byte_perm((uint32_t)e.x, (uint32_t)e.y, 0x7632) & m2) | 0x64006400u);
+        a[3] = half2_sub_1024((__byte_perm((uint32_t)e.z, (uint32_t)e.w, 0x7632) & m2) | 0x64006400u);
 #pragma unroll
         for (int w = 0; w < EPG / 4; w++) {
             uint32_t u[4], bq[4][2];
@@ -138,62 +143,43 @@ __device__ __forceinline__ void attn_rows(const int8_t *q, int q_ld, int nb, int
     };
     const int nkb = n16 >> 4;
     int tot[LONGK ? NT : 1][4];
-    if (SHARED || NB == 1) {
-        constexpr int UB = 2;  // steps whose loads are in flight together
-        auto run = [&](int kb, int end) {
-            for (; kb + UB <= end; kb += UB) {
-                Vec raw[UB][4];
+    constexpr int UB = 2;  // steps whose loads are in flight together
+    auto run = [&](int kb, int end) {
+        for (; kb + UB <= end; kb += UB) {
+            Vec raw[UB][4];
 #pragma unroll
-                for (int u = 0; u < UB; u++) vload(kb + u, 0, raw[u]);
+            for (int u = 0; u < UB; u++) vload(kb + u, raw[u]);
 #pragma unroll
-                for (int u = 0; u < UB; u++) step(kb + u, raw[u], m01, m2);
-            }
-            for (; kb < end; kb++) {
-                Vec raw[4];
-                vload(kb, 0, raw);
-                step(kb, raw, m01, m2);
-            }
-        };
-        if (!LONGK) {
-            run(0, nkb);
-        } else {
-#pragma unroll
-            for (int j = 0; j < NT; j++)
-#pragma unroll
-                for (int i = 0; i < 4; i++) tot[LONGK ? j : 0][i] = 0;
-#pragma unroll 1
-            for (int k0 = 0; k0 < nkb; k0 += ATT_CORE_MAX_KEYS / 16) {
-                run(k0, min(nkb, k0 + ATT_CORE_MAX_KEYS / 16));
-#pragma unroll
-                for (int j = 0; j < NT; j++)
-#pragma unroll
-                    for (int i = 0; i < 4; i++) {
-                        tot[LONGK ? j : 0][i] += __float2int_rn(acc[j][i]);
-                        acc[j][i] = 0.0f;
-                    }
-            }
-#pragma unroll
-            for (int j = 0; j < NT; j++)
-#pragma unroll
-                for (int i = 0; i < 4; i++) acc[j][i] = __int_as_float(tot[LONGK ? j : 0][i]);  // carried as bits
+            for (int u = 0; u < UB; u++) step(kb + u, raw[u]);
         }
-    } else {
-        static_assert(!LONGK || SHARED || NB == 1, "long rows are read one query row or a shared set at a time");
-        for (int kb = 0; kb < nkb; kb++) {
-            const bool one = rows.same_block(kb);
+        for (; kb < end; kb++) {
             Vec raw[4];
-            vload(kb, 0, raw);
-            if (one) {
-                step(kb, raw, m01, m2);
-            } else {
-                // the rows hold different values: one product per row, the others' weights masked
-#pragma unroll 1
-                for (int b = 0; b < nb; b++) {
-                    if (b) vload(kb, b, raw);
-                    step(kb, raw, qb == b ? m01 : 0u, qb == b ? m2 : 0u);
-                }
-            }
+            vload(kb, raw);
+            step(kb, raw);
         }
+    };
+    if (!LONGK) {
+        run(0, nkb);
+    } else {
+#pragma unroll
+        for (int j = 0; j < NT; j++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) tot[LONGK ? j : 0][i] = 0;
+#pragma unroll 1
+        for (int k0 = 0; k0 < nkb; k0 += ATT_CORE_MAX_KEYS / 16) {
+            run(k0, min(nkb, k0 + ATT_CORE_MAX_KEYS / 16));
+#pragma unroll
+            for (int j = 0; j < NT; j++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    tot[LONGK ? j : 0][i] += __float2int_rn(acc[j][i]);
+                    acc[j][i] = 0.0f;
+                }
+        }
+#pragma unroll
+        for (int j = 0; j < NT; j++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) acc[j][i] = __int_as_float(tot[LONGK ? j : 0][i]);  // carried as bits
     }
     // lanes g < 4 finish the elements EPG 2 t + j of row g, lanes g >= 4 those
     // from EPG (2 t + 1) of row g - 4

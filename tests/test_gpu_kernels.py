@@ -263,6 +263,18 @@ def test_layernorm_warp_rows(M, d, scale):
     assert np.array_equal(host(oq), ref_q)
 
 
+@pytest.mark.parametrize("R,H,dh,T", [(1217, 3, 32, 65), (1217, 3, 64, 31), (1000, 5, 64, 48), (912, 4, 32, 33)])
+def test_attention_decode_many_warps(R, H, dh, T):
+    """Grids around the 24 warps per SM from which more, smaller warps share an
+    SM (a last block of three warps; exactly 24), keys in part of a group of 32."""
+    q = synth.uniform_int8(5, "q", (R, H, dh))
+    Kc, Vc = synth.uniform_int8(6, "k", (R, H, T, dh)), synth.uniform_int8(7, "v", (R, H, T, dh))
+    n_keys = (1 + np.arange(R) % T).astype(np.int32)
+    ctx = torch.zeros((R, H, dh), dtype=torch.int8, device="cuda")
+    mnmt.mnmt_attention_decode(dev(q), dev(Kc), dev(Vc), dev(n_keys), R, H, dh, T, np.float32(1e-4), np.float32(0.8), ctx)
+    assert np.array_equal(host(ctx), O.attention_decode(q, Kc, Vc, n_keys, np.float32(1e-4), np.float32(0.8)))
+
+
 @pytest.mark.parametrize("R,H,dh,T", [(1, 1, 64, 1), (3, 5, 32, 17), (2, 3, 128, 33), (5, 4, 64, 512), (2, 2, 64, 513), (2, 3, 32, 1024),
                                       (1, 2, 128, 1023)])
 @pytest.mark.parametrize("flat", [False, True])
