@@ -400,7 +400,7 @@ def measure_decode_step(w, flush, steps_run, cluster):
     peak, kind = _peaks()
     achieved = algo / (avg_us * 1e-6) / 1e9
     unit = ("decode_cluster_kernel + vocab_greedy_kernel (one graph launch)" if cluster
-            else "multi-kernel decode step (one graph launch)")
+            else "batched decode step (one graph launch)")
     traffic, stamp = STEP_TRAFFIC.get((wl.name, cluster), (None, None))
     if traffic is not None and stamp != _source_hash(STEP_SOURCES):
         traffic = None
