@@ -745,11 +745,11 @@ __global__ void __launch_bounds__(256) beam_select_kernel(BeamArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// The same step for vocabularies of 4096 to 4096 NV entries (rows of whole,
-// aligned float4s), one block of 1024 threads per row and the row in registers:
+// The same step for vocabularies of 4096 to 32768 entries (rows of whole,
+// aligned float4s), one block of NT threads per row and the row in registers:
 // the logits are read once, and the block that finishes a sentence's last row
 // selects for the sentence (no second kernel).
-//   threshold  the KC-th largest of the 32 warps' maxima: at least KC logits
+//   threshold  the KC-th largest of 32 maxima (of warps or half warps): at least KC logits
 //              reach it and few more (about 9 of them for KC = 8), so listing
 //              those that do is a compare per logit and a handful of insertions;
 //   candidates the row's KC best logits, taken from that list by warp 1 while
@@ -757,20 +757,22 @@ __global__ void __launch_bounds__(256) beam_select_kernel(BeamArgs a) {
 //              full scan where the candidates may not be exact.
 // Bound by issue (exp_own per logit) and the latency of its serial parts.
 // 128 rows of 32000 (32 x beam 4): step 128 -> 113 us with one launch less;
-// 512 rows: 621 -> 607.
+// 512 rows: 621 -> 607.  More rows than SMs: 512 threads, so that two rows share
+// an SM and one's serial parts run under the other's; half of such a row is kept in
+// shared memory (512 rows: 554 -> 543 us a step, 256 rows 494 -> 490).
 // ---------------------------------------------------------------------------
-constexpr int BRR_THREADS = 1024;
 constexpr int BRR_LIST = 256;
+constexpr size_t BRR_ROW_SMEM = 8 * 512 * 16;  // half a row of 32768
 
-template <int KM, int NV>
-__global__ void __launch_bounds__(BRR_THREADS, 1) beam_rows_reg_kernel(BeamArgs a) {
+template <int KM, int NV, int NT, int NS>
+__global__ void __launch_bounds__(NT, 1024 / NT) beam_rows_reg_kernel(BeamArgs a) {
     pdl_grid_wait();
     if (*a.done) return;
-    constexpr int KC = KM + 4, NT = BRR_THREADS;
+    constexpr int KC = KM + 4, NW = NT / 32, HM = 32 / NW;  // maxima per warp
     const int r = blockIdx.x, k = a.k, V = a.V;
     const int lb = r % k;  // beam index within the sentence
     unsigned long long *out = a.cand + (size_t)r * k;
-    extern __shared__ int anc_old[];  // [k][T]
+    extern __shared__ __align__(16) int anc_old[];  // [k][T]; before: [NS][NT] float4s of the row
     __shared__ float s_mx[32], s_lam;
     __shared__ long long s_z[32];
     __shared__ unsigned long long s_list[BRR_LIST], s_cand[KC], s_key[32];
@@ -784,22 +786,36 @@ __global__ void __launch_bounds__(BRR_THREADS, 1) beam_rows_reg_kernel(BeamArgs 
         const float *l = a.logits + (size_t)r * V;
         const float4 *l4 = reinterpret_cast<const float4 *>(l);
         const int n4 = V >> 2;
-        float4 v[NV];
+        constexpr int NR = NV - NS;  // float4s of a thread in registers; NS more in its own slots of shared memory
+        float4 *sv = reinterpret_cast<float4 *>(anc_old) + threadIdx.x;
+        float4 v[NR];
         float mx = NI;
-#pragma unroll
-        for (int i = 0; i < NV; i++) {
+        auto load = [&](int i) {
             const int n = i * NT + threadIdx.x;
-            v[i] = n < n4 ? l4[n] : make_float4(NI, NI, NI, NI);
+            return n < n4 ? l4[n] : make_float4(NI, NI, NI, NI);
+        };
+        if (NS > 0) {
+            float4 u[NS > 0 ? NS : 1];
+#pragma unroll
+            for (int i = 0; i < NS; i++) u[i] = load(NR + i);
+#pragma unroll
+            for (int i = 0; i < NS; i++) {
+                sv[i * NT] = u[i];
+                mx = fmaxf(mx, fmaxf(fmaxf(u[i].x, u[i].y), fmaxf(u[i].z, u[i].w)));
+            }
         }
 #pragma unroll
-        for (int i = 0; i < NV; i++) mx = fmaxf(mx, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
-        mx = warp_max_f(mx);
-        if (lane == 0) s_mx[warp] = mx;
+        for (int i = 0; i < NR; i++) v[i] = load(i);
+#pragma unroll
+        for (int i = 0; i < NR; i++) mx = fmaxf(mx, fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)));
+#pragma unroll
+        for (int o = 16 / HM; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+        if (lane % (32 / HM) == 0) s_mx[HM * warp + lane / (32 / HM)] = mx;
         if (threadIdx.x == 0) s_cnt = 0;
         __syncthreads();
         const float wm = s_mx[lane];
         const float m = warp_max_f(wm);
-        int rank = 0;  // of this lane's warp maximum (ties by lane)
+        int rank = 0;  // of this lane's maximum (ties by lane)
 #pragma unroll
         for (int i = 0; i < 32; i++) {
             const float o = __shfl_sync(0xFFFFFFFFu, wm, i);
@@ -808,12 +824,11 @@ __global__ void __launch_bounds__(BRR_THREADS, 1) beam_rows_reg_kernel(BeamArgs 
         const unsigned at = __ballot_sync(0xFFFFFFFFu, rank == KC - 1);
         const float thr = at ? __shfl_sync(0xFFFFFFFFu, wm, __ffs(at) - 1) : NI;
         uint32_t z = 0;  // at most 4 NV weights of 2^24
-#pragma unroll
-        for (int i = 0; i < NV; i++) {
-            z += (uint32_t)(softmax_weight(__fsub_rn(v[i].x, m)) + softmax_weight(__fsub_rn(v[i].y, m)) +
-                            softmax_weight(__fsub_rn(v[i].z, m)) + softmax_weight(__fsub_rn(v[i].w, m)));
-            if (fmaxf(fmaxf(v[i].x, v[i].y), fmaxf(v[i].z, v[i].w)) >= thr && i * NT + (int)threadIdx.x < n4) {
-                const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+        auto take = [&](const float4 &x, int i) {
+            z += (uint32_t)(softmax_weight(__fsub_rn(x.x, m)) + softmax_weight(__fsub_rn(x.y, m)) +
+                            softmax_weight(__fsub_rn(x.z, m)) + softmax_weight(__fsub_rn(x.w, m)));
+            if (fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w)) >= thr && i * NT + (int)threadIdx.x < n4) {
+                const float e[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
                 for (int q = 0; q < 4; q++)
                     if (e[q] >= thr) {
@@ -821,14 +836,18 @@ __global__ void __launch_bounds__(BRR_THREADS, 1) beam_rows_reg_kernel(BeamArgs 
                         if (p < BRR_LIST) s_list[p] = pack_key(e[q], (uint32_t)(4 * (i * NT + (int)threadIdx.x) + q));
                     }
             }
-        }
+        };
+#pragma unroll
+        for (int i = 0; i < NR; i++) take(v[i], i);
+#pragma unroll
+        for (int i = 0; i < NS; i++) take(sv[i * NT], NR + i);
         const long long zw = (long long)__reduce_add_sync(0xFFFFFFFFu, z & 0xFFFFu) +
                              ((long long)__reduce_add_sync(0xFFFFFFFFu, z >> 16) << 16);
         if (lane == 0) s_z[warp] = zw;
         __syncthreads();
         const int cnt = s_cnt;
         if (warp == 0) {
-            const long long Z = warp_sum_ll(s_z[lane]);
+            const long long Z = warp_sum_ll(lane < NW ? s_z[lane] : 0ll);
             // lambda = ln Z - 24 ln 2 (log of the normaliser of the 2^-24 weights)
             if (lane == 0) s_lam = __double2float_rn(__dadd_rn(log_own(__ll2double_rn(Z)), -0x1.0a2b23f3bab73p+4));
         } else if (warp == 1 && cnt <= BRR_LIST) {
@@ -902,9 +921,19 @@ __global__ void __launch_bounds__(BRR_THREADS, 1) beam_rows_reg_kernel(BeamArgs 
 
 template <int KM>
 static cudaError_t launch_beam_rows_reg(const BeamArgs &a, cudaStream_t st) {
-    const size_t smem = (size_t)a.k * a.T * sizeof(int);
-    if (a.V <= 8192) launch_pdl(beam_rows_reg_kernel<KM, 2>, a.B * a.k, BRR_THREADS, smem, st, a);
-    else launch_pdl(beam_rows_reg_kernel<KM, 8>, a.B * a.k, BRR_THREADS, smem, st, a);
+    size_t smem = (size_t)a.k * a.T * sizeof(int);
+    const int R = a.B * a.k;
+    if (R <= device_sm_count()) {
+        if (a.V <= 8192) launch_pdl(beam_rows_reg_kernel<KM, 2, 1024, 0>, R, 1024, smem, st, a);
+        else launch_pdl(beam_rows_reg_kernel<KM, 8, 1024, 0>, R, 1024, smem, st, a);
+    } else {
+        if (a.V <= 8192) {
+            launch_pdl(beam_rows_reg_kernel<KM, 4, 512, 0>, R, 512, smem, st, a);
+        } else {
+            if (smem < BRR_ROW_SMEM) smem = BRR_ROW_SMEM;
+            launch_pdl(beam_rows_reg_kernel<KM, 16, 512, 8>, R, 512, smem, st, a);
+        }
+    }
     return cudaGetLastError();
 }
 
@@ -965,17 +994,24 @@ __global__ void finalize_kernel(FinalArgs a) {
 // Opt the beam reorder kernels into the shared memory of their largest shape
 // (k = 16 hypotheses x 1024 positions); once per process, before any capture.
 cudaError_t rows_init() {
-    const int anc = BEAM_MAX * 1024 * (int)sizeof(int);
+    const int anc = BEAM_MAX * 1024 * (int)sizeof(int);  // also BRR_ROW_SMEM
+    static_assert(BEAM_MAX * 1024 * sizeof(int) >= BRR_ROW_SMEM, "one limit for both uses");
     cudaError_t err = cudaFuncSetAttribute(beam_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, anc);
     auto reg = [&](auto k) {
         if (err == cudaSuccess) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, anc);
     };
-    reg(beam_rows_reg_kernel<4, 2>);
-    reg(beam_rows_reg_kernel<4, 8>);
-    reg(beam_rows_reg_kernel<8, 2>);
-    reg(beam_rows_reg_kernel<8, 8>);
-    reg(beam_rows_reg_kernel<16, 2>);
-    reg(beam_rows_reg_kernel<16, 8>);
+    reg(beam_rows_reg_kernel<4, 2, 1024, 0>);
+    reg(beam_rows_reg_kernel<4, 8, 1024, 0>);
+    reg(beam_rows_reg_kernel<4, 4, 512, 0>);
+    reg(beam_rows_reg_kernel<4, 16, 512, 8>);
+    reg(beam_rows_reg_kernel<8, 2, 1024, 0>);
+    reg(beam_rows_reg_kernel<8, 8, 1024, 0>);
+    reg(beam_rows_reg_kernel<8, 4, 512, 0>);
+    reg(beam_rows_reg_kernel<8, 16, 512, 8>);
+    reg(beam_rows_reg_kernel<16, 2, 1024, 0>);
+    reg(beam_rows_reg_kernel<16, 8, 1024, 0>);
+    reg(beam_rows_reg_kernel<16, 4, 512, 0>);
+    reg(beam_rows_reg_kernel<16, 16, 512, 8>);
     return err;
 }
 

@@ -516,3 +516,24 @@ def test_beam_rows_in_registers(V, beam, flat, stream):
     o_ids, o_len, o_sc = O.translate(blob, ids, lens, beam, T)
     assert np.array_equal(g_ids, o_ids) and np.array_equal(g_len, o_len)
     assert np.array_equal(g_sc.view(np.uint32), o_sc.view(np.uint32))
+
+
+@pytest.mark.parametrize("V,beam,B", [(4096, 4, 39), (8192, 5, 31), (8196, 8, 20), (20000, 16, 10), (32764, 4, 39), (32768, 3, 51)])
+@pytest.mark.parametrize("flat", [False, True])
+def test_beam_rows_two_to_an_sm(V, beam, B, flat, stream):
+    """More rows than SMs: blocks of 512 threads, half of a row above 8192
+    entries in shared memory; flat: as above, ties in either half."""
+    cfg = synth.ModelConfig(1, 1, 64, 1, 64, V, 64, 1, 1, max_pos=32)
+    lo = V - 900 if flat and V % 8 else 0
+    bias = {lo + i: 40.0 for i in range(0, 900)} if flat else None
+    blob = synth.build_blob(cfg, 19, gamma_range=(0.5, 1.5), out_bias=bias)
+    ids, lens = synth.source_batch(V, B, 3, 9, 8)
+    T = 5
+    tr = mnmt.Translator(blob, B, ids.shape[1], beam, T, stream)
+    try:
+        g_ids, g_len, g_sc = tr.translate(ids, lens, T)
+    finally:
+        tr.close()
+    o_ids, o_len, o_sc = O.translate(blob, ids, lens, beam, T, n_threads=4)
+    assert np.array_equal(g_ids, o_ids) and np.array_equal(g_len, o_len)
+    assert np.array_equal(g_sc.view(np.uint32), o_sc.view(np.uint32))
