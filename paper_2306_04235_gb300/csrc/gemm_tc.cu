@@ -35,6 +35,8 @@
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "epilogue.cuh"
 #include "internal.h"
@@ -496,32 +498,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc(const __grid_constant
 // 256 columns: 64 KB of operands feed 128 x 256 x 64 products per SM, as much as
 // shared memory moves (128 bytes a cycle, written once and read once) in the 512
 // cycles that the tensor core takes; 128 columns: 620 cycles a k-block for half
-// of the products.  Four stages, 128 KB in flight, are what two staging blocks a
-// warp leave room for.
+// of the products.  The ring's depth is what the staging blocks leave room for:
+// four stages with codes, five with fp32 outputs, whose two column constants are
+// then single and whose ring has no slack (16384 x 512 x 2048 42.5 -> 39.2 us,
+// 8192 x 8192 x 2048 193 -> 182).
 // Tried and not better: k-blocks brought to L2 ahead of the ring, pairs starting
 // at different k-blocks, residuals of the second two blocks brought to L2 early.
 // us, 128 x 256 tiles of one CTA -> here (before and after, inputs larger than L2):
-//   16384 x 512 x 2048 residual    57.6 -> 43.0;  K = 512     35.6 -> 24.5
-//   16384 x 2048 x 512 codes       46.5 -> 40.2;  N = 1536    38.5 -> 33.6
-//   6400 x 512 x 2048 residual     29.1 -> 24.3;  K = 512     20.9 -> 15.7
-//   512 x 32000 x 512 fp32         45.8 -> 30.0;  256 rows    27.2 -> 19.6
-//   8192 x 8192 x 1024 codes       96.8 -> 90.2;  2048, fp32 281.3 -> 196 (1400 TFLOP/s)
+//   16384 x 512 x 2048 residual    57.6 -> 39.2;  K = 512     35.6 -> 23.8
+//   16384 x 2048 x 512 codes       46.5 -> 39.7;  N = 1536    38.5 -> 33.6
+//   6400 x 512 x 2048 residual     29.1 -> 22.3;  K = 512     20.9 -> 15.4
+//   512 x 32000 x 512 fp32         45.8 -> 29.3;  256 rows    27.2 -> 18.9
+//   8192 x 8192 x 1024 codes       96.8 -> 90.6;  2048, fp32 281.3 -> 182 (1510 TFLOP/s)
 // ---------------------------------------------------------------------------
 constexpr int T2_BLK = 4096;  // one staging block: 32 rows x 128 bytes
 
-template <int BN>
+template <int BN, bool F32>
 struct T2Layout {
-    static constexpr int STAGES = BN == 256 ? 4 : 6;
+    static constexpr int STAGES = BN == 256 ? (F32 ? 5 : 4) : 6;
+    static constexpr int NC = F32 ? 2 : 3, CBUF = BN == 256 && F32 ? 1 : 2;  // column constants, buffers of them
     static constexpr uint32_t A_BYTES = TC_BM * TC_BK * 2;
     static constexpr uint32_t STAGE = A_BYTES + (BN / 2) * TC_BK * 2;     // A rows, then W rows
     static constexpr uint32_t OFF_STG = STAGES * STAGE;                   // [8 warps][2] blocks
-    static constexpr uint32_t OFF_COLS = OFF_STG + TC_EPI_WARPS * 2 * T2_BLK;  // [2][3][BN] fp32
-    static constexpr uint32_t OFF_BARS = OFF_COLS + 2 * 3 * BN * 4;
+    static constexpr uint32_t OFF_COLS = OFF_STG + TC_EPI_WARPS * 2 * T2_BLK;  // [CBUF][NC][BN] fp32
+    static constexpr uint32_t OFF_BARS = OFF_COLS + CBUF * NC * BN * 4;
     // full, empty, acc_full[2], acc_empty[2], done, residual[8 warps][2]
     static constexpr int NBARS = 2 * STAGES + 5 + 2 * TC_EPI_WARPS;
     static constexpr uint32_t OFF_MISC = OFF_BARS + NBARS * 8;
     static constexpr uint32_t BYTES = OFF_MISC + 16;
-    static constexpr size_t SMEM = 1024 + BYTES;
+    // five stages leave no slack to align the ring: the kernel checks that
+    // shared memory starts on 1024 bytes
+    static constexpr uint32_t SLACK = BN == 256 && F32 ? 0 : 1024;
+    static constexpr size_t SMEM = SLACK + BYTES;
 };
 
 __device__ __forceinline__ uint32_t t2_mapa(uint32_t local, uint32_t rank) {
@@ -658,20 +666,25 @@ __device__ __forceinline__ int8_t *epi_dst16(const Epi &e, int row, int col, int
 }
 
 // outs: 1 = tmO describes the output matrix (fp32, or codes), 2 = tmH its fp16 copy
-template <int BN, int NCH>
+// F32: fp32 outputs (with or without residuals), else codes or the argmax
+template <int BN, int NCH, bool F32>
 __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constant__ CUtensorMap tmA,
                                                             const __grid_constant__ CUtensorMap tmB,
                                                             const __grid_constant__ CUtensorMap tmO,
                                                             const __grid_constant__ CUtensorMap tmH, int outs, int M, int N,
                                                             int K, Epi e, int *status) {
     pdl_grid_wait();
-    using L = T2Layout<BN>;
+    using L = T2Layout<BN, F32>;
     constexpr uint32_t IDESC = idesc_f16(2 * TC_BM, BN);
     constexpr int STAGES = L::STAGES, ACC_COLS = NCH * BN;
     constexpr int NBUF = 2 * ACC_COLS <= 512 ? 2 : 1;  // accumulator buffers
     if (e.skip && *e.skip) return;  // one flag for every CTA of the grid
 
-    extern __shared__ uint8_t tc_raw[];
+    extern __shared__ __align__(1024) uint8_t tc_raw[];
+    if (L::SLACK == 0 && (s_addr(tc_raw) & 1023)) {  // the same for every CTA of the grid
+        if (threadIdx.x == 0) set_status(status, MNMT_ECUDA);
+        return;
+    }
     uint8_t *sm = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(tc_raw) + 1023) & ~(uintptr_t)1023);
     float *cols = reinterpret_cast<float *>(sm + L::OFF_COLS);
     const uint32_t bars = s_addr(sm + L::OFF_BARS);
@@ -790,8 +803,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constan
         constexpr int PL = NBUF == 2 ? 1 : NB;     // blocks read at a time: a single buffer is released at once
         const int ew = warp - 2, q = warp & 3, cw = RB * (ew >> 2);  // rows 32 q .., columns cw ..
         const int t = e.t_ptr ? *e.t_ptr : 0;
-        const bool f32m = e.mode == EPI_RESID || e.mode == EPI_F32, plain = e.mode == EPI_Q8 || e.mode == EPI_RELU_Q8;
-        const bool tma = outs & 1, h16 = outs & 2, cache = !f32m && !plain && e.mode != EPI_ARGMAX && epi_vec_ok(e) && N % 16 == 0;
+        constexpr bool f32m = F32;
+        const bool plain = !F32 && (e.mode == EPI_Q8 || e.mode == EPI_RELU_Q8), argmax = !F32 && e.mode == EPI_ARGMAX;
+        const bool with_resid = F32 && e.mode == EPI_RESID;
+        const bool tma = outs & 1, h16 = outs & 2, cache = !f32m && !plain && !argmax && epi_vec_ok(e) && N % 16 == 0;
         uint8_t *blk = sm + L::OFF_STG + ew * 2 * T2_BLK;
         const uint32_t blk_s = s_addr(blk);
         uint32_t rphase = 0;  // of the two residual barriers, a bit each
@@ -803,7 +818,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constan
             if (ti < BN && tile < tiles && n < N) {
                 k_sw = e.s_w[n];
                 k_b = e.bias[n];
-                k_inv = e.inv_out ? e.inv_out[n] : 0.0f;
+                if (!F32) k_inv = e.inv_out ? e.inv_out[n] : 0.0f;
             }
         };
         fetch(pair);
@@ -811,14 +826,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constan
         for (int tile = pair; tile < tiles; tile += pairs, lt++) {
             const int n0 = tile_n(tile), row0 = tile_m(tile) + (int)rank * TC_BM + 32 * q, col0 = n0 + cw;
             const bool mine = row0 < M && col0 < N;
-            float *c_sc = cols + (lt & 1) * 3 * BN, *c_b = c_sc + BN, *c_inv = c_b + BN;
+            float *c_sc = cols + (L::CBUF == 2 ? lt & 1 : 0) * L::NC * BN, *c_b = c_sc + BN, *c_inv = c_b + BN;
+            if (L::CBUF == 1 && lt > 0) epi_bar_sync();  // the previous tile's constants have been read
             if (ti < BN) {
                 c_sc[ti] = __fmul_rn(e.s_x, k_sw);
                 c_b[ti] = k_b;
-                c_inv[ti] = k_inv;
+                if (!F32) c_inv[ti] = k_inv;
             }
             fetch(tile + pairs);
-            const bool resid = tma && e.mode == EPI_RESID && mine;
+            const bool resid = tma && with_resid && mine;
             // one thread: the residuals of block b into their staging block, which is free
             auto load_resid = [&](int b) {
                 const uint32_t rb = resid_bar(2 * ew + (b & 1));
@@ -899,7 +915,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constan
                     const float(&acc)[32] = a[PL > 1 ? b : 0];
                     const float *scb = sc + 32 * b, *bsb = bs + 32 * b, *invb = inv + 32 * b;
                     uint8_t *p = blk + (b & 1) * T2_BLK;
-                    if (e.mode == EPI_ARGMAX) {
+                    if (argmax) {
 #pragma unroll
                         for (int g = 0; g < 8; g++) {
                             const float4 s4 = *reinterpret_cast<const float4 *>(scb + 4 * g), b4 = *reinterpret_cast<const float4 *>(bsb + 4 * g);
@@ -915,7 +931,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constan
                             }
                         }
                     } else if (f32m && tma) {
-                        if (e.mode == EPI_RESID) {
+                        if (with_resid) {
                             if (!mbar_wait(resid_bar(2 * ew + (b & 1)), (rphase >> (b & 1)) & 1)) {
                                 *abort_flag = 1;
                                 set_status(status, MNMT_ETIMEOUT);
@@ -934,7 +950,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constan
                         if (lane == 0) {
                             t2_store(&tmO, col0 + 32 * b, row0, blk_s + (b & 1) * T2_BLK);
                             t2_store_commit();
-                            if (NB == 4 && b == 1 && e.mode == EPI_RESID) {  // the second pair of blocks
+                            if (NB == 4 && b == 1 && with_resid) {  // the second pair of blocks
                                 t2_store_wait_read<1>();
                                 if (col0 + 64 < N) load_resid(2);
                                 t2_store_wait_read<0>();
@@ -974,7 +990,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) linear_tc2(const __grid_constan
                     }
                 }
             }
-            if (e.mode == EPI_ARGMAX) {  // pack_key(value, column)
+            if (argmax) {  // pack_key(value, column)
                 if (row0 + lane < M) atomicMax(e.keys + row0 + lane, ((unsigned long long)bk << 32) | (0xFFFFFFFFu - bi));
             } else if (plain && tma) {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1400,12 +1416,12 @@ cudaError_t tc_launch_sk(const CUtensorMap &ta, const CUtensorMap &tb, int M, in
     return cudaLaunchKernelEx(&cfg, linear_tc_sk<S>, ta, tb, M, N, K, e, status);
 }
 
-template <int BN, int NCH>
+template <int BN, int NCH, bool F32>
 cudaLaunchConfig_t tc2_config(int pairs, cudaStream_t st, cudaLaunchAttribute (&attr)[2], bool pdl) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(2 * pairs));
     cfg.blockDim = dim3(TC_THREADS);
-    cfg.dynamicSmemBytes = T2Layout<BN>::SMEM;
+    cfg.dynamicSmemBytes = T2Layout<BN, F32>::SMEM;
     cfg.stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
@@ -1418,14 +1434,14 @@ cudaLaunchConfig_t tc2_config(int pairs, cudaStream_t st, cudaLaunchAttribute (&
     return cfg;
 }
 
-template <int BN, int NCH>
+template <int BN, int NCH, bool F32>
 cudaError_t tc2_init() {
-    cudaError_t err = cudaFuncSetAttribute(linear_tc2<BN, NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T2Layout<BN>::SMEM);
+    cudaError_t err = cudaFuncSetAttribute(linear_tc2<BN, NCH, F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T2Layout<BN, F32>::SMEM);
     if (err != cudaSuccess) return err;
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = tc2_config<BN, NCH>(64, nullptr, attr, false);
+    cudaLaunchConfig_t cfg = tc2_config<BN, NCH, F32>(64, nullptr, attr, false);
     int n = 0;
-    err = cudaOccupancyMaxActiveClusters(&n, linear_tc2<BN, NCH>, &cfg);
+    err = cudaOccupancyMaxActiveClusters(&n, linear_tc2<BN, NCH, F32>, &cfg);
     if (err == cudaSuccess && (g_pairs == 0 || n < g_pairs)) g_pairs = n;
     return err;
 }
@@ -1443,12 +1459,12 @@ bool make_out_map(CUtensorMap *tm, CUtensorMapDataType type, int esize, void *p,
                     CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int NCH>
+template <int BN, int NCH, bool F32>
 cudaError_t tc2_launch(const CUtensorMap &ta, const CUtensorMap &tb, int M, int N, int K, const Epi &e, int *status, long tiles,
                        cudaStream_t st) {
     CUtensorMap to = ta, th = ta;
     int outs = 0;
-    if (e.mode == EPI_RESID || e.mode == EPI_F32) {
+    if (F32) {
         outs = make_out_map(&to, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, e.f32, N, M, e.ldf, 32);
     } else if ((e.mode == EPI_Q8 || e.mode == EPI_RELU_Q8) && make_out_map(&to, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, e.out, N, M, e.ldo, BN / 2)) {
         outs = !e.out16 ? 1 : make_out_map(&th, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, e.out16, N, M, e.ldo, 64) ? 3 : 0;
@@ -1457,8 +1473,8 @@ cudaError_t tc2_launch(const CUtensorMap &ta, const CUtensorMap &tb, int M, int 
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cs = cudaStreamCaptureStatusNone;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg =
-        tc2_config<BN, NCH>((int)(tiles < g_pairs ? tiles : g_pairs), st, attr, cs != cudaStreamCaptureStatusActive);
-    return cudaLaunchKernelEx(&cfg, linear_tc2<BN, NCH>, ta, tb, to, th, outs, M, N, K, e, status);
+        tc2_config<BN, NCH, F32>((int)(tiles < g_pairs ? tiles : g_pairs), st, attr, cs != cudaStreamCaptureStatusActive);
+    return cudaLaunchKernelEx(&cfg, linear_tc2<BN, NCH, F32>, ta, tb, to, th, outs, M, N, K, e, status);
 }
 
 constexpr int TC_STAGES = 6;
@@ -1483,10 +1499,14 @@ cudaError_t linear_tc_init() {
     if (err == cudaSuccess) err = tc_attr<128, 2, TC_STAGES, 2>();
     if (err == cudaSuccess) err = tc_attr<256, 1, TC_STAGES_WIDE, 2>();
     if (err == cudaSuccess) err = tc_attr<256, 2, TC_STAGES_WIDE, 1>();
-    if (err == cudaSuccess) err = tc2_init<128, 1>();
-    if (err == cudaSuccess) err = tc2_init<128, 2>();
-    if (err == cudaSuccess) err = tc2_init<256, 1>();
-    if (err == cudaSuccess) err = tc2_init<256, 2>();
+    if (err == cudaSuccess) err = tc2_init<128, 1, false>();
+    if (err == cudaSuccess) err = tc2_init<128, 1, true>();
+    if (err == cudaSuccess) err = tc2_init<128, 2, false>();
+    if (err == cudaSuccess) err = tc2_init<128, 2, true>();
+    if (err == cudaSuccess) err = tc2_init<256, 1, false>();
+    if (err == cudaSuccess) err = tc2_init<256, 1, true>();
+    if (err == cudaSuccess) err = tc2_init<256, 2, false>();
+    if (err == cudaSuccess) err = tc2_init<256, 2, true>();
     if (err == cudaSuccess) err = tc_attr<64, 1, TC_STAGES_NARROW, 2>();
     if (err == cudaSuccess) err = tc_attr<64, 2, TC_STAGES_NARROW, 2>();
     if (err == cudaSuccess) err = tc_sk_init<2>();
@@ -1538,12 +1558,15 @@ cudaError_t launch_linear_tc(const __half *A16, int lda, const __half *W16, int 
     CUtensorMap ta, tb;
     if (!make_map(&ta, A16, K, M, lda, TC_BM) || !make_map(&tb, W16, K, N, ldw, wide ? 256 : pair256 ? 128 : pair || narrow ? 64 : 128))
         return cudaErrorInvalidValue;
-    if (pair256)
-        return two_chunks ? tc2_launch<256, 2>(ta, tb, M, N, K, e, status, p256, st)
-                          : tc2_launch<256, 1>(ta, tb, M, N, K, e, status, p256, st);
-    if (pair)
-        return two_chunks ? tc2_launch<128, 2>(ta, tb, M, N, K, e, status, p128, st)
-                          : tc2_launch<128, 1>(ta, tb, M, N, K, e, status, p128, st);
+    auto go = [&](auto f32) {
+        constexpr bool F = decltype(f32)::value;
+        if (pair256)
+            return two_chunks ? tc2_launch<256, 2, F>(ta, tb, M, N, K, e, status, p256, st)
+                              : tc2_launch<256, 1, F>(ta, tb, M, N, K, e, status, p256, st);
+        return two_chunks ? tc2_launch<128, 2, F>(ta, tb, M, N, K, e, status, p128, st)
+                          : tc2_launch<128, 1, F>(ta, tb, M, N, K, e, status, p128, st);
+    };
+    if (pair) return f32m ? go(std::true_type{}) : go(std::false_type{});
     if (narrow) {
         // split K over a cluster when the 128 x 64 tiles leave SMs idle: S CTAs
         // per tile, each with at most 16 k-blocks (one exact chunk); K of at
