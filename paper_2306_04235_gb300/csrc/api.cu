@@ -588,6 +588,7 @@ struct mnmt_session {
     int graph_B = -1, graph_S = -1;
     // cluster decode step (small greedy batches)
     DcParams *d_dc = nullptr;
+    DcParams dc_host = {};    // what was last copied there
     float *dc_ln = nullptr;  // the cluster step's LayerNorm vectors, contiguous
     bool use_cluster = false;
     int dc_S = 0;  // host source of the parameter block's S when it is updated
@@ -596,6 +597,7 @@ struct mnmt_session {
     int dc_flags = -1;  // the compiled-in model bits of its step kernel (dc_flags)
     // batched decode step on clusters of 8 dr_nb rows
     DrParams *d_dr = nullptr;
+    DrParams dr_host = {};    // what was last copied there
     uint8_t *dr_w = nullptr;  // the decoder's weights as it consumes them
     bool rows_ok = false;   // the model and the session allow it
     bool use_rows = false;
@@ -1203,7 +1205,7 @@ int setup_cluster_step(mnmt_session *s) {
     if (s->k != 1 || R > DC_RMAX || c.n_dec > DC_LMAX || nc == 0 || d > 512 || F > 2048 || d % (16 * nc) ||
         F % (16 * nc) || (3 * d) % (16 * nc))
         return MNMT_OK;
-    DcParams P;
+    DcParams &P = s->dc_host;
     std::memset(&P, 0, sizeof(P));
     P.R = R; P.d = d; P.H = H; P.dh = dh; P.F = F; P.E = c.d_embed; P.V = c.vocab; P.T = s->Tcap; P.S = s->S;
     P.n_dec = c.n_dec; P.pre_ln = c.pre_ln; P.factorised = m->factorised; P.nc = nc;
@@ -1262,8 +1264,7 @@ int setup_cluster_step(mnmt_session *s) {
     P.S = s->S;
     const int flags = dc_flags(c, m, R, P.att_lw);
     if (!decode_cluster_fits(dh, nc, smem, m->wq != 8, R == 1, flags)) return MNMT_OK;
-    CK(cudaMemcpyAsync(s->d_dc, &P, sizeof(P), cudaMemcpyHostToDevice, m->stream));
-    CK(cudaStreamSynchronize(m->stream));  // P lives on this stack frame
+    CK(cudaMemcpyAsync(s->d_dc, &P, sizeof(P), cudaMemcpyHostToDevice, m->stream));  // as in setup_rows_step
     s->use_cluster = true;
     s->dc_nc = nc;
     s->dc_smem = smem;
@@ -1287,7 +1288,7 @@ int setup_rows_step(mnmt_session *s) {
     if (!s->rows_ok || s->use_cluster || (env && env[0] == '0')) return MNMT_OK;
     const int R = s->B * s->k;
     static_assert(sizeof(DrParams) % 16 == 0, "the parameter block is copied in 16-byte chunks");
-    DrParams P;
+    DrParams &P = s->dr_host;
     std::memset(&P, 0, sizeof(P));
     P.R = R; P.d = c.d_model; P.H = c.n_heads; P.F = c.d_ffn; P.E = c.d_embed; P.V = c.vocab; P.T = s->Tcap;
     P.n_dec = c.n_dec; P.beam = s->k;
@@ -1346,8 +1347,9 @@ int setup_rows_step(mnmt_session *s) {
         s->dr_packed = s->dr_hpc;
     }
     P.S = s->S;
+    // pageable, so staged by the time the call returns; no synchronisation: the
+    // steps are captured while the encoder runs (100 us of a new session's first step)
     CK(cudaMemcpyAsync(s->d_dr, &P, sizeof(P), cudaMemcpyHostToDevice, m->stream));
-    CK(cudaStreamSynchronize(m->stream));  // P lives on this stack frame
     return MNMT_OK;
 }
 
