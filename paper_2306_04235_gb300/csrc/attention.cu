@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(32 * ENC_WARPS) attn_encoder(AttnEncArgs a, in
             }
         }
         const size_t o = ((size_t)b * S + qi) * a.d + h * DH + lane * EPL;
-        const float iz = __frcp_rn(ll2float(Z));
+        const float iz = softmax_inv(ll2float(Z));
 #pragma unroll
         for (int u = 0; u < EPL; u++) {
             const int8_t v = q8_context_hl(hi[u], lo[u], iz, a.rho, [&]() {
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(ENC_TC_THREADS) attn_encoder_tc(AttnEncArgs a,
     }
     // N = a0 + 2^8 a1 + 2^16 a2: fl(2^8 a1 + a0) is off by at most 2^8 + 1, which
     // makes at most rho 2^-15 of t (Z >= 2^24)
-    const float iz0 = __frcp_rn(ll2float(Z0)), iz1 = __frcp_rn(ll2float(Z1));
+    const float iz0 = softmax_inv(ll2float(Z0)), iz1 = softmax_inv(ll2float(Z1));
     const float slack = __fmul_rn(fabsf(a.rho), 0x1p-15f);
     uint8_t *Os = Qs + warp * 16 * RB;  // this warp's own query rows: the output as fp16
     __syncwarp();

@@ -96,7 +96,7 @@ __device__ __forceinline__ void attn_rows(const int8_t *q, int q_ld, int nb, int
             z += (uint32_t)E;
         }
         Z[b] = warp_sum_exact((long long)z);
-        iz[b] = __frcp_rn(ll2float(Z[b]));
+        iz[b] = softmax_inv(ll2float(Z[b]));
     }
     __syncwarp();
 

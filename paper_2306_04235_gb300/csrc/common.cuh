@@ -106,10 +106,10 @@ MNMT_DEV int exp_bound(float v) {
 // ---------------------------------------------------------------------------
 // e^x for x <= 0: Cody-Waite reduction with ln2 split into a 16-bit head and
 // a tail, degree-7 Taylor polynomial of e^r by Horner in fused multiply-adds,
-// scaled by 2^n through the exponent field; 0 below -87.
+// scaled by 2^n through the exponent field; 0 below -87 and for a NaN.
 // ---------------------------------------------------------------------------
 MNMT_DEV float exp_own(float x) {
-    if (x < -87.0f) return 0.0f;
+    if (!(x >= -87.0f)) return 0.0f;
     // n = rne(x log2(e)) in [-126, 0] by adding 1.5 2^23 (ulp 1 there: the sum
     // rounds the fraction half to even and its low bits hold n)
     const float t = __fadd_rn(__fmul_rn(x, 0x1.715476p+0f), 12582912.0f);
@@ -392,8 +392,13 @@ MNMT_DEV float rn32_div(long long n, long long z) {
     return n < 0 ? -q : q;
 }
 
+// fl(1 / fl(Z)) for q8_context.  Z >= 2^24 (the largest score's weight), or 0
+// where no score is a number or the largest is infinite: every weight is then 0
+// (a NaN difference has weight 0), N = 0, and the context is the code of 0.
+MNMT_DEV float softmax_inv(float z) { return __frcp_rn(fmaxf(z, 1.0f)); }
+
 // q8(nearest float to N / Z, rho), the quantised attention context of Eq. 2,
-// from an approximation fN of N and invZ = fl(1 / fl(Z)), Z >= 2^24: t = fl(fl(fN invZ) rho) is off the exact chain by
+// from an approximation fN of N and invZ = softmax_inv(fl(Z)): t = fl(fl(fN invZ) rho) is off the exact chain by
 // at most eight relative roundings of 2^-24 (two in fN, fl(Z), fl(1/Z), two
 // products; the quotient and the product of the exact chain; < 2^-20) plus
 // `slack`, what fN's absolute error makes of t.  Where t lies further from a

@@ -441,7 +441,7 @@ __device__ __forceinline__ void dc_attention(const DcParams &P, int l, int cross
             // context, the KPI lanes of a group sharing its 4 elements
             if (live) {
                 constexpr int UPL = 4 / KPI;
-                const float iz = __frcp_rn(ll2float(z));
+                const float iz = softmax_inv(ll2float(z));
 #pragma unroll
                 for (int u = 0; u < 4; u++)
                     if (u / UPL == kg)
@@ -466,7 +466,7 @@ __device__ __forceinline__ void dc_attention(const DcParams &P, int l, int cross
                     Z += pz[ii * wpi + w];
                 }
                 const int m2 = dc_row_of<RM>(it2, H, R), h2 = it2 - m2 * H;
-                const float c = q8_context(ll2float(N), __frcp_rn(ll2float(Z)), rho, 0.0f, [&]() { return dc_q8_exact(N, Z, rho); });
+                const float c = q8_context(ll2float(N), softmax_inv(ll2float(Z)), rho, 0.0f, [&]() { return dc_q8_exact(N, Z, rho); });
                 ctx[(size_t)m2 * P.d + h2 * DH + e] = (int8_t)(__float_as_uint(__fadd_rn(c, 12582912.0f)) & 0xFFu);
             }
         }

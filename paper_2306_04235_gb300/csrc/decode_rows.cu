@@ -467,7 +467,7 @@ __device__ __noinline__ void dr_attention(const DrParams &P, const int8_t *q, in
     };
     float z0, z1, z2;
     pieces(acc[8], z0, z1, z2);
-    const float iz = __frcp_rn(__fmaf_rn(z2, 65536.0f, __fmaf_rn(z1, 256.0f, z0)));  // two roundings, Z >= 2^24
+    const float iz = softmax_inv(__fmaf_rn(z2, 65536.0f, __fmaf_rn(z1, 256.0f, z0)));  // two roundings, Z >= 2^24
     const float slack = __fmul_rn(fabsf(rho), 0x1p-15f);
     uint32_t words[2] = {0u, 0u};
 #pragma unroll

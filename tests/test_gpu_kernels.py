@@ -295,3 +295,18 @@ def test_attention_core_edges(R, H, dh, T, flat):
             mnmt.mnmt_attention_decode(dev(q), dev(Kc), dev(Vc), dev(n_keys), R, H, dh, T, sigma, np.float32(0.97), ctx[off:])
             got = host(ctx[off: off + R * H * dh]).reshape(R, H, dh)
             assert np.array_equal(got, O.attention_decode(q, Kc, Vc, n_keys, sigma, np.float32(0.97)))
+
+
+@pytest.mark.parametrize("R,H,dh,T", [(3, 2, 32, 1), (5, 2, 64, 17), (700, 2, 64, 33), (2, 3, 128, 160), (3, 2, 32, 600), (2, 1, 64, 1024)])
+@pytest.mark.parametrize("sigma", [np.inf, -np.inf, np.nan, 3e38])
+@pytest.mark.parametrize("rho", [1.25, -1.0, 1e30])
+def test_attention_of_infinite_scores(R, H, dh, T, sigma, rho):
+    """Scores that overflow fp32 or are not numbers: their differences from the
+    maximum are NaN, whose weight is 0, so no key has a weight and the context
+    is the code of 0 (in every form of the incremental kernel)."""
+    q = synth.uniform_int8(1, "q", (R, H, dh), 60, 127)
+    Kc, Vc = synth.uniform_int8(2, "k", (R, H, T, dh), 60, 127), synth.uniform_int8(3, "v", (R, H, T, dh))
+    n_keys = np.array([max(1, T - 3 * (i % 7)) for i in range(R)], np.int32)
+    ctx = torch.full((R, H, dh), 55, dtype=torch.int8, device="cuda")
+    mnmt.mnmt_attention_decode(dev(q), dev(Kc), dev(Vc), dev(n_keys), R, H, dh, T, sigma, rho, ctx)
+    assert not host(ctx).any()

@@ -537,3 +537,38 @@ def test_beam_rows_two_to_an_sm(V, beam, B, flat, stream):
     o_ids, o_len, o_sc = O.translate(blob, ids, lens, beam, T, n_threads=4)
     assert np.array_equal(g_ids, o_ids) and np.array_equal(g_len, o_len)
     assert np.array_equal(g_sc.view(np.uint32), o_sc.view(np.uint32))
+
+
+@pytest.mark.parametrize("B,beam,S,cluster", [(2, 1, 9, "1"), (1, 1, 9, "1"), (6, 2, 9, "1"), (3, 4, 9, "0"), (100, 1, 9, "1"), (12, 1, 33, "0")])
+def test_infinite_attention_scale(B, beam, S, cluster, stream, monkeypatch):
+    """Query and key scales whose product overflows: the codes are all zero, the
+    scores 0 * inf, no key has a weight, and every context is the code of 0 -- as
+    with large finite scales and zero value codes.  Both encoder attentions, the
+    single-cluster, the batched and the kernel-per-operation step."""
+    cfg = synth.ModelConfig(1, 2, 128, 2, 256, 300, 128, 1, 1, max_pos=64)
+    blob = synth.build_blob(cfg, 23, gamma_range=(0.5, 1.5), cross_gains=synth.NO_GAINS)
+    lin = np.float32(synth.activation_scales(cfg)["lin"])
+
+    def scaled(s_qk, s_v):  # every attention block's {s_in, s_q, s_k, s_v, s_ctx, gamma, 0, 0}
+        f = np.frombuffer(blob, np.float32).copy()
+        at = [i for i in np.nonzero(f[:-8] == lin)[0] if (f[i: i + 4] == lin).all() and not f[i + 5: i + 7].any()]
+        assert len(at) == cfg.n_enc + 2 * cfg.n_dec
+        for i in at:
+            f[i: i + 2], f[i + 2] = s_qk, s_v
+        return f.tobytes()
+
+    blobs = {"finite": scaled(1e15, 1e15), "infinite": scaled(1e30, lin)}
+    monkeypatch.setenv("MNMT_DECODE_CLUSTER", cluster)
+    ids, lens = synth.source_batch(cfg.vocab, B, max(1, S // 2), S, 8)
+    ids = np.pad(ids, ((0, 0), (0, S - ids.shape[1])))
+    T, out = 6, {}
+    for name, b in blobs.items():
+        tr = mnmt.Translator(b, B, S, beam, T, stream)
+        try:
+            out[name] = list(tr.translate(ids, lens, T)) + [mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_ENC_OUT), mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_DEC_OUT)]
+        finally:
+            tr.close()
+    o_ids, o_len, o_sc = O.translate(blobs["finite"], ids, lens, beam, T)
+    assert np.array_equal(out["finite"][0], o_ids) and np.array_equal(out["finite"][2].view(np.uint32), o_sc.view(np.uint32))
+    for a, b in zip(out["finite"], out["infinite"]):
+        assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
