@@ -1456,8 +1456,12 @@ int sync_state(mnmt_session *s) {
 
 }  // namespace
 
-extern "C" int mnmt_encode(mnmt_session *s, const int32_t *src_ids, const int32_t *src_lens, int32_t B,
-                           int32_t S_pad, int32_t flags) {
+// mnmt_encode for a search of at most max_len steps.  The limit travels in the
+// arguments of the kernel that resets the search: a host buffer copied
+// asynchronously could be rewritten by the next call on the session before the
+// stream reaches the copy (translations with device pointers queue up).
+static int encode_batch(mnmt_session *s, const int32_t *src_ids, const int32_t *src_lens, int32_t B, int32_t S_pad,
+                        int32_t max_len, int32_t flags) {
     if (!s) return fail(MNMT_EINVAL, "session is null");
     if (s->poisoned) return fail(s->poisoned, "session poisoned by an earlier failure");
     if (!src_ids || !src_lens || B < 1 || B > s->Bmax || S_pad < 1 || S_pad > s->Smax)
@@ -1490,17 +1494,22 @@ extern "C" int mnmt_encode(mnmt_session *s, const int32_t *src_ids, const int32_
     ia.t_ptr = s->state + ST_T;
     ia.done = s->state + ST_DONE;
     ia.ticket = s->state + ST_TICKET;
+    ia.tmax_ptr = s->state + ST_TMAX;
+    ia.tmax = max_len;
     ia.R = B * s->k;
     ia.k = s->k;
     ia.T = s->Tcap;
     ia.bos = m->c.bos_id;
     ia.pad = m->c.pad_id;
     CK(launch_search_init(ia, st));
-    s->max_len = s->Tcap;
-    s->h_state[ST_TMAX] = s->Tcap;
-    CK(cudaMemcpyAsync(s->state + ST_TMAX, s->h_state + ST_TMAX, 4, cudaMemcpyHostToDevice, st));
+    s->max_len = max_len;
     s->steps = 0;
     return MNMT_OK;
+}
+
+extern "C" int mnmt_encode(mnmt_session *s, const int32_t *src_ids, const int32_t *src_lens, int32_t B,
+                           int32_t S_pad, int32_t flags) {
+    return encode_batch(s, src_ids, src_lens, B, S_pad, s ? s->Tcap : 0, flags);
 }
 
 extern "C" int mnmt_decode_steps(mnmt_session *s, int32_t n) {
@@ -1546,12 +1555,9 @@ extern "C" int mnmt_translate(mnmt_session *s, const int32_t *src_ids, const int
     if (!s) return fail(MNMT_EINVAL, "session is null");
     if (max_len < 1 || max_len > s->Tcap) return fail(MNMT_EINVAL, "max_len %d outside [1, %d]", max_len, s->Tcap);
     if (!out_ids || !out_lens || !out_scores) return fail(MNMT_EINVAL, "null output");
-    int rc = mnmt_encode(s, src_ids, src_lens, B, S_pad, flags);
+    int rc = encode_batch(s, src_ids, src_lens, B, S_pad, max_len, flags);
     if (rc) return rc;
     cudaStream_t st = s->m->stream;
-    s->max_len = max_len;
-    s->h_state[ST_TMAX] = max_len;
-    CK(cudaMemcpyAsync(s->state + ST_TMAX, s->h_state + ST_TMAX, 4, cudaMemcpyHostToDevice, st));
     if ((rc = ensure_graph(s))) return poison(s, rc);
     // Chunks of GRAPH_STEPS steps with one chunk of look-ahead: a copy of the
     // state after the chunks queued so far is taken, the next chunk is queued,

@@ -207,8 +207,8 @@ struct InitArgs {
     int32_t *tok, *fin, *anc, *hist, *parents;
     float *cum;
     unsigned long long *keys;
-    int *t_ptr, *done, *ticket;
-    int R, k, T, bos, pad;
+    int *t_ptr, *done, *ticket, *tmax_ptr;
+    int R, k, T, bos, pad, tmax;  // tmax: steps of this translation
 };
 cudaError_t launch_search_init(const InitArgs &a, cudaStream_t st);
 

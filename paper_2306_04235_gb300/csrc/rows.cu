@@ -369,6 +369,7 @@ __global__ void search_init_kernel(InitArgs a) {
     }
     if (i == 0) {
         *a.t_ptr = 0;
+        *a.tmax_ptr = a.tmax;
         *a.done = 0;
         a.ticket[0] = 0;
         a.ticket[1] = 0;

@@ -572,3 +572,30 @@ def test_infinite_attention_scale(B, beam, S, cluster, stream, monkeypatch):
     assert np.array_equal(out["finite"][0], o_ids) and np.array_equal(out["finite"][2].view(np.uint32), o_sc.view(np.uint32))
     for a, b in zip(out["finite"], out["infinite"]):
         assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
+
+
+@pytest.mark.parametrize("beam,B", [(1, 3), (1, 9), (3, 4)])
+def test_queued_translations_keep_their_step_limits(beam, B, stream):
+    """Two device-pointer translations queued on one session while the stream is
+    busy: each runs to its own max_len (the second call's must not reach the
+    first), as when they run one after the other."""
+    cfg = MINI["fact"]
+    tr = mnmt.Translator(synth.build_blob(cfg, 41, gamma_range=(0.5, 1.5)), B, 12, beam, 8, stream)
+    try:
+        ids, lens = synth.source_batch(cfg.vocab, B, 3, 12, 42)
+        ids = np.pad(ids, ((0, 0), (0, 12 - ids.shape[1])))
+        refs = [tr.translate(ids, lens, T) for T in (8, 3)]
+        d_ids, d_lens = torch.from_numpy(ids).cuda(), torch.from_numpy(lens).cuda()
+        outs = [(torch.zeros((B, T), dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda"),
+                 torch.zeros(B, device="cuda")) for T in (8, 3)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(100_000_000)
+        for T, o in zip((8, 3), outs):
+            mnmt.mnmt_translate(tr.session, d_ids, d_lens, B, 12, T, mnmt.DEVICE_PTRS, *o)
+        torch.cuda.synchronize()
+        for ref, out in zip(refs, outs):
+            for a, b in zip(ref, out):
+                assert np.array_equal(a.view(np.uint32), b.cpu().numpy().view(np.uint32))
+    finally:
+        tr.close()
