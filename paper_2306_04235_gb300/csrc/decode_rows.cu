@@ -125,9 +125,14 @@ MNMT_DEV void dr_prefetch(const void *p, int bytes) {
 }
 // barrier over the compute warps
 MNMT_DEV void dr_sync() { asm volatile("bar.sync 1, %0;" ::"n"(DR_WARPS * 32) : "memory"); }
+// barrier over all warps
+MNMT_DEV void dr_sync_all() { asm volatile("bar.sync 0, %0;" ::"n"(DR_THREADS) : "memory"); }
 
 // state of a CTA's pipeline that every wait shares: once a wait has given up,
 // the later ones return at once (the step's results are void: status is set)
+// and the CTA leaves by dr_leave's longer way.  A thread whose wait for an
+// exchange has given up sends nothing more and arms no exchange barrier (it has
+// not seen the phase end); the peers that miss its bytes give up too.
 struct DrWait {
     int *status;
     volatile uint32_t *abort_flag;
@@ -151,11 +156,29 @@ struct DrPipe {
     int slots;
     DrWait wait;
 };
+// the CTA's abort flag, behind the barriers
+MNMT_DEV volatile uint32_t *dr_abort(const DrParams &P) {
+    return reinterpret_cast<volatile uint32_t *>(const_cast<uint8_t *>(reinterpret_cast<const uint8_t *>(&P)) + P.off_bar +
+                                                 8 * (2 * DR_MAX_SLOTS + 2));
+}
 MNMT_DEV DrPipe dr_pipe(const DrParams &P) {
     const uint8_t *sm = reinterpret_cast<const uint8_t *>(&P);
     const uint32_t bars = dr_smem(sm + P.off_bar);
-    return DrPipe{sm + P.off_ring, bars, bars + 8u * DR_MAX_SLOTS, bars + 16u * DR_MAX_SLOTS, P.slots,
-                  DrWait{P.status, reinterpret_cast<volatile uint32_t *>(const_cast<uint8_t *>(sm) + P.off_bar + 8 * (2 * DR_MAX_SLOTS + 2))}};
+    return DrPipe{sm + P.off_ring, bars, bars + 8u * DR_MAX_SLOTS, bars + 16u * DR_MAX_SLOTS, P.slots, DrWait{P.status, dr_abort(P)}};
+}
+
+// The way out of a CTA whose wait has timed out (every thread).  Other CTAs of
+// the cluster may still send to it: it stays until all of them have ended or
+// come here too (the cluster barrier counts ended threads as arrived, and every
+// wait on the way is bounded), and then for as long again as a store needs to
+// land many times over.  A CTA without a timed-out wait just ends: every byte
+// that the others send it in a step has arrived by its last exchange.
+constexpr unsigned long long DR_LAND_NS = 100000;
+__device__ __noinline__ void dr_leave() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;\n" ::: "memory");
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < DR_LAND_NS) {
+    }
 }
 
 // this warp's tiles of one linear over k-blocks [0, nkb): acc[i][nt] = W tile x
@@ -318,7 +341,7 @@ __device__ __noinline__ long long dr_fx_scale(float v, int shift) { return fx_sc
 // loops over (32 keys, set of rows that reads them).  A row's position j lives at
 // kc / vc + (base[b] + prow[b][j]) rs + 64 j; `same` has a bit per 16 keys at
 // which the rows read the same keys and values.  Z comes out of the products
-// too, as one more column tile of ones.  The codes go to every CTA (send).
+// too, as one more column tile of ones.  The codes go to the first nc CTAs.
 // Bound by the latency of each step's loads and chains (two warps a scheduler):
 // with a lane per key and a row after the other, 102 to 124 keys of 4 rows took
 // 8.5 thousand cycles of scores, 4 to 6.5 of softmax and 11 to 14 of values, in
@@ -493,7 +516,8 @@ __device__ __noinline__ void dr_attention(const DrParams &P, const int8_t *q, in
 // once that has arrived (bar, par; then re-armed for `arm` bytes).  Partial
 // extremes and sums meet in `part_s` behind the row's named barrier; the centred
 // row's largest magnitude follows from the extremes (subtraction is monotone).
-// Leaves the codes of the row in `codes`, behind a last barrier.
+// Leaves the codes of the row in `codes`, behind a last barrier.  False if the
+// wait has given up.
 struct DrLnRow {
     float *r;
     const float *y;
@@ -503,7 +527,7 @@ struct DrLnRow {
     bool live;
 };
 template <int EPL>
-__device__ __noinline__ void dr_layernorm(const DrParams &P, const DrLnRow w, const float *gp, const float *bp, float inv,
+__device__ __noinline__ bool dr_layernorm(const DrParams &P, const DrLnRow w, const float *gp, const float *bp, float inv,
                                           float gamma, const DrWait wait, uint32_t bar, uint32_t par, uint32_t arm) {
     const int lane = threadIdx.x & 31, e0 = w.part * (P.d / w.wpr) + lane;
     auto sync = [&]() {
@@ -517,11 +541,12 @@ __device__ __noinline__ void dr_layernorm(const DrParams &P, const DrLnRow w, co
         bv[i] = __ldg(bp + e0 + 32 * i);
         v[i] = w.live ? w.r[e0 + 32 * i] : 0.0f;
     }
+    bool ok = true;
     if (bar) {
-        wait(bar, par);
-        if (threadIdx.x == 0 && arm) mbar_expect_tx(bar, arm);
+        ok = wait(bar, par);
+        if (threadIdx.x == 0 && arm && ok) mbar_expect_tx(bar, arm);
     }
-    if (!w.live) return;
+    if (!w.live) return ok;
     unsigned am = 0, hi = 0, lo = 0xFFFFFFFFu;
 #pragma unroll
     for (int i = 0; i < EPL; i++) {
@@ -597,6 +622,7 @@ __device__ __noinline__ void dr_layernorm(const DrParams &P, const DrLnRow w, co
     for (int i = 0; i < EPL; i++)
         w.codes[e0 + 32 * i] = (int8_t)q8_bits(__fadd_rn(__fmul_rn(__fmul_rn(v[i], rstd), gv[i]), bv[i]), inv);
     sync();
+    return ok;
 }
 
 // One warp: the caches that layer l's attention of these rows and heads reads,
@@ -640,7 +666,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
     const int slots = P.slots;
     const uint32_t bars = dr_smem(smem + P.off_bar), full = bars, empty = bars + 8u * DR_MAX_SLOTS,
                    xbars = empty + 8u * DR_MAX_SLOTS;
-    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + P.off_bar + 8 * (2 * DR_MAX_SLOTS + 2));
+    volatile uint32_t *abort_flag = dr_abort(P);
     const int nx = 9 * P.n_dec;
     auto xbytes = [&](int x) -> uint32_t {
         const int k = dr_exchange_kind(x);
@@ -672,7 +698,8 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
         uint32_t s = 0, par = 1, i = 0;
         auto feed = [&](uint32_t end) {  // one thread: slots up to `end`; false after a timed-out wait
             for (; i < end; i++) {
-                if (i >= (uint32_t)slots && !wait(empty + 8u * s, par)) return false;
+                // (the flag after the wait: warps that have given up pass slots unread)
+                if (i >= (uint32_t)slots && (!wait(empty + 8u * s, par) || *abort_flag)) return false;
                 mbar_expect_tx(full + 8u * s, DR_SLOT);
                 bulk_load(dr_smem(ring + s * DR_SLOT), src + (size_t)i * DR_SLOT, DR_SLOT, full + 8u * s);
                 if (++s == (uint32_t)slots) {
@@ -692,11 +719,16 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                 ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
             }
         }
-        // after a timed-out wait: the copies in flight land (bounded) before the CTA ends
-        if (lane == 0 && *abort_flag)
-            for (uint32_t k = i > (uint32_t)slots ? i - slots : 0; k < i; k++) mbar_wait(full + 8u * (k % slots), (k / slots) & 1);
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
+        dr_sync_all();  // the compute warps are through
+        if (*abort_flag) {
+            // the copies in flight land (bounded) before the CTA ends
+            if (lane == 0)
+                for (uint32_t k = i > (uint32_t)slots ? i - slots : 0; k < i; k++) mbar_wait(full + 8u * (k % slots), (k / slots) & 1);
+            __syncwarp();
+            dr_leave();
+        }
         return;
     }
 
@@ -784,12 +816,14 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
     asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory");
 
     int x = 0;        // exchanges so far
+    int live = nc;    // CTAs that this thread sends to: all, or none after a timed-out wait
     uint32_t it = 0;  // ring slots so far
     // wait for exchange x's bytes; arm its barrier for exchange x + 2
     auto receive = [&]() {
         const uint32_t bar = xbars + 8u * (uint32_t)(x & 1);
-        wait(bar, (uint32_t)(x >> 1) & 1u);
-        if (threadIdx.x == 0 && x + 2 < nx) mbar_expect_tx(bar, xbytes(x + 2));
+        const bool ok = live && wait(bar, (uint32_t)(x >> 1) & 1u);
+        if (!ok) live = 0;
+        if (threadIdx.x == 0 && x + 2 < nx && ok) mbar_expect_tx(bar, xbytes(x + 2));
         x++;
     };
     // LayerNorm of the owned rows, 2^ln_w warps per row; add: after the linear
@@ -799,7 +833,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
         const int lw = P.ln_w, wpr = 1 << lw, slot = warp >> lw, part = warp & (wpr - 1), gt = threadIdx.x & (wpr * 32 - 1);
         uint32_t bar = 0, par = 0, arm = 0;
         if (add) {
-            bar = xbars + 8u * (uint32_t)(x & 1);
+            bar = live ? xbars + 8u * (uint32_t)(x & 1) : 0u;
             par = (uint32_t)(x >> 1) & 1u;
             arm = x + 2 < nx ? xbytes(x + 2) : 0u;
             x++;
@@ -809,15 +843,17 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
             uint8_t *ls = lns + slot * (256 + d);
             const DrLnRow w{rbuf + (size_t)rr * d, add ? ybuf + (size_t)rr * d : nullptr, reinterpret_cast<uint32_t *>(ls),
                             reinterpret_cast<int8_t *>(ls + 256), part, wpr, slot, rr < nown};
+            bool ok;
             switch (P.ln_epl) {
-                case 2: dr_layernorm<2>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
-                case 3: dr_layernorm<3>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
-                case 4: dr_layernorm<4>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
-                case 6: dr_layernorm<6>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
-                case 8: dr_layernorm<8>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
-                case 12: dr_layernorm<12>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
-                default: dr_layernorm<16>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
+                case 2: ok = dr_layernorm<2>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
+                case 3: ok = dr_layernorm<3>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
+                case 4: ok = dr_layernorm<4>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
+                case 6: ok = dr_layernorm<6>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
+                case 8: ok = dr_layernorm<8>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
+                case 12: ok = dr_layernorm<12>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
+                default: ok = dr_layernorm<16>(P, w, gp, bp, inv, gamma, wait, bar, par, arm); break;
             }
+            if (!ok) live = 0;
             bar = 0;
             if (rr >= nown) break;
             const int row = own0 + rr, rg = r0 + row, chunks = d >> 4;
@@ -846,7 +882,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                 if (q0 < per) {
                     const uint4 v = *reinterpret_cast<const uint4 *>(ls + 256 + 16 * ch);
                     const uint32_t local = dr_smem(actA + (size_t)row * sa + 16 * ch);
-                    for (int q = q0; q < nc; q += per) dr_send4(dr_mapa(local, q), v, dr_mapa(xbar, q));
+                    for (int q = q0; q < live; q += per) dr_send4(dr_mapa(local, q), v, dr_mapa(xbar, q));
                 }
             }
             if (rr + (DR_WARPS >> lw) < nown) {  // the slot's partials and codes are free again
@@ -860,7 +896,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
         dr_sync();
         const uint32_t xbar = xbars + 8u * (uint32_t)(x & 1);
         const float *sy = reinterpret_cast<const float *>(stage);
-        for (int i = threadIdx.x; i < RB * HC / 4; i += DR_WARPS * 32) {
+        for (int i = threadIdx.x; i < RB * HC / 4 && live; i += DR_WARPS * 32) {
             const int row = i / (HC / 4), ch = i % (HC / 4), o = meta[2 * RB + row];
             const uint4 v = *reinterpret_cast<const uint4 *>(sy + row * (HC + 4) + 4 * ch);
             const uint32_t local = dr_smem(ybuf + (size_t)(row - o * RB / nc) * d + HC * c + 4 * ch);
@@ -907,7 +943,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                 auto run = [&](auto rows_c) {
                     dr_attention<decltype(rows_c)::value>(P, qbuf + (c0 + b0) * HC + hl * 64, HC, b1 - b0, n,
                                                           cross ? Y.sigma2 : Y.sigma1, cross ? Y.rho2 : Y.rho1, scw, kc, vc, rs,
-                                                          base, pr, same, out + (uint32_t)(b0 * sa), sa, xbar, nc);
+                                                          base, pr, same, out + (uint32_t)(b0 * sa), sa, xbar, live);
                 };
                 if (AR > 1 && b1 - b0 == 1) run(std::integral_constant<int, 1>{});
                 else run(std::integral_constant<int, AR>{});
@@ -916,7 +952,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
             // rows past the batch send zeros: every exchange has its full size
             for (int i = lane; i < (AR - wnb) * 8; i += 32) {
                 const uint32_t local = out + (uint32_t)((wnb + (i >> 3)) * sa + 8 * (i & 7));
-                for (int k = 0; k < nc; k++) dr_send2(dr_mapa(local, k), 0u, 0u, dr_mapa(xbar, k));
+                for (int k = 0; k < live; k++) dr_send2(dr_mapa(local, k), 0u, 0u, dr_mapa(xbar, k));
             }
         }
     };
@@ -971,7 +1007,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                 const int row = k / cpr, ch = k - row * cpr;
                 const uint4 v = *reinterpret_cast<const uint4 *>(stage + row * fst + 16 * ch);
                 const uint32_t local = dr_smem(actH + (size_t)row * sh + c * fc + 16 * ch);
-                for (int q = 0; q < nc; q++) {
+                for (int q = 0; q < live; q++) {
                     const int dst = c + q < nc ? c + q : c + q - nc;
                     dr_send4(dr_mapa(local, dst), v, dr_mapa(xbar, dst));
                 }
@@ -990,8 +1026,11 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
                 last ? P.inv_dout : sub == 0 ? Z.inv_in2 : sub == 1 ? Z.inv_in3 : Z.inv_in1, true, Lout.gam, last);
         if (!last) receive();
     }
-    // everything sent to this CTA has arrived (its last exchange was received)
-    // and every weight copy was consumed; its own stores carry their data
+    // unless a wait timed out: everything sent to this CTA has arrived (its last
+    // exchange was received) and every weight copy was consumed; its own stores
+    // carry their data
+    dr_sync_all();
+    if (*abort_flag) dr_leave();
 }
 
 const void *dr_kernel(int nb, int hpc) {
