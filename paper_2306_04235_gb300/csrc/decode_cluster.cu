@@ -144,6 +144,15 @@ MNMT_DEV int dc_row_of(int i, int d, int R) {  // i / d for i < R d, R <= RM
     return r;
 }
 
+// What a CTA remembers behind the barriers of its weight ring: has a wait given
+// up, and how many phases' slices were issued.
+struct DcFate {
+    uint32_t abort, fed;
+};
+MNMT_DEV volatile DcFate *dc_fate(const DcParams &P) {
+    return reinterpret_cast<volatile DcFate *>(const_cast<uint8_t *>(reinterpret_cast<const uint8_t *>(&P)) + P.off_bar + 8 * DC_NB);
+}
+
 // ring slot layout: W rows (rows * K bytes), then s[rows], b[rows], inv[rows] (fp32)
 // Phase ph's slice goes to slot ph % DC_NB as up to five 1-D bulk copies (the
 // copy engine moves them: no per-thread copy instructions queue ahead of the
@@ -155,6 +164,7 @@ MNMT_DEV void dc_prefetch(const DcParams &P, int ph, int c, uint8_t *ring, uint3
     if ((int)threadIdx.x != who || ph >= 1 + 6 * P.n_dec) return;
     const DcPhase &f = P.phase[ph];
     const uint32_t bar = bars + 8u * (uint32_t)(ph % DC_NB);
+    dc_fate(P)->fed = (uint32_t)ph + 1u;
     if (!f.rows) {
         mbar_arrive(bar);
         return;
@@ -173,16 +183,54 @@ MNMT_DEV void dc_prefetch(const DcParams &P, int ph, int c, uint8_t *ring, uint3
     if (f.m) bulk_load(dst + wb + 3 * vb, f.m + c * f.rows, vb, bar);
 }
 
-// wait for phase ph's slice; a wait that gives up records MNMT_ETIMEOUT
+// A wait that gives up records MNMT_ETIMEOUT (the step's results are void) and
+// lets every later wait of the CTA give up at once.  No slice is issued any more
+// (n_dec = -1: dc_prefetch sees no phases left): its slot may still be filling.  All of this
+// is out of line; the step is sensitive to the size of its code.
+__device__ __noinline__ void dc_wait_slow(DcParams &P, uint32_t bar, uint32_t parity) {
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try(bar, parity)) {
+        if (dc_fate(P)->abort || global_ns() - t0 > MNMT_WAIT_NS) {
+            dc_fate(P)->abort = 1;
+            P.n_dec = -1;
+            set_status(P.status, MNMT_ETIMEOUT);
+            return;
+        }
+    }
+}
+MNMT_DEV void dc_wait(const DcParams &P, uint32_t bar, uint32_t parity) {
+    if (!mbar_test(bar, parity)) dc_wait_slow(const_cast<DcParams &>(P), bar, parity);
+}
+// wait for phase ph's slice
 MNMT_DEV void dc_wait_slice(const DcParams &P, int ph, uint32_t bars) {
-    if (!mbar_wait(bars + 8u * (uint32_t)(ph % DC_NB), (uint32_t)(ph / DC_NB) & 1u)) set_status(P.status, MNMT_ETIMEOUT);
+    dc_wait(P, bars + 8u * (uint32_t)(ph % DC_NB), (uint32_t)(ph / DC_NB) & 1u);
+}
+
+// The way out of a CTA whose wait has given up (every thread).  Its own copies
+// land (bounded); then, as other CTAs of the cluster may still send to it, it
+// stays until all of them have ended or come here too (the cluster barrier
+// counts ended threads as arrived, and every wait on the way is bounded) and
+// for as long again as a store needs to land many times over.  It has sent its
+// part of every phase, so the others are not held up.
+constexpr unsigned long long DC_LAND_NS = 100000;
+__device__ __noinline__ void dc_leave(const DcParams &P, uint32_t bars) {
+    if (threadIdx.x == 0) {
+        const int fed = (int)dc_fate(P)->fed;
+        for (int ph = fed > DC_NB ? fed - DC_NB : 0; ph < fed; ph++)
+            mbar_wait(bars + 8u * (uint32_t)(ph % DC_NB), (uint32_t)(ph / DC_NB) & 1u);
+    }
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;\n" ::: "memory");
+    const unsigned long long t0 = global_ns();
+    while (global_ns() - t0 < DC_LAND_NS) {
+    }
 }
 
 // Exchange between the CTAs of the cluster.  A phase's slice goes to every
 // CTA (itself included) as st.async stores, each completing its bytes on the
-// receiver's exchange mbarrier for that phase (two, used by alternate
-// phases); a CTA waits on its own barrier until the whole vector has arrived
-// instead of a cluster-wide barrier.  No store can overwrite data a receiver
+// receiver's exchange mbarrier of that phase (one per phase, armed once: no
+// barrier is armed again that a late store could still complete); a CTA waits on
+// its own barrier until the whole vector has arrived instead of a cluster-wide
+// barrier.  No store can overwrite data a receiver
 // still reads: a CTA sends phase ph + 1 only after receiving phase ph from
 // every CTA, i.e. after every CTA finished the GEMV of phase ph (and with it
 // every read of the buffers that phase ph + 1 overwrites).
@@ -518,14 +566,18 @@ __global__ void __launch_bounds__(DC_THREADS, 1) decode_cluster_kernel(const DcP
         const int n16 = (int)(sizeof(DcParams) / 16);
         for (int i = threadIdx.x; i < n16; i += DC_THREADS)
             reinterpret_cast<int4 *>(smem)[i] = reinterpret_cast<const int4 *>(Pp)[i];
-        if (threadIdx.x == 0) {
-            // the weight ring's mbarriers and the two exchange barriers, one
-            // arrival per phase each; the exchange barriers of phases 0 and 1
-            // are armed with the bytes they receive
-            const uint32_t b0 = dc_smem_u32(smem + Pp->off_bar);
-            for (int i = 0; i < DC_NB + 2; i++) mbar_init(b0 + 8u * (uint32_t)i, 1u);
+        // the weight ring's mbarriers (one arrival per phase) and a phase's
+        // exchange barrier each, armed with the bytes it receives
+        const uint32_t b0 = dc_smem_u32(smem + Pp->off_bar);
+        const int nbar = DC_NB + 1 + 1 + 6 * Pp->n_dec;  // between them: DcFate
+        for (int i = threadIdx.x; i < nbar; i += DC_THREADS) {
+            if (i == DC_NB) {
+                reinterpret_cast<volatile DcFate *>(smem + Pp->off_bar + 8 * DC_NB)->abort = 0;
+                continue;
+            }
+            mbar_init(b0 + 8u * (uint32_t)i, 1u);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-            for (int i = 0; i < 2; i++) mbar_expect_tx(b0 + 8u * (uint32_t)(DC_NB + i), dc_xbytes(*Pp, i));
+            if (i > DC_NB) mbar_expect_tx(b0 + 8u * (uint32_t)i, dc_xbytes(*Pp, i - DC_NB - 1));
         }
         __syncthreads();
         // the barriers are set before any CTA of the cluster may store into
@@ -539,7 +591,7 @@ __global__ void __launch_bounds__(DC_THREADS, 1) decode_cluster_kernel(const DcP
     const bool pre_ln = FL < 0 ? P.pre_ln != 0 : (FL & 1) != 0;
     const bool factorised = FL < 0 ? P.factorised != 0 : (FL & 2) != 0;
     constexpr int TW = FL < 0 ? -1 : ((FL >> 2) & 1);  // row width above 256 (bit 2); bits 3-4: log2 warps per attention item
-    const uint32_t bars = dc_smem_u32(smem + P.off_bar), xbars = bars + 8u * DC_NB;
+    const uint32_t bars = dc_smem_u32(smem + P.off_bar), xbars = bars + 8u * (DC_NB + 1);
     cg::cluster_group cl = cg::this_cluster();
     const int c = (int)cl.block_rank();
     const int nc = P.nc;
@@ -564,7 +616,7 @@ __global__ void __launch_bounds__(DC_THREADS, 1) decode_cluster_kernel(const DcP
     int *tok_s = reinterpret_cast<int *>(smem + P.off_red + 128 + 8 * DH * 8);  // [R]
     unsigned *mm = reinterpret_cast<unsigned *>(smem + P.off_part);               // [R][nc][2] slice max / min of r
     long long *part_l = reinterpret_cast<long long *>(smem + P.off_part + 512);    // [2][64] LN partials, [R] (mu, eb)
-    const int nphase = 1 + 6 * P.n_dec;
+    const int nphase = 1 + 6 * P.n_dec;  // (read here: a wait that gives up clears P.n_dec)
 
     // the LayerNorm vectors of every layer (+ the final LN), the first DC_NB
     // weight slices and the cross keys / values the step attends to
@@ -835,7 +887,7 @@ __global__ void __launch_bounds__(DC_THREADS, 1) decode_cluster_kernel(const DcP
         // thread issuing bulk copies is held for a few hundred ns)
         dc_prefetch(P, ph + DC_NB, c, ring, bars, DC_THREADS - 32);
         // ---- publish the slice to every CTA ----
-        const uint32_t xbar = xbars + 8u * (uint32_t)(ph & 1);
+        const uint32_t xbar = xbars + 8u * (uint32_t)ph;
         if (out_f32) {
             // the slice's largest and smallest residual value per row (rows <= 32),
             // for the next LayerNorm's grids
@@ -859,12 +911,11 @@ __global__ void __launch_bounds__(DC_THREADS, 1) decode_cluster_kernel(const DcP
             dc_bcast(P.phase[ph], stage, R, rows, reinterpret_cast<uint8_t *>(full), width, n0, nc, xbar);
         }
         // the whole vector of this phase, from every CTA
-        if (!mbar_wait(xbar, (uint32_t)(ph >> 1) & 1u)) set_status(P.status, MNMT_ETIMEOUT);
-        if (threadIdx.x == 0 && ph + 2 < nphase) mbar_expect_tx(xbar, dc_xbytes(P, ph + 2));
+        dc_wait(P, xbar, 0u);
         DC_STAMP(stamp, 7 + 4 * ph);
         if (kind == K_W2 && !pre_ln) {
             // post-LN: the FFN's LayerNorm normalises the stream in place
-            const bool last = l + 1 == P.n_dec;
+            const bool last = ph == nphase - 1;
             const float inv = last ? P.inv_dout : P.layer[l + 1].inv_in1;
             dc_layernorm<RM, TW>(r_full, R, d, lnl + 4 * d, lnl + 5 * d, inv, a_full, 1, P.status, mm, nc, part_l, P.ln_kd, P.ln_dodd, P.ln_zm);
         }
@@ -872,7 +923,7 @@ __global__ void __launch_bounds__(DC_THREADS, 1) decode_cluster_kernel(const DcP
     DC_STAMP(stamp, 100);
     // ---- final LayerNorm + quantisation -> vocabulary input ----
     if (pre_ln)
-        dc_layernorm<RM, TW>(r_full, R, d, lnp + (size_t)6 * P.n_dec * d, lnp + (size_t)(6 * P.n_dec + 1) * d,
+        dc_layernorm<RM, TW>(r_full, R, d, lnp + (size_t)(nphase - 1) * d, lnp + (size_t)nphase * d,
                      P.inv_dout, a_full, 0, P.status, mm, nc, part_l, P.ln_kd, P.ln_dodd, P.ln_zm);
     __syncthreads();
     if (c == 0) {
@@ -883,8 +934,9 @@ __global__ void __launch_bounds__(DC_THREADS, 1) decode_cluster_kernel(const DcP
     }
     DC_STAMP(stamp, 101);
     if (pend && c == 0 && threadIdx.x == 0) dc_commit_greedy(P, t - 1, s_out, s_fin, 0);
-    // no closing cluster barrier: the last exchange has delivered everything
-    // any CTA stores into this one
+    // no closing cluster barrier unless a wait gave up: the last exchange has
+    // delivered everything any CTA stores into this one
+    if (dc_fate(P)->abort) dc_leave(P, bars);
     DC_STAMP(stamp, 102);
 }
 
@@ -1117,7 +1169,7 @@ size_t dc_layout(DcParams &P, size_t max_smem) {
     P.off_red = take(128 + (size_t)DC_WARPS * P.dh * 8 + 16 * 4);  // reductions, context partials, tokens
     P.off_part = take(512 + 1024 + 64);  // slice extremes [R][nc][2], LN partials [2][64], per-row (mu, eb)
     if (R * d > 64 * 32) return (size_t)-1;                         // 64 warp chunks of partials
-    P.off_bar = take(8 * (DC_NB + 2));  // weight ring, then the two exchange barriers
+    P.off_bar = take(8 * (DC_NB + 1 + 1 + 6 * (size_t)P.n_dec));  // weight ring, DcFate, a phase's exchange barrier each
     int slot = 0;
     for (int ph = 0; ph < 1 + 6 * P.n_dec; ph++) {
         const DcPhase &f = P.phase[ph];
