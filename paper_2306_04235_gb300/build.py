@@ -20,7 +20,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libmnmt.so")
 SOURCES = ["api.cu", "linear.cu", "linear_w4.cu", "gemm_tc.cu", "attention.cu", "rows.cu", "decode_cluster.cu",
            "decode_rows.cu",            "noalloc.cu", "fakequant.cu"]
-HEADERS = ["attn_core.cuh", "common.cuh", "decode_rows.h", "epilogue.cuh", "internal.h", "mbarrier.cuh"]
+HEADERS = ["attn_core.cuh", "common.cuh", "decode_rows.h", "epilogue.cuh", "internal.h", "mbarrier.cuh", "routes.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

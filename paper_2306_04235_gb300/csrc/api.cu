@@ -27,6 +27,7 @@
 
 #include "decode_rows.h"
 #include "internal.h"
+#include "routes.h"
 
 using namespace mnmt;
 
@@ -246,6 +247,7 @@ struct Lin {
     int bits;                 // 8 or 4
     const uint8_t *wp;        // 4-bit: packed codes [n][k/2]
     const float *m;           // 4-bit min-max rows: row offsets (null: symmetric)
+    LinRole role;
 };
 struct LnP {
     const float *g, *b;
@@ -390,6 +392,7 @@ extern "C" int mnmt_load_weights_ex(const void *blob, size_t bytes, void *cuda_s
         l.bits = o.bits;
         l.wp = nullptr;
         l.m = nullptr;
+        l.role = LIN_LAYER;
         if (o.bits == 4) {
             l.wp = m->d_blob + o.w;
             l.m = o.minmax ? reinterpret_cast<const float *>(m->d_blob + o.m) : nullptr;
@@ -441,6 +444,7 @@ extern "C" int mnmt_load_weights_ex(const void *blob, size_t bytes, void *cuda_s
         s.rho = s.s_v / s.s_ctx;
         s.qkv = dlin(o.qkv);
         s.o = dlin(o.o);
+        s.o.role = LIN_SQUARE;
         s.inv_qkv = nullptr;
         return s;
     };
@@ -459,6 +463,7 @@ extern "C" int mnmt_load_weights_ex(const void *blob, size_t bytes, void *cuda_s
     }
     for (int l = 0; l < c.n_dec; l++) {
         m->dec_self.push_back(mk_self(L.dec_self[l]));
+        m->dec_self.back().qkv.role = LIN_CACHE;
         const CrossOff &o = L.dec_cross[l];
         CrossBlk x;
         x.ln = dln(o.ln_g, o.ln_b);
@@ -469,6 +474,8 @@ extern "C" int mnmt_load_weights_ex(const void *blob, size_t bytes, void *cuda_s
         x.q = dlin(o.q);
         x.kv = dlin(o.kv);
         x.o = dlin(o.o);
+        x.q.role = x.o.role = LIN_SQUARE;
+        x.kv.role = LIN_CACHE;
         m->dec_cross.push_back(x);
         m->dec_ffn.push_back(mk_ffn(L.dec_ffn[l]));
     }
@@ -490,6 +497,7 @@ extern "C" int mnmt_load_weights_ex(const void *blob, size_t bytes, void *cuda_s
     m->out.b = reinterpret_cast<const float *>(m->d_blob + L.out_b);
     m->out.n = c.vocab;
     m->out.k = d;
+    m->out.role = LIN_OUT;
     // the tensor-core linears read the weight codes as fp16: convert the whole
     // blob once (the fp32 regions become unused garbage); offsets stay 16-byte
     // aligned, so W16 = d_blob16 + (W - d_blob) is 32-byte aligned.  A lean
@@ -776,21 +784,10 @@ const __half *w16_of(const mnmt_model *m, const int8_t *w) {
 
 // does the linear l of M rows run on the tcgen05 kernel (then its input comes
 // from the fp16 mirror its producer wrote), or on the kernels that read int8
-// codes?  The latter start faster (no TMEM, no barriers; mma.sync), the former
-// has the throughput and splits a long K.  Both measured in graphs, us:
-//   0.13 GMAC, K = 256 (512 x 1024): 3.7 / 5.3;  0.4 GMAC, K = 512: 6.9 / 6.3;
-//   0.8 GMAC, K = 512 (1024 x 1536): 9.4 / 8.9;  1.6 GMAC: 18.4 / 11.3
-//   K = 768: equal up to 0.15 GMAC; K = 1024 (512 x 256): 8.6 / 7.1, but the
-//   GEMV's 16-row chunks (narrow layers of up to 64 rows): 3.3 / 6.4
-//   fp32 rows of 32000 logits, K = 256: 32 rows 11.4 / 9.4, 128 rows 12.8 / 15.6,
-//   192 rows 20.6 / 16.1, 512 rows 34.4 / 25.9; K = 512: 128 rows 20.1 / 17.6, 512
-//   rows 60.3 / 30.8; of 8000, K = 256: 256 rows 7.5 / 9.3, 640 rows 15.7 / 14.8
+// codes?
 bool tc_linear(const mnmt_session *s, int M, const Lin &l, bool f32_out = false) {
-    if (!s->use_tc || (size_t)M < TC_MIN_ROWS) return false;
-    if (f32_out && l.k <= 256 && M >= 128) return (double)M * l.n * l.k > 1.2e9;
-    const long tiles64 = (long)((M + 63) / 64) * ((l.n + 63) / 64);
-    if (M <= 64 && l.k <= 1024 && tiles64 < 8) return false;
-    return l.k > 768 || (double)M * l.n * l.k > 3e8;
+    const mnmt_config &c = s->m->c;
+    return s->use_tc && (size_t)M >= TC_MIN_ROWS && route_linear_tc(l.role, M, c.d_model, c.d_ffn, l.n, l.k, f32_out);
 }
 
 // fp16 mirror of one of the session's int8 activation buffers

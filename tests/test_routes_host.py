@@ -1,0 +1,64 @@
+"""The rules that choose a call's kernel by its sizes (csrc/routes.h), against
+measured times of both sides (tests/golden/*_routes.txt): the choice may not be
+slower than the best by more than the times repeat, nor than the code that the
+choice replaced."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2306_04235_gb300", "csrc")
+GOLDEN = os.path.join(ROOT, "tests", "golden")
+
+pytestmark = pytest.mark.skipif(shutil.which("g++") is None, reason="needs a host compiler")
+
+
+def _decide(tmp_path, expr, rows):
+    """The values of the C++ expression `expr` of ints a[] for every row."""
+    src = tmp_path / "r.cpp"
+    src.write_text(f"""#include "routes.h"
+#include <cstdio>
+using namespace mnmt;
+int main() {{
+    int n, a[16];
+    while (scanf("%d", &n) == 1) {{
+        for (int i = 0; i < n; i++) if (scanf("%d", a + i) != 1) return 1;
+        printf("%d\\n", (int)({expr}));
+    }}
+}}
+""")
+    exe = tmp_path / "r"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    text = "\n".join(f"{len(r)} " + " ".join(map(str, r)) for r in rows)
+    out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True).stdout
+    return [int(x) for x in out.split()]
+
+
+def _table(name, kind):
+    for line in open(os.path.join(GOLDEN, name)):
+        f = line.split()
+        if f and f[0] == kind:
+            yield f[1:]
+
+
+@pytest.mark.parametrize("kind", ["enc", "dec"])
+def test_session_linears_take_the_faster_family(kind, tmp_path):
+    rows = [([int(x) for x in f[:3]], float(f[3]), [float(x) for x in f[4:]]) for f in _table("linear_routes.txt", kind)]
+    assert len(rows) > 60
+    roles = "LIN_LAYER, LIN_SQUARE, LIN_CACHE".split(", ")
+    got = [_decide(tmp_path, f"route_linear_tc({r}, a[0], a[1], a[2], a[1], a[1], false)", [x[0] for x in rows]) for r in roles]
+    for (m, start, t), layer, square, cache in zip(rows, *got):
+        column = 0 if not cache and not layer else 1 if not layer else 2 if not square else 3
+        assert cache or not layer
+        best = min(t)
+        assert t[column] <= 1.06 * best, (m, t, column)
+        assert not start or t[column] <= 1.01 * start + 2, (m, start, t, column)
+
+
+def test_vocabulary_projection_takes_the_faster_family(tmp_path):
+    rows = [([int(x) for x in f[:4]], float(f[4]), float(f[5])) for f in _table("linear_routes.txt", "out")]
+    got = _decide(tmp_path, "route_linear_tc(LIN_OUT, a[0], a[2], 4 * a[2], a[1], a[2], a[3])", [x[0] for x in rows])
+    for (m, t8, tc), choice in zip(rows, got):
+        assert (tc if choice else t8) <= 1.06 * min(t8, tc), (m, t8, tc, choice)
