@@ -198,7 +198,11 @@ int mnmt_translate(mnmt_session *s, const int32_t *src_ids, const int32_t *src_l
  *                                                  decoder rows after a step)
  *   MNMT_TAP_HISTORY    int32 [max_len][B*beam]   token chosen per step and hypothesis
  *   MNMT_TAP_PARENTS    int32 [max_len][B*beam]   parent beam per step and hypothesis
- *   MNMT_TAP_ANCESTRY   int32 [B*beam][max_len]   physical cache row holding each position */
+ *   MNMT_TAP_ANCESTRY   int32 [B*beam][max_len]   physical cache row holding each position
+ *   MNMT_TAP_STEP       int32 [4]                 the decode step of the batch encoded last: kind (0 a
+ *                                                  kernel per operation, 1 the single cluster, 2 the
+ *                                                  batched step), then for kind 2 rows per cluster,
+ *                                                  heads per CTA, clusters (else 0) */
 enum {
     MNMT_TAP_ENC_OUT = 1,
     MNMT_TAP_CROSS_K = 2,
@@ -210,7 +214,8 @@ enum {
     MNMT_TAP_RESID = 8,
     MNMT_TAP_HISTORY = 9,
     MNMT_TAP_PARENTS = 10,
-    MNMT_TAP_ANCESTRY = 11
+    MNMT_TAP_ANCESTRY = 11,
+    MNMT_TAP_STEP = 12
 };
 int64_t mnmt_debug_tap(mnmt_session *s, int32_t tap, int32_t layer, void *host_dst, size_t bytes);
 

@@ -1654,6 +1654,16 @@ extern "C" int64_t mnmt_debug_tap(mnmt_session *s, int32_t tap, int32_t layer, v
             src = s->anc;
             n = R * s->Tcap * 4;
             break;
+        case MNMT_TAP_STEP: {  // known to the host
+            if (s->B < 1) return fail(MNMT_EINVAL, "no batch encoded yet");
+            if (int rc = ensure_graph(s)) return rc;
+            const int32_t v[4] = {s->use_cluster ? 1 : s->use_rows ? 2 : 0, s->use_rows ? 8 * s->dr_nb : 0,
+                                  s->use_rows ? s->dr_hpc : 0, s->use_rows ? s->dr_clusters : 0};
+            if (!host_dst) return (int64_t)sizeof(v);
+            if (bytes != sizeof(v)) return fail(MNMT_EINVAL, "tap %d holds %zu bytes, not %zu", tap, sizeof(v), bytes);
+            std::memcpy(host_dst, v, sizeof(v));
+            return MNMT_OK;
+        }
         default:
             return fail(MNMT_EINVAL, "unknown tap %d", tap);
     }

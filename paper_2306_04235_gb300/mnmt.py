@@ -20,7 +20,7 @@ OK, EINVAL, ENOMEM, ECUDA, ETIMEOUT, EFORMAT, EOVERFLOW = 0, -1, -2, -3, -4, -5,
 DEVICE_PTRS = 1
 EPI_Q8, EPI_RELU_Q8, EPI_RESID, EPI_F32, EPI_ARGMAX = 0, 1, 2, 3, 4
 (TAP_ENC_OUT, TAP_CROSS_K, TAP_CROSS_V, TAP_SELF_K, TAP_SELF_V, TAP_DEC_OUT, TAP_LOGITS, TAP_RESID,
- TAP_HISTORY, TAP_PARENTS, TAP_ANCESTRY) = range(1, 12)
+ TAP_HISTORY, TAP_PARENTS, TAP_ANCESTRY, TAP_STEP) = range(1, 13)
 
 _lock = threading.Lock()
 _lib = None

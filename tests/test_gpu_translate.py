@@ -430,23 +430,23 @@ def test_tensor_core_and_imma_paths_bit_identical(stream):
                               b.view(np.uint32) if b.dtype == np.float32 else b)
 
 
-@pytest.mark.parametrize("d,H,F,n_dec,beam,B,wq", [
-    (128, 2, 128, 1, 1, 5, synth.WQ_INT8),     # 64 FFN columns per CTA, two CTAs, one ragged cluster
-    (128, 2, 512, 2, 3, 3, synth.WQ_INT8),     # sentences straddling warps; 256 columns
-    (256, 4, 768, 2, 5, 7, synth.WQ_INT4),     # 192 columns, 4-bit rows, 5 beams over 4-row chunks
-    (384, 6, 768, 1, 4, 9, synth.WQ_INT8),     # odd factor of d, owned rows of unequal number
-    (384, 6, 384, 1, 1, 40, synth.WQ_INT8),
-    (512, 8, 2048, 2, 2, 13, synth.WQ_INT8),   # K = 2048
-    (512, 8, 2048, 1, 4, 33, synth.WQ_INT8),   # 16 rows per cluster
-    (512, 8, 1536, 1, 4, 100, synth.WQ_INT8),  # 32 rows per cluster
-    (512, 8, 2048, 1, 4, 128, synth.WQ_INT8),  # two heads per CTA, 16 rows
-    (512, 8, 1024, 1, 4, 150, synth.WQ_INT8),  # two heads per CTA, 32 rows
+@pytest.mark.parametrize("d,H,F,n_dec,beam,B,wq,step", [
+    (128, 2, 128, 1, 1, 5, synth.WQ_INT8, [2, 8, 1, 1]),       # 64 FFN columns per CTA, two CTAs, one ragged cluster
+    (128, 2, 512, 2, 3, 3, synth.WQ_INT8, [2, 8, 1, 2]),       # sentences straddling warps; 256 columns
+    (256, 4, 768, 2, 5, 7, synth.WQ_INT4, [2, 8, 1, 5]),       # 192 columns, 4-bit rows, 5 beams over 4-row chunks
+    (384, 6, 768, 1, 4, 9, synth.WQ_INT8, [2, 8, 1, 5]),       # odd factor of d, owned rows of unequal number
+    (384, 6, 384, 1, 1, 40, synth.WQ_INT8, [2, 8, 1, 5]),
+    (512, 8, 2048, 2, 2, 13, synth.WQ_INT8, [2, 8, 1, 4]),     # K = 2048
+    (512, 8, 2048, 1, 4, 33, synth.WQ_INT8, [2, 16, 1, 9]),    # 16 rows per cluster
+    (512, 8, 1536, 1, 4, 100, synth.WQ_INT8, [2, 32, 1, 13]),  # 32 rows per cluster
+    (512, 8, 2048, 1, 4, 128, synth.WQ_INT8, [2, 16, 2, 32]),  # two heads per CTA, 16 rows
+    (512, 8, 1024, 1, 4, 150, synth.WQ_INT8, [2, 32, 2, 19]),  # two heads per CTA, 32 rows
 ])
-def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, B, wq, stream, monkeypatch):
-    """The batched decode step against the kernel-per-operation one, bit for
-    bit: tokens, scores, the last decoder output, residual and self cache, over
-    steps that cross a 16-key block, and again after the padded source length
-    changes (the captured steps are kept)."""
+def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, B, wq, step, stream, monkeypatch):
+    """The batched decode step, in the form named, against the oracle and against
+    the kernel-per-operation step, bit for bit: tokens, scores, the last decoder
+    output, residual and self cache, over steps that cross a 16-key block, and
+    again after the padded source length changes (the captured steps are kept)."""
     cfg = synth.ModelConfig(1, n_dec, d, H, F, 300, d, 1, 1, max_pos=64)
     blob = synth.build_blob(cfg, 91, gamma_range=(0.5, 1.5), wq=wq)
     T, out = 20, {}
@@ -459,6 +459,7 @@ def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, 
                 ids, lens = synth.source_batch(cfg.vocab, B, 1, S, seed)
                 ids = np.pad(ids, ((0, 0), (0, S - ids.shape[1])))
                 res += list(tr.translate(ids, lens, T))
+                assert mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_STEP, 0, np.int32).tolist() == (step if env == "1" else [0] * 4)
                 res += [mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_DEC_OUT), mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_RESID, 0, np.uint32),
                         mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_SELF_K, n_dec - 1), mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_SELF_V, 0)]
             out[env] = res
@@ -466,6 +467,10 @@ def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, 
             tr.close()
     for a, b in zip(out["1"], out["0"]):
         assert np.array_equal(a.view(np.uint8), b.view(np.uint8))
+    o_ids, o_len, o_sc = O.translate(blob, ids, lens, beam, T, n_threads=16)  # of the second batch
+    g_ids, g_len, g_sc = out["1"][7:10]
+    assert np.array_equal(g_ids, o_ids) and np.array_equal(g_len, o_len)
+    assert np.array_equal(g_sc.view(np.uint32), o_sc.view(np.uint32))
 
 
 @pytest.mark.parametrize("beam,B,n_dec", [(1, 260, 1), (4, 65, 1), (3, 23, 4)])
@@ -485,6 +490,7 @@ def test_batched_cluster_step_with_caches_beyond_l2(beam, B, n_dec, stream, monk
         tr = mnmt.Translator(blob, B, 33, beam, T, stream)
         try:
             out[env] = list(tr.translate(ids, lens, 20)) + [mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_DEC_OUT)]
+            assert mnmt.mnmt_debug_tap(tr.session, mnmt.TAP_STEP, 0, np.int32)[0] == (2 if env == "1" else 0)
         finally:
             tr.close()
     for a, b in zip(out["1"], out["0"]):
