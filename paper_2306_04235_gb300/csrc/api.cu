@@ -1269,13 +1269,10 @@ int setup_cluster_step(mnmt_session *s) {
     return MNMT_OK;
 }
 
-// The batched step (decode_rows.cu) where the single-cluster step does not
-// apply: as few rows per cluster as still keep every cluster resident at once
-// (a second wave of clusters would double the step), one head per CTA before
-// two: 15 clusters of eight CTAs fit on 152 SMs, 36 of four.  It was faster than
-// the kernel-per-operation step at every batch measured (12+2 layers, d = 256,
-// beam 4, 1 .. 64 sentences: 139 -> 115 .. 216 -> 158 us per step; 6+6 layers,
-// d = 512, 1 .. 128 sentences: 314 -> 292 .. 665 -> 621).
+// The batched step (decode_rows.cu) where the single-cluster step does not apply
+// and the batch fits it (route_rows_variant): as few rows per cluster as still
+// keep every cluster resident at once, one head per CTA before two: 15 clusters
+// of eight CTAs fit on 152 SMs, 36 of four.
 // MNMT_DECODE_CLUSTER=0 forces the kernel-per-operation step.
 int setup_rows_step(mnmt_session *s) {
     mnmt_model *m = s->m;
@@ -1315,18 +1312,18 @@ int setup_rows_step(mnmt_session *s) {
     }
     // laid out for the session's longest source: only S changes with the batch
     P.S = s->Smax;
-    for (const auto &v : {std::pair<int, int>{1, 1}, {2, 1}, {4, 1}, {2, 2}, {4, 2}}) {
+    for (const auto &v : {std::pair<int, int>{1, 1}, {2, 1}, {4, 1}, {2, 2}}) {
         const int nb = v.first, hpc = v.second;
         const size_t smem = dr_layout(P, nb, hpc, 227 * 1024);
         if (smem == (size_t)-1) continue;
         const int clusters = (R + 8 * nb - 1) / (8 * nb), fit = dr_max_clusters(nb, hpc, P.nc, smem);
-        if (fit < 1) continue;
+        if (!route_rows_variant(nb, hpc, s->k, clusters, fit)) continue;
         s->use_rows = true;
         s->dr_nb = nb;
         s->dr_hpc = hpc;
         s->dr_clusters = clusters;
         s->dr_smem = smem;
-        if (clusters <= fit) break;
+        break;
     }
     if (!s->use_rows) return MNMT_OK;
     dr_layout(P, s->dr_nb, s->dr_hpc, 227 * 1024);

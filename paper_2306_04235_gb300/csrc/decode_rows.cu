@@ -1034,7 +1034,7 @@ __global__ void __launch_bounds__(DR_THREADS, 1) decode_rows_kernel(const DrPara
 }
 
 const void *dr_kernel(int nb, int hpc) {
-    if (hpc == 2) return nb == 2 ? (const void *)decode_rows_kernel<2, 2> : (const void *)decode_rows_kernel<4, 2>;
+    if (hpc == 2) return (const void *)decode_rows_kernel<2, 2>;
     return nb == 1 ? (const void *)decode_rows_kernel<1, 1> : nb == 2 ? (const void *)decode_rows_kernel<2, 1>
                                                                       : (const void *)decode_rows_kernel<4, 1>;
 }
@@ -1136,7 +1136,7 @@ int dr_max_clusters(int nb, int hpc, int nc, size_t smem) {
 
 cudaError_t decode_rows_init() {
     cudaError_t err = cudaSuccess;
-    const int v[5][2] = {{1, 1}, {2, 1}, {4, 1}, {2, 2}, {4, 2}};
+    const int v[4][2] = {{1, 1}, {2, 1}, {4, 1}, {2, 2}};
     for (const auto &x : v)
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(dr_kernel(x[0], x[1]), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);

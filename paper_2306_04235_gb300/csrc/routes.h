@@ -47,4 +47,22 @@ inline bool route_linear_tc(LinRole role, int M, int d, int F, int n, int k, boo
     return role != LIN_SQUARE || d > 512 || (d > 384 && (double)M * n * k > 3e8);
 }
 
+// May the batched decode step run on `clusters` clusters of 8 nb rows with hpc
+// heads per CTA, of which `fit` are resident at once?  (Tried with 1, 2 and 4
+// times 8 rows of one head per CTA, then 16 rows of two; else a kernel per
+// operation.)  A second wave of clusters doubles the step; 32 rows, or two heads,
+// to a warp's chain are worth it only where beams share their keys.  Steps of
+// 24, us, batched / kernel per operation:
+//   one wave of 8 or 16 rows: d 128, 480 rows 66 / 95; d 256, 576 rows 110 / 128; d 512,
+//     6 layers, 240 rows 205 / 251
+//   32 rows: d 512, 400 rows, beam 1 267 / 229, beam 4 279 / 278; d 256, beam 4,
+//     640 rows 203 / 197, 1152 rows 251 / 253; d 384, beam 4, 640 rows 154 / 163
+//   16 rows of two heads: d 512, 576 rows, beam 1 281 / 267, beam 2 306 / 311, beam 4
+//     293 / 314; steps of 128, beam 2, 444 rows 342 / 309, beam 4, 576 rows 318 / 353
+//   32 rows of two heads: d 512, beam 4, 640 rows 404 / 324, beam 1 427 / 274
+//   two waves: d 512, beam 1, 1200 rows 805 / 348
+inline bool route_rows_variant(int nb, int hpc, int beam, int clusters, int fit) {
+    return clusters <= fit && ((nb <= 2 && hpc == 1) || beam >= 4);
+}
+
 }  // namespace mnmt

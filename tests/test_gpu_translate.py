@@ -440,7 +440,9 @@ def test_tensor_core_and_imma_paths_bit_identical(stream):
     (512, 8, 2048, 1, 4, 33, synth.WQ_INT8, [2, 16, 1, 9]),    # 16 rows per cluster
     (512, 8, 1536, 1, 4, 100, synth.WQ_INT8, [2, 32, 1, 13]),  # 32 rows per cluster
     (512, 8, 2048, 1, 4, 128, synth.WQ_INT8, [2, 16, 2, 32]),  # two heads per CTA, 16 rows
-    (512, 8, 1024, 1, 4, 150, synth.WQ_INT8, [2, 32, 2, 19]),  # two heads per CTA, 32 rows
+    (512, 8, 1024, 1, 4, 144, synth.WQ_INT8, [2, 16, 2, 36]),  # as many clusters as are resident at once
+    (512, 8, 1024, 1, 4, 150, synth.WQ_INT8, [0, 0, 0, 0]),    # more: a kernel per operation
+    (512, 8, 1024, 1, 1, 250, synth.WQ_INT8, [0, 0, 0, 0]),    # 32 rows without beams: the same
 ])
 def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, B, wq, step, stream, monkeypatch):
     """The batched decode step, in the form named, against the oracle and against
@@ -473,7 +475,7 @@ def test_batched_cluster_step_equals_kernel_per_operation(d, H, F, n_dec, beam, 
     assert np.array_equal(g_sc.view(np.uint32), o_sc.view(np.uint32))
 
 
-@pytest.mark.parametrize("beam,B,n_dec", [(1, 260, 1), (4, 65, 1), (3, 23, 4)])
+@pytest.mark.parametrize("beam,B,n_dec", [(1, 240, 2), (4, 65, 1), (3, 23, 4)])
 def test_batched_cluster_step_with_caches_beyond_l2(beam, B, n_dec, stream, monkeypatch):
     """Sessions whose caches exceed L2 bring a layer's to it ahead of its
     attention: the first step (no own keys yet), sentences of one token, beams

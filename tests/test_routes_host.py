@@ -62,3 +62,22 @@ def test_vocabulary_projection_takes_the_faster_family(tmp_path):
     got = _decide(tmp_path, "route_linear_tc(LIN_OUT, a[0], a[2], 4 * a[2], a[1], a[2], a[3])", [x[0] for x in rows])
     for (m, t8, tc), choice in zip(rows, got):
         assert (tc if choice else t8) <= 1.06 * min(t8, tc), (m, t8, tc, choice)
+
+
+# clusters of n CTAs that are resident at once on 152 SMs
+FIT = {1: 152, 2: 76, 3: 45, 4: 36, 6: 23, 8: 15}
+
+
+def test_batched_step_runs_where_it_is_faster(tmp_path):
+    rows = [([int(x) for x in f[:4]], *map(float, f[4:])) for f in _table("rows_routes.txt", "rows")]
+    assert len(rows) > 100
+    taken = [0] * len(rows)
+    for nb, hpc in ((1, 1), (2, 1), (4, 1), (2, 2)):
+        args = [(beam, -(-r // (8 * nb)), FIT.get(heads // hpc, 0)) for (r, heads, beam, _), *_ in rows]
+        for i, ok in enumerate(_decide(tmp_path, f"route_rows_variant({nb}, {hpc}, a[0], a[1], a[2])", args)):
+            taken[i] |= ok
+    for (m, batched, per_op, start), use in zip(rows, taken):
+        t = batched if use else per_op
+        # (one line for short and long sources: two beams cross between them)
+        assert t <= 1.10 * min(batched, per_op), (m, batched, per_op, use)
+        assert t <= 1.01 * start, (m, t, start)
