@@ -42,6 +42,7 @@
 #include "internal.h"
 #include "mbarrier.cuh"
 #include "mnmt.h"
+#include "routes.h"
 
 namespace mnmt {
 namespace {
@@ -158,7 +159,7 @@ __device__ __forceinline__ void q8_pack16(const float (&a)[16], const float *sc,
 
 // the 16-column epilogue below applies (every destination row segment of 16
 // outputs is contiguous and 16-byte aligned)
-__device__ __forceinline__ bool epi_vec_ok(const Epi &e) {
+__host__ __device__ __forceinline__ bool epi_vec_ok(const Epi &e) {
     const auto al = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
     switch (e.mode) {
         case EPI_Q8:
@@ -1533,28 +1534,12 @@ cudaError_t launch_linear_tc(const __half *A16, int lda, const __half *W16, int 
     const bool two_chunks = K > TC_KB_PER_CHUNK * TC_BK;
     const int nkb = (K + TC_BK - 1) / TC_BK;
     const long mt = (M + TC_BM - 1) / TC_BM, mt2 = (M + 2 * TC_BM - 1) / (2 * TC_BM);
-    const long tiles_128 = mt * ((N + 127) / 128), tiles64 = mt * ((N + SK_BN - 1) / SK_BN);
-    const bool f32m = e.mode == EPI_RESID || e.mode == EPI_F32;
-    // CTA pairs, by the waves of 256 x 256 tiles on the pairs and of 128 x 128
-    // tiles on the SMs.  A pair starts later (cluster, 512 TMEM columns) and its
-    // tile takes longer; with K = 512 and codes out 7.2 + 4.4 us a wave against
-    // 4.4 + 3.5, so it wins where 5 w256 + 3 < 4 w128 (M 4000, N 2048: 15.9 us
-    // against 18.0; M 4400, N 1536, where it does not: 15.8 against 15.0).  The fp32 outputs of
-    // 128 x 128 tiles are slower, two waves (M 5000, N 512, residual 20.2; M 300,
-    // N 8192 14.6) than one of pairs (14.7; 12.8); with equal waves they are not.
+    const long tiles64 = mt * ((N + SK_BN - 1) / SK_BN);
     const long p256 = mt2 * ((N + 255) / 256), p128 = mt2 * ((N + 127) / 128);
-    const long w256 = g_pairs > 0 ? (p256 + g_pairs - 1) / g_pairs : 0, w128 = (tiles_128 + g_num_sms - 1) / g_num_sms;
-    const bool pair256 = g_pairs > 0 && N >= 256 && tiles_128 >= g_num_sms && (f32m ? w256 < w128 : 5 * w256 + 3 < 4 * w128);
-    // 256 x 128 tiles: one wave of pairs where 128 x 64 tiles need two and K is
-    // long (M 4000, N 512, K 2048, residual: 18.1 us against 23.1; K 1024: 13.9
-    // against 15.1; K 512: equal; M 2300, N 1024, K 1024, codes: 11.9 against 13.8)
-    const bool pair128 = !pair256 && nkb >= TC_KB_PER_CHUNK && p128 <= g_pairs && tiles64 > g_num_sms;
-    // 128 x 256 tiles of one CTA: one wave that would be two of 128 x 128 (M 1500,
-    // N 2048, codes: K 512 9.5 us against 10.6, K 1024 13.3 against 15.4, K 2048
-    // 19.1 against 23.9; M 2400, N 2048, K 512, residual: 20.1 against 21.1)
-    const long tiles_wide = mt * ((N + 255) / 256);
-    const bool wide = !pair256 && !pair128 && N >= 256 && w128 == 2 && tiles_wide <= g_num_sms;
-    const bool pair = pair256 || pair128, narrow = !pair && tiles_128 < g_num_sms;
+    const bool f32m = e.mode == EPI_RESID || e.mode == EPI_F32;
+    const bool vec = f32m || e.mode == EPI_ARGMAX || (N % 16 == 0 && epi_vec_ok(e));
+    const TcTiles tt = route_tc_tiles(M, N, nkb, f32m, e.mode == EPI_ARGMAX, vec, g_num_sms, g_pairs);
+    const bool pair256 = tt == TC_PAIR256, pair = pair256 || tt == TC_PAIR128, wide = tt == TC_WIDE, narrow = tt == TC_NARROW;
     CUtensorMap ta, tb;
     if (!make_map(&ta, A16, K, M, lda, TC_BM) || !make_map(&tb, W16, K, N, ldw, wide ? 256 : pair256 ? 128 : pair || narrow ? 64 : 128))
         return cudaErrorInvalidValue;

@@ -47,6 +47,59 @@ inline bool route_linear_tc(LinRole role, int M, int d, int F, int n, int k, boo
     return role != LIN_SQUARE || d > 512 || (d > 384 && (double)M * n * k > 3e8);
 }
 
+// Output tiles of a tcgen05 linear: 256 x 256 or 256 x 128 on CTA pairs, 128 x 256,
+// 128 x 128 or (split K where it leaves SMs idle) 128 x 64 on single CTAs.
+enum TcTiles { TC_PAIR256, TC_PAIR128, TC_WIDE, TC_128, TC_NARROW };
+
+// sms SMs, `pairs` CTA pairs resident at once; nkb k-blocks of 64; f32: fp32
+// outputs; rows16: output rows that 16-byte stores can write.
+//   Codes and argmax: a pair starts later (cluster, 512 TMEM columns) and its tile
+//   takes longer, and K above 1024 leaves 256 columns one accumulator buffer, so by
+//   time, t + a nkb + waves x (b + c nkb) us, fitted to 2300 calls of 300 to 16384
+//   rows (K 64 to 2048; 2 to 4 % rms, with two chunks 3 to 8 %), with 3 % asked for
+//   before leaving 128 x 128, or up to K = 512 pairs for wide (6400 x 1536, K = 512
+//   pair256 15.3, wide 15.1 alone, but 1383 / 1392 a first step).
+//   Measured (128 x 128 / wide / pair256): 4000 x 2048, K = 64 13.7 / 11.6 / 12.7, K = 512 18.0
+//   / 14.2 / 15.9; 3000 x 2048, K = 1024 20.6 / 17.9 / 18.7, K = 2048 33.3 / 29.9 / 29.6; 1500 x
+//   2048, K = 512 10.6 / 9.5 / 11.6
+//   Rows that cannot be stored 16 bytes at a time go through the pairs' staging
+//   blocks (3000 x 1000, K = 512: 51.7 / 58.2 / 25.1).
+//   fp32 outputs of 128 x 128 tiles are slower: one wave of pairs against two of
+//   those (M 5000, N 512, residual 14.7 / 20.2; M 300, N 8192 12.8 / 14.6); with
+//   equal waves they are not.
+//   pair128: one wave where 128 x 64 tiles need two and K is long (M 4000, N 512,
+//   residual: K 2048 18.1 / 23.1, K 1024 13.9 / 15.1, K 512 equal; M 2300, N 1024,
+//   K 1024, codes 11.9 / 13.8).
+//   fp32 wide: one wave that would be two of 128 x 128 (M 2400, N 2048, K 512, residual
+//   20.1 / 21.1).
+inline TcTiles route_tc_tiles(int M, int N, int nkb, bool f32, bool argmax, bool rows16, int sms, int pairs) {
+    const auto up = [](long a, long b) { return (a + b - 1) / b; };
+    const long mt = up(M, 128), mt2 = up(M, 256);
+    const long t128 = mt * up(N, 128), wide = mt * up(N, 256), p256 = mt2 * up(N, 256);
+    const bool pair128 = pairs > 0 && nkb >= 16 && mt2 * up(N, 128) <= pairs && mt * up(N, 64) > sms;
+    if (t128 < sms) return pair128 ? TC_PAIR128 : TC_NARROW;
+    const long w128 = up(t128, sms), ww = up(wide, sms), w256 = pairs > 0 ? up(p256, pairs) : 0;
+    if (N >= 256 && f32) {
+        if (w256 > 0 && w256 < w128) return TC_PAIR256;
+        if (!pair128 && w128 == 2 && ww == 1) return TC_WIDE;
+    } else if (N >= 256) {
+        // [argmax][two chunks of K][pair256, wide, 128 x 128] {t, a, b, c}
+        static constexpr double fit[2][2][3][4] = {
+            {{{4.69, 0.162, 3.69, 0.116}, {3.09, 0.153, 4.24, 0.125}, {3.24, 0.137, 2.41, 0.142}},
+             {{6.78, -0.026, 5.19, 0.206}, {3.99, -0.073, 11.89, 0.053}, {4.53, 0.015, 4.32, 0.149}}},
+            {{{4.24, 0.138, 3.21, 0.139}, {2.89, 0.215, 4.82, 0.064}, {3.11, 0.150, 2.55, 0.133}},
+             {{6.88, -0.034, 4.62, 0.214}, {4.09, -0.058, 12.17, 0.041}, {5.90, -0.030, 3.03, 0.193}}}};
+        const auto time = [&](int v, long w) {
+            const double *c = fit[argmax][nkb > 16][v];
+            return c[0] + c[1] * nkb + (double)w * (c[2] + c[3] * nkb);
+        };
+        const double tp = time(0, w256), tw = time(1, ww), t1 = time(2, w128);
+        if (w256 > 0 && (!rows16 || (tp < 0.97 * t1 && tp < (nkb > 8 ? 1.0 : 1.03) * tw))) return TC_PAIR256;
+        if (!pair128 && tw < 0.97 * t1) return TC_WIDE;
+    }
+    return pair128 ? TC_PAIR128 : TC_128;
+}
+
 // May the batched decode step run on `clusters` clusters of 8 nb rows with hpc
 // heads per CTA, of which `fit` are resident at once?  (Tried with 1, 2 and 4
 // times 8 rows of one head per CTA, then 16 rows of two; else a kernel per

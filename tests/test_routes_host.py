@@ -31,7 +31,7 @@ int main() {{
 """)
     exe = tmp_path / "r"
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)], check=True)
-    text = "\n".join(f"{len(r)} " + " ".join(map(str, r)) for r in rows)
+    text = "\n".join(f"{len(r)} " + " ".join(str(int(x)) for x in r) for r in rows)
     out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True).stdout
     return [int(x) for x in out.split()]
 
@@ -81,3 +81,15 @@ def test_batched_step_runs_where_it_is_faster(tmp_path):
         # (one line for short and long sources: two beams cross between them)
         assert t <= 1.10 * min(batched, per_op), (m, batched, per_op, use)
         assert t <= 1.01 * start, (m, t, start)
+
+
+def test_tcgen05_tiles_are_the_faster_ones(tmp_path):
+    rows = [([int(x) for x in f[:4]], float(f[4]), [float(x) for x in f[5:]]) for f in _table("tc_routes.txt", "tc")]
+    assert len(rows) > 300
+    args = [(m, n, -(-k // 64), mode == 2, mode == 4, mode != 0 or n % 16 == 0) for (m, n, k, mode), *_ in rows]
+    got = _decide(tmp_path, "route_tc_tiles(a[0], a[1], a[2], a[3], a[4], a[5], 152, 76)", args)
+    loss = []
+    for (m, start, t), choice in zip(rows, got):
+        assert t[choice] <= 1.05 * start + 0.3, (m, start, t, choice)
+        loss.append(t[choice] / min(t))
+    assert sum(loss) / len(loss) < 1.03
