@@ -16,6 +16,7 @@
 // inference kernels on the same codes.
 #include "common.cuh"
 #include "internal.h"
+#include "routes.h"
 
 namespace mnmt {
 
@@ -42,10 +43,12 @@ MNMT_DEV float fq_code(float x, float inv, float r, int minmax, FqRange rg, floa
 // an integer-valued |q| <= 255 as an int
 MNMT_DEV int fq_int(float q) { return (int)(__float_as_uint(__fadd_rn(q, 12582912.0f)) - 0x4B400000u); }
 
-MNMT_DEV bool fq_al16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+__host__ __device__ __forceinline__ bool fq_al16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// Forward, four elements per thread and step where every array is 16-byte
-// aligned.  Bound by the 8 bytes per element (12 with codes) it moves.
+// Forward, four elements per thread and step (groups; route_fake_quant) where
+// every array is 16-byte aligned.  Bound by the 8 bytes per element (12 with
+// codes) it moves.
+template <bool GROUPS>
 __global__ void fq_forward_kernel(const float *__restrict__ x, size_t n, float s, float r, int bits, int minmax,
                                   float *__restrict__ y, int32_t *__restrict__ codes) {
     const float inv = __fdiv_rn(1.0f, s);
@@ -56,7 +59,7 @@ __global__ void fq_forward_kernel(const float *__restrict__ x, size_t n, float s
         return minmax ? __fadd_rn(v, r) : v;
     };
     size_t done = 0;
-    if (fq_al16(x) && fq_al16(y) && fq_al16(codes)) {
+    if (GROUPS) {
         for (size_t i = tid; i < n / 4; i += nt) {
             const float4 v = reinterpret_cast<const float4 *>(x)[i];
             const float q0 = fq_code(v.x, inv, r, minmax, rg, nullptr), q1 = fq_code(v.y, inv, r, minmax, rg, nullptr);
@@ -89,6 +92,7 @@ MNMT_DEV float fq_two_sum(float a, float b, float &e) {
 // and the third level is added plainly (2^-72 of the largest term, far below
 // fp64's own 2^-53).  Groups whose products leave the range in which that
 // holds (2^-80 .. 2^120) are summed in fp64 term by term.  2 M elements: 14.8 us.
+template <bool GROUPS>
 __global__ void __launch_bounds__(256) fq_backward_kernel(const float *__restrict__ x, const float *__restrict__ g, size_t n, float s,
                                    float r, int bits, int minmax, float *__restrict__ gx, double *gs, double *gr) {
     const float inv = __fdiv_rn(1.0f, s);
@@ -96,7 +100,7 @@ __global__ void __launch_bounds__(256) fq_backward_kernel(const float *__restric
     double as = 0.0, ar = 0.0;
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (size_t)gridDim.x * blockDim.x;
     size_t done = 0;
-    if (fq_al16(x) && fq_al16(g) && fq_al16(gx)) {
+    if (GROUPS) {
         for (size_t i = tid; i < n / 8; i += nt) {
             float xv[8], gv[8], ev[8], ov[8];
             *reinterpret_cast<float4 *>(xv) = reinterpret_cast<const float4 *>(x)[2 * i];
@@ -221,7 +225,9 @@ static int fq_grid(size_t n, int per) {
 cudaError_t launch_fake_quant(const float *x, size_t n, float s, float r, int bits, int minmax, float *y,
                               int32_t *codes, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    fq_forward_kernel<<<fq_grid(n, 4), 256, 0, st>>>(x, n, s, r, bits, minmax, y, codes);
+    const FqLaunch l = route_fake_quant(n, fq_al16(x) && fq_al16(y) && fq_al16(codes), false, minmax, device_sm_count());
+    if (l.groups) fq_forward_kernel<true><<<l.blocks, 256, 0, st>>>(x, n, s, r, bits, minmax, y, codes);
+    else fq_forward_kernel<false><<<l.blocks, 256, 0, st>>>(x, n, s, r, bits, minmax, y, codes);
     return cudaGetLastError();
 }
 
@@ -230,7 +236,9 @@ cudaError_t launch_fake_quant_backward(const float *x, const float *g, size_t n,
     cudaError_t e = cudaMemsetAsync(gs, 0, sizeof(double), st);
     if (e == cudaSuccess && gr) e = cudaMemsetAsync(gr, 0, sizeof(double), st);
     if (e != cudaSuccess || n == 0) return e;
-    fq_backward_kernel<<<fq_grid(n, 8), 256, 0, st>>>(x, g, n, s, r, bits, minmax, gx, gs, gr);
+    const FqLaunch l = route_fake_quant(n, fq_al16(x) && fq_al16(g) && fq_al16(gx), true, minmax, device_sm_count());
+    if (l.groups) fq_backward_kernel<true><<<l.blocks, 256, 0, st>>>(x, g, n, s, r, bits, minmax, gx, gs, gr);
+    else fq_backward_kernel<false><<<l.blocks, 256, 0, st>>>(x, g, n, s, r, bits, minmax, gx, gs, gr);
     return cudaGetLastError();
 }
 

@@ -2,6 +2,8 @@
 // functions, so that the rules can be compared with measured times anywhere.
 #pragma once
 
+#include <stddef.h>
+
 namespace mnmt {
 
 // what a linear of a session does (it decides the kernel with the sizes)
@@ -98,6 +100,24 @@ inline TcTiles route_tc_tiles(int M, int N, int nkb, bool f32, bool argmax, bool
         if (!pair128 && tw < 0.97 * t1) return TC_WIDE;
     }
     return pair128 ? TC_PAIR128 : TC_128;
+}
+
+// Fake quantisation of n elements: groups of 4 (forward) or 8 (backward) per
+// thread and step, or single elements, and the blocks of 256 threads for it.
+//   Single elements where an array is not 16-byte aligned, and where groups would
+//   leave too few threads: a step's chain is then longer than its loads are worth
+//   (us, single / groups: forward 10007 1.56 / 1.70, 65536 1.66 / 1.60; backward 100
+//   7.1 / 8.2, 65536 8.9 / 8.7; min-max form 65536 8.7 / 10.3, 300000 11.6 / 11.0).
+struct FqLaunch {
+    bool groups;
+    int blocks;
+};
+inline FqLaunch route_fake_quant(size_t n, bool aligned, bool backward, bool minmax, int sms) {
+    FqLaunch l;
+    l.groups = aligned && n >= (size_t)(!backward ? 32768 : minmax ? 262144 : 4096);
+    const size_t per = l.groups ? (backward ? 8 : 4) : 1, b = (n / per + 255) / 256, cap = (size_t)8 * sms;
+    l.blocks = (int)(b < 1 ? 1 : b > cap ? cap : b);
+    return l;
 }
 
 // May the batched decode step run on `clusters` clusters of 8 nb rows with hpc

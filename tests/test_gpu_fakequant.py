@@ -111,3 +111,25 @@ def test_fake_quant_backward_non_finite():
         rgx, rgs, _ = O.fake_quant_backward(x, g, np.float32(0.041), 8, 0.0, False)
         assert np.array_equal(host(gx).view(np.uint32), rgx.view(np.uint32))
         assert np.array_equal(np.array([float(host(gs)[0])]), np.array([rgs]), equal_nan=True)
+
+
+@pytest.mark.parametrize("n", [4095, 4096, 32767, 32769, 262143, 262145])
+@pytest.mark.parametrize("minmax", [False, True])
+@pytest.mark.parametrize("off", [0, 1])
+def test_fake_quant_group_limits(n, minmax, off):
+    """Both sides of the sizes from which elements are taken in groups, aligned
+    and not.  Bound of the sums: fp64 addition of n terms."""
+    s, r = np.float32(0.041), np.float32(-1.7) if minmax else np.float32(0)
+    x, g = _x(n, n + off, 0.6), _x(n + 3, n + off, 1.0)
+    dx, dg = dev(x)[off:], dev(g)[off:]
+    y, gx = (torch.empty(n + off, dtype=torch.float32, device="cuda")[off:] for _ in range(2))
+    codes = torch.empty(n + off, dtype=torch.int32, device="cuda")[off:]
+    gs, gr = (torch.empty(1, dtype=torch.float64, device="cuda") for _ in range(2))
+    mnmt.mnmt_fake_quant(dx, n, s, r, 4, minmax, y, codes)
+    mnmt.mnmt_fake_quant_backward(dx, dg, n, s, gx, gs, gr, r, 4, minmax)
+    ry, rq = O.fake_quant(x[off:], s, 4, r, minmax)
+    rgx, rgs, rgr = O.fake_quant_backward(x[off:], g[off:], s, 4, r, minmax)
+    assert np.array_equal(host(y).view(np.uint32), ry.view(np.uint32)) and np.array_equal(host(codes), rq)
+    assert np.array_equal(host(gx).view(np.uint32), rgx.view(np.uint32))
+    bound = n * 2.0 ** -53 * float(np.abs(g[off:].astype(np.float64)).sum()) * 15
+    assert abs(float(host(gs)[0]) - rgs) <= bound and abs(float(host(gr)[0]) - rgr) <= bound

@@ -93,3 +93,18 @@ def test_tcgen05_tiles_are_the_faster_ones(tmp_path):
         assert t[choice] <= 1.05 * start + 0.3, (m, start, t, choice)
         loss.append(t[choice] / min(t))
     assert sum(loss) / len(loss) < 1.03
+
+
+def test_fake_quant_threads_are_not_idle(tmp_path):
+    """Single elements get a thread each up to 8 blocks per SM; groups only where
+    every array is aligned and they fill the blocks that single elements would."""
+    sizes = [1, 100, 4095, 4096, 10007, 32767, 32768, 65536, 262143, 262144, 1 << 22]
+    rows = [(n, al, bw, mm) for n in sizes for al in (0, 1) for bw in (0, 1) for mm in (0, 1)]
+    call = "route_fake_quant(a[0], a[1], a[2], a[3], 152)"
+    groups, blocks = _decide(tmp_path, call + ".groups", rows), _decide(tmp_path, call + ".blocks", rows)
+    for (n, al, bw, mm), g, b in zip(rows, groups, blocks):
+        per = (8 if bw else 4) if g else 1
+        assert b == max(1, min(8 * 152, -(-(n // per) // 256)))
+        assert not g or al
+        if al:
+            assert g == (n >= (262144 if bw and mm else 4096 if bw else 32768))
