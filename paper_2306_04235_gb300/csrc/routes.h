@@ -102,6 +102,15 @@ inline TcTiles route_tc_tiles(int M, int N, int nkb, bool f32, bool argmax, bool
     return pair128 ? TC_PAIR128 : TC_128;
 }
 
+// LayerNorm of M rows of d: a warp per row (whole float4s, up to 1024 elements) or
+// a block per row?  A warp per row from two rows per SM on, from three where the
+// block kernel divides d among its threads without remainder (us, block / warp:
+// 301 x 384 3.8 / 3.1, 301 x 512 2.75 / 3.2, 400 x 512 3.1 / 3.1, 512 x 512 3.6 / 3.2, 301 x 1024,
+// codes only 3.6 / 4.4, 512 x 1024 4.9 / 4.5, 16384 x 512 38.1 / 20.6).
+inline bool route_layernorm_warp(int M, int d) {
+    return d % 4 == 0 && d <= 1024 && M > (d == 512 || d == 1024 ? 448 : 300);
+}
+
 // Fake quantisation of n elements: groups of 4 (forward) or 8 (backward) per
 // thread and step, or single elements, and the blocks of 256 threads for it.
 //   Single elements where an array is not 16-byte aligned, and where groups would

@@ -10,6 +10,7 @@
 // the same mean and rstd bits.
 #include "common.cuh"
 #include "internal.h"
+#include "routes.h"
 
 namespace mnmt {
 
@@ -21,8 +22,6 @@ namespace mnmt {
 // exact fixed-point sums combine across warps through shared memory.  The
 // row, gamma and beta are loaded together before the skip flag is tested.
 // ---------------------------------------------------------------------------
-constexpr int LN_WARP_MIN_ROWS = 300;
-
 template <int VPT, int LN_T>
 __global__ void __launch_bounds__(LN_T) layernorm_kernel(LnArgs a) {
     pdl_grid_wait();
@@ -246,14 +245,12 @@ cudaError_t launch_layernorm_t(const LnArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// A warp per row from about two rows per SM on (512 x 512: 3.4 against 4.1 us,
-// 256 x 512: 3.3 against 3.1, 16384 x 512: 21.8 against 38.8), for rows of
-// whole, aligned float4s up to 1024 elements; else the block-per-row kernel,
-// with 256 threads per row up to 1024 rows (shorter chains), else 128.
+// A warp per row by route_layernorm_warp, for aligned rows; else the block-per-row
+// kernel, with 256 threads per row up to 1024 rows (shorter chains), else 128.
 cudaError_t launch_layernorm(const LnArgs &a, cudaStream_t st) {
     if (a.M <= 0) return cudaSuccess;
     const auto al = [](const void *p, uintptr_t m) { return (reinterpret_cast<uintptr_t>(p) & m) == 0; };
-    if (a.M > LN_WARP_MIN_ROWS && a.d % 4 == 0 && a.d <= 1024 && al(a.r, 15) && al(a.g, 15) && al(a.b, 15) &&
+    if (route_layernorm_warp(a.M, a.d) && al(a.r, 15) && al(a.g, 15) && al(a.b, 15) &&
         al(a.out_f, 15) && al(a.out_q, 3) && al(a.out16, 7)) {
         switch ((a.d + 127) / 128) {
             case 1: return launch_layernorm_warp<1>(a, st);

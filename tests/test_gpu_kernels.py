@@ -239,10 +239,11 @@ def test_linear_fp16_products_edges(M, N, K, mode):
     assert np.array_equal(got.view(v), ref.view(v))
 
 
-@pytest.mark.parametrize("M,d", [(301, 4), (301, 128), (333, 132), (301, 384), (700, 516), (301, 768), (301, 1020), (302, 1024), (2500, 512)])
+@pytest.mark.parametrize("M,d", [(301, 4), (301, 128), (333, 132), (301, 384), (700, 516), (301, 768), (301, 1020), (302, 1024),
+                                 (448, 512), (449, 512), (449, 1024), (2500, 512)])
 @pytest.mark.parametrize("scale", [1.0, 1e-12, 1e-25, 3e6])
 def test_layernorm_warp_rows(M, d, scale):
-    """The warp-per-row LayerNorm (more than 300 rows): ragged and whole
+    """The warp-per-row LayerNorm (more than 300 rows, 448 of 512 or 1024): ragged and whole
     float4 counts per lane, odd factors of d, rows within fx_sum's range and,
     at the two small scales, the term-by-term forms of the variance and of both
     sums; rows with values far below the largest (every piece of a term)."""

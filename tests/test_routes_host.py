@@ -108,3 +108,10 @@ def test_fake_quant_threads_are_not_idle(tmp_path):
         assert not g or al
         if al:
             assert g == (n >= (262144 if bw and mm else 4096 if bw else 32768))
+
+
+def test_layernorm_takes_the_faster_kernel(tmp_path):
+    rows = [([int(x) for x in f[:2]], float(f[3]), float(f[4])) for f in _table("ln_routes.txt", "ln")]
+    assert len(rows) > 100
+    for (m, block, warp), choice in zip(rows, _decide(tmp_path, "route_layernorm_warp(a[0], a[1])", [x[0] for x in rows])):
+        assert (warp if choice else block) <= 1.06 * min(block, warp), (m, block, warp, choice)
