@@ -138,7 +138,10 @@ void mnmt_session_free(mnmt_session *s);
 
 /* Device bytes held by a model (blob, derived constants, fp16 operand copy
  * unless lean) or by a session (its one arena: caches, activations, search
- * state).  Nothing else is allocated on the device by the library after these
+ * state and, where the batched decode step can run -- pre-LN, head width 64, 2 to
+ * 8 heads and an even number, no min-max rows, beams or more than 4 sentences,
+ * lengths up to 512, not lean -- the decoder's weights as that step reads them,
+ * n_dec (6 d^2 + 2 d F) bytes, packed at the first decode).  Nothing else is allocated on the device by the library after these
  * objects are created, so model + session bytes are the library's peak device
  * memory for a translation.  Negative MNMT_EINVAL for a null handle. */
 int64_t mnmt_model_device_bytes(const mnmt_model *model);
@@ -224,8 +227,9 @@ int64_t mnmt_debug_tap(mnmt_session *s, int32_t tap, int32_t layer, void *host_d
  * sentences whose shapes fit one cluster's shared memory), 0 = the multi-kernel
  * step (whose decoder layers run as one kernel where the model's shape allows
  * it, else a kernel per operation); negative on error.  Setting MNMT_DECODE_CLUSTER=0 in the environment
- * before the first decode of a batch forces the kernel-per-operation step.  Both give
- * bit-identical results. */
+ * before the first decode of a batch forces the kernel-per-operation step (and
+ * before the session is created keeps the batched step's weights out of it).
+ * All give bit-identical results. */
 int mnmt_session_decode_path(mnmt_session *s);
 
 /* Thread-local description of the last error on this thread ("" if none). */

@@ -661,10 +661,19 @@ extern "C" int mnmt_session_create_ex(mnmt_model *m, int32_t max_batch, int32_t 
         return at;
     };
     // the batched decode step (decode_rows.cu), where greedy batches too small
-    // for it have the single-cluster one: its packed weights live in the arena
-    const char *tc_env = std::getenv("MNMT_TC");
-    const bool rows_ok = tc_ok && !(tc_env && tc_env[0] == '0') && c.pre_ln && m->dec_self[0].qkv.w &&
-                         (beam > 1 || max_batch > DC_RMAX) && dr_shape_ok(c.d_model, c.n_heads, c.d_ffn, c.d_embed, c.n_dec);
+    // for it have the single-cluster one and one of its forms has room for the
+    // session's lengths: its packed weights live in the arena
+    const char *tc_env = std::getenv("MNMT_TC"), *dc_env = std::getenv("MNMT_DECODE_CLUSTER");
+    bool rows_ok = tc_ok && !(tc_env && tc_env[0] == '0') && !(dc_env && dc_env[0] == '0') && c.pre_ln && m->dec_self[0].qkv.w &&
+                   (beam > 1 || max_batch > DC_RMAX) && dr_shape_ok(c.d_model, c.n_heads, c.d_ffn, c.d_embed, c.n_dec);
+    if (rows_ok) {
+        DrParams &P = s->dr_host;
+        P.d = c.d_model; P.H = c.n_heads; P.F = c.d_ffn; P.n_dec = c.n_dec; P.T = max_len; P.S = max_src_len;
+        bool room = false;
+        for (const auto &v : DR_FORMS)
+            room = room || (route_rows_variant(v[0], v[1], beam, 1, 1) && dr_layout(P, v[0], v[1], 227 * 1024) != (size_t)-1);
+        rows_ok = room;
+    }
     const size_t drw_bytes = rows_ok ? dr_bytes(c.d_model, c.d_ffn, c.n_dec) : 0;
     const size_t qkv_bytes = lean ? std::max(ME * 3 * d, rows * F) : ME * 3 * d;
     size_t o_resid = piece(rows * d * 4), o_act = piece(rows * (d > F ? d : F)), o_qkv = piece(qkv_bytes),
@@ -1312,8 +1321,8 @@ int setup_rows_step(mnmt_session *s) {
     }
     // laid out for the session's longest source: only S changes with the batch
     P.S = s->Smax;
-    for (const auto &v : {std::pair<int, int>{1, 1}, {2, 1}, {4, 1}, {2, 2}}) {
-        const int nb = v.first, hpc = v.second;
+    for (const auto &v : DR_FORMS) {
+        const int nb = v[0], hpc = v[1];
         const size_t smem = dr_layout(P, nb, hpc, 227 * 1024);
         if (smem == (size_t)-1) continue;
         const int clusters = (R + 8 * nb - 1) / (8 * nb), fit = dr_max_clusters(nb, hpc, P.nc, smem);

@@ -1136,8 +1136,7 @@ int dr_max_clusters(int nb, int hpc, int nc, size_t smem) {
 
 cudaError_t decode_rows_init() {
     cudaError_t err = cudaSuccess;
-    const int v[4][2] = {{1, 1}, {2, 1}, {4, 1}, {2, 2}};
-    for (const auto &x : v)
+    for (const auto &x : DR_FORMS)
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(dr_kernel(x[0], x[1]), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     return err;

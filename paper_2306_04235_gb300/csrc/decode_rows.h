@@ -10,6 +10,7 @@ namespace mnmt {
 
 // ---- decode step of larger batches: clusters of H / hpc CTAs (hpc heads each), 8 nb rows each ----
 constexpr int DR_LMAX = 16;  // decoder layers
+constexpr int DR_FORMS[4][2] = {{1, 1}, {2, 1}, {4, 1}, {2, 2}};  // nb, hpc in the order of preference
 struct DrLin {
     const float *s, *b, *inv;  // inv: requantisation constants (or null)
     float sx, gam;             // input scale; residual gain (W_o, W_2)

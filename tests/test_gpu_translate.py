@@ -607,3 +607,30 @@ def test_queued_translations_keep_their_step_limits(beam, B, stream):
                 assert np.array_equal(a.view(np.uint32), b.cpu().numpy().view(np.uint32))
     finally:
         tr.close()
+
+
+def test_session_holds_packed_weights_only_where_the_batched_step_can_run(stream, monkeypatch):
+    """Lengths above 512, or the step switched off when the session is created:
+    no packed decoder weights in the session (and a kernel per operation)."""
+    cfg = synth.ModelConfig(1, 2, 256, 4, 1024, 300, 256, 1, 1, max_pos=600)
+    packed = cfg.n_dec * (6 * 256 * 256 + 2 * 256 * 1024)
+    model = mnmt.mnmt_load_weights(synth.build_blob(cfg, 3), stream)
+    ids, lens = synth.source_batch(cfg.vocab, 4, 8, 8, 4)
+
+    def session(T):
+        s = mnmt.mnmt_session_create(model, 4, 8, 4, T)
+        try:
+            mnmt.mnmt_encode(s, ids, lens, 4, ids.shape[1])
+            return mnmt.mnmt_session_device_bytes(s), int(mnmt.mnmt_debug_tap(s, mnmt.TAP_STEP, 0, np.int32)[0])
+        finally:
+            mnmt.mnmt_session_free(s)
+
+    try:
+        monkeypatch.setenv("MNMT_DECODE_CLUSTER", "1")
+        (with_, kind), (long_, kind_long) = session(512), session(513)
+        monkeypatch.setenv("MNMT_DECODE_CLUSTER", "0")
+        off, kind_off = session(512)
+    finally:
+        mnmt.mnmt_model_free(model)
+    assert (kind, kind_long, kind_off) == (2, 0, 0)
+    assert with_ - off >= packed and with_ - long_ > 0.9 * packed
