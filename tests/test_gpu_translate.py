@@ -526,15 +526,20 @@ def test_beam_rows_in_registers(V, beam, flat, stream):
     assert np.array_equal(g_sc.view(np.uint32), o_sc.view(np.uint32))
 
 
-@pytest.mark.parametrize("V,beam,B", [(4096, 4, 39), (8192, 5, 31), (8196, 8, 20), (20000, 16, 10), (32764, 4, 39), (32768, 3, 51)])
+@pytest.mark.parametrize("V,beam,B,lo", [(4096, 4, 39, 0), (8192, 5, 31, 0), (8196, 8, 20, 7296), (20000, 16, 10, 19100),
+                                         (32764, 4, 39, 31864), (32768, 3, 51, 15934), (32768, 4, 39, 0)])
 @pytest.mark.parametrize("flat", [False, True])
-def test_beam_rows_two_to_an_sm(V, beam, B, flat, stream):
-    """More rows than SMs: blocks of 512 threads, half of a row above 8192
-    entries in shared memory; flat: as above, ties in either half."""
+def test_beam_rows_two_to_an_sm(V, beam, B, lo, flat, stream):
+    """More rows than SMs: blocks of 512 threads, above 8192 entries those from
+    16384 on in shared memory; flat: 900 equal logits from id lo on, in either half
+    or across both (the list overflows and the row is scanned in full)."""
     cfg = synth.ModelConfig(1, 1, 64, 1, 64, V, 64, 1, 1, max_pos=32)
-    lo = V - 900 if flat and V % 8 else 0
     bias = {lo + i: 40.0 for i in range(0, 900)} if flat else None
     blob = synth.build_blob(cfg, 19, gamma_range=(0.5, 1.5), out_bias=bias)
+    if flat:  # equal logits: the tied embedding rows of the biased ids zeroed
+        b = bytearray(blob)
+        b[64 + lo * 64: 64 + (lo + 900) * 64] = bytes(900 * 64)
+        blob = bytes(b)
     ids, lens = synth.source_batch(V, B, 3, 9, 8)
     T = 5
     tr = mnmt.Translator(blob, B, ids.shape[1], beam, T, stream)
