@@ -1350,7 +1350,8 @@ int setup_rows_step(mnmt_session *s) {
         s->dr_packed = s->dr_hpc;
     }
     P.S = s->S;
-    // pageable, so staged by the time the call returns; no synchronisation: the
+    // pageable and below 64 KB, so staged by the time the call returns (checked by
+    // rewriting the source at once behind a busy stream); no synchronisation: the
     // steps are captured while the encoder runs (100 us of a new session's first step)
     CK(cudaMemcpyAsync(s->d_dr, &P, sizeof(P), cudaMemcpyHostToDevice, m->stream));
     return MNMT_OK;

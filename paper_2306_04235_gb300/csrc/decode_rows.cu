@@ -20,8 +20,10 @@
 //   * the fp32 residual lives with the CTA that owns the row: the W_o / W_2
 //     outputs go to the row's owner, which adds them, normalises and sends the
 //     codes to every CTA; exchanges are st.async stores completing on the
-//     receiver's mbarrier (two, alternating), as in the single-cluster step.
-// No cluster waits for another, so any number of clusters runs.  The
+//     receiver's mbarrier (two, alternating, armed by the receiver for the
+//     phase after next).
+// No cluster waits for another, so it would run in any number of waves; one is
+// where it is faster (route_rows_variant).  The
 // arithmetic is that of the other kernels (exact integer sums, the same fp32
 // roundings), so results are bit-identical.
 // Bound by the chain of short phases (time stamps of one step, 16 clusters of

@@ -11,7 +11,7 @@
 //                  row is streamed once with 16-byte coalesced loads, the M
 //                  activation rows sit in shared memory, products use dp4a and
 //                  a lane group's partial sums meet by warp shuffles.  Bound by
-//                  weight bytes (HBM or L2).
+//                  latency (start, loads, reduction).
 //   linear_mma     other M > 16: CTA tiles of the int8 GEMM on the warp-level
 //                  fp16 tensor-core instruction (mma.sync m16n8k16), the codes
 //                  staged as bytes and widened to fp16 in registers; cp.async
@@ -453,7 +453,7 @@ static cudaError_t launch_small_u(const int8_t *A, int lda, const int8_t *W, int
                                   cudaStream_t st) {
     constexpr int CPB = (SM_THREADS / 32) * (32 / LPC) * U;
     int blocks = (N + CPB - 1) / CPB;
-    if (blocks > 4 * 152) blocks = 4 * 152;
+    if (blocks > 4 * device_sm_count()) blocks = 4 * device_sm_count();
     const dim3 grid(blocks, (M + MT - 1) / MT);  // row chunks of MT, one per grid row
     launch_pdl(linear_smallm<MT, LPC, U>, grid, SM_THREADS, (size_t)MT * K, st, A, lda, W, M, N, K, e);
     return cudaGetLastError();
@@ -466,7 +466,7 @@ static cudaError_t launch_small_t(const int8_t *A, int lda, const int8_t *W, int
                                   cudaStream_t st) {
     constexpr int CPB2 = (SM_THREADS / 32) * (32 / LPC) * 2;
     const long blocks = (long)((N + CPB2 - 1) / CPB2) * ((M + MT - 1) / MT);
-    return blocks >= 152 ? launch_small_u<MT, LPC, 2>(A, lda, W, M, N, K, e, st)
+    return blocks >= device_sm_count() ? launch_small_u<MT, LPC, 2>(A, lda, W, M, N, K, e, st)
                          : launch_small_u<MT, LPC, 1>(A, lda, W, M, N, K, e, st);
 }
 
@@ -506,7 +506,7 @@ cudaError_t launch_linear(const int8_t *A, int lda, const int8_t *W, int M, int 
     const long tiles64 = (long)((M + 63) / 64) * ((N + 63) / 64);
     if (M <= SMALL_CHUNKED_MAX_M && K <= 2048 && tiles64 < 8) return launch_small<16>(A, lda, W, M, N, K, e, st);
     long tiles_big = (long)((M + 127) / 128) * ((N + 127) / 128);
-    if (tiles_big >= 152) return launch_mma<128, 128, 2, 4, 4>(A, lda, W, M, N, K, e, st);
+    if (tiles_big >= device_sm_count()) return launch_mma<128, 128, 2, 4, 4>(A, lda, W, M, N, K, e, st);
     return launch_mma<64, 64, 2, 2, 4>(A, lda, W, M, N, K, e, st);
 }
 

@@ -227,6 +227,9 @@ cudaError_t launch_layernorm_warp(const LnArgs &a, cudaStream_t st) {
     int kd = 0;
     while (((a.d >> kd) & 1) == 0) kd++;
     const unsigned z = (unsigned)a.d >> kd;
+    // Blocks walk over the rows; the cap bounds how many share them.  Registers let
+    // fewer be resident (2 of <4>, 1 of <6> and <8>), so the last ones of a full
+    // grid start when a first one has finished its rows.
     const int blocks = (a.M + 7) / 8, cap = device_sm_count() * (NV <= 4 ? 3 : 2);
     launch_pdl(layernorm_warp_kernel<NV>, blocks < cap ? blocks : cap, 256, 0, st, a, kd, z,
                z > 1 ? ~0ull / (unsigned long long)z : 0ull);  // floor(2^64 / z), z odd

@@ -133,13 +133,14 @@ def test_linear_tc_equals_imma_path():
 
 
 @pytest.mark.parametrize("M,N,K", [(19300, 528, 64), (9700, 1008, 1032), (4801, 2001, 512), (9600, 1024, 2048),
-                                   (2500, 512, 2048), (1301, 1000, 1032), (1501, 2000, 1032), (3100, 1008, 512)])
+                                   (4001, 2000, 64), (3000, 2048, 1024), (2500, 512, 2048),
+                                   (1301, 1000, 1032), (1501, 2000, 1032), (3100, 1008, 512)])
 @pytest.mark.parametrize("mode", [mnmt.EPI_Q8, mnmt.EPI_RELU_Q8, mnmt.EPI_RESID, mnmt.EPI_F32, mnmt.EPI_ARGMAX])
 def test_linear_tc_large_grids(M, N, K, mode):
-    """Grids of several 256x256 tiles per CTA pair, of one wave of 256x128 or 128x256 tiles,
-    ragged in M and N, with and without 16-byte rows, one and two accumulator
-    chunks: the first, last and tile-edge rows against the oracle, all rows
-    against the int8 kernel."""
+    """Grids of several 256x256 tiles per CTA pair, of one wave of 256x128 tiles, of one and
+    two waves of 128x256 tiles and of five of 128x128, ragged in M and N, with and without
+    16-byte rows, one and two accumulator chunks: the first, last and tile-edge rows
+    against the oracle, all rows against the int8 kernel."""
     A, W, s_w, b, inv, s_x = _inputs(M + 3 * N + K, M, N, K)
     gamma = np.float32(0.875)
     Kp = (K + 63) // 64 * 64  # the int8 kernel's reductions, padded with zeros

@@ -48,7 +48,7 @@ def test_lean_translation_equals_default_and_oracle(name, stream):
 @pytest.mark.parametrize("beam,B", [(3, 60), (1, 150)])
 def test_lean_batched_search_equals_oracle(beam, B, stream):
     """>= 128 decoder rows: the default session runs its linears on the tensor
-    cores, the lean one on the int8 IMMA kernels; both equal the oracle."""
+    cores, the lean one on the int8 kernels; both equal the oracle."""
     cfg = synth.ModelConfig(2, 2, 128, 4, 256, 500, 128, 1, 1, max_pos=64)
     blob = synth.build_blob(cfg, 51, gamma_range=(0.5, 1.5))
     ids, lens = synth.source_batch(cfg.vocab, B, 1, 30, 52)

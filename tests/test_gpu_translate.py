@@ -416,7 +416,7 @@ def test_tensor_core_rows_match_oracle(kind, beam, stream):
 
 def test_tensor_core_and_imma_paths_bit_identical(stream):
     """The same batched beam workload through the tcgen05 linears and through
-    the IMMA linears (MNMT_TC=0): identical outputs."""
+    the int8 linears (MNMT_TC=0): identical outputs."""
     cfg, blob, ids, lens, beam, T = synth.workload_inputs("small-b32-s10to80-beam4-t128")
     outs = []
     for on in (True, False):

@@ -39,7 +39,7 @@ def test_noalloc_argmax_equals_keyed_argmax_twice(M):
 
 @pytest.mark.parametrize("M,N,K", [(4096, 32000, 256), (3, 8000, 2048), (16, 32000, 512)])
 def test_noalloc_argmax_at_the_row_limit_and_long_k(M, N, K):
-    """The full 4096-row scratch (tensor-core / IMMA tile path), and the GEMV
+    """The full 4096-row scratch (`mma.sync` tile path), and the GEMV
     path at K = 2048: two calls in a row equal the keyed call, and sampled rows
     equal the oracle's argmax of its fp32 logits (ties to the lowest id)."""
     stream = torch.cuda.current_stream()
