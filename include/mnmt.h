@@ -141,9 +141,9 @@ void mnmt_session_free(mnmt_session *s);
  * state and, where the batched decode step can run -- pre-LN, head width 64, 2 to
  * 8 heads and an even number, no min-max rows, beams or more than 4 sentences,
  * lengths up to 512, not lean -- the decoder's weights as that step reads them,
- * n_dec (6 d^2 + 2 d F) bytes, packed at the first decode).  Nothing else is allocated on the device by the library after these
- * objects are created, so model + session bytes are the library's peak device
- * memory for a translation.  Negative MNMT_EINVAL for a null handle. */
+ * n_dec (6 d^2 + 2 d F) bytes, packed at the first decode).  Nothing else is
+ * allocated on the device by the library after these objects are created, so
+ * model + session bytes are the library's peak device memory for a translation.  Negative MNMT_EINVAL for a null handle. */
 int64_t mnmt_model_device_bytes(const mnmt_model *model);
 int64_t mnmt_session_device_bytes(const mnmt_session *s);
 
